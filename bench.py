@@ -222,6 +222,44 @@ def run_reference(args, inst, rank, world):
     print(json.dumps(line), flush=True)
 
 
+def contract_flops(m, n, n_a=0):
+    """(algorithmic, issued) operations of the bit-row contraction: 2 m per reported pair, and
+    the 128 x 240 tiles that hold one over the padded K (the first tile of a 256-row block runs
+    whenever the block does)."""
+    bm, bn, tiles = 128, 240, 0
+    for c0 in range(n_a, n, bn):
+        clim = min(c0 + bn, n)
+        for r0 in range(0, n_a or n, 2 * bm):
+            if n_a:
+                tiles += 1 + (r0 + bm < n_a)
+            elif r0 + 1 < clim:
+                tiles += 1 + (r0 + bm + 1 < clim)
+    npairs = n_a * (n - n_a) if n_a else n * (n - 1) // 2
+    return 2.0 * npairs * m, 2.0 * tiles * bm * bn * ((m + 255) // 256 * 256)
+
+
+def contract_roofline(m, n, n_a, seconds, peaks, peak_kind, traffic):
+    alg, issued = contract_flops(m, n, n_a)
+    # fp4 dense peak: the measured bf16 peak x the nominal fp4 / bf16 ratio (13.5 / 2.25)
+    peak = 6.0 * peaks.get("bf16_tflops", 1900.0)
+    return {"bound": "tensor", "achieved": alg / seconds / 1e12, "peak": peak, "unit": "TFLOP/s",
+            "frac": alg / seconds / 1e12 / peak, "kernel": "k_contract", "traffic": traffic,
+            "peak_kind": f"fp4 dense = 6 x {peak_kind} bf16 burst (nominal 13.5/2.25 ratio)",
+            "algorithmic_flops": "2 m per reported pair",
+            "issued_definition": "128 x 240 tiles that hold a reported pair, over the padded K",
+            "issued_TFLOPs": issued / seconds / 1e12, "issued_frac": issued / seconds / 1e12 / peak}
+
+
+def scan_roofline(wp_scan, scan_s, alu_peak, sms, peaks, peak_kind, traffic):
+    achieved = OPS_PER_WORD_PAIR * wp_scan / scan_s / 1e12
+    return {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s",
+            "frac": achieved / alu_peak, "kernel": "k_compare", "traffic": traffic,
+            "peak_kind": f"{sms} SMs x 128 INT32 lanes x {peaks.get('sm_max_mhz', 2070.0):.0f} MHz "
+                         f"({peak_kind} max clock)",
+            "algorithmic_ops": f"{OPS_PER_WORD_PAIR} x {wp_scan:.4g} word pairs (the scan-routed pairs' "
+                               f"max(|B_i|,|B_j|)/4) per scan time {1e3 * scan_s:.3f} ms"}
+
+
 def dense_leg(args, inst, off, tids, n_out_ref, peaks, peak_kind, steps=None, warmup=None, workload=None):
     """The dense-bitmap tensor-core comparison path on the same workload."""
     import torch
@@ -245,31 +283,11 @@ def dense_leg(args, inst, off, tids, n_out_ref, peaks, peak_kind, steps=None, wa
     torch.cuda.synchronize()
     assert k == n_out_ref, (k, n_out_ref)
     elapsed = ev0.elapsed_time(ev1) / 1e3
-    # tensor work actually issued: 128 x 240 tiles that hold a pair i < j, over the padded K (the
-    # first tile of a 256-row block runs whenever the block does)
-    n, bm, bn = inst.n, 128, 240
-    tiles = 0
-    for c0 in range(0, n, bn):
-        clim = min(c0 + bn, n)
-        for r0 in range(0, n, 2 * bm):
-            if r0 + 1 < clim:
-                tiles += 1 + (r0 + bm + 1 < clim)
-    kpad = (inst.m + 255) // 256 * 256
-    flops_issued = 2.0 * tiles * bm * bn * kpad
-    flops_alg = 2.0 * npairs * inst.m  # 2 m per pair i < j
     g = statistics.mean(gemm) / 1e3
-    # fp4 dense peak: the measured bf16 peak x the nominal fp4 / bf16 ratio (13.5 / 2.25)
-    peak = 6.0 * peaks.get("bf16_tflops", 1900.0)
     return {"value": npairs * steps / elapsed, "unit": UNIT, "ms_per_step": 1e3 * elapsed / steps,
             "phases_ms": {"bitmap": statistics.mean(build), "tensor_kernel": statistics.mean(gemm)},
-            "roofline": {"bound": "tensor", "achieved": flops_alg / g / 1e12, "peak": peak, "unit": "TFLOP/s",
-                         "frac": flops_alg / g / 1e12 / peak, "kernel": "k_contract",
-                         "traffic": _traffic(workload or args.workload, "k_contract", "dense.cu"),
-                         "peak_kind": f"fp4 dense = 6 x {peak_kind} bf16 burst (nominal 13.5/2.25 ratio)",
-                         "algorithmic_flops": "2 m n(n-1)/2 (pairs i < j only)",
-                         "issued_definition": "128 x 240 tiles that hold a pair i < j, over the padded K",
-                         "issued_TFLOPs": flops_issued / g / 1e12,
-                         "issued_frac": flops_issued / g / 1e12 / peak},
+            "roofline": contract_roofline(inst.m, inst.n, 0, g, peaks, peak_kind,
+                                          _traffic(workload or args.workload, "k_contract", "dense.cu")),
             "dtype": "e2m1 {0,1} operands, fp32 accumulate (exact integers <= 2^24)"}
 
 
@@ -352,7 +370,10 @@ def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None
     wp_probe = info["probe_word_pairs"]
     wp_scan = wp - wp_probe
     alu_peak, sms = _alu_peak(dev, peaks)
-    achieved = OPS_PER_WORD_PAIR * wp_scan / scan_s / 1e12
+    contract = scan_s == 0.0  # the supports came from the bit rows, not from a BatMap route
+    roofline = (contract_roofline(inst.m, inst.n, 0, cmp_s, peaks, peak_kind,
+                                  _traffic(workload, "k_contract", "dense.cu")) if contract else
+                scan_roofline(wp_scan, scan_s, alu_peak, sms, peaks, peak_kind, _traffic(workload)))
     logical_gbs = 8.0 * wp / cmp_s / 1e9
     rec = {
         "value": npairs * steps / elapsed, "unit": UNIT, "steps": steps, "warmup": warmup,
@@ -360,13 +381,7 @@ def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None
         "config": {"workload": workload, "desc": _desc(workload), "m": inst.m, "n": inst.n,
                    "s": inst.s, "pairs": npairs, "tids": int(inst.tids.size), "batmap_bytes": info["bytes"],
                    "width_classes": info["n_classes"], "l2": "inputs larger than L2 (no flush)"},
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s",
-                     "frac": achieved / alu_peak, "kernel": "k_compare",
-                     "traffic": _traffic(workload),
-                     "peak_kind": f"{sms} SMs x 128 INT32 lanes x {peaks.get('sm_max_mhz', 2070.0):.0f} MHz "
-                                  f"({peak_kind} max clock)",
-                     "algorithmic_ops": f"{OPS_PER_WORD_PAIR} x {wp_scan:.4g} word pairs (the scan-routed pairs' "
-                                        f"max(|B_i|,|B_j|)/4) per scan time {1e3 * scan_s:.3f} ms"},
+        "roofline": roofline,
         "logical_hbm": {"achieved_GBps": logical_gbs, "peak_GBps": peaks["hbm_gbs"],
                         "frac": logical_gbs / peaks["hbm_gbs"],
                         "definition": "sum over pairs of 2*max(|B_i|,|B_j|) bytes / compare time (Sec. IV-A)"},
@@ -377,7 +392,7 @@ def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None
         "frequent_pairs": n_out, "failed_insertions": info["n_failed"], "gpu_launches": int(launches),
         "clocks": clocks,
     }
-    if wp_probe > 0:
+    if wp_probe > 0 and not contract:
         probe_s = statistics.mean(probe_ms) / 1e3
         rec["compare_equiv"] = {
             "frac": OPS_PER_WORD_PAIR * wp / cmp_s / 1e12 / alu_peak,
@@ -708,7 +723,9 @@ def run_cross(args):
     wp_scan = info["word_pairs"] - info["probe_word_pairs"]
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     alu_peak = sms * 128 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
-    achieved = OPS_PER_WORD_PAIR * wp_scan / scan_s / 1e12
+    roofline = (contract_roofline(union.m, union.n, na, statistics.mean(t["compare_ms"] for t in phases) / 1e3, peaks,
+                                  peak_kind, None) if scan_s == 0.0 else
+                scan_roofline(wp_scan, scan_s, alu_peak, sms, peaks, peak_kind, None))
     line = {"metric": "A x B pair supports/sec (sparse boolean matrix multiplication), bit-exact",
             "workload": "cross", "unit": UNIT, "value": npairs * args.steps / elapsed, "n_gpus": 1,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * elapsed / args.steps,
@@ -717,12 +734,7 @@ def run_cross(args):
                        "desc": "A: Zipf(1) sizes at mean density 1%; B: Bernoulli p=0.002",
                        "tids": int(union.tids.size), "batmap_bytes": int(info["bytes"]),
                        "l2": "inputs larger than L2 (no flush)"},
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s",
-                         "frac": achieved / alu_peak, "kernel": "k_compare", "traffic": None,
-                         "peak_kind": f"{sms} SMs x 128 INT32 lanes x {peaks.get('sm_max_mhz', 2070.0):.0f} MHz "
-                                      f"({peak_kind} max clock)",
-                         "algorithmic_ops": f"{OPS_PER_WORD_PAIR} x {wp_scan:.4g} word pairs (the scan-routed pairs' "
-                                        f"max(|B_i|,|B_j|)/4) per scan time {1e3 * scan_s:.3f} ms"},
+            "roofline": roofline,
             "phases_ms": {p: statistics.mean(t[p] for t in phases)
                           for p in ("build_ms", "compare_ms", "scan_ms", "probe_ms", "compact_ms")},
             "probe_routed_share": info["probe_word_pairs"] / max(info["word_pairs"], 1.0),

@@ -132,7 +132,8 @@ typedef struct batmap_info {
     double word_pairs;       /* sum over reported pairs of max(|B_i|,|B_j|)/4  */
     uint32_t d;              /* copies per element: 2 (2-of-3) or 3 (3-of-4)   */
     uint32_t reserved;
-    double probe_word_pairs; /* part of word_pairs counted by the probe route  */
+    double probe_word_pairs; /* part of word_pairs that the BatMap schedule
+                                gives to the probe route                       */
     double probe_words;      /* words the probe route reads: sum over probe-
                                 routed pairs of min(|B_i|,|B_j|)/4             */
 } batmap_info;
@@ -295,10 +296,15 @@ batmap_status batmap_export_layout(const batmap_set *set, uint8_t *h_bytes,
 
 /*
  * Support of every item pair and the frequent pairs (Sec. I problem
- * statement; Sec. III-B/C all-pairs comparison, failure correction).  Pairs
- * of similar width run the cyclic scan; pairs whose widths differ by
- * 2^probe_log or more run the probe route (batmap_params.probe_log); both
- * count the same slot pairs.
+ * statement; Sec. III-B/C all-pairs comparison, failure correction).  Two
+ * routes give the same supports; the build picks the one it estimates faster:
+ *   - the contraction of the family's bit rows (Sec. I-B), which the build then
+ *     keeps beside the BatMaps (n * ceil(m / 256) * 32 bytes), on the tensor
+ *     cores.  Taken only with tile, shape_mask and probe_log left at 0, and
+ *     only if the bit rows fit in half of the free memory;
+ *   - the BatMaps: pairs of similar width run the cyclic scan, pairs whose
+ *     widths differ by 2^probe_log or more the probe route
+ *     (batmap_params.probe_log); both count the same slot pairs.
  *   s       : support threshold; pairs with support >= s are reported.
  *   d_pairs : device uint32[3*cap]: triples (i, j, support) with original
  *             item ids i < j, in lexicographic (i, j) order.  May be NULL
@@ -355,11 +361,12 @@ typedef struct batmap_timing {
     float build_ms;     /* whole batmap_build, first to last enqueued operation */
     float place_ms;     /* 2-of-3 placement kernel                              */
     float finalize_ms;  /* byte writing + failure lists + correction entries    */
-    float compare_ms;   /* the all-pairs compare: scan and probe kernels        */
+    float compare_ms;   /* the all-pairs compare: contraction, or scan and probe */
     float compact_ms;   /* failure correction + threshold compaction            */
     float pairs_ms;     /* whole pair_support_all                               */
     float scan_ms;      /* frequent_triples / _quadruples: the witness scan;
-                           pair_support_all: the cyclic-scan compare kernels    */
+                           pair_support_all: the cyclic-scan compare kernels (0
+                           when the supports came from the bit rows)            */
     float probe_ms;     /* frequent_triples / _quadruples and pair_support_all:
                            the probe kernel of width-skewed tuples              */
 } batmap_timing;
@@ -368,7 +375,8 @@ typedef struct batmap_timing {
 batmap_status batmap_get_timing(const batmap_set *set, batmap_timing *t);
 
 /* Release the scratch the library caches between calls (the placement table
- * of batmap_build, one uint32 per BatMap byte; the dense path's bitmap and
+ * of batmap_build, one uint32 per BatMap byte; at most six arrays of freed
+ * sets; the dense path's bitmap and
  * workspace; pair_support_host's device copies of its inputs and output).
  * Call when no other call of the library is running. */
 void batmap_release_scratch(void);
@@ -387,16 +395,16 @@ typedef struct batmap_out {
 
 /*
  * Many independent mining instances in one pass: the compare work of all k
- * sets runs in ONE persistent launch that pulls (instance, tile, k-range)
- * units from a shared queue, followed by the per-instance correction and
+ * sets runs in ONE persistent launch per route that pulls (instance, tile,
+ * k-range) units from a shared queue, followed by the per-instance correction and
  * compaction.  Results equal k separate pair_support_all calls.
  *   sets : k built handles.   s : host uint32[k] thresholds.
  *   outs : host batmap_out[k]; n_out is filled in for each instance.
  * Returns BATMAP_ERR_CAPACITY if any instance overflowed its buffer (that
  * instance's first cap triples are written).  Synchronises the stream.
  * Afterwards batmap_get_timing of every set of the batch reports the batched
- * pass: compare_ms = the one compare launch over all instances (the span of
- * its CTAs on the GPU's global timer), pairs_ms = the whole pass (events
+ * pass: compare_ms = the compare launches over all instances (the span of
+ * their CTAs on the GPU's global timer), pairs_ms = the whole pass (events
  * around it), compact_ms = the rest (zeroing, corrections, compactions).
  */
 batmap_status pair_support_batch(batmap_set *const *sets, const uint32_t *s, uint32_t k,
@@ -483,15 +491,15 @@ batmap_status batmap_serve(const batmap_pool *pool, const uint32_t *h_qoff, cons
  * m*n bits, where a support is AND + popcount).  Builds the item x transaction
  * bit matrix (packed, one bit per pair) and computes all supports as the dense
  * contraction M M^T on the tensor cores: each K step's bits are expanded to
- * e4m3 {0, 1} bytes in shared memory and multiplied with tcgen05
- * kind::f8f6f4 (FP32 accumulation in tensor memory, exact because every
- * product is 0 or 1 and every partial sum an integer below 2^24), then the
- * same threshold compaction as pair_support_all.
+ * e2m1 {0, 1} nibbles in shared memory and multiplied with tcgen05
+ * kind::mxf4 under unit block scales (FP32 accumulation in tensor memory, exact
+ * because every product is 0 or 1 and every partial sum an integer of at most
+ * 2^24), then the same threshold compaction as pair_support_all.
  *   m, n, d_offsets, d_tids : CSR tidlists as in batmap_build (1 <= m <= 2^24).
  *   s, d_pairs, cap, n_out, d_full : as in pair_support_all.
  *   timing  : optional host struct; build_ms = bitmap build, compare_ms = the
  *             tensor-core kernel, compact_ms = compaction.
- * The bit matrix (n rows of ceil(m/128)*128 bits) and scratch are cached
+ * The bit matrix (n rows of ceil(m/256)*256 bits) and scratch are cached
  * inside the library between calls.  Synchronises the stream.
  */
 batmap_status pair_support_dense(uint32_t m, uint32_t n, const uint64_t *d_offsets, const uint32_t *d_tids,

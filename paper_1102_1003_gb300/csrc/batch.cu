@@ -10,6 +10,7 @@
 #include <mutex>
 #include <string>
 
+#include "bits.cuh"
 #include "common.cuh"
 #include "compare.cuh"
 
@@ -24,7 +25,10 @@ struct BatchPlan {
     std::vector<uint32_t *> C;
     DevBuf<InstView> d_views;
     DevBuf<WorkUnit> d_units;
-    DevBuf<uint32_t> d_counter;
+    DevBuf<uint32_t> d_counter;           // COMPARE_COUNTERS, then the contraction's counter and flag
+    DevBuf<MmView> d_mviews;              // instances whose supports come from their bit rows
+    DevBuf<MmUnit> d_munits;
+    std::vector<char> zero;               // per instance: its supports are added into
     DevBuf<uint64_t> d_totals;
     UnitParts parts;
     cudaStream_t stream = nullptr;
@@ -60,12 +64,14 @@ static void enqueue_batch(BatchPlan *P, batmap_set *const *sets, const uint32_t 
                           const batmap_out *outs, cudaStream_t st) {
     for (uint32_t q = 0; q < k; q++) {
         const uint64_t np = sets[q]->npairs();
-        if (np) BM_CUDA(cudaMemsetAsync(P->C[q], 0, np * sizeof(uint32_t), st));
+        if (np && P->zero[q]) BM_CUDA(cudaMemsetAsync(P->C[q], 0, np * sizeof(uint32_t), st));
     }
-    BM_CUDA(cudaMemsetAsync(P->d_counter.p, 0, COMPARE_COUNTERS * sizeof(uint32_t), st));
+    BM_CUDA(cudaMemsetAsync(P->d_counter.p, 0, (COMPARE_COUNTERS + 2) * sizeof(uint32_t), st));
     BM_CUDA(cudaMemsetAsync(P->d_stamps.p, 0xFF, sizeof(unsigned long long), st));
     BM_CUDA(cudaMemsetAsync(P->d_stamps.p + 1, 0, sizeof(unsigned long long), st));
     launch_compare(P->d_views.p, P->d_units.p, P->parts, P->d_counter.p, st, P->d_stamps.p);
+    launch_contract(P->d_mviews.p, MmView{}, P->d_munits.p, (uint32_t)P->d_munits.n, P->d_counter.p + COMPARE_COUNTERS,
+                    st, P->d_stamps.p);
     for (uint32_t q = 0; q < k; q++)
         enqueue_correct_compact(sets[q], P->C[q], s[q], outs[q].d_pairs, outs[q].cap, P->d_totals.p + q, st);
 }
@@ -78,6 +84,12 @@ static BatchPlan *make_plan(batmap_set *const *sets, const uint32_t *s, uint32_t
     std::vector<InstView> views(k);
     std::vector<WorkUnit> units;
     P->C.resize(k);
+    P->zero.assign(k, 1);
+    std::vector<MmView> mviews;
+    std::vector<MmUnit> munits;
+    double mm_total = 0.0;  // seconds of all contractions, each alone
+    for (uint32_t q = 0; q < k; q++)
+        if (sets[q]->contract) mm_total += contract_seconds(sets[q]->n, sets[q]->n_a, sets[q]->kblocks);
     for (uint32_t q = 0; q < k; q++) {
         batmap_set *S = sets[q];
         uint32_t *C = outs[q].d_full;
@@ -88,9 +100,15 @@ static BatchPlan *make_plan(batmap_set *const *sets, const uint32_t *s, uint32_t
         P->C[q] = C;
         views[q] = InstView{reinterpret_cast<const uint4 *>(S->d_bm.p), S->d_line_off.p, S->d_wshift.p,
                             S->d_order.p, C, S->n, S->n_a, S->shift};
-        for (WorkUnit u : S->units) {
-            u.inst = q;
-            units.push_back(u);
+        if (S->contract) {
+            const double own = contract_seconds(S->n, S->n_a, S->kblocks);
+            P->zero[q] = contract_units(S->n, S->n_a, S->kblocks, (uint32_t)mviews.size(), mm_total - own, &munits);
+            mviews.push_back(contract_view(S, C));
+        } else {
+            for (WorkUnit u : S->units) {
+                u.inst = q;
+                units.push_back(u);
+            }
         }
         prepare_compaction(S);
     }
@@ -98,7 +116,15 @@ static BatchPlan *make_plan(batmap_set *const *sets, const uint32_t *s, uint32_t
     P->parts = unit_parts(units);
     P->d_views.alloc(k);
     P->d_units.alloc(units.size());
-    P->d_counter.alloc(COMPARE_COUNTERS);
+    P->d_counter.alloc(COMPARE_COUNTERS + 2);
+    std::stable_sort(munits.begin(), munits.end(),
+                     [](const MmUnit &a, const MmUnit &b) { return a.kb1 - a.kb0 > b.kb1 - b.kb0; });
+    P->d_mviews.alloc(mviews.size());
+    P->d_munits.alloc(munits.size());
+    if (!munits.empty()) {
+        BM_CUDA(cudaMemcpyAsync(P->d_mviews.p, mviews.data(), mviews.size() * sizeof(MmView), cudaMemcpyHostToDevice, st));
+        BM_CUDA(cudaMemcpyAsync(P->d_munits.p, munits.data(), munits.size() * sizeof(MmUnit), cudaMemcpyHostToDevice, st));
+    }
     P->d_totals.alloc(k);
     P->d_stamps.alloc(2);
     BM_CUDA(cudaMemcpyAsync(P->d_views.p, views.data(), k * sizeof(InstView), cudaMemcpyHostToDevice, st));
@@ -107,6 +133,7 @@ static BatchPlan *make_plan(batmap_set *const *sets, const uint32_t *s, uint32_t
                                 cudaMemcpyHostToDevice, st));
     BM_CUDA(cudaStreamSynchronize(st));
     prepare_compare();
+    prepare_contract();
     P->ev.create();
 
     // capture the whole batch (zeroing, one compare launch, k compactions)
@@ -155,9 +182,12 @@ void run_batch(batmap_set *const *sets, const uint32_t *s, uint32_t k, batmap_ou
     P->ev.record(1, st);
     std::vector<uint64_t> totals(k);
     unsigned long long stamps[2] = {0, 0};
+    uint32_t mm_state[2] = {0, 0};
+    BM_CUDA(cudaMemcpyAsync(mm_state, P->d_counter.p + COMPARE_COUNTERS, sizeof(mm_state), cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaMemcpyAsync(totals.data(), P->d_totals.p, k * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaMemcpyAsync(stamps, P->d_stamps.p, sizeof(stamps), cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaStreamSynchronize(st));
+    BM_REQUIRE(!mm_state[1], BATMAP_ERR_TIMEOUT, "tensor-core kernel: a bounded pipeline wait timed out");
     // every set of the batch reports the batched pass: the one compare launch
     // over all instances (its CTAs' globaltimer span) and the rest of the pass
     // (zeroing, corrections, compactions)

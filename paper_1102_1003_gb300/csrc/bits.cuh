@@ -52,9 +52,18 @@ double contract_seconds(uint32_t n, uint32_t n_a, uint32_t kblocks);
 bool contract_units(uint32_t n, uint32_t n_a, uint32_t kblocks, uint32_t inst, double others,
                     std::vector<MmUnit> *out);
 void prepare_contract();  // kernel attributes (before stream capture)
-// One persistent launch over the units (longest first).  d_state: two zeroed
-// words, [0] the queue counter, [1] <- 1 if a bounded wait gave up.
-void launch_contract(const MmView *d_views, const MmUnit *d_units, uint32_t count, uint32_t *d_state,
-                     cudaStream_t st, unsigned long long *d_stamps = nullptr, uint32_t test_spin = 0);
+// One persistent launch over the units (longest first), of the instances at
+// d_views or, if that is NULL, of `one`.  d_state: two zeroed words, [0] the
+// queue counter, [1] <- 1 if a bounded wait gave up.
+void launch_contract(const MmView *d_views, const MmView &one, const MmUnit *d_units, uint32_t count,
+                     uint32_t *d_state, cudaStream_t st, unsigned long long *d_stamps = nullptr,
+                     uint32_t test_spin = 0);
+
+// Decides whether a set's pair supports come from its bit rows; if so, allocates
+// them and enqueues their build (d_flags as in enqueue_bits) and the units.
+void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids, int *d_flags, bool sorted_only);
+// Supports of all pairs of a set planned that way into C.
+void enqueue_contract(batmap_set *S, uint32_t *C, cudaStream_t st);
+MmView contract_view(const batmap_set *S, uint32_t *C);
 
 }  // namespace bm

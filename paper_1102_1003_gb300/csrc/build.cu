@@ -14,6 +14,7 @@
 #include <mutex>
 #include <numeric>
 
+#include "bits.cuh"
 #include "common.cuh"
 #include "items.cuh"
 #include "perm.cuh"
@@ -325,7 +326,10 @@ struct CachedBuf {
     size_t cap;
 };
 std::mutex g_bm_cache_mu;
-std::vector<CachedBuf> g_bm_cache;  // at most two, oldest first
+std::vector<CachedBuf> g_bm_cache;  // at most BM_CACHE, oldest first
+// A set holds a BatMap array, bit rows and the units of the contraction; a level of itemset mining
+// frees two sets.
+constexpr size_t BM_CACHE = 6;
 }  // namespace
 
 uint8_t *bm_buffer_take(size_t bytes, size_t *capacity) {
@@ -354,7 +358,7 @@ void bm_buffer_give(uint8_t *p, size_t capacity) {
     cudaDeviceSynchronize();
     std::lock_guard<std::mutex> lock(g_bm_cache_mu);
     g_bm_cache.push_back({p, capacity});
-    if (g_bm_cache.size() > 2) {
+    if (g_bm_cache.size() > BM_CACHE) {
         cudaFree(g_bm_cache.front().p);
         g_bm_cache.erase(g_bm_cache.begin());
     }
@@ -491,23 +495,27 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     BM_CUDA(cudaMemcpyAsync(d_base.p, base.data(), n * 8ull, cudaMemcpyHostToDevice, st));
     ItemView v{d_offsets, d_tids, d_base.p, d_rlog.p, d_ch_item.p, d_ch_start.p};
 
-    // ---- validation ----
+    // ---- bit rows (where the pair supports come from them) and validation ----
+    DevBuf<int> d_err(4);  // [0] a bad list or permutation, [2], [3] the bit rows' flags
+    BM_CUDA(cudaMemsetAsync(d_err.p, 0, 4 * sizeof(int), st));
+    plan_contract(S, d_offsets, d_tids, d_err.p + 2, P.validate != 0);
     if (P.validate) {
-        DevBuf<int> d_err(1);
         DevBuf<uint32_t> d_bits(d_perm ? 3ull * ((m + 31) / 32) : 0);
-        BM_CUDA(cudaMemsetAsync(d_err.p, 0, sizeof(int), st));
         if (d_perm) BM_CUDA(cudaMemsetAsync(d_bits.p, 0, d_bits.bytes(), st));
-        k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_err.p);
-        BM_CHECK_LAUNCH();
+        if (!S->contract) {  // the bit rows' build checks every list
+            k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_err.p);
+            BM_CHECK_LAUNCH();
+        }
         if (d_perm) {  // computed permutations are bijections by construction
             k_validate_perm<<<grid_for(3ull * m), 256, 0, st>>>(d_perm, m, 3, d_bits.p, d_err.p);
             BM_CHECK_LAUNCH();
         }
-        int err = 0;
-        BM_CUDA(cudaMemcpyAsync(&err, d_err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        int err[4] = {0, 0, 0, 0};
+        BM_CUDA(cudaMemcpyAsync(err, d_err.p, sizeof(err), cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
-        BM_REQUIRE(err != 1, BATMAP_ERR_ARG, "tids must be strictly increasing per item and < m");
-        BM_REQUIRE(err != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
+        BM_REQUIRE(err[0] != 1 && !err[2] && !err[3], BATMAP_ERR_ARG,
+                   "tids must be strictly increasing per item and < m");
+        BM_REQUIRE(err[0] != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
     }
 
     // ---- place + finalize ----
@@ -586,7 +594,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     }
 
     E.record(4, st);
-    if (!S->skip_schedule) build_schedule(S);
+    if (!S->skip_schedule && !S->contract) build_schedule(S);
     E.record(1, st);
     BM_CUDA(cudaStreamSynchronize(st));
     S->timing.build_ms = E.ms(0, 1);

@@ -6,6 +6,7 @@
 #include <new>
 #include <string>
 
+#include "bits.cuh"
 #include "common.cuh"
 #include "compare.cuh"
 
@@ -194,6 +195,7 @@ batmap_status batmap_get_info(const batmap_set *S, batmap_info *info) {
     return guarded([&] {
         BM_REQUIRE(S && info, BATMAP_ERR_ARG, "NULL argument");
         std::memset(info, 0, sizeof(*info));
+        if (S->contract && S->units.empty()) host_schedule(const_cast<batmap_set *>(S));
         info->m = S->m;
         info->n = S->n;
         info->shift = S->shift;
@@ -245,23 +247,32 @@ static void pair_support_impl(batmap_set *S, uint32_t s, uint32_t *d_pairs, uint
         S->d_C.ensure(npairs);
         C = S->d_C.p;
     }
-    static thread_local InstView h_view;
-    h_view = InstView{reinterpret_cast<const uint4 *>(S->d_bm.p), S->d_line_off.p, S->d_wshift.p,
-                      S->d_order.p, C, S->n, S->n_a, S->shift};
     S->d_total.ensure(1);
-    S->d_view.ensure(1);
     S->pairs_ev.create();
     S->pairs_ev.record(0, st);
-    BM_CUDA(cudaMemcpyAsync(S->d_view.p, &h_view, sizeof(InstView), cudaMemcpyHostToDevice, st));
-    enqueue_compare(S, C, S->d_view.p, st);  // records events 1, 2 around the launch
+    if (S->contract) {
+        S->pairs_ev.record(1, st);
+        enqueue_contract(S, C, st);
+        S->pairs_ev.record(2, st);
+    } else {
+        static thread_local InstView h_view;
+        h_view = InstView{reinterpret_cast<const uint4 *>(S->d_bm.p), S->d_line_off.p, S->d_wshift.p,
+                          S->d_order.p, C, S->n, S->n_a, S->shift};
+        S->d_view.ensure(1);
+        BM_CUDA(cudaMemcpyAsync(S->d_view.p, &h_view, sizeof(InstView), cudaMemcpyHostToDevice, st));
+        enqueue_compare(S, C, S->d_view.p, st);  // records events 1, 2 around the launch
+    }
     enqueue_correct_compact(S, C, s, d_pairs, cap, S->d_total.p, st);
     S->pairs_ev.record(3, st);
     uint64_t total = 0;
+    uint32_t state[2] = {0, 0};
     BM_CUDA(cudaMemcpyAsync(&total, S->d_total.p, 8, cudaMemcpyDeviceToHost, st));
+    if (S->contract) BM_CUDA(cudaMemcpyAsync(state, S->d_mm.p, sizeof(state), cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaStreamSynchronize(st));
+    BM_REQUIRE(!state[1], BATMAP_ERR_TIMEOUT, "tensor-core kernel: a bounded pipeline wait timed out");
     S->timing.compare_ms = S->pairs_ev.ms(1, 2);
-    S->timing.scan_ms = S->pairs_ev.ms(1, 4);
-    S->timing.probe_ms = S->pairs_ev.ms(4, 2);
+    S->timing.scan_ms = S->contract ? 0.f : S->pairs_ev.ms(1, 4);
+    S->timing.probe_ms = S->contract ? 0.f : S->pairs_ev.ms(4, 2);
     S->timing.compact_ms = S->pairs_ev.ms(2, 3);
     S->timing.pairs_ms = S->pairs_ev.ms(0, 3);
     *n_out = total;

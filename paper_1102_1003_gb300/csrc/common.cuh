@@ -73,9 +73,9 @@ struct DevBuf {
     size_t bytes() const { return n * sizeof(T); }
 };
 
-// The BatMap array of a built set comes from a small cache: a freed set's
-// array (after a device synchronisation, as cudaFree would do) is kept for the
-// next build, at most two arrays, reused when no larger than twice the request
+// The large arrays of a built set come from a small cache: a freed set's
+// arrays (after a device synchronisation, as cudaFree would do) are kept for the
+// next build, at most six, reused when no larger than twice the request
 // plus 64 MiB, so repeated builds do not map and unmap hundreds of MB each.
 uint8_t *bm_buffer_take(size_t bytes, size_t *capacity);
 void bm_buffer_give(uint8_t *p, size_t capacity);
@@ -203,10 +203,15 @@ struct batmap_set {
     std::vector<uint64_t> byte_off;       // byte offset of BatMap, sorted order
     std::vector<uint32_t> wshift_sorted;  // e per sorted position
     std::vector<uint32_t> class_begin;    // sorted positions where a width class starts (+ n)
-    std::vector<bm::WorkUnit> units;      // compare schedule, longest first
+    std::vector<bm::WorkUnit> units;      // compare schedule, longest first (contract: made when asked for)
 
     // device data
     bm::BmBuf d_bm;                       // all BatMaps, width-sorted order
+    bool contract = false;                // pair supports by the contraction of bit rows (dense.cu)
+    bool mm_add = false;                  // its units add into zeroed supports
+    uint32_t mm_count = 0, kblocks = 0;
+    bm::BmBuf d_bits;                     // bit rows, original item order
+    bm::BmBuf d_mm;                       // queue counter and timeout flag (64 bytes), then the units
     bm::DevBuf<uint32_t> d_line_off;      // [n] sorted
     bm::DevBuf<uint32_t> d_wshift;        // [n] sorted
     bm::DevBuf<uint32_t> d_order;         // [n]

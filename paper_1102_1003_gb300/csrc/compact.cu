@@ -87,7 +87,7 @@ void enqueue_correct_compact(batmap_set *S, uint32_t *C, uint32_t s, uint32_t *d
                              uint64_t *d_total, cudaStream_t st) {
     const uint64_t n = S->n;
     const uint64_t npairs = S->npairs();
-    if (S->n_corr) {
+    if (S->n_corr && !S->contract) {  // the contraction counts every element
         uint64_t g = std::min<uint64_t>((S->n_corr + 255) / 256, 1u << 16);
         k_apply_corrections<<<(unsigned)g, 256, 0, st>>>(S->d_corr.p, S->n_corr, n, S->n_a, C);
         BM_CHECK_LAUNCH();

@@ -1030,12 +1030,16 @@ static void probe_stats(const batmap_set *S, const std::vector<WorkUnit> &units,
 
 bool tuned_shape_eff(double *eff);  // batch.cu
 
-void build_schedule(batmap_set *S) {
+void host_schedule(batmap_set *S) {
     S->units.clear();
     double eff[NUM_SHAPES];
     const bool tuned = tuned_shape_eff(eff);
     schedule_units(S, S->params.tile, tuned ? eff : nullptr, 0.0, &S->units);
     probe_stats(S, S->units, &S->probe_word_pairs, &S->probe_words);
+}
+
+void build_schedule(batmap_set *S) {
+    host_schedule(S);
     S->d_units.alloc(S->units.size());
     if (!S->units.empty())
         BM_CUDA(cudaMemcpyAsync(S->d_units.p, S->units.data(), S->units.size() * sizeof(WorkUnit),

@@ -27,6 +27,7 @@ int device_sms();
 // throughput of each shape (autotuner); `force_shape` (1..NUM_SHAPES) pins
 // one shape; target_cost <= 0 picks about 32 units per SM.
 void build_schedule(batmap_set *S);
+void host_schedule(batmap_set *S);  // the units without their upload
 void schedule_units(const batmap_set *S, uint32_t force_shape, const double *shape_eff,
                     double target_cost, std::vector<WorkUnit> *out);
 

@@ -151,7 +151,7 @@ __device__ __forceinline__ uint64_t global_ns() {
 
 // Persistent: one CTA per SM pulls units until the queue is empty.
 __global__ void __launch_bounds__(THREADS, 1)
-k_contract(const MmView *__restrict__ views, const MmUnit *__restrict__ units, uint32_t count,
+k_contract(const MmView *__restrict__ views, const MmView one, const MmUnit *__restrict__ units, uint32_t count,
            uint32_t *__restrict__ state, uint32_t spin, uint32_t no_loads, unsigned long long *stamps) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -199,7 +199,7 @@ k_contract(const MmView *__restrict__ views, const MmUnit *__restrict__ units, u
     uint32_t step0 = 0, round = 0;  // K steps and units done: the rings' and the accumulators' phases
     for (uint32_t u = s_unit; u < count; round++) {
         const MmUnit U = units[u];
-        const MmView V = views[U.inst];
+        const MmView V = views ? views[U.inst] : one;
         const uint32_t nk = U.kb1 - U.kb0;
         const uint32_t clim = min(U.c0 + (uint32_t)BN, V.n);  // columns [c0, clim)
         // does the second A tile hold a pair that is reported?
@@ -437,13 +437,70 @@ void prepare_contract() {
     });
 }
 
-void launch_contract(const MmView *d_views, const MmUnit *d_units, uint32_t count, uint32_t *d_state,
-                     cudaStream_t st, unsigned long long *d_stamps, uint32_t test_spin) {
+void launch_contract(const MmView *d_views, const MmView &one, const MmUnit *d_units, uint32_t count,
+                     uint32_t *d_state, cudaStream_t st, unsigned long long *d_stamps, uint32_t test_spin) {
     if (!count) return;
     prepare_contract();
     dense::k_contract<<<std::min<uint32_t>(count, (uint32_t)device_sms()), dense::THREADS, dense::SMEM, st>>>(
-        d_views, d_units, count, d_state, test_spin ? test_spin : dense::SPIN_LIMIT, test_spin ? 1u : 0u, d_stamps);
+        d_views, one, d_units, count, d_state, test_spin ? test_spin : dense::SPIN_LIMIT, test_spin ? 1u : 0u, d_stamps);
     BM_CHECK_LAUNCH();
+}
+
+// ---- built sets ----------------------------------------------------------------------
+//
+// A set's supports come from its bit rows where that is estimated faster than
+// the BatMap scan, the bits' build included.  The scan costs four integer
+// instructions per 32-bit word pair: 7e12 word pairs/s on large instances
+// (9.5 ms for the 6.6e10 of the m = 10^6, n = 2,000 Zipf workload after the probe
+// route), and about 40 us of latency on the smallest; the contraction 256 x 240
+// pairs x 256 transactions per SM in MM_STEP_S.  BatMaps are at least m / 42
+// bytes wide, so the scan wins only where tiles are mostly padding: few items
+// over many transactions.  A caller who sets tile, shape_mask or probe_log asks
+// for a BatMap route and gets it.  The bits are left out (and the scan taken)
+// where they would take more than half of the free memory.
+constexpr double SCAN_WORD_PAIRS_PER_S = 7e12, SCAN_MIN_S = 40e-6, BITS_BYTES_PER_S = 4e12;
+
+static bool room_for(uint64_t bytes) {
+    if (bytes <= (64ull << 20)) return true;
+    size_t free_b = 0, total_b = 0;
+    BM_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    return bytes <= free_b / 2;
+}
+
+void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids, int *d_flags, bool sorted_only) {
+    const batmap_params &P = S->params;
+    S->contract = false;
+    if (S->skip_schedule || P.tile || P.shape_mask || P.probe_log || !S->npairs() || !S->n_elements) return;
+    const BitsLayout L = bits_block_major(S->n, S->m);
+    const uint64_t bytes = L.kb_stride * L.kblocks;
+    const double bits_s = ((double)bytes + 4.0 * (double)S->n_elements) / BITS_BYTES_PER_S;
+    if (bits_s + contract_seconds(S->n, S->n_a, L.kblocks) > SCAN_MIN_S + S->word_pairs / SCAN_WORD_PAIRS_PER_S) return;
+    if (!room_for(bytes)) return;
+    try {
+        S->d_bits.alloc(bytes);
+    } catch (const Error &e) {
+        if (e.code != BATMAP_ERR_NOMEM) throw;
+        cudaGetLastError();  // not an error of this call: the scan needs no bits
+        return;
+    }
+    std::vector<MmUnit> units;
+    S->mm_add = contract_units(S->n, S->n_a, L.kblocks, 0, 0.0, &units);
+    S->mm_count = (uint32_t)units.size();
+    S->kblocks = L.kblocks;
+    S->d_mm.alloc(64 + units.size() * sizeof(MmUnit));
+    BM_CUDA(cudaMemcpyAsync(S->d_mm.p + 64, units.data(), units.size() * sizeof(MmUnit), cudaMemcpyHostToDevice,
+                            S->stream));
+    enqueue_bits(d_off, d_tids, S->n, S->m, L, S->d_bits.p, d_flags, sorted_only, S->stream);
+    S->contract = true;
+}
+
+MmView contract_view(const batmap_set *S, uint32_t *C) { return MmView{S->d_bits.p, C, S->n, S->n_a}; }
+
+void enqueue_contract(batmap_set *S, uint32_t *C, cudaStream_t st) {
+    if (S->mm_add) BM_CUDA(cudaMemsetAsync(C, 0, S->npairs() * sizeof(uint32_t), st));
+    BM_CUDA(cudaMemsetAsync(S->d_mm.p, 0, 64, st));
+    launch_contract(nullptr, contract_view(S, C), reinterpret_cast<const MmUnit *>(S->d_mm.p + 64), S->mm_count,
+                    reinterpret_cast<uint32_t *>(S->d_mm.p), st);
 }
 
 // ---- pair_support_dense ------------------------------------------------------------
@@ -453,7 +510,6 @@ struct DenseWork {
     DevBuf<uint8_t> bits;
     DevBuf<uint32_t> C;
     DevBuf<MmUnit> units;
-    DevBuf<MmView> view;
     DevBuf<uint32_t> state;   // queue counter, timeout flag, bit flags (tid >= m, unsorted)
     DevBuf<uint64_t> blocksums, total;
     PhaseEvents ev;
@@ -492,7 +548,6 @@ void run_dense(uint32_t m, uint32_t n, const uint64_t *d_off, const uint32_t *d_
         C = W.C.p;
     }
     W.state.ensure(4);
-    W.view.ensure(1);
     W.total.ensure(1);
     W.bits.ensure(std::max<uint64_t>((uint64_t)L.kblocks * L.kb_stride, 32));
     BM_CUDA(cudaMemsetAsync(W.state.p, 0, 4 * sizeof(uint32_t), st));
@@ -506,8 +561,7 @@ void run_dense(uint32_t m, uint32_t n, const uint64_t *d_off, const uint32_t *d_
         if (add && npairs) BM_CUDA(cudaMemsetAsync(C, 0, npairs * sizeof(uint32_t), st));
         W.units.ensure(units.size());
         BM_CUDA(cudaMemcpyAsync(W.units.p, units.data(), units.size() * sizeof(MmUnit), cudaMemcpyHostToDevice, st));
-        BM_CUDA(cudaMemcpyAsync(W.view.p, &view, sizeof(view), cudaMemcpyHostToDevice, st));
-        launch_contract(W.view.p, W.units.p, (uint32_t)units.size(), W.state.p, st, nullptr,
+        launch_contract(nullptr, view, W.units.p, (uint32_t)units.size(), W.state.p, st, nullptr,
                         g_dense_timeout_test.exchange(0));
     }
     W.ev.record(2, st);

@@ -71,3 +71,60 @@ def test_largest_supports():
     full = torch.zeros(10, dtype=torch.int32, device="cuda")
     pkg.pair_support_dense(m, off, tids, 1, full=full)
     assert full.tolist() == want
+
+
+@pytest.mark.parametrize("na,nb", [(1, 1), (1, 241), (127, 240), (129, 239), (256, 241), (257, 480), (300, 7)])
+def test_cross_tile_edges(na, nb):
+    """Cross mode: rows end with family A inside a tile, columns start at family B."""
+    import torch
+    import paper_1102_1003_gb300 as pkg
+    inst = datagen.zipf_tidlists(20_011, na + nb, 0.05, seed=na * 1000 + nb)
+    off, tids, _ = device_inputs(inst, 0)
+    ref = oracle.pairs_full(inst.offsets, inst.tids, threads=THREADS)
+    a, b = np.meshgrid(np.arange(na), np.arange(nb), indexing="ij")
+    want = ref[oracle.packed_index(inst.n, a.ravel(), na + b.ravel())]
+    for probe_log in (0, 2):  # the library's choice, and a BatMap route
+        s = pkg.batmap_build_cross(inst.m, na, off, tids, params=pkg.batmap_default_params(probe_log=probe_log))
+        full = torch.full((na * nb,), -1, dtype=torch.int32, device="cuda")
+        pkg.pair_support_all(s, 1, full=full)
+        assert np.array_equal(full.cpu().numpy().astype(np.uint32), want), probe_log
+
+
+def test_batch_of_both_routes():
+    """One batched pass over sets on either route, small and large, split and whole K."""
+    import torch
+    import paper_1102_1003_gb300 as pkg
+    insts = [datagen.zipf_tidlists(150_000, 700, 0.02, seed=1, s=150), datagen.bernoulli_tidlists(900, 33, 0.2, seed=2, s=3),
+             datagen.zipf_tidlists(40_000, 250, 0.04, seed=3, s=40), datagen.bernoulli_tidlists(300, 2, 0.5, seed=4, s=1)]
+    sets, fulls, bufs, refs = [], [], [], []
+    for q, inst in enumerate(insts):
+        off, tids, _ = device_inputs(inst, 0)
+        p = pkg.batmap_default_params(probe_log=2) if q == 2 else None
+        sets.append(pkg.batmap_build(inst.m, off, tids, params=p))
+        refs.append(oracle.pairs_full(inst.offsets, inst.tids, threads=THREADS))
+        fulls.append(torch.full((refs[-1].size,), -1, dtype=torch.int32, device="cuda"))
+        bufs.append(torch.empty((refs[-1].size, 3), dtype=torch.int32, device="cuda"))
+    for rep in range(2):
+        n_out = pkg.pair_support_batch(sets, [i.s for i in insts], bufs, fulls)
+        for q, inst in enumerate(insts):
+            assert np.array_equal(fulls[q].cpu().numpy().astype(np.uint32), refs[q]), (rep, q)
+            want = oracle.threshold_from_full(refs[q], inst.n, inst.s)
+            assert n_out[q] == want.shape[0]
+            assert np.array_equal(bufs[q][:n_out[q]].cpu().numpy().astype(np.uint32), want)
+            fulls[q].fill_(-1)
+
+
+def test_invalid_lists_refused_with_bit_rows():
+    """The bit rows' build stands in for the list check: the same lists are refused."""
+    import torch
+    import paper_1102_1003_gb300 as pkg
+    inst = datagen.bernoulli_tidlists(70_000, 50, 0.1, seed=8)
+    off, tids, _ = device_inputs(inst, 0)
+    e = int(inst.offsets[7]) + 4_000  # inside item 7
+    for at, value in ((e, int(inst.tids[e + 1])), (e, 70_000), (e, 0), (int(inst.offsets[50]) - 1, 1 << 30)):
+        bad = tids.clone()
+        bad[at] = value
+        with pytest.raises(pkg.BatmapError) as err:
+            pkg.batmap_build(inst.m, off, bad)
+        assert err.value.code == pkg.BATMAP_ERR_ARG
+    pkg.batmap_build(inst.m, off, tids)

@@ -50,7 +50,6 @@ WORKLOAD_DESC = {
     "bern_m4m_n8192_p5": "density sweep, m=4,194,304, n=8,192, Bernoulli p=0.05",
 }
 OPS_PER_WORD_PAIR = 4  # LOP3, IADD, LOP3, IDP4A per 32-bit word pair
-WITNESS_OPS = 5        # per word-triple against the pair's prepared pattern: 2 masked XORs, IADD, AND-NOT, IDP4A
 
 
 def _peaks():
@@ -827,51 +826,29 @@ def run_triples(args):
                     for c, v in zip(cand_ref[pick].tolist(), sup.tolist()))
     peaks, peak_kind = _peaks()
     wit_s = statistics.mean(r[4]["compare_ms"] for r in rec) / 1e3
-    scan_s = statistics.mean(r[4]["scan_ms"] for r in rec) / 1e3
-    probe_s = statistics.mean(r[4]["probe_ms"] for r in rec) / 1e3
-    sz = inst.sizes
-    r0 = info3["r0"]
-    rr = np.array([max(r0, 1 << int(np.ceil(np.log2(max(2 * int(x), 1))))) for x in sz], dtype=np.int64)
-    rc = rr[cand_ref]
-    wt = int(rc.max(axis=1).sum())
-    # the library's route: the probe kernel takes the candidates whose widest
-    # BatMap is at least 8x the narrowest, the scan kernel the rest
-    probe = rc.max(axis=1) >= 8 * rc.min(axis=1)
-    wt_scan = int(rc[~probe].max(axis=1).sum())
-    narrow = np.argmin(rc, axis=1)
-    probe_words = int(rc[probe].min(axis=1).sum())
-    probe_slots = int(3 * sz[cand_ref[np.arange(cand_ref.shape[0]), narrow]][probe].sum())
+    words = n_cand * ((inst.m + 255) // 256 * 8)
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    alu_peak = sms * 128 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
-    achieved = WITNESS_OPS * wt_scan / scan_s / 1e12
+    popc_peak = sms * 16 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
+    achieved = words / wit_s / 1e12
     line = {"metric": "candidate itemset supports/sec (Apriori level 3 over 3-of-4 BatMaps), bit-exact",
             "workload": "triples", "unit": "candidate-supports/s", "value": n_cand * args.steps / elapsed,
             "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * elapsed / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u8", "data": "synthetic",
             "config": {"workload": "triples", "m": inst.m, "n": inst.n, "s": s, "tids": int(inst.tids.size),
                        "desc": "Zipf(1) items at mean density 2%", "frequent_pairs": n_pairs,
-                       "candidates": n_cand, "frequent_triples": n_trip, "batmap3_bytes": int(info3["bytes"]),
-                       "word_triples": wt},
+                       "candidates": n_cand, "frequent_triples": n_trip, "batmap3_bytes": int(info3["bytes"])},
             "phases_ms": {"build_2of3": statistics.mean(r[3]["build_ms"] for r in rec),
                           "pairs": statistics.mean(r[3]["pairs_ms"] for r in rec),
                           "build_3of4": statistics.mean(r[4]["build_ms"] for r in rec),
-                          "witness": 1e3 * wit_s, "witness_scan": 1e3 * scan_s, "witness_probe": 1e3 * probe_s,
+                          "supports": 1e3 * wit_s,
                           "candidates_compact": statistics.mean(r[4]["compact_ms"] for r in rec)},
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s",
-                         "frac": achieved / alu_peak, "kernel": "k_witness_group",
-                         "traffic": _traffic("triples", "k_witness_group", "witness.cu"),
-                         "peak_kind": f"{sms} SMs x 128 INT32 lanes x {peaks.get('sm_max_mhz', 2070.0):.0f} MHz "
+            "roofline": {"bound": "alu", "achieved": achieved, "peak": popc_peak, "unit": "Tops/s",
+                         "frac": achieved / popc_peak, "kernel": "k_bits_support",
+                         "traffic": _traffic("triples", "k_bits_support", "bits.cu"),
+                         "peak_kind": f"popcount: {sms} SMs x 16 lanes x {peaks.get('sm_max_mhz', 2070.0):.0f} MHz "
                                       f"({peak_kind} max clock)",
-                         "algorithmic_ops": f"{WITNESS_OPS} x {wt_scan:.4g} word-triples (max_j r_j words per "
-                                            f"scan-routed candidate, {int((~probe).sum())} of {probe.size})",
-                         "note": "the 3-of-4 BatMaps (24.6 MB) are L2-resident"},
-            "probe": {"kernel": "k_witness_probe", "candidates": int(probe.sum()), "ms": 1e3 * probe_s,
-                      "traffic": _traffic("triples", "k_witness_probe", "witness.cu"),
-                      "narrow_words": probe_words, "slots": probe_slots,
-                      "slots_per_s": probe_slots / probe_s if probe_s > 0 else None,
-                      "bound": "L2 latency: two random byte probes per nonempty slot of the narrowest BatMap",
-                      "slots_definition": "3 |S| of each probed candidate's narrowest set (copies stored)",
-                      "scan_equivalent_word_triples": int(rc[probe].max(axis=1).sum())},
+                         "algorithmic_ops": f"{words:.4g} popcounts (one per candidate and 32 transactions)",
+                         "note": "the bit rows (12.5 MB) are L2-resident"},
             "gpu_launches": int(launches), "failed_insertions_3of4": info3["n_failed"],
             "parity": {"pairs_exact": exact_pairs, "sampled_candidates": int(pick.size), "exact": bool(ok_sample)},
             "clocks": clocks}
@@ -974,12 +951,9 @@ def run_quads(args):
                           "pairs": statistics.mean(r[4]["pairs_ms"] for r in rec),
                           "build_4of5": statistics.mean(r[5]["build_ms"] for r in rec),
                           "triples": statistics.mean(r[6]["pairs_ms"] for r in rec),
-                          "triple_witness_scan": statistics.mean(r[6]["scan_ms"] for r in rec),
-                          "triple_witness_probe": statistics.mean(r[6]["probe_ms"] for r in rec),
                           "quadruples": statistics.mean(r[7]["pairs_ms"] for r in rec),
-                          "quadruple_witness": statistics.mean(r[7]["compare_ms"] for r in rec),
-                          "quadruple_witness_scan": statistics.mean(r[7]["scan_ms"] for r in rec),
-                          "quadruple_witness_probe": statistics.mean(r[7]["probe_ms"] for r in rec)},
+                          "triple_supports": statistics.mean(r[6]["compare_ms"] for r in rec),
+                          "quadruple_supports": statistics.mean(r[7]["compare_ms"] for r in rec)},
             "gpu_launches": int(launches), "failed_insertions_4of5": info4["n_failed"],
             "parity": {"pairs_exact": exact_pairs, "sampled_triple_candidates": k3, "triples_exact": bool(ok3),
                        "sampled_quadruple_candidates": k4, "quadruples_exact": bool(ok4)},

@@ -205,7 +205,11 @@ batmap_status batmap_build_cross(const batmap_params *p, uint32_t m, uint32_t n_
  *            copy for d >= 3), or NULL for the computed permutations of
  *            p->perm_seed (rows t = 0 .. d).  Other arguments as batmap_build.
  * Items keep their original order (no width sort); h_bytes of
- * batmap_export_layout follow it.  Errors: BATMAP_ERR_ARG for d outside
+ * batmap_export_layout follow it.  For d = 3 and 4 the build also keeps the
+ * family's bit rows (n * ceil(m / 256) * 32 bytes) unless they would take more
+ * than half of the free memory or p->tile, shape_mask or probe_log is set; the
+ * k-way supports are then the AND + popcount of the rows, else the witness rule
+ * on the BatMaps.  Errors: BATMAP_ERR_ARG for d outside
  * {2, 3, 4} or invalid input.
  */
 batmap_status batmap_build_d(const batmap_params *p, uint32_t d, uint32_t m, uint32_t n,
@@ -214,7 +218,8 @@ batmap_status batmap_build_d(const batmap_params *p, uint32_t d, uint32_t m, uin
 
 /*
  * |S_a1 ∩ ... ∩ S_ak| for n_q queries of k item ids (1 <= k <= d) on a set
- * built with d = 3 or d = 4, by the witness rule: the slot of table t counts
+ * built with d = 3 or d = 4, from its bit rows or, without them, by the witness
+ * rule: the slot of table t counts
  * iff the code bits of the k bytes agree and are nonzero and t is the
  * smallest table missed by none of the k sets (read from the bytes' missing-
  * table fields); failed common elements are added from the F lists.
@@ -238,13 +243,14 @@ batmap_status itemset_support(batmap_set *set, uint32_t k, uint64_t n_q, const u
  *   d_out   : device uint32[4 * cap], (a, b, c, support), lexicographic.
  *   n_out   : host, number of frequent triples (all of them, even > cap).
  *   n_candidates : host, may be NULL; number of candidates counted.
- * The set may be built with d = 3 or d = 4.  Candidates whose widest BatMap
+ * The set may be built with d = 3 or d = 4.  With bit rows every candidate is an
+ * AND + popcount (k_bits_support).  Without: candidates whose widest BatMap
  * is at least 8x (d = 3) or 2x (d = 4) the narrowest are counted by probing
  * the narrowest set's slots in the others (Sec. V: look up the elements of
  * the smallest set); the rest by the witness scan (grouped by pair for d = 3,
  * one warp per candidate for d = 4).  Both count the same elements.
  * Synchronises `stream`.  Timing: compare_ms = the support kernels (scan_ms
- * the scan, probe_ms the probe), compact_ms = candidate generation +
+ * the scan, probe_ms the probe; both 0 with bit rows), compact_ms = candidate generation +
  * compaction, pairs_ms = the call.  Errors: BATMAP_ERR_ARG,
  * BATMAP_ERR_CAPACITY (cap < *n_out; the first cap triples are written).
  */

@@ -121,4 +121,129 @@ void enqueue_bits(const uint64_t *d_off, const uint32_t *d_tids, uint32_t n, uin
     }
 }
 
+bool take_bits(BmBuf *buf, uint64_t bytes) {
+    if (bytes > (64ull << 20)) {
+        size_t free_b = 0, total_b = 0;
+        BM_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        if (bytes > free_b / 2) return false;
+    }
+    try {
+        buf->alloc(bytes);
+    } catch (const Error &e) {
+        if (e.code != BATMAP_ERR_NOMEM) throw;
+        cudaGetLastError();  // not an error of this call: the BatMap routes need no bits
+        return false;
+    }
+    return true;
+}
+
+// ---- k-way supports ------------------------------------------------------------
+//
+// A group of W warps takes G consecutive queries.  The queries of a candidate
+// list are in lexicographic order, so most share all ids but the last: their
+// common AND is formed once per 16-byte chunk, and each query costs one load,
+// four ANDs and four popcounts per chunk.  Queries that differ earlier go one by
+// one.  Rows come from L2 (12.5 MB at m = 100,000, n = 1,000) and, for the shared
+// ones, from L1; popcount issues at 16 per clock and SM, so 511,714 triples of
+// 3,128 words take at least 0.32 ms, and their rows 6.4 GB of L2 reads.
+template <int K, int G, int W>
+__global__ void __launch_bounds__(256) k_bits_support(const uint4 *__restrict__ bits, uint32_t chunks,
+                                                      const uint32_t *__restrict__ items, uint64_t nq,
+                                                      uint32_t *__restrict__ out) {
+    const uint32_t t = threadIdx.x % (32 * W);
+    const uint64_t groups = (uint64_t)gridDim.x * (8 / W);
+    __shared__ uint32_t s_sum[8];
+    for (uint64_t q0 = (blockIdx.x * (uint64_t)(8 / W) + threadIdx.x / (32 * W)) * G; q0 < nq; q0 += groups * G) {
+        const uint32_t gn = (uint32_t)min((uint64_t)G, nq - q0);
+        const uint32_t *it = items + q0 * K;
+        bool same = true;
+        for (uint32_t j = 1; j < gn; j++)
+#pragma unroll
+            for (int p = 0; p < K - 1; p++) same &= __ldg(&it[j * K + p]) == __ldg(&it[p]);
+        uint32_t cnt[G];
+#pragma unroll
+        for (int j = 0; j < G; j++) cnt[j] = 0;
+        if (same) {
+            const uint4 *pre[K], *last[G];
+#pragma unroll
+            for (int p = 0; p < K - 1; p++) pre[p] = bits + (uint64_t)__ldg(&it[p]) * chunks;
+#pragma unroll
+            for (int j = 0; j < G; j++) last[j] = bits + (uint64_t)__ldg(&it[((uint32_t)j < gn ? j : 0) * K + K - 1]) * chunks;
+            for (uint32_t c = t; c < chunks; c += 32 * W) {
+                uint4 v = make_uint4(~0u, ~0u, ~0u, ~0u), y[G];
+#pragma unroll
+                for (int j = 0; j < G; j++) y[j] = __ldg(last[j] + c);
+#pragma unroll
+                for (int p = 0; p < K - 1; p++) {
+                    const uint4 x = __ldg(pre[p] + c);
+                    v.x &= x.x; v.y &= x.y; v.z &= x.z; v.w &= x.w;
+                }
+#pragma unroll
+                for (int j = 0; j < G; j++)
+                    cnt[j] += __popc(v.x & y[j].x) + __popc(v.y & y[j].y) + __popc(v.z & y[j].z) + __popc(v.w & y[j].w);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                if ((uint32_t)j >= gn) break;
+                const uint4 *row[K];
+#pragma unroll
+                for (int p = 0; p < K; p++) row[p] = bits + (uint64_t)__ldg(&it[j * K + p]) * chunks;
+#pragma unroll 2
+                for (uint32_t c = t; c < chunks; c += 32 * W) {
+                    uint4 v = __ldg(row[0] + c);
+#pragma unroll
+                    for (int p = 1; p < K; p++) {
+                        const uint4 x = __ldg(row[p] + c);
+                        v.x &= x.x; v.y &= x.y; v.z &= x.z; v.w &= x.w;
+                    }
+                    cnt[j] += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < G; j++) {
+            const uint32_t sum = __reduce_add_sync(0xffffffffu, cnt[j]);
+            if (W == 1) {
+                if (t == 0 && (uint32_t)j < gn) out[q0 + j] = sum;
+            } else {  // G == 1: one query per block
+                if ((threadIdx.x & 31u) == 0) s_sum[threadIdx.x >> 5] = sum;
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    uint32_t all = 0;
+                    for (int w = 0; w < 8; w++) all += s_sum[w];
+                    out[q0] = all;
+                }
+                __syncthreads();
+            }
+        }
+    }
+}
+
+template <int K>
+static void launch_bits_support(const uint4 *bits, uint32_t chunks, const uint32_t *items, uint64_t nq, uint32_t *out,
+                                cudaStream_t st) {
+    // few queries: a block each, so that one long row does not wait on one warp
+    constexpr uint64_t FEW = 152 * 8;
+    if (nq <= FEW) {
+        k_bits_support<K, 1, 8><<<(unsigned)nq, 256, 0, st>>>(bits, chunks, items, nq, out);
+    } else {
+        constexpr int G = K == 1 ? 1 : K == 4 ? 4 : 8;
+        const uint64_t blocks = (nq + 8ull * G - 1) / (8ull * G);
+        k_bits_support<K, G, 1><<<(unsigned)std::min<uint64_t>(blocks, 1u << 20), 256, 0, st>>>(bits, chunks, items, nq, out);
+    }
+    BM_CHECK_LAUNCH();
+}
+
+void enqueue_bits_support(const uint8_t *d_bits, uint32_t kblocks, uint32_t k, const uint32_t *d_items, uint64_t nq,
+                          uint32_t *d_support, cudaStream_t st) {
+    if (!nq) return;
+    const uint4 *bits = reinterpret_cast<const uint4 *>(d_bits);
+    const uint32_t chunks = kblocks * 2;
+    if (k == 1) launch_bits_support<1>(bits, chunks, d_items, nq, d_support, st);
+    if (k == 2) launch_bits_support<2>(bits, chunks, d_items, nq, d_support, st);
+    if (k == 3) launch_bits_support<3>(bits, chunks, d_items, nq, d_support, st);
+    if (k == 4) launch_bits_support<4>(bits, chunks, d_items, nq, d_support, st);
+}
+
 }  // namespace bm

@@ -29,6 +29,15 @@ inline BitsLayout bits_row_major(uint32_t m) { return {32ull * bits_blocks(m), 3
 void enqueue_bits(const uint64_t *d_off, const uint32_t *d_tids, uint32_t n, uint32_t m, const BitsLayout &L,
                   uint8_t *d_bits, int *d_flags, bool sorted_only, cudaStream_t st);
 
+// Allocates `bytes` of bit rows unless they would take more than half of the
+// free memory; false (and no rows) if so, or if the allocation fails.
+bool take_bits(BmBuf *buf, uint64_t bytes);
+
+// |S_a1 cap .. cap S_ak| of nq queries of k ids each (1 <= k <= 4) over
+// row-major bit rows: AND and popcount.
+void enqueue_bits_support(const uint8_t *d_bits, uint32_t kblocks, uint32_t k, const uint32_t *d_items, uint64_t nq,
+                          uint32_t *d_support, cudaStream_t st);
+
 // ---- contraction -----------------------------------------------------------------
 
 struct MmView {          // one instance

@@ -460,13 +460,6 @@ void launch_contract(const MmView *d_views, const MmView &one, const MmUnit *d_u
 // where they would take more than half of the free memory.
 constexpr double SCAN_WORD_PAIRS_PER_S = 7e12, SCAN_MIN_S = 40e-6, BITS_BYTES_PER_S = 4e12;
 
-static bool room_for(uint64_t bytes) {
-    if (bytes <= (64ull << 20)) return true;
-    size_t free_b = 0, total_b = 0;
-    BM_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    return bytes <= free_b / 2;
-}
-
 void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids, int *d_flags, bool sorted_only) {
     const batmap_params &P = S->params;
     S->contract = false;
@@ -475,14 +468,7 @@ void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids,
     const uint64_t bytes = L.kb_stride * L.kblocks;
     const double bits_s = ((double)bytes + 4.0 * (double)S->n_elements) / BITS_BYTES_PER_S;
     if (bits_s + contract_seconds(S->n, S->n_a, L.kblocks) > SCAN_MIN_S + S->word_pairs / SCAN_WORD_PAIRS_PER_S) return;
-    if (!room_for(bytes)) return;
-    try {
-        S->d_bits.alloc(bytes);
-    } catch (const Error &e) {
-        if (e.code != BATMAP_ERR_NOMEM) throw;
-        cudaGetLastError();  // not an error of this call: the scan needs no bits
-        return;
-    }
+    if (!take_bits(&S->d_bits, bytes)) return;
     std::vector<MmUnit> units;
     S->mm_add = contract_units(S->n, S->n_a, L.kblocks, 0, 0.0, &units);
     S->mm_count = (uint32_t)units.size();

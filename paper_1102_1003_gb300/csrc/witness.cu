@@ -28,6 +28,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "bits.cuh"
 #include "common.cuh"
 #include "items.cuh"
 #include "scan.cuh"
@@ -264,12 +265,21 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     }
     ItemView v{d_offsets, d_tids, S->d_base.p, S->d_rlog.p, d_ch_item.p, d_ch_start.p};
 
+    // bit rows for the k-way supports, in the items' order: a row is m / 8 bytes where the BatMap
+    // has at least m / 16 (d = 3) or m / 6 (d = 4), and costs an AND and a popcount per 32
+    // transactions, whatever the item's size.  tile, shape_mask or probe_log ask for the BatMap
+    // kernels, as for pairs.
+    DevBuf<int> d_err(4);  // [0] a bad list or permutation, [2], [3] the bit rows' flags
+    BM_CUDA(cudaMemsetAsync(d_err.p, 0, 4 * sizeof(int), st));
+    const BitsLayout BL = bits_row_major(m);
+    S->kblocks = BL.kblocks;
+    const bool with_bits = T && !P.tile && !P.shape_mask && !P.probe_log && take_bits(&S->d_bits, BL.row_stride * n);
+    if (with_bits) enqueue_bits(d_offsets, d_tids, n, m, BL, S->d_bits.p, d_err.p + 2, P.validate != 0, st);
+
     if (P.validate) {
-        DevBuf<int> d_err(1);
         DevBuf<uint32_t> d_bits(d_perm ? (uint64_t)TABLES * ((m + 31) / 32) : 0);
-        BM_CUDA(cudaMemsetAsync(d_err.p, 0, sizeof(int), st));
         if (d_perm) BM_CUDA(cudaMemsetAsync(d_bits.p, 0, d_bits.bytes(), st));
-        if (nch) {
+        if (nch && !with_bits) {  // the bit rows' build checks every list
             k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_err.p);
             BM_CHECK_LAUNCH();
         }
@@ -277,11 +287,12 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
             k_validate_perm<<<grid_for((uint64_t)TABLES * m), 256, 0, st>>>(d_perm, m, TABLES, d_bits.p, d_err.p);
             BM_CHECK_LAUNCH();
         }
-        int err = 0;
-        BM_CUDA(cudaMemcpyAsync(&err, d_err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        int err[4] = {0, 0, 0, 0};
+        BM_CUDA(cudaMemcpyAsync(err, d_err.p, sizeof(err), cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
-        BM_REQUIRE(err != 1, BATMAP_ERR_ARG, "tids must be strictly increasing per item and < m");
-        BM_REQUIRE(err != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
+        BM_REQUIRE(err[0] != 1 && !err[2] && !err[3], BATMAP_ERR_ARG,
+                   "tids must be strictly increasing per item and < m");
+        BM_REQUIRE(err[0] != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
     }
 
     S->n_failed = 0;
@@ -1134,6 +1145,10 @@ void witness_support(batmap_set *S, uint32_t k, uint64_t nq, const uint32_t *d_i
         BM_CUDA(cudaStreamSynchronize(st));
         BM_REQUIRE(h == 0, BATMAP_ERR_ARG, "item id >= n in a query");
     }
+    if (S->d_bits.p) {
+        enqueue_bits_support(S->d_bits.p, S->kblocks, k, d_items, nq, d_support, st);
+        return;
+    }
     const View V{reinterpret_cast<const uint32_t *>(S->d_bm.p), S->d_base.p, S->d_rlog.p, S->perm,
                  S->d_fail_off.p, S->d_fail_tid.p, S->m, S->n, S->shift};
     launch_witness(V, S->d, k, d_items, nq, d_support, st);
@@ -1145,7 +1160,8 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
                       uint64_t cap, uint64_t *n_out, uint64_t *n_cand, cudaStream_t st) {
     using namespace wit;
     BM_REQUIRE(S && (S->d == 3 || S->d == 4), BATMAP_ERR_ARG, "frequent_triples needs a set built with d = 3 or 4");
-    const bool grouped = S->d == 3;  // the grouped kernel reads the 3-of-4 format
+    const bool by_bits = S->d_bits.p != nullptr;
+    const bool grouped = S->d == 3 && !by_bits;  // the grouped kernel reads the 3-of-4 format
     BM_REQUIRE(n_out, BATMAP_ERR_ARG, "n_out is NULL");
     BM_REQUIRE(np == 0 || d_pairs, BATMAP_ERR_ARG, "d_pairs is NULL");
     BM_REQUIRE(cap == 0 || d_out, BATMAP_ERR_ARG, "d_out is NULL with cap > 0");
@@ -1203,7 +1219,9 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
     if (nc) {
         const View V{reinterpret_cast<const uint32_t *>(S->d_bm.p), S->d_base.p, S->d_rlog.p, S->perm,
                      S->d_fail_off.p, S->d_fail_tid.p, S->m, S->n, S->shift};
-        if (grouped) {
+        if (by_bits) {
+            enqueue_bits_support(S->d_bits.p, S->kblocks, 3, cand.p, nc, sup.p, st);
+        } else if (grouped) {
             const uint64_t wpb = WG_TPB / 32;
             const unsigned grid = (unsigned)std::min<uint64_t>((n_units + wpb - 1) / wpb, 152ull * 64);
             k_witness_group<<<grid, WG_TPB, 0, st>>>(V, d_pairs, cnt.p, cand.p, units.p, n_units, sup.p);
@@ -1239,8 +1257,8 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
     S->timing.compare_ms = E.ms(1, 2);
     S->timing.compact_ms = E.ms(0, 1) + E.ms(2, 3);
     S->timing.pairs_ms = E.ms(0, 3);
-    const bool split = nc > 0;  // event 4 sits between the scan and the probe kernels (both routes)
-    S->timing.scan_ms = split ? E.ms(1, 4) : S->timing.compare_ms;
+    const bool split = nc > 0 && !by_bits;  // event 4 sits between the scan and the probe kernels
+    S->timing.scan_ms = split ? E.ms(1, 4) : 0.f;
     S->timing.probe_ms = split ? E.ms(4, 2) : 0.f;
     *n_out = total;
     if (total > cap)
@@ -1290,7 +1308,8 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
     if (nc) {
         const View V{reinterpret_cast<const uint32_t *>(S->d_bm.p), S->d_base.p, S->d_rlog.p, S->perm,
                      S->d_fail_off.p, S->d_fail_tid.p, S->m, S->n, S->shift};
-        witness_routed5(V, 4, cand.p, nc, S->d_rlog.p, sup.p, E, st);
+        if (S->d_bits.p) enqueue_bits_support(S->d_bits.p, S->kblocks, 4, cand.p, nc, sup.p, st);
+        else witness_routed5(V, 4, cand.p, nc, S->d_rlog.p, sup.p, E, st);
     }
     E.record(2, st);
     uint64_t total = 0;
@@ -1309,8 +1328,9 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
     E.record(3, st);
     BM_CUDA(cudaStreamSynchronize(st));
     S->timing.compare_ms = E.ms(1, 2);
-    S->timing.scan_ms = nc ? E.ms(1, 4) : 0.f;  // event 4 sits between the scan and the probe kernels
-    S->timing.probe_ms = nc ? E.ms(4, 2) : 0.f;
+    const bool split = nc > 0 && !S->d_bits.p;  // event 4 sits between the scan and the probe kernels
+    S->timing.scan_ms = split ? E.ms(1, 4) : 0.f;
+    S->timing.probe_ms = split ? E.ms(4, 2) : 0.f;
     S->timing.compact_ms = E.ms(0, 1) + E.ms(2, 3);
     S->timing.pairs_ms = E.ms(0, 3);
     *n_out = total;

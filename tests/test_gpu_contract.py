@@ -128,3 +128,49 @@ def test_invalid_lists_refused_with_bit_rows():
             pkg.batmap_build(inst.m, off, bad)
         assert err.value.code == pkg.BATMAP_ERR_ARG
     pkg.batmap_build(inst.m, off, tids)
+
+
+@pytest.mark.parametrize("d", [3, 4])
+@pytest.mark.parametrize("m", [200, 8_191, 8_193, 40_007])
+def test_kway_supports_of_bit_rows_and_batmaps(d, m):
+    """k_bits_support (few and many queries, runs of queries sharing all ids but the last
+    that start and end inside its groups) and the BatMap kernels give the merge counts."""
+    import torch
+    import paper_1102_1003_gb300 as pkg
+    inst = datagen.zipf_tidlists(m, 60, 0.1, seed=m + d)
+    off, tids, _ = device_inputs(inst, 0)
+    sets = [pkg.batmap_build_d(d, m, off, tids, params=pkg.batmap_default_params(probe_log=pl)) for pl in (0, 3)]
+    rng = np.random.default_rng(m)
+    for k in range(1, d + 1):
+        few = rng.integers(0, inst.n, (37, k))
+        runs = [np.concatenate([np.tile(rng.integers(0, inst.n, (1, k - 1)), (r, 1)),
+                                rng.integers(0, inst.n, (r, 1))], axis=1) for r in rng.integers(1, 21, 260)]
+        for qs in (few, np.concatenate(runs)):
+            qs = np.ascontiguousarray(qs, np.int32)
+            want = oracle.kway_counts(inst.offsets, inst.tids, qs.tolist())
+            for s in sets:
+                got = pkg.itemset_support(s, torch.from_numpy(qs).cuda()).cpu().numpy().astype(np.uint64)
+                assert np.array_equal(got, want), (k, qs.shape)
+
+
+@pytest.mark.parametrize("d", [3, 4])
+def test_frequent_itemsets_same_on_both_routes(d):
+    """Triples (and quadruples) of a set with bit rows equal those of the BatMap kernels."""
+    import paper_1102_1003_gb300 as pkg
+    inst = datagen.zipf_tidlists(30_000, 200, 0.04, seed=9)
+    off, tids, _ = device_inputs(inst, 0)
+    s = 40
+    b2 = pkg.batmap_build(inst.m, off, tids)
+    _, pairs = pkg.pair_support_all(b2, s)
+    got = []
+    for pl in (0, 3):
+        b = pkg.batmap_build_d(d, inst.m, off, tids, params=pkg.batmap_default_params(probe_log=pl))
+        n3, t3, c3 = pkg.frequent_triples(b, s, pairs)
+        r = [n3, c3, t3.cpu().numpy()]
+        if d == 4:
+            n4, t4, c4 = pkg.frequent_quadruples(b, s, t3)
+            r += [n4, c4, t4.cpu().numpy()]
+        got.append(r)
+    assert got[0][0] > 0
+    for x, y in zip(*got):
+        assert np.array_equal(x, y)

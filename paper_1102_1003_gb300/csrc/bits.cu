@@ -1,88 +1,175 @@
 // Bit rows from CSR tidlists (the bitmap vertical representation, Sec. I-B).
 //
-// One warp writes one item's bits of one 32,768-transaction chunk: it finds
-// the chunk's tids by two 32-way searches (about log32 |S| dependent reads),
-// ORs them into 4 KiB of shared memory and stores the 128 blocks of 32 bytes.
-// Every byte of the matrix is written once, so nothing is zeroed before, no
-// global atomic is used and the lists' order is checked on the way.
-// Bound: HBM, 4 bytes read per tid and 1 bit written per (item, transaction).
+// One warp writes one item's bits of a run of 16,384-transaction chunks: it finds
+// the run's tids by two 32-way searches side by side (about log32 |S| dependent
+// reads), then walks them in blocks of 256 (16-byte loads, the next block on its
+// way), ORs a chunk's into 2 KiB of shared memory and stores its 64 blocks of 32
+// bytes.  Every byte of the matrix is written once, so nothing is zeroed before,
+// no global atomic is used and the lists' order is checked on the way.
+// Bound: HBM, 4 bytes read per tid and 1 bit written per (item, transaction);
+// short lists by the latency of the searches (hence runs), skewed families by
+// the warps of full lists, one tid per bit, which end last (hence runs only
+// where there are warps enough).
 #include <algorithm>
 
 #include "bits.cuh"
 
 namespace bm {
 
-constexpr uint32_t CHUNK_KB = 128;                   // blocks per warp
-constexpr uint32_t CHUNK_BITS = CHUNK_KB * BITS_K;   // 32,768
+constexpr uint32_t CHUNK_KB = 64;                    // blocks per warp
+constexpr uint32_t CHUNK_BITS = CHUNK_KB * BITS_K;   // 16,384
 constexpr int BW = 8;                                // warps per CTA
 
-// First index in a[0 .. n) whose value is >= v, by the whole warp.  A function
-// of the list and v alone, so neighbouring chunks agree on their border even
-// when the list is not sorted.
-__device__ __forceinline__ uint64_t warp_lower_bound(const uint32_t *__restrict__ a, uint64_t n, uint32_t v,
-                                                     uint32_t lane) {
-    uint64_t lo = 0, hi = n;
-    while (lo < hi) {
-        const uint64_t step = (hi - lo + 31) >> 5;
-        const uint64_t p = lo + lane * step + (step - 1);
-        const bool below = p < hi && __ldg(&a[p]) < v;
-        const uint32_t c = __popc(__ballot_sync(0xffffffffu, below));
-        const uint64_t top = lo + c * step + (step - 1);  // the first probe not below, if c < 32
-        lo = min(lo + c * step, hi);
-        if (c < 32) hi = min(hi, top);
+// One round of a 32-way search for the first index in [lo, hi) whose value is
+// >= v, by the whole warp.  The result of all rounds is a function of the list
+// and v alone, so neighbouring chunks agree on their border even when the list
+// is not sorted.
+__device__ __forceinline__ void search_round(const uint32_t *__restrict__ a, uint64_t &lo, uint64_t &hi, uint32_t v,
+                                             uint32_t lane) {
+    if (lo >= hi) return;  // done (warp-uniform): a further round could move the result of an unsorted list
+    const uint64_t step = (hi - lo + 31) >> 5;
+    const uint64_t p = lo + lane * step + (step - 1);
+    const bool below = p < hi && __ldg(&a[p]) < v;
+    const uint32_t c = __popc(__ballot_sync(0xffffffffu, below));
+    const uint64_t top = lo + c * step + (step - 1);  // the first probe not below, if c < 32
+    lo = min(lo + c * step, hi);
+    if (c < 32) hi = min(hi, top);
+}
+
+// BLOCK tids of one list from place f on, four per lane and 16-byte load; place f
+// stands for element f - skew, which starts a 16-byte boundary.  Places before
+// `begin` hold `before` (the predecessor of the first), those from `end` on 0.
+constexpr int BQ = 2;                  // loads in flight per lane and block
+constexpr uint32_t BLOCK = 128 * BQ;
+struct TidBlock {
+    uint32_t x[BQ][4];
+};
+__device__ __forceinline__ void load_block(TidBlock &B, const uint32_t *__restrict__ a, uint64_t f, uint32_t skew,
+                                           uint64_t begin, uint64_t end, uint32_t before, uint32_t lane) {
+#pragma unroll
+    for (int q = 0; q < BQ; q++) {
+        const uint64_t i = f + 128u * q + 4u * lane;
+        if (i >= begin && i + 4 <= end) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(a + (i - skew)));
+            B.x[q][0] = v.x; B.x[q][1] = v.y; B.x[q][2] = v.z; B.x[q][3] = v.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                B.x[q][j] = i + j < begin ? before : i + j < end ? __ldg(&a[i + j - skew]) : 0;
+        }
     }
-    return lo;
 }
 
 __global__ void __launch_bounds__(32 * BW)
 k_bits(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tids, uint32_t n, uint32_t m, BitsLayout L,
-       uint8_t *__restrict__ out, int *__restrict__ flags) {
+       uint32_t run, uint8_t *__restrict__ out, int *__restrict__ flags) {
     __shared__ __align__(16) uint32_t s_bits[BW][CHUNK_BITS / 32];
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t *bits = s_bits[threadIdx.x >> 5];
     uint4 *bits4 = reinterpret_cast<uint4 *>(bits);
-    const uint32_t nchunk = (L.kblocks + CHUNK_KB - 1) / CHUNK_KB;
-    const uint64_t tasks = (uint64_t)n * nchunk, warps = (uint64_t)gridDim.x * BW;
+    const uint32_t nchunk = (L.kblocks + CHUNK_KB - 1) / CHUNK_KB, nrun = (nchunk + run - 1) / run;
+    const uint64_t tasks = (uint64_t)n * nrun, warps = (uint64_t)gridDim.x * BW;
     bool bad_tid = false, unsorted = false;
-    // neighbouring warps: neighbouring items of the same chunk, whose 32-byte pieces share lines
+    // neighbouring warps: neighbouring items of the same chunks, whose 32-byte pieces share lines
     for (uint64_t w = blockIdx.x * (uint64_t)BW + (threadIdx.x >> 5); w < tasks; w += warps) {
-        const uint32_t item = (uint32_t)(w % n), chunk = (uint32_t)(w / n);
-#pragma unroll
-        for (uint32_t j = 0; j < CHUNK_BITS / 32 / 4; j += 32) bits4[j + lane] = make_uint4(0, 0, 0, 0);
+        const uint32_t item = (uint32_t)(w % n), c0 = (uint32_t)(w / n) * run, c1 = min(c0 + run, nchunk);
         const uint64_t b = off[item], size = off[item + 1] - b;
         const uint32_t *a = tids + b;
-        const uint32_t x0 = chunk * CHUNK_BITS, x1 = x0 + CHUNK_BITS;  // m <= 2^30: no overflow
-        const bool last = chunk + 1 == nchunk;
-        const uint64_t e0 = chunk ? warp_lower_bound(a, size, x0, lane) : 0;
-        const uint64_t e1 = last ? size : warp_lower_bound(a, size, x1, lane);
+        const uint32_t first = c0 * CHUNK_BITS, past = c1 * CHUNK_BITS;  // m <= 2^30: no overflow
+        uint64_t e0 = 0, h0 = c0 ? size : 0, e1 = c1 == nchunk ? size : 0, h1 = size;
+        while (e0 < h0 || e1 < h1) {
+            search_round(a, e0, h0, first, lane);
+            search_round(a, e1, h1, past, lane);
+        }
         unsorted |= e1 < e0;
-        __syncwarp();
-        for (uint64_t e = e0; e < e1; e += 128) {
-            uint32_t x[4], y[4];
+        const uint32_t skew = (uint32_t)(reinterpret_cast<uintptr_t>(a + e0) >> 2) & 3u;
+        const uint64_t begin = e0 + skew, end = e1 + skew;  // places of the run's elements
+        uint32_t carry = e0 ? __ldg(&a[e0 - 1]) : 0;         // predecessor of the block's first tid
+        uint64_t f = e0;                                     // the block in hand; the one behind it is on its way
+        TidBlock B, N;
+        load_block(B, a, f, skew, begin, end, carry, lane);
+        load_block(N, a, f + BLOCK, skew, begin, end, carry, lane);
+        uint32_t b0 = 0;       // the block's first tid (carry: its last)
+        bool fresh = true, plain = false;
+        for (uint32_t c = c0; c < c1; c++) {
+            const uint32_t x0 = c * CHUNK_BITS;
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const uint64_t i = e + 32u * q + lane;
-                x[q] = i < e1 ? __ldg(&a[i]) : 0xFFFFFFFFu;
-                y[q] = i < e1 && i + 1 < size ? __ldg(&a[i + 1]) : 0xFFFFFFFFu;
+            for (uint32_t j = 0; j < CHUNK_BITS / 32 / 4; j += 32) bits4[j + lane] = make_uint4(0, 0, 0, 0);
+            __syncwarp();
+            for (;;) {
+                if (fresh) {
+                    // a new block.  plain: all places hold tids of the run, ascending and below m
+                    const uint32_t last = __shfl_sync(0xffffffffu, B.x[BQ - 1][3], 31);
+                    b0 = __shfl_sync(0xffffffffu, B.x[0][0], 0);
+                    plain = f >= begin && f + BLOCK <= end && b0 >= first && last < past && last < m &&
+                            (f == 0 || carry < b0);
+                    bool ok = true;
+#pragma unroll
+                    for (int q = 0; q < BQ; q++) {
+                        const uint32_t up = __shfl_up_sync(0xffffffffu, B.x[q][3], 1);
+                        const uint32_t head = q ? __shfl_sync(0xffffffffu, B.x[q ? q - 1 : 0][3], 31) : 0;
+                        const uint32_t prev = lane ? up : head;
+                        ok &= (q == 0 && lane == 0) || prev < B.x[q][0];
+                        ok &= B.x[q][0] < B.x[q][1] && B.x[q][1] < B.x[q][2] && B.x[q][2] < B.x[q][3];
+                    }
+                    plain = plain && __all_sync(0xffffffffu, ok);
+                    if (!plain) {  // place by place
+#pragma unroll
+                        for (int q = 0; q < BQ; q++) {
+                            const uint64_t i = f + 128u * q + 4u * lane;
+                            uint32_t prev = __shfl_up_sync(0xffffffffu, B.x[q][3], 1);
+                            if (lane == 0) prev = carry;
+#pragma unroll
+                            for (int j = 0; j < 4; j++) {
+                                const uint32_t y = B.x[q][j];
+                                if (i + j >= begin && i + j < end) {
+                                    // (the list's first tid has no predecessor)
+                                    unsorted |= (i + j != skew && !(prev < y)) || y < first || y >= past;
+                                    bad_tid |= y >= m;
+                                }
+                                prev = y;
+                            }
+                            carry = __shfl_sync(0xffffffffu, B.x[q][3], 31);
+                        }
+                    }
+                    carry = last;
+                }
+#pragma unroll
+                for (int q = 0; q < BQ; q++) {
+                    const uint64_t i = f + 128u * q + 4u * lane;
+                    uint32_t word = 0, mask = 0;  // bits of one word are set together
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const uint32_t y = B.x[q][j];
+                        if (y - x0 < CHUNK_BITS && (plain || (y < m && i + j >= begin && i + j < end))) {
+                            const uint32_t v = (y - x0) >> 5;
+                            if (v != word && mask) {
+                                atomicOr(&bits[word], mask);
+                                mask = 0;
+                            }
+                            word = v;
+                            mask |= 1u << (y & 31u);
+                        }
+                    }
+                    if (mask) atomicOr(&bits[word], mask);
+                }
+                // the chunk goes on in the next block if this one's last tid (carry) lies before its end
+                fresh = f + BLOCK < end && carry < x0 + CHUNK_BITS;
+                if (!fresh) break;
+                f += BLOCK;
+                B = N;
+                load_block(N, a, f + BLOCK, skew, begin, end, carry, lane);
             }
+            __syncwarp();
+            uint8_t *row = out + item * L.row_stride;
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-                if (e + 32u * q + lane >= e1) continue;
-                unsorted |= !(x[q] < y[q]);
-                if (x[q] >= m) bad_tid = true;
-                else if (x[q] - x0 < CHUNK_BITS) atomicOr(&bits[(x[q] - x0) >> 5], 1u << (x[q] & 31u));
-                else unsorted = true;
+            for (uint32_t j = 0; j < CHUNK_KB * 2; j += 32) {
+                const uint32_t i = j + lane, kb = c * CHUNK_KB + (i >> 1);
+                if (kb < L.kblocks) *reinterpret_cast<uint4 *>(row + kb * L.kb_stride + 16u * (i & 1u)) = bits4[i];
             }
+            __syncwarp();
         }
-        __syncwarp();
-        uint8_t *row = out + item * L.row_stride;
-        const uint32_t kb0 = chunk * CHUNK_KB;
-#pragma unroll
-        for (uint32_t j = 0; j < CHUNK_KB * 2; j += 32) {
-            const uint32_t i = j + lane, kb = kb0 + (i >> 1);
-            if (kb < L.kblocks) *reinterpret_cast<uint4 *>(row + kb * L.kb_stride + 16u * (i & 1u)) = bits4[i];
-        }
-        __syncwarp();
+        unsorted |= f + BLOCK < end;  // (a sorted run ends with its last block)
     }
     if (bad_tid) atomicExch(&flags[0], 1);
     if (unsorted) atomicExch(&flags[1], 1);
@@ -111,9 +198,13 @@ __global__ void k_bits_unsorted(const uint64_t *__restrict__ off, const uint32_t
 void enqueue_bits(const uint64_t *d_off, const uint32_t *d_tids, uint32_t n, uint32_t m, const BitsLayout &L,
                   uint8_t *d_bits, int *d_flags, bool sorted_only, cudaStream_t st) {
     if (!n) return;
-    const uint64_t tasks = (uint64_t)n * ((L.kblocks + CHUNK_KB - 1) / CHUNK_KB);
+    const uint32_t nchunk = (L.kblocks + CHUNK_KB - 1) / CHUNK_KB;
+    // chunks per warp: about 200,000 warps (many rounds of the chip) before a warp takes several,
+    // which saves it their searches
+    const uint32_t run = (uint32_t)std::min<uint64_t>(16, std::max<uint64_t>(1, (uint64_t)n * nchunk / 200000));
+    const uint64_t tasks = (uint64_t)n * ((nchunk + run - 1) / run);
     const unsigned grid = (unsigned)std::min<uint64_t>((tasks + BW - 1) / BW, 1u << 20);
-    k_bits<<<grid, 32 * BW, 0, st>>>(d_off, d_tids, n, m, L, d_bits, d_flags);
+    k_bits<<<grid, 32 * BW, 0, st>>>(d_off, d_tids, n, m, L, run, d_bits, d_flags);
     BM_CHECK_LAUNCH();
     if (!sorted_only) {
         k_bits_unsorted<<<dim3(8, std::min<uint32_t>(n, 128u)), 256, 0, st>>>(d_off, d_tids, n, m, L, d_bits, d_flags);

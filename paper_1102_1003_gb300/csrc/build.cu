@@ -3,9 +3,9 @@
 //   validate  : tids strictly increasing and < m per item; each permutation
 //               row a bijection of [0, m)
 //   size      : s, r_0, r_i, widths 3 r_i, width-sorted order (host)
-//   place     : parallel generalised cuckoo INSERT into uint32 tables
-//   finalize  : every element with exactly two copies gets its two bytes
-//               (indicator << 7 | code); the rest are failed insertions
+//   place     : parallel generalised cuckoo INSERT; every element with exactly
+//               two copies gets its two bytes (indicator << 7 | code); the
+//               rest are failed insertions (place.cu)
 //   failures  : F_i in (item, tid) order, then the correction entries: one
 //               (min, max) item pair per failed common transaction
 //   schedule  : compare work units (host, compare.cu)
@@ -18,6 +18,7 @@
 #include "common.cuh"
 #include "items.cuh"
 #include "perm.cuh"
+#include "place.cuh"
 #include "scan.cuh"
 
 namespace bm {
@@ -55,133 +56,7 @@ __global__ void k_validate_perm(const uint32_t *perm, uint32_t m, uint32_t rows,
     }
 }
 
-// ---- placement: parallel 2-of-3 cuckoo insertion (Sec. II-A) --------------------
-//
-// Each thread carries one copy of one element.  Copy c starts in table c; a
-// copy is swapped into its slot of table t; the evicted occupant (if any)
-// continues in table t+1 (cyclic order 1,2,3,1,...).  Swapping a copy with
-// the other copy of the same element leaves the table unchanged and the
-// element continues in the next table, so the two copies always end in two
-// distinct tables.  Atomic exchanges conserve copies; a chain that exceeds
-// 3*MaxLoop moves drops the copy it holds, and finalize then reports that
-// element as a failed insertion.
-__global__ void k_place(ItemView v, const PermView P, uint32_t shift, uint32_t max_moves,
-                        uint32_t *__restrict__ table) {
-    const uint32_t m = P.m;
-    uint32_t item;
-    uint64_t e0, e1;
-    chunk_range(v, blockIdx.x >> 1, &item, &e0, &e1);
-    const uint32_t copy = blockIdx.x & 1u;
-    const uint64_t base = v.base[item];
-    const uint32_t r = 1u << v.rlog[item];
-    for (uint64_t e = e0 + threadIdx.x; e < e1; e += TPB) {
-        uint32_t x = v.tids[e];
-        if (x >= m) continue;  // rejected by validation; never index past perm
-        uint32_t t = copy;
-        for (uint32_t mv = 0; mv < max_moves; mv++) {
-            uint32_t pi = P(t, x);
-            uint64_t pos = base + slot_of(t, pi, r, shift);
-            uint32_t old = atomicExch(&table[pos], x);
-            if (old == EMPTY) break;
-            x = old;  // old == x: same element, continue in the next table
-            t = (t == 2) ? 0 : t + 1;
-        }
-    }
-}
-
-struct Copies {
-    uint32_t pi[3];
-    uint64_t pos[3];
-    uint32_t has;  // bit t set: a copy sits in table t
-};
-
-__device__ __forceinline__ Copies find_copies(uint32_t x, uint64_t base, uint32_t r, uint32_t shift,
-                                              const PermView &P, const uint32_t *__restrict__ table) {
-    Copies c;
-    c.has = 0;
-#pragma unroll
-    for (uint32_t t = 0; t < 3; t++) {
-        c.pi[t] = P(t, x);
-        c.pos[t] = base + slot_of(t, c.pi[t], r, shift);
-        if (table[c.pos[t]] == x) c.has |= 1u << t;
-    }
-    return c;
-}
-
-__device__ __forceinline__ bool two_copies(uint32_t has) { return __popc(has) == 2; }
-
-// Writes the two bytes of every element stored twice.  The indicator is 1 on
-// the copy whose twin sits in the cyclic predecessor table (Fig. 3).
-// Also counts the block's failed insertions into blocksums[block] (the count
-// pass of the ordered compaction that lists them).
-__global__ void k_finalize(ItemView v, const PermView P, uint32_t shift, const uint32_t *__restrict__ table,
-                           uint8_t *__restrict__ out, uint64_t *__restrict__ blocksums) {
-    const uint32_t m = P.m;
-    __shared__ uint32_t s_fail;
-    if (threadIdx.x == 0) s_fail = 0;
-    __syncthreads();
-    uint32_t item;
-    uint64_t e0, e1;
-    chunk_range(v, blockIdx.x, &item, &e0, &e1);
-    const uint64_t base = v.base[item];
-    const uint32_t r = 1u << v.rlog[item];
-    uint32_t fails = 0;
-    for (uint64_t e = e0 + threadIdx.x; e < e1; e += TPB) {
-        uint32_t x = v.tids[e];
-        if (x >= m) continue;
-        Copies c = find_copies(x, base, r, shift, P, table);
-        if (!two_copies(c.has)) {
-            fails++;
-            continue;
-        }
-#pragma unroll
-        for (uint32_t t = 0; t < 3; t++) {
-            if (c.has & (1u << t)) {
-                uint32_t pred = (t + 2) % 3;
-                uint32_t ind = (c.has >> pred) & 1u;
-                out[c.pos[t]] = (uint8_t)element_byte(c.pi[t], shift, ind);
-            }
-        }
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) fails += __shfl_xor_sync(0xffffffffu, fails, d);
-    if ((threadIdx.x & 31) == 0 && fails) atomicAdd(&s_fail, fails);
-    __syncthreads();
-    if (threadIdx.x == 0) blocksums[blockIdx.x] = s_fail;
-}
-
-// ---- failed insertions, in (item, tid) order --------------------------------------
-
-// Rank of each failing element inside its block, in element order.
-template <bool WRITE>
-__global__ void k_failures(ItemView v, const PermView P, uint32_t shift, const uint32_t *__restrict__ table,
-                           uint64_t *blocksums, uint32_t *f_item, uint32_t *f_tid) {
-    const uint32_t m = P.m;
-    uint32_t item;
-    uint64_t e0, e1;
-    chunk_range(v, blockIdx.x, &item, &e0, &e1);
-    const uint64_t base = v.base[item];
-    const uint32_t r = 1u << v.rlog[item];
-    uint64_t running = WRITE ? blocksums[blockIdx.x] : 0;
-    if (WRITE && blocksums[blockIdx.x + 1] == running) return;  // no failure in this block
-    for (int j = 0; j < PER_THREAD; j++) {
-        uint64_t e = e0 + (uint64_t)j * TPB + threadIdx.x;
-        bool fail = false;
-        uint32_t x = 0;
-        if (e < e1) {
-            x = v.tids[e];
-            fail = x < m && !two_copies(find_copies(x, base, r, shift, P, table).has);
-        }
-        uint64_t tot;
-        uint64_t rank = block_exclusive_scan(fail ? 1 : 0, &tot);
-        if (WRITE && fail) {
-            f_item[running + rank] = item;
-            f_tid[running + rank] = x;
-        }
-        running += tot;
-    }
-    if (!WRITE && threadIdx.x == 0) blocksums[blockIdx.x] = running;
-}
+// ---- failed insertions ------------------------------------------------------------
 
 // f_off[i] = first failure of item i (lower bound in the sorted f_item list).
 __global__ void k_fail_offsets(const uint32_t *f_item, uint64_t nfail, uint32_t n, uint64_t *f_off) {
@@ -300,10 +175,11 @@ static uint32_t shift_bits(uint32_t m, uint32_t min_shift) {
     return s;
 }
 
-// The placement scratch (one uint32 per BatMap byte) is kept between builds
-// so that repeated builds do not pay for allocating and freeing it; it is
-// released when a build needs less than a quarter of it or on
-// batmap_release_scratch().  Builds are serialised on it.
+// The placement scratch (the regions of place.cu: 96 MiB, or two of the widest
+// item's tables if that is more) is kept between builds so that repeated builds
+// do not pay for allocating and freeing it; it is released when a build needs
+// less than a quarter of it or on batmap_release_scratch().  Builds are
+// serialised on it.
 std::mutex g_scratch_mu;
 static DevBuf<uint32_t> g_scratch;
 
@@ -464,20 +340,23 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         BM_CUDA(cudaMemcpyAsync(S->d_wshift.p, S->wshift_sorted.data(), n * 4, cudaMemcpyHostToDevice, st));
         BM_CUDA(cudaMemcpyAsync(S->d_order.p, S->order.data(), n * 4, cudaMemcpyHostToDevice, st));
     }
-    if (S->bytes) BM_CUDA(cudaMemsetAsync(S->d_bm.p, 0, S->bytes, st));
 
     // per-element chunks: block b handles elements [ch_start[b], +CHUNK) of item ch_item[b]
     std::vector<uint32_t> ch_item;
     std::vector<uint64_t> ch_start;
-    for (uint32_t i = 0; i < n; i++)
+    std::vector<uint32_t> chunk0(n);
+    for (uint32_t i = 0; i < n; i++) {
+        chunk0[i] = (uint32_t)ch_item.size();
         for (uint64_t s = off[i]; s < off[i + 1]; s += CHUNK) {
             ch_item.push_back(i);
             ch_start.push_back(s);
         }
+    }
     const uint32_t nch = (uint32_t)ch_item.size();
 
     S->d_fail_off.alloc(n + 1);
     if (T == 0) {
+        if (S->bytes) BM_CUDA(cudaMemsetAsync(S->d_bm.p, 0, S->bytes, st));
         BM_CUDA(cudaMemsetAsync(S->d_fail_off.p, 0, (n + 1) * sizeof(uint64_t), st));
         if (!S->skip_schedule) build_schedule(S);
         E.record(1, st);
@@ -518,19 +397,30 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         BM_REQUIRE(err[0] != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
     }
 
-    // ---- place + finalize ----
+    // ---- placement and bytes ----
     {
-        DevBuf<uint32_t> &table = scratch_table(S->bytes);
-        BM_CUDA(cudaMemsetAsync(table.p, 0xFF, S->bytes * sizeof(uint32_t), st));
-        const uint32_t max_moves = 3u * std::max<uint32_t>(P.max_loop, 1u);
         E.record(2, st);
-        k_place<<<2u * nch, TPB, 0, st>>>(v, PV, S->shift, max_moves, table.p);
-        BM_CHECK_LAUNCH();
-        E.record(3, st);
-        // failed insertions, ordered by (item, tid): counted by finalize, listed below
         DevBuf<uint64_t> bs(nch + 1), d_tot(1);
-        k_finalize<<<nch, TPB, 0, st>>>(v, PV, S->shift, table.p, S->d_bm.p, bs.p);
-        BM_CHECK_LAUNCH();
+        DevBuf<uint32_t> d_mask((uint64_t)nch * (CHUNK / 32)), d_chunk0(n);
+        BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
+        BM_CUDA(cudaMemcpyAsync(d_chunk0.p, chunk0.data(), n * 4ull, cudaMemcpyHostToDevice, st));
+        std::vector<PlaceItem> list(n);
+        for (uint32_t i = 0; i < n; i++) list[i] = {i, rlog[i], off[i + 1] - off[i]};
+        DevBuf<uint32_t> d_list(n), d_queue(PLACE_QUEUES);
+        PlaceJob J{};
+        J.off = d_offsets;
+        J.tids = d_tids;
+        J.base = d_base.p;
+        J.chunk0 = d_chunk0.p;
+        J.shift = S->shift;
+        J.max_moves = 3u * std::max<uint32_t>(P.max_loop, 1u);
+        J.out = S->d_bm.p;
+        J.fails = bs.p;
+        J.mask = d_mask.p;
+        J.queue = d_queue.p;
+        enqueue_place(3, J, PV, std::move(list), d_list.p, st);
+        E.record(3, st);
+        // failed insertions, ordered by (item, tid): counted and marked by the placement
         k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, d_tot.p, 1);
         BM_CHECK_LAUNCH();
         uint64_t nfail = 0;
@@ -540,8 +430,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         DevBuf<uint32_t> f_item(nfail);
         S->d_fail_tid.alloc(nfail);
         if (nfail) {
-            k_failures<true><<<nch, TPB, 0, st>>>(v, PV, S->shift, table.p, bs.p, f_item.p,
-                                                  S->d_fail_tid.p);
+            k_failures<<<nch, TPB, 0, st>>>(v, d_mask.p, bs.p, f_item.p, S->d_fail_tid.p);
             BM_CHECK_LAUNCH();
         }
         k_fail_offsets<<<(n + 1 + 255) / 256, 256, 0, st>>>(f_item.p, nfail, n, S->d_fail_off.p);

@@ -1,0 +1,36 @@
+// Placement of the elements of all items and the bytes of their BatMaps, for
+// 2-of-3, 3-of-4 and 4-of-5 sets.
+#pragma once
+
+#include "items.cuh"
+
+namespace bm {
+
+struct PlaceJob {
+    const uint64_t *off;     // CSR
+    const uint32_t *tids;
+    const uint64_t *base;    // [n] first byte of item i in `out`
+    const uint32_t *chunk0;  // [n] first chunk (CHUNK elements) of item i
+    const uint32_t *items;   // a launch's items, all of range 2^rlog (set by the launches)
+    uint32_t count, rlog, shift, max_moves;
+    uint8_t *out;            // BatMap bytes (every byte of the items is written)
+    uint64_t *fails;         // [chunks] zeroed; failed insertions per chunk
+    uint32_t *mask;          // [chunks * CHUNK / 32] bit e: element e of the chunk failed
+    uint32_t *queue;         // PLACE_QUEUES words
+};
+
+// Places all items of the list (ids, any order; d_list: room for as many ids on
+// the device); tables: d + 1 (3, 4 or 5).
+struct PlaceItem {
+    uint32_t item, rlog;
+    uint64_t size;
+};
+constexpr uint32_t PLACE_QUEUES = 64;
+void enqueue_place(uint32_t tables, const PlaceJob &job, const PermView &P, std::vector<PlaceItem> list,
+                   uint32_t *d_list, cudaStream_t st);
+
+// F_i of every chunk with failures, in (item, tid) order: offsets[b] = first
+// entry of chunk b (exclusive scan of the counts, with the total behind it).
+__global__ void k_failures(ItemView v, const uint32_t *mask, const uint64_t *offsets, uint32_t *f_item, uint32_t *f_tid);
+
+}  // namespace bm

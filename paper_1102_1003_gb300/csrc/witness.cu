@@ -31,6 +31,7 @@
 #include "bits.cuh"
 #include "common.cuh"
 #include "items.cuh"
+#include "place.cuh"
 #include "scan.cuh"
 
 namespace bm {
@@ -67,124 +68,6 @@ __device__ __forceinline__ uint32_t code6(uint32_t pi, uint32_t shift) { return 
 
 // ---- build ------------------------------------------------------------------
 
-// Parallel INSERT with d = NT - 1 copies: copy c of every element starts in
-// table c; a copy is swapped into its slot and the evicted occupant continues
-// in the next table (0, 1, .., NT - 1, 0, ...).  Swapping with another copy
-// of the same element leaves the slot unchanged and the element moves on, so
-// copies of one element never share a table.  A chain longer than max_moves
-// drops the copy it holds (the element then fails).
-template <uint32_t NT>
-__global__ void k_place(ItemView v, const PermView P, uint32_t shift, uint32_t max_moves,
-                        uint32_t *__restrict__ table) {
-    constexpr uint32_t NC = Fmt<NT>::COPIES;
-    const uint32_t m = P.m;
-    uint32_t item;
-    uint64_t e0, e1;
-    chunk_range(v, blockIdx.x / NC, &item, &e0, &e1);
-    const uint32_t copy = blockIdx.x % NC;
-    const uint64_t base = v.base[item];
-    const uint32_t r = 1u << v.rlog[item];
-    for (uint64_t e = e0 + threadIdx.x; e < e1; e += TPB) {
-        uint32_t x = v.tids[e];
-        if (x >= m) continue;  // rejected by validation; never index past perm
-        uint32_t t = copy;
-        for (uint32_t mv = 0; mv < max_moves; mv++) {
-            const uint32_t pi = P(t, x);
-            const uint32_t old = atomicExch(&table[base + slot_nt<NT>(t, pi, r, shift)], x);
-            if (old == EMPTY) break;
-            x = old;
-            t = (t + 1u == NT) ? 0u : t + 1u;
-        }
-    }
-}
-
-template <uint32_t NT>
-struct CopiesN {
-    uint32_t pi[NT];
-    uint64_t pos[NT];
-    uint32_t has;  // bit t: a copy sits in table t
-};
-
-template <uint32_t NT>
-__device__ __forceinline__ CopiesN<NT> find_copies(uint32_t x, uint64_t base, uint32_t r, uint32_t shift,
-                                                   const PermView &P, const uint32_t *__restrict__ table) {
-    CopiesN<NT> c;
-    c.has = 0;
-#pragma unroll
-    for (uint32_t t = 0; t < NT; t++) {
-        c.pi[t] = P(t, x);
-        c.pos[t] = base + slot_nt<NT>(t, c.pi[t], r, shift);
-        if (table[c.pos[t]] == x) c.has |= 1u << t;
-    }
-    return c;
-}
-
-// Bytes of every element stored d times; failures counted per block.
-template <uint32_t NT>
-__global__ void k_finalize(ItemView v, const PermView P, uint32_t shift, const uint32_t *__restrict__ table,
-                           uint8_t *__restrict__ out, uint64_t *__restrict__ blocksums) {
-    const uint32_t m = P.m;
-    __shared__ uint32_t s_fail;
-    if (threadIdx.x == 0) s_fail = 0;
-    __syncthreads();
-    uint32_t item;
-    uint64_t e0, e1;
-    chunk_range(v, blockIdx.x, &item, &e0, &e1);
-    const uint64_t base = v.base[item];
-    const uint32_t r = 1u << v.rlog[item];
-    uint32_t fails = 0;
-    for (uint64_t e = e0 + threadIdx.x; e < e1; e += TPB) {
-        const uint32_t x = v.tids[e];
-        if (x >= m) continue;
-        const CopiesN<NT> c = find_copies<NT>(x, base, r, shift, P, table);
-        if (__popc(c.has) != (int)Fmt<NT>::COPIES) {
-            fails++;
-            continue;
-        }
-        const uint32_t missing = __ffs(~c.has & ((1u << NT) - 1u)) - 1;
-#pragma unroll
-        for (uint32_t t = 0; t < NT; t++)
-            if (c.has & (1u << t))
-                out[c.pos[t]] = (uint8_t)((missing << Fmt<NT>::CODE_BITS) | code6(c.pi[t], shift));
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) fails += __shfl_xor_sync(0xffffffffu, fails, d);
-    if ((threadIdx.x & 31) == 0 && fails) atomicAdd(&s_fail, fails);
-    __syncthreads();
-    if (threadIdx.x == 0) blocksums[blockIdx.x] = s_fail;
-}
-
-// Failed insertions in (item, tid) order: block offsets come from the scan
-// of the finalize counts.
-template <uint32_t NT>
-__global__ void k_failures(ItemView v, const PermView P, uint32_t shift, const uint32_t *__restrict__ table,
-                           const uint64_t *blocksums, uint32_t *f_item, uint32_t *f_tid) {
-    const uint32_t m = P.m;
-    uint32_t item;
-    uint64_t e0, e1;
-    chunk_range(v, blockIdx.x, &item, &e0, &e1);
-    uint64_t running = blocksums[blockIdx.x];
-    if (blocksums[blockIdx.x + 1] == running) return;  // no failure in this block
-    const uint64_t base = v.base[item];
-    const uint32_t r = 1u << v.rlog[item];
-    for (int j = 0; j < PER_THREAD; j++) {
-        const uint64_t e = e0 + (uint64_t)j * TPB + threadIdx.x;
-        bool fail = false;
-        uint32_t x = 0;
-        if (e < e1) {
-            x = v.tids[e];
-            fail = x < m && __popc(find_copies<NT>(x, base, r, shift, P, table).has) != (int)Fmt<NT>::COPIES;
-        }
-        uint64_t tot;
-        const uint64_t rank = block_exclusive_scan(fail ? 1 : 0, &tot);
-        if (fail) {
-            f_item[running + rank] = item;
-            f_tid[running + rank] = x;
-        }
-        running += tot;
-    }
-}
-
 // Smallest s >= min_shift with m <= code_max * 2^s (codes 1..code_max, 0 = empty).
 static uint32_t shift_bits_codes(uint32_t m, uint32_t min_shift, uint32_t code_max) {
     uint32_t s = min_shift;
@@ -194,7 +77,7 @@ static uint32_t shift_bits_codes(uint32_t m, uint32_t min_shift, uint32_t code_m
 
 template <uint32_t NT>
 void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids, const uint32_t *d_perm) {
-    constexpr uint32_t TABLES = NT, COPIES = Fmt<NT>::COPIES;
+    constexpr uint32_t TABLES = NT;
     std::lock_guard<std::mutex> scratch_lock(g_scratch_mu);
     const uint32_t m = S->m, n = S->n;
     cudaStream_t st = S->stream;
@@ -246,16 +129,19 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     if (d_perm) BM_CUDA(cudaMemcpyAsync(S->d_perm.p, d_perm, (uint64_t)TABLES * m * 4, cudaMemcpyDeviceToDevice, st));
     S->perm = make_perm_view(d_perm ? S->d_perm.p : nullptr, m, P.perm_seed);
     const PermView PV = S->perm;
-    if (S->bytes) BM_CUDA(cudaMemsetAsync(S->d_bm.p, 0, S->bytes, st));
+    if (S->bytes && !T) BM_CUDA(cudaMemsetAsync(S->d_bm.p, 0, S->bytes, st));
     S->d_fail_off.alloc(n + 1);
 
     std::vector<uint32_t> ch_item;
     std::vector<uint64_t> ch_start;
-    for (uint32_t i = 0; i < n; i++)
+    std::vector<uint32_t> chunk0(n);
+    for (uint32_t i = 0; i < n; i++) {
+        chunk0[i] = (uint32_t)ch_item.size();
         for (uint64_t s0 = off[i]; s0 < off[i + 1]; s0 += CHUNK) {
             ch_item.push_back(i);
             ch_start.push_back(s0);
         }
+    }
     const uint32_t nch = (uint32_t)ch_item.size();
     DevBuf<uint32_t> d_ch_item(nch);
     DevBuf<uint64_t> d_ch_start(nch);
@@ -297,16 +183,27 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
 
     S->n_failed = 0;
     if (nch) {
-        DevBuf<uint32_t> &table = scratch_table(S->bytes);
-        BM_CUDA(cudaMemsetAsync(table.p, 0xFF, S->bytes * sizeof(uint32_t), st));
-        const uint32_t max_moves = TABLES * std::max<uint32_t>(P.max_loop, 1u);
         E.record(2, st);
-        k_place<NT><<<COPIES * nch, TPB, 0, st>>>(v, PV, S->shift, max_moves, table.p);
-        BM_CHECK_LAUNCH();
-        E.record(3, st);
         DevBuf<uint64_t> bs(nch + 1), d_tot(1);
-        k_finalize<NT><<<nch, TPB, 0, st>>>(v, PV, S->shift, table.p, S->d_bm.p, bs.p);
-        BM_CHECK_LAUNCH();
+        DevBuf<uint32_t> d_mask((uint64_t)nch * (CHUNK / 32)), d_queue(PLACE_QUEUES);
+        DevBuf<uint32_t> d_list(n), d_chunk0(n);
+        std::vector<PlaceItem> list(n);
+        for (uint32_t i = 0; i < n; i++) list[i] = {i, rlog[i], off[i + 1] - off[i]};
+        BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
+        BM_CUDA(cudaMemcpyAsync(d_chunk0.p, chunk0.data(), n * 4ull, cudaMemcpyHostToDevice, st));
+        PlaceJob J{};
+        J.off = d_offsets;
+        J.tids = d_tids;
+        J.base = S->d_base.p;
+        J.chunk0 = d_chunk0.p;
+        J.shift = S->shift;
+        J.max_moves = TABLES * std::max<uint32_t>(P.max_loop, 1u);
+        J.out = S->d_bm.p;
+        J.fails = bs.p;
+        J.mask = d_mask.p;
+        J.queue = d_queue.p;
+        enqueue_place(NT, J, PV, std::move(list), d_list.p, st);
+        E.record(3, st);
         k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, d_tot.p, 1);
         BM_CHECK_LAUNCH();
         uint64_t nfail = 0;
@@ -316,8 +213,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
         DevBuf<uint32_t> f_item(nfail);
         S->d_fail_tid.alloc(nfail);
         if (nfail) {
-            k_failures<NT><<<nch, TPB, 0, st>>>(v, PV, S->shift, table.p, bs.p, f_item.p,
-                                            S->d_fail_tid.p);
+            k_failures<<<nch, TPB, 0, st>>>(v, d_mask.p, bs.p, f_item.p, S->d_fail_tid.p);
             BM_CHECK_LAUNCH();
         }
         k_fail_offsets<<<(n + 1 + 255) / 256, 256, 0, st>>>(f_item.p, nfail, n, S->d_fail_off.p);

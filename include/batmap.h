@@ -365,8 +365,8 @@ batmap_status batmap_autotune(batmap_set *const *sets, uint32_t k, double *shape
  */
 typedef struct batmap_timing {
     float build_ms;     /* whole batmap_build, first to last enqueued operation */
-    float place_ms;     /* 2-of-3 placement kernel                              */
-    float finalize_ms;  /* byte writing + failure lists + correction entries    */
+    float place_ms;     /* placement and byte writing                           */
+    float finalize_ms;  /* failure lists + correction entries                   */
     float compare_ms;   /* the all-pairs compare: contraction, or scan and probe */
     float compact_ms;   /* failure correction + threshold compaction            */
     float pairs_ms;     /* whole pair_support_all                               */
@@ -381,8 +381,8 @@ typedef struct batmap_timing {
 batmap_status batmap_get_timing(const batmap_set *set, batmap_timing *t);
 
 /* Release the scratch the library caches between calls (the placement table
- * of batmap_build, one uint32 per BatMap byte; at most six arrays of freed
- * sets; the dense path's bitmap and
+ * of batmap_build, up to 96 MiB or two of its widest item's, four bytes per
+ * slot; at most six arrays of freed sets; the dense path's bitmap and
  * workspace; pair_support_host's device copies of its inputs and output).
  * Call when no other call of the library is running. */
 void batmap_release_scratch(void);
@@ -534,7 +534,7 @@ void batmap_test_dense_timeout(uint32_t spin_limit);
  * synchronisation cudaMalloc / cudaFree may perform, cannot let the library
  * allocate.  This call performs the same support-threshold compaction as
  * pair_support_all and allocates nothing: its scratch is a fixed device array
- * of 512 KiB + 8 bytes inside the library, which every GPU that loads the
+ * of 512 KiB + 16 bytes inside the library, which every GPU that loads the
  * library holds until the process exits.
  *   d_full  : device uint32[n(n-1)/2], supports of all pairs i < j as the
  *             packed upper triangle written by pair_support_all's d_full.

@@ -19,6 +19,7 @@ namespace bm {
 void enqueue_correct_compact(batmap_set *S, uint32_t *C, uint32_t s, uint32_t *d_pairs, uint64_t cap,
                              uint64_t *d_total, cudaStream_t st);
 void prepare_compaction(batmap_set *S);
+void check_total(uint64_t total);
 
 struct BatchPlan {
     std::vector<uint64_t> key;
@@ -196,6 +197,7 @@ void run_batch(batmap_set *const *sets, const uint32_t *s, uint32_t k, batmap_ou
     const float cc = all > cmp ? all - cmp : 0.f;
     bool overflow = false;
     for (uint32_t q = 0; q < k; q++) {
+        check_total(totals[q]);
         outs[q].n_out = totals[q];
         overflow |= totals[q] > outs[q].cap;
         sets[q]->timing.compare_ms = cmp;

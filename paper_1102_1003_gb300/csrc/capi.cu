@@ -28,6 +28,7 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
                          uint64_t cap, uint64_t *n_out, uint64_t *n_cand, cudaStream_t st);
 void enqueue_correct_compact(batmap_set *S, uint32_t *C, uint32_t s, uint32_t *d_pairs, uint64_t cap,
                              uint64_t *d_total, cudaStream_t st);
+void check_total(uint64_t total);
 void run_batch(batmap_set *const *sets, const uint32_t *s, uint32_t k, batmap_out *outs, cudaStream_t st);
 void autotune(batmap_set *const *sets, uint32_t k, double *eff_out, cudaStream_t st);
 void release_scratch();
@@ -270,6 +271,7 @@ static void pair_support_impl(batmap_set *S, uint32_t s, uint32_t *d_pairs, uint
     if (S->contract) BM_CUDA(cudaMemcpyAsync(state, S->d_mm.p, sizeof(state), cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaStreamSynchronize(st));
     BM_REQUIRE(!state[1], BATMAP_ERR_TIMEOUT, "tensor-core kernel: a bounded pipeline wait timed out");
+    check_total(total);
     S->timing.compare_ms = S->pairs_ev.ms(1, 2);
     S->timing.scan_ms = S->contract ? 0.f : S->pairs_ev.ms(1, 4);
     S->timing.probe_ms = S->contract ? 0.f : S->pairs_ev.ms(4, 2);

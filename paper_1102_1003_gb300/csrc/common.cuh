@@ -233,6 +233,6 @@ struct batmap_set {
     bm::DevBuf<uint32_t> d_C;             // packed upper triangle when no d_full
     bm::DevBuf<uint32_t> d_counters;      // work-queue counter
     bm::DevBuf<bm::InstView> d_view;      // device copy of this set's InstView
-    bm::DevBuf<uint64_t> d_blocksums;     // compaction block counts / offsets
+    bm::DevBuf<uint64_t> d_blocksums;     // compaction tile states
     bm::DevBuf<uint64_t> d_total;         // compaction total
 };

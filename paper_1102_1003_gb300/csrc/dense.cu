@@ -49,7 +49,8 @@
 namespace bm {
 
 void enqueue_threshold(const uint32_t *C, uint64_t n, uint32_t s, uint32_t *d_pairs, uint64_t cap,
-                       DevBuf<uint64_t> *blocksums, uint64_t *d_total, cudaStream_t st);
+                       DevBuf<uint64_t> *state, uint64_t *d_total, cudaStream_t st);
+void check_total(uint64_t total);
 
 namespace dense {
 
@@ -566,6 +567,7 @@ void run_dense(uint32_t m, uint32_t n, const uint64_t *d_off, const uint32_t *d_
     if (tout) *tout = W.timing;
     BM_REQUIRE(state[2] == 0, BATMAP_ERR_ARG, "tids must be < m");
     BM_REQUIRE(state[1] == 0, BATMAP_ERR_TIMEOUT, "dense tensor-core kernel: a bounded pipeline wait timed out");
+    check_total(total);
     *n_out = total;
     if (total > cap)
         throw Error{BATMAP_ERR_CAPACITY, "d_pairs too small: " + std::to_string(total) + " pairs qualify"};

@@ -7,7 +7,7 @@
 // perform.  This entry point takes the packed supports (the d_full output of
 // pair_support_all) and writes the frequent pairs with the same kernels as
 // the compaction inside pair_support_all, but its only scratch -- per-block
-// counts and their prefix sums -- lives in a fixed device array declared in
+// states and a counter -- lives in a fixed device array declared in
 // this file.  With lazy module loading (the CUDA default) the array's memory
 // is reserved when this file's module is first loaded on a device, which is
 // the first call's address lookup; a caller that must not see that happen
@@ -19,19 +19,20 @@
 
 namespace bm {
 
-// Compaction of compact.cu: block counts of 4096 packed positions each.
+// Compaction of compact.cu: a state word per tile of 4096 packed positions, and the tile counter.
 uint64_t threshold_blocks(uint64_t n);
 void enqueue_threshold_into(const uint32_t *C, uint64_t n, uint32_t s, uint32_t *d_pairs, uint64_t cap,
-                            uint64_t *blocksums, uint64_t *d_total, cudaStream_t st);
+                            uint64_t *state, uint64_t *d_total, cudaStream_t st);
+void check_total(uint64_t total);
 
-// Capacity of the fixed scratch: one 64-bit count per block of 4096 pairs.
+// Capacity of the fixed scratch: one 64-bit state per tile of 4096 pairs.
 constexpr uint64_t NOALLOC_BLOCK_PAIRS = 4096;
 constexpr uint64_t NOALLOC_MAX_BLOCKS = 65536;  // 2^28 pairs, n <= 23,170 items
 constexpr uint64_t NOALLOC_MAX_PAIRS = NOALLOC_BLOCK_PAIRS * NOALLOC_MAX_BLOCKS;
 
-// [0, NOALLOC_MAX_BLOCKS): block counts, then their exclusive prefix sums;
-// [NOALLOC_MAX_BLOCKS]: the number of qualifying pairs.  512 KiB + 8 B.
-static __device__ __align__(256) uint64_t g_noalloc_scratch[NOALLOC_MAX_BLOCKS + 1];
+// The tile states and, behind the last, the tile counter; the last word: the
+// number of qualifying pairs.  512 KiB + 16 B.
+static __device__ __align__(256) uint64_t g_noalloc_scratch[NOALLOC_MAX_BLOCKS + 2];
 
 // Device address of g_noalloc_scratch, looked up once per device.
 static std::mutex g_na_mu;
@@ -61,12 +62,13 @@ void threshold_noalloc(const uint32_t *d_full, uint32_t n, uint32_t s, uint32_t 
                "pair_threshold_noalloc supports at most 2^28 pairs (n <= 23170); use pair_support_all");
     BM_REQUIRE(npairs == 0 || d_full != nullptr, BATMAP_ERR_ARG, "d_full is NULL");
     uint64_t *scratch = noalloc_scratch_for_current_device();
-    uint64_t *d_total = scratch + NOALLOC_MAX_BLOCKS;
+    uint64_t *d_total = scratch + NOALLOC_MAX_BLOCKS + 1;
     BM_REQUIRE(threshold_blocks(n) <= NOALLOC_MAX_BLOCKS, BATMAP_ERR_INTERNAL, "block size mismatch");
     enqueue_threshold_into(d_full, n, s, d_pairs, cap, scratch, d_total, st);
     uint64_t total = 0;
     BM_CUDA(cudaMemcpyAsync(&total, d_total, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaStreamSynchronize(st));
+    check_total(total);
     *n_out = total;
     if (total > cap)
         throw Error{BATMAP_ERR_CAPACITY, "d_pairs too small: " + std::to_string(total) + " pairs qualify"};

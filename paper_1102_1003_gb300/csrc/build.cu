@@ -56,6 +56,35 @@ __global__ void k_validate_perm(const uint32_t *perm, uint32_t m, uint32_t rows,
     }
 }
 
+// Chunk b: elements [ch_start[b], + CHUNK) of item ch_item[b].
+__global__ void k_chunks(const uint64_t *off, const uint32_t *chunk0, uint32_t *ch_item, uint64_t *ch_start) {
+    const uint32_t i = blockIdx.x;
+    const uint64_t e0 = off[i], e1 = off[i + 1];
+    for (uint64_t c = threadIdx.x; e0 + c * CHUNK < e1; c += blockDim.x) {
+        ch_item[chunk0[i] + c] = i;
+        ch_start[chunk0[i] + c] = e0 + c * CHUNK;
+    }
+}
+
+// Number of correction entries of a set with bit rows, which needs no list of
+// them: a failed (a, x) makes one with every other item holding x, less one per
+// pair of items that both failed x.  One warp per failure counts the items in
+// x's column; seen: m zeroed words.
+__global__ void k_count_corrections(const uint32_t *f_tid, uint64_t nfail, const uint8_t *bits, uint32_t n,
+                                    uint32_t *seen, unsigned long long *count) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
+    for (uint64_t k = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32; k < nfail; k += warps) {
+        const uint32_t x = f_tid[k];
+        const uint8_t *col = bits + (uint64_t)(x >> 8) * 32u * n + 4u * ((x >> 5) & 7u);
+        uint32_t items = 0;
+        for (uint32_t c = lane; c < n; c += 32)
+            items += (*reinterpret_cast<const uint32_t *>(col + 32ull * c) >> (x & 31u)) & 1u;
+        items = __reduce_add_sync(0xffffffffu, items);
+        if (lane == 0) atomicAdd(count, (unsigned long long)items - 1ull - atomicAdd(&seen[x], 1u));
+    }
+}
+
 // ---- failed insertions ------------------------------------------------------------
 
 // f_off[i] = first failure of item i (lower bound in the sorted f_item list).
@@ -192,9 +221,10 @@ void release_scratch() {
     std::lock_guard<std::mutex> lock(g_scratch_mu);
     g_scratch.release();
     bm_buffer_release_all();
+    release_arenas();
 }
 
-// ---- cache of BatMap arrays ----------------------------------------------------------
+// ---- kept device memory and events ---------------------------------------------------
 
 namespace {
 struct CachedBuf {
@@ -202,23 +232,29 @@ struct CachedBuf {
     size_t cap;
 };
 std::mutex g_bm_cache_mu;
-std::vector<CachedBuf> g_bm_cache;  // at most BM_CACHE, oldest first
-// A set holds a BatMap array, bit rows and the units of the contraction; a level of itemset mining
-// frees two sets.
-constexpr size_t BM_CACHE = 6;
+std::vector<CachedBuf> g_bm_cache[2];  // arrays of up to LARGE_BUF bytes, larger ones; oldest first
+constexpr size_t LARGE_BUF = 64ull << 20, BM_CACHE[2] = {32, 4};
+thread_local int t_released = 0;
+
+std::mutex g_event_mu;
+std::vector<cudaEvent_t> g_events;  // at most MAX_EVENTS
+constexpr size_t MAX_EVENTS = 256;
 }  // namespace
 
 uint8_t *bm_buffer_take(size_t bytes, size_t *capacity) {
     {
         std::lock_guard<std::mutex> lock(g_bm_cache_mu);
-        int best = -1;
-        for (int i = 0; i < (int)g_bm_cache.size(); i++) {
-            const size_t c = g_bm_cache[i].cap;
-            if (c >= bytes && c <= 2 * bytes + (64ull << 20) && (best < 0 || c < g_bm_cache[best].cap)) best = i;
-        }
-        if (best >= 0) {
-            const CachedBuf b = g_bm_cache[best];
-            g_bm_cache.erase(g_bm_cache.begin() + best);
+        CachedBuf *best = nullptr;
+        std::vector<CachedBuf> *from = nullptr;
+        for (auto &cache : g_bm_cache)
+            for (auto &b : cache)
+                if (b.cap >= bytes && b.cap <= 2 * bytes + (1u << 20) && (!best || b.cap < best->cap)) {
+                    best = &b;
+                    from = &cache;
+                }
+        if (best) {
+            const CachedBuf b = *best;
+            from->erase(from->begin() + (best - from->data()));
             *capacity = b.cap;
             return b.p;
         }
@@ -231,19 +267,143 @@ uint8_t *bm_buffer_take(size_t bytes, size_t *capacity) {
 
 void bm_buffer_give(uint8_t *p, size_t capacity) {
     // no queued work may still use the array when it is handed out again
-    cudaDeviceSynchronize();
+    if (!t_released) cudaDeviceSynchronize();
     std::lock_guard<std::mutex> lock(g_bm_cache_mu);
-    g_bm_cache.push_back({p, capacity});
-    if (g_bm_cache.size() > BM_CACHE) {
-        cudaFree(g_bm_cache.front().p);
-        g_bm_cache.erase(g_bm_cache.begin());
+    const int k = capacity > LARGE_BUF;
+    g_bm_cache[k].push_back({p, capacity});
+    if (g_bm_cache[k].size() > BM_CACHE[k]) {
+        cudaFree(g_bm_cache[k].front().p);
+        g_bm_cache[k].erase(g_bm_cache[k].begin());
     }
 }
 
 void bm_buffer_release_all() {
     std::lock_guard<std::mutex> lock(g_bm_cache_mu);
-    for (auto &b : g_bm_cache) cudaFree(b.p);
-    g_bm_cache.clear();
+    for (auto &cache : g_bm_cache) {
+        for (auto &b : cache) cudaFree(b.p);
+        cache.clear();
+    }
+}
+
+ReleaseScope::ReleaseScope() {
+    cudaDeviceSynchronize();
+    t_released++;
+}
+ReleaseScope::~ReleaseScope() { t_released--; }
+
+void PhaseEvents::create() {
+    if (ok) return;
+    std::lock_guard<std::mutex> lock(g_event_mu);
+    for (int i = 0; i < N; i++) {
+        if (!g_events.empty()) {
+            ev[i] = g_events.back();
+            g_events.pop_back();
+        } else {
+            BM_CUDA(cudaEventCreate(&ev[i]));
+        }
+    }
+    ok = true;
+}
+
+PhaseEvents::~PhaseEvents() {
+    std::lock_guard<std::mutex> lock(g_event_mu);
+    for (int i = 0; i < N; i++) {
+        if (!ev[i]) continue;
+        if (g_events.size() < MAX_EVENTS) g_events.push_back(ev[i]);
+        else cudaEventDestroy(ev[i]);
+    }
+}
+
+struct Arena {
+    struct Block {
+        uint8_t *p;
+        size_t cap, used;
+    };
+    std::vector<Block> blocks;
+    void *pinned = nullptr;
+    size_t total() const {
+        size_t t = 0;
+        for (const Block &b : blocks) t += b.cap;
+        return t;
+    }
+    void add(size_t cap) {
+        Block b{nullptr, cap, 0};
+        BM_CUDA(cudaMalloc(&b.p, cap));
+        blocks.push_back(b);
+    }
+    void clear() {
+        for (const Block &b : blocks) cudaFree(b.p);
+        blocks.clear();
+    }
+    ~Arena() {
+        clear();
+        if (pinned) cudaFreeHost(pinned);
+    }
+};
+
+namespace {
+std::mutex g_arena_mu;
+std::vector<Arena *> g_arenas;
+constexpr size_t MAX_ARENAS = 4, ARENA_BYTES = 256ull << 20;
+}  // namespace
+
+Workspace::Workspace(cudaStream_t st) : arena_(nullptr), st_(st) {
+    std::lock_guard<std::mutex> lock(g_arena_mu);
+    if (!g_arenas.empty()) {
+        arena_ = g_arenas.back();
+        g_arenas.pop_back();
+    } else {
+        arena_ = new Arena();
+    }
+}
+
+Workspace::~Workspace() {
+    if (!synced_) cudaStreamSynchronize(st_);
+    // what took several blocks gets one next time
+    const size_t total = arena_->total();
+    try {
+        if (arena_->blocks.size() > 1 || total > ARENA_BYTES) {
+            arena_->clear();
+            if (total <= ARENA_BYTES) arena_->add(total);
+        }
+    } catch (const Error &) {
+        cudaGetLastError();  // no memory to keep: the next call allocates what it needs
+    }
+    for (auto &b : arena_->blocks) b.used = 0;
+    std::lock_guard<std::mutex> lock(g_arena_mu);
+    if (g_arenas.size() < MAX_ARENAS) g_arenas.push_back(arena_);
+    else delete arena_;
+}
+
+void *Workspace::bytes(size_t count) {
+    if (!count) return nullptr;
+    count = (count + 255) / 256 * 256;
+    if (arena_->blocks.empty() || arena_->blocks.back().cap - arena_->blocks.back().used < count)
+        arena_->add(std::max<size_t>(count, 1u << 20));
+    Arena::Block &b = arena_->blocks.back();
+    void *p = b.p + b.used;
+    b.used += count;
+    return p;
+}
+
+void *Workspace::host() {
+    if (!arena_->pinned) BM_CUDA(cudaMallocHost(&arena_->pinned, PINNED));
+    return arena_->pinned;
+}
+
+void release_arenas() {
+    std::lock_guard<std::mutex> lock(g_arena_mu);
+    for (Arena *a : g_arenas) delete a;
+    g_arenas.clear();
+}
+
+// The CSR offsets to the host (synchronises).
+void read_offsets(Workspace &ws, std::vector<uint64_t> &off, const uint64_t *d_offsets, cudaStream_t st) {
+    const size_t bytes = off.size() * sizeof(uint64_t);
+    void *to = bytes <= Workspace::PINNED ? ws.host() : off.data();
+    BM_CUDA(cudaMemcpyAsync(to, d_offsets, bytes, cudaMemcpyDeviceToHost, st));
+    BM_CUDA(cudaStreamSynchronize(st));
+    if (to != off.data()) std::memcpy(off.data(), to, bytes);
 }
 
 void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
@@ -251,6 +411,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     std::lock_guard<std::mutex> scratch_lock(g_scratch_mu);
     const uint32_t m = S->m, n = S->n;
     cudaStream_t st = S->stream;
+    Workspace ws(st);
     const batmap_params &P = S->params;
     PhaseEvents &E = S->build_ev;
     E.create();
@@ -260,9 +421,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     std::vector<uint64_t> off(n + 1, 0);
     if (n) {
         BM_REQUIRE(d_offsets != nullptr, BATMAP_ERR_ARG, "d_offsets is NULL");
-        BM_CUDA(cudaMemcpyAsync(off.data(), d_offsets, (n + 1) * sizeof(uint64_t),
-                                cudaMemcpyDeviceToHost, st));
-        BM_CUDA(cudaStreamSynchronize(st));
+        read_offsets(ws, off, d_offsets, st);
     }
     BM_REQUIRE(off[0] == 0, BATMAP_ERR_ARG, "offsets[0] must be 0");
     for (uint32_t i = 0; i < n; i++)
@@ -283,18 +442,22 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         S->range[i] = 1u << rlog[i];
     }
     S->order.resize(n);
-    std::iota(S->order.begin(), S->order.end(), 0u);
     // width-sorted (stable by id); in cross mode family A [0, n_a) first
     const uint32_t na = S->n_a;
-    std::stable_sort(S->order.begin(), S->order.end(), [&](uint32_t a, uint32_t b) {
-        const bool fa = na && a >= na, fb = na && b >= na;
-        return fa != fb ? fb : rlog[a] < rlog[b];
-    });
+    {
+        uint32_t at[65] = {};
+        auto key = [&](uint32_t i) { return rlog[i] + (na && i >= na ? 32u : 0u); };
+        for (uint32_t i = 0; i < n; i++) at[key(i) + 1]++;
+        for (int k = 0; k < 64; k++) at[k + 1] += at[k];
+        for (uint32_t i = 0; i < n; i++) S->order[at[key(i)]++] = i;
+    }
     S->rank.assign(n, 0);
     S->byte_off.assign(n, 0);
     S->wshift_sorted.assign(n, 0);
-    std::vector<uint64_t> base(n, 0);
-    std::vector<uint32_t> line_off(n, 0);
+    // per-item arrays for the device: base (64 bits) | line_off | wshift | order | rlog | chunk0
+    std::vector<uint32_t> meta(7ull * n);
+    uint64_t *base = reinterpret_cast<uint64_t *>(meta.data());
+    uint32_t *line_off = meta.data() + 2ull * n, *chunk0 = meta.data() + 6ull * n;
     uint64_t pos = 0;
     S->class_begin.clear();
     for (uint32_t q = 0; q < n; q++) {
@@ -332,27 +495,21 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
 
     // ---- device metadata ----
     S->d_bm.alloc(S->bytes);
-    S->d_line_off.alloc(n);
-    S->d_wshift.alloc(n);
-    S->d_order.alloc(n);
-    if (n) {
-        BM_CUDA(cudaMemcpyAsync(S->d_line_off.p, line_off.data(), n * 4, cudaMemcpyHostToDevice, st));
-        BM_CUDA(cudaMemcpyAsync(S->d_wshift.p, S->wshift_sorted.data(), n * 4, cudaMemcpyHostToDevice, st));
-        BM_CUDA(cudaMemcpyAsync(S->d_order.p, S->order.data(), n * 4, cudaMemcpyHostToDevice, st));
-    }
-
-    // per-element chunks: block b handles elements [ch_start[b], +CHUNK) of item ch_item[b]
-    std::vector<uint32_t> ch_item;
-    std::vector<uint64_t> ch_start;
-    std::vector<uint32_t> chunk0(n);
+    uint32_t nch = 0;  // chunk b: CHUNK elements of one item
     for (uint32_t i = 0; i < n; i++) {
-        chunk0[i] = (uint32_t)ch_item.size();
-        for (uint64_t s = off[i]; s < off[i + 1]; s += CHUNK) {
-            ch_item.push_back(i);
-            ch_start.push_back(s);
-        }
+        chunk0[i] = nch;
+        nch += (uint32_t)((off[i + 1] - off[i] + CHUNK - 1) / CHUNK);
     }
-    const uint32_t nch = (uint32_t)ch_item.size();
+    if (n) {
+        std::copy(S->wshift_sorted.begin(), S->wshift_sorted.end(), meta.begin() + 3ull * n);
+        std::copy(S->order.begin(), S->order.end(), meta.begin() + 4ull * n);
+        std::copy(rlog.begin(), rlog.end(), meta.begin() + 5ull * n);
+        S->d_meta.alloc(meta.size());
+        S->d_line_off.p = S->d_meta.p + 2ull * n;
+        S->d_wshift.p = S->d_meta.p + 3ull * n;
+        S->d_order.p = S->d_meta.p + 4ull * n;
+        BM_CUDA(cudaMemcpyAsync(S->d_meta.p, meta.data(), meta.size() * 4, cudaMemcpyHostToDevice, st));
+    }
 
     S->d_fail_off.alloc(n + 1);
     if (T == 0) {
@@ -366,52 +523,54 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         return;
     }
 
-    DevBuf<uint32_t> d_ch_item(nch), d_rlog(n);
-    DevBuf<uint64_t> d_ch_start(nch), d_base(n);
-    BM_CUDA(cudaMemcpyAsync(d_ch_item.p, ch_item.data(), nch * 4ull, cudaMemcpyHostToDevice, st));
-    BM_CUDA(cudaMemcpyAsync(d_ch_start.p, ch_start.data(), nch * 8ull, cudaMemcpyHostToDevice, st));
-    BM_CUDA(cudaMemcpyAsync(d_rlog.p, rlog.data(), n * 4ull, cudaMemcpyHostToDevice, st));
-    BM_CUDA(cudaMemcpyAsync(d_base.p, base.data(), n * 8ull, cudaMemcpyHostToDevice, st));
-    ItemView v{d_offsets, d_tids, d_base.p, d_rlog.p, d_ch_item.p, d_ch_start.p};
+    const uint64_t *d_base = reinterpret_cast<const uint64_t *>(S->d_meta.p);
+    const uint32_t *d_chunk0 = S->d_meta.p + 6ull * n;
+    WsBuf<uint32_t> d_ch_item(ws, nch);
+    WsBuf<uint64_t> d_ch_start(ws, nch);
+    ItemView v{d_offsets, d_tids, d_base, S->d_meta.p + 5ull * n, d_ch_item.p, d_ch_start.p};
+    auto make_chunks = [&] {
+        k_chunks<<<n, 64, 0, st>>>(d_offsets, d_chunk0, d_ch_item.p, d_ch_start.p);
+        BM_CHECK_LAUNCH();
+    };
+    // what the host reads back: flags ([0] a bad list or permutation, [2], [3] the bit rows'), failed
+    // insertions, correction entries
+    struct Stat {
+        int err[4];
+        unsigned long long nfail, ncorr;
+    };
+    WsBuf<Stat> d_stat(ws, 1);
+    Stat *stat = static_cast<Stat *>(ws.host());
+    BM_CUDA(cudaMemsetAsync(d_stat.p, 0, sizeof(Stat), st));
 
-    // ---- bit rows (where the pair supports come from them) and validation ----
-    DevBuf<int> d_err(4);  // [0] a bad list or permutation, [2], [3] the bit rows' flags
-    BM_CUDA(cudaMemsetAsync(d_err.p, 0, 4 * sizeof(int), st));
-    plan_contract(S, d_offsets, d_tids, d_err.p + 2, P.validate != 0);
-    if (P.validate) {
-        DevBuf<uint32_t> d_bits(d_perm ? 3ull * ((m + 31) / 32) : 0);
-        if (d_perm) BM_CUDA(cudaMemsetAsync(d_bits.p, 0, d_bits.bytes(), st));
-        if (!S->contract) {  // the bit rows' build checks every list
-            k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_err.p);
-            BM_CHECK_LAUNCH();
-        }
-        if (d_perm) {  // computed permutations are bijections by construction
-            k_validate_perm<<<grid_for(3ull * m), 256, 0, st>>>(d_perm, m, 3, d_bits.p, d_err.p);
-            BM_CHECK_LAUNCH();
-        }
-        int err[4] = {0, 0, 0, 0};
-        BM_CUDA(cudaMemcpyAsync(err, d_err.p, sizeof(err), cudaMemcpyDeviceToHost, st));
-        BM_CUDA(cudaStreamSynchronize(st));
-        BM_REQUIRE(err[0] != 1 && !err[2] && !err[3], BATMAP_ERR_ARG,
-                   "tids must be strictly increasing per item and < m");
-        BM_REQUIRE(err[0] != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
+    // ---- bit rows (where the pair supports come from them) and validation; the placement is safe on
+    // lists and permutations that are refused behind it ----
+    plan_contract(S, d_offsets, d_tids, d_stat.p->err + 2, P.validate != 0);
+    if (P.validate && !S->contract) {  // (the bit rows' build checks every list)
+        make_chunks();
+        k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_stat.p->err);
+        BM_CHECK_LAUNCH();
+    }
+    if (P.validate && d_perm) {  // computed permutations are bijections by construction
+        WsBuf<uint32_t> d_bits(ws, 3ull * ((m + 31) / 32));
+        BM_CUDA(cudaMemsetAsync(d_bits.p, 0, d_bits.bytes(), st));
+        k_validate_perm<<<grid_for(3ull * m), 256, 0, st>>>(d_perm, m, 3, d_bits.p, d_stat.p->err);
+        BM_CHECK_LAUNCH();
     }
 
     // ---- placement and bytes ----
     {
         E.record(2, st);
-        DevBuf<uint64_t> bs(nch + 1), d_tot(1);
-        DevBuf<uint32_t> d_mask((uint64_t)nch * (CHUNK / 32)), d_chunk0(n);
+        WsBuf<uint64_t> bs(ws, nch + 1);
+        WsBuf<uint32_t> d_mask(ws, (uint64_t)nch * (CHUNK / 32));
         BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
-        BM_CUDA(cudaMemcpyAsync(d_chunk0.p, chunk0.data(), n * 4ull, cudaMemcpyHostToDevice, st));
         std::vector<PlaceItem> list(n);
         for (uint32_t i = 0; i < n; i++) list[i] = {i, rlog[i], off[i + 1] - off[i]};
-        DevBuf<uint32_t> d_list(n), d_queue(PLACE_QUEUES);
+        WsBuf<uint32_t> d_list(ws, n), d_queue(ws, PLACE_QUEUES);
         PlaceJob J{};
         J.off = d_offsets;
         J.tids = d_tids;
-        J.base = d_base.p;
-        J.chunk0 = d_chunk0.p;
+        J.base = d_base;
+        J.chunk0 = d_chunk0;
         J.shift = S->shift;
         J.max_moves = 3u * std::max<uint32_t>(P.max_loop, 1u);
         J.out = S->d_bm.p;
@@ -421,27 +580,44 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         enqueue_place(3, J, PV, std::move(list), d_list.p, st);
         E.record(3, st);
         // failed insertions, ordered by (item, tid): counted and marked by the placement
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, d_tot.p, 1);
+        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, reinterpret_cast<uint64_t *>(&d_stat.p->nfail), 1);
         BM_CHECK_LAUNCH();
-        uint64_t nfail = 0;
-        BM_CUDA(cudaMemcpyAsync(&nfail, d_tot.p, 8, cudaMemcpyDeviceToHost, st));
+        BM_CUDA(cudaMemsetAsync(S->d_fail_off.p, 0, (n + 1) * sizeof(uint64_t), st));
+        if (!S->skip_schedule && !S->contract) build_schedule(S);
+        E.record(4, st);
+        E.record(1, st);
+        BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(Stat), cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
+        if (P.validate) {
+            BM_REQUIRE(stat->err[0] != 1 && !stat->err[2] && !stat->err[3], BATMAP_ERR_ARG,
+                       "tids must be strictly increasing per item and < m");
+            BM_REQUIRE(stat->err[0] != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
+        }
+        const uint64_t nfail = stat->nfail;
         S->n_failed = nfail;
-        DevBuf<uint32_t> f_item(nfail);
+        WsBuf<uint32_t> f_item(ws, nfail);
         S->d_fail_tid.alloc(nfail);
         if (nfail) {
+            make_chunks();
             k_failures<<<nch, TPB, 0, st>>>(v, d_mask.p, bs.p, f_item.p, S->d_fail_tid.p);
             BM_CHECK_LAUNCH();
+            k_fail_offsets<<<(n + 1 + 255) / 256, 256, 0, st>>>(f_item.p, nfail, n, S->d_fail_off.p);
+            BM_CHECK_LAUNCH();
         }
-        k_fail_offsets<<<(n + 1 + 255) / 256, 256, 0, st>>>(f_item.p, nfail, n, S->d_fail_off.p);
-        BM_CHECK_LAUNCH();
 
         // ---- correction entries ----
         S->n_corr = 0;
-        if (nfail) {
+        if (nfail && S->contract && m <= (1u << 24) && nfail * n <= (1u << 24)) {
+            // supports count every element: only the number of entries is reported
+            WsBuf<uint32_t> seen(ws, m);
+            BM_CUDA(cudaMemsetAsync(seen.p, 0, seen.bytes(), st));
+            k_count_corrections<<<grid_for(32 * nfail), 256, 0, st>>>(S->d_fail_tid.p, nfail, S->d_bits.p, n, seen.p,
+                                                                      &d_stat.p->ncorr);
+            BM_CHECK_LAUNCH();
+        } else if (nfail) {
             const uint64_t nwords = (m + 31) / 32;
-            DevBuf<uint32_t> bits(nwords);
-            DevBuf<uint64_t> wrank(nwords + 1), d_nu(1);
+            WsBuf<uint32_t> bits(ws, nwords);
+            WsBuf<uint64_t> wrank(ws, nwords + 1), d_nu(ws, 1);
             BM_CUDA(cudaMemsetAsync(bits.p, 0, bits.bytes(), st));
             k_mark_failed<<<grid_for(nfail), 256, 0, st>>>(S->d_fail_tid.p, nfail, bits.p);
             BM_CHECK_LAUNCH();
@@ -451,8 +627,8 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
             uint64_t nu = 0;
             BM_CUDA(cudaMemcpyAsync(&nu, d_nu.p, 8, cudaMemcpyDeviceToHost, st));
             BM_CUDA(cudaStreamSynchronize(st));
-            DevBuf<uint64_t> fptr(nu + 1), cursor(nu + 1), d_sum(1);
-            DevBuf<uint32_t> fitems(nfail);
+            WsBuf<uint64_t> fptr(ws, nu + 1), cursor(ws, nu + 1), d_sum(ws, 1);
+            WsBuf<uint32_t> fitems(ws, nfail);
             BM_CUDA(cudaMemsetAsync(fptr.p, 0, fptr.bytes(), st));
             BM_CUDA(cudaMemsetAsync(cursor.p, 0, cursor.bytes(), st));
             k_count_per_tid<<<grid_for(nfail), 256, 0, st>>>(S->d_fail_tid.p, nfail, bits.p, wrank.p, fptr.p);
@@ -463,29 +639,30 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
                                                            wrank.p, fptr.p,
                                                            (unsigned long long *)cursor.p, fitems.p);
             BM_CHECK_LAUNCH();
-            DevBuf<unsigned long long> counter(1);
-            BM_CUDA(cudaMemsetAsync(counter.p, 0, 8, st));
-            k_corrections<false><<<nch, TPB, 0, st>>>(v, m, bits.p, wrank.p, fptr.p, fitems.p, counter.p,
+            k_corrections<false><<<nch, TPB, 0, st>>>(v, m, bits.p, wrank.p, fptr.p, fitems.p, &d_stat.p->ncorr,
                                                        nullptr);
             BM_CHECK_LAUNCH();
-            unsigned long long ncorr = 0;
-            BM_CUDA(cudaMemcpyAsync(&ncorr, counter.p, 8, cudaMemcpyDeviceToHost, st));
-            BM_CUDA(cudaStreamSynchronize(st));
-            S->n_corr = ncorr;
-            if (ncorr) {
-                S->d_corr.alloc(2 * ncorr);
-                BM_CUDA(cudaMemsetAsync(counter.p, 0, 8, st));
-                k_corrections<true><<<nch, TPB, 0, st>>>(v, m, bits.p, wrank.p, fptr.p, fitems.p,
-                                                          counter.p, S->d_corr.p);
-                BM_CHECK_LAUNCH();
+            if (!S->contract) {
+                BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(Stat), cudaMemcpyDeviceToHost, st));
+                BM_CUDA(cudaStreamSynchronize(st));
+                if (stat->ncorr) {
+                    S->d_corr.alloc(2 * stat->ncorr);
+                    BM_CUDA(cudaMemsetAsync(&d_stat.p->ncorr, 0, 8, st));
+                    k_corrections<true><<<nch, TPB, 0, st>>>(v, m, bits.p, wrank.p, fptr.p, fitems.p,
+                                                              &d_stat.p->ncorr, S->d_corr.p);
+                    BM_CHECK_LAUNCH();
+                }
             }
         }
+        if (nfail) {
+            E.record(4, st);
+            E.record(1, st);
+            BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(Stat), cudaMemcpyDeviceToHost, st));
+            BM_CUDA(cudaStreamSynchronize(st));
+            S->n_corr = stat->ncorr;
+        }
     }
-
-    E.record(4, st);
-    if (!S->skip_schedule && !S->contract) build_schedule(S);
-    E.record(1, st);
-    BM_CUDA(cudaStreamSynchronize(st));
+    ws.done();
     S->timing.build_ms = E.ms(0, 1);
     S->timing.place_ms = E.ms(2, 3);
     S->timing.finalize_ms = E.ms(3, 4);

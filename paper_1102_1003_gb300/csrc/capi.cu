@@ -189,6 +189,7 @@ void batmap_free(batmap_set *set) {
     if (!set) return;
     cudaStreamSynchronize(set->stream);
     release_batch_plan();  // a cached batch graph may point into this set
+    ReleaseScope released;
     delete set;
 }
 
@@ -248,7 +249,12 @@ static void pair_support_impl(batmap_set *S, uint32_t s, uint32_t *d_pairs, uint
         S->d_C.ensure(npairs);
         C = S->d_C.p;
     }
-    S->d_total.ensure(1);
+    Workspace ws(st);
+    uint64_t *d_total = reinterpret_cast<uint64_t *>(S->d_mm.p + 8);  // contract: beside the queue's state
+    if (!S->contract) {
+        S->d_total.ensure(1);
+        d_total = S->d_total.p;
+    }
     S->pairs_ev.create();
     S->pairs_ev.record(0, st);
     if (S->contract) {
@@ -263,14 +269,20 @@ static void pair_support_impl(batmap_set *S, uint32_t s, uint32_t *d_pairs, uint
         BM_CUDA(cudaMemcpyAsync(S->d_view.p, &h_view, sizeof(InstView), cudaMemcpyHostToDevice, st));
         enqueue_compare(S, C, S->d_view.p, st);  // records events 1, 2 around the launch
     }
-    enqueue_correct_compact(S, C, s, d_pairs, cap, S->d_total.p, st);
+    enqueue_correct_compact(S, C, s, d_pairs, cap, d_total, st);
     S->pairs_ev.record(3, st);
-    uint64_t total = 0;
-    uint32_t state[2] = {0, 0};
-    BM_CUDA(cudaMemcpyAsync(&total, S->d_total.p, 8, cudaMemcpyDeviceToHost, st));
-    if (S->contract) BM_CUDA(cudaMemcpyAsync(state, S->d_mm.p, sizeof(state), cudaMemcpyDeviceToHost, st));
+    struct Back {
+        uint32_t queue, timeout;
+        uint64_t total;
+    };
+    Back *back = static_cast<Back *>(ws.host());
+    back->timeout = 0;
+    if (S->contract) BM_CUDA(cudaMemcpyAsync(back, S->d_mm.p, sizeof(Back), cudaMemcpyDeviceToHost, st));
+    else BM_CUDA(cudaMemcpyAsync(&back->total, d_total, 8, cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaStreamSynchronize(st));
-    BM_REQUIRE(!state[1], BATMAP_ERR_TIMEOUT, "tensor-core kernel: a bounded pipeline wait timed out");
+    ws.done();
+    const uint64_t total = back->total;
+    BM_REQUIRE(!back->timeout, BATMAP_ERR_TIMEOUT, "tensor-core kernel: a bounded pipeline wait timed out");
     check_total(total);
     S->timing.compare_ms = S->pairs_ev.ms(1, 2);
     S->timing.scan_ms = S->contract ? 0.f : S->pairs_ev.ms(1, 4);

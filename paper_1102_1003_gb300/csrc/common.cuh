@@ -73,43 +73,80 @@ struct DevBuf {
     size_t bytes() const { return n * sizeof(T); }
 };
 
-// The large arrays of a built set come from a small cache: a freed set's
-// arrays (after a device synchronisation, as cudaFree would do) are kept for the
-// next build, at most six, reused when no larger than twice the request
-// plus 64 MiB, so repeated builds do not map and unmap hundreds of MB each.
+// The arrays of built sets come from a cache: a freed set's arrays (after a
+// device synchronisation, as cudaFree would do) are kept for the next build, at
+// most four of more than 64 MiB and 32 smaller ones, reused when no larger than
+// twice the request plus 1 MiB.  A small build makes about thirty allocations,
+// which cost more than its kernels.
 uint8_t *bm_buffer_take(size_t bytes, size_t *capacity);
 void bm_buffer_give(uint8_t *p, size_t capacity);
 void bm_buffer_release_all();
 
-struct BmBuf {
-    uint8_t *p = nullptr;
+// While one lives, arrays given back on this thread wait for no further work:
+// its constructor has waited for all of the device's.
+struct ReleaseScope {
+    ReleaseScope();
+    ~ReleaseScope();
+};
+
+template <typename T>
+struct CacheBuf {
+    T *p = nullptr;
     size_t n = 0, cap = 0;
-    BmBuf() = default;
-    BmBuf(const BmBuf &) = delete;
-    BmBuf &operator=(const BmBuf &) = delete;
-    ~BmBuf() { release(); }
-    void alloc(size_t bytes) {
+    CacheBuf() = default;
+    CacheBuf(const CacheBuf &) = delete;
+    CacheBuf &operator=(const CacheBuf &) = delete;
+    ~CacheBuf() { release(); }
+    void alloc(size_t count) {
         release();
-        if (bytes) p = bm_buffer_take(bytes, &cap);
-        n = bytes;
+        if (count) p = reinterpret_cast<T *>(bm_buffer_take(count * sizeof(T), &cap));
+        n = count;
     }
+    void ensure(size_t count) { if (count > n) alloc(count); }
     void release() {
-        if (p) bm_buffer_give(p, cap);
+        if (p) bm_buffer_give(reinterpret_cast<uint8_t *>(p), cap);
         p = nullptr;
         n = cap = 0;
     }
 };
+using BmBuf = CacheBuf<uint8_t>;
 
-// Events bracketing phases of a call on its stream.
+// Device scratch of one call that synchronises its stream before it returns:
+// pieces of an arena that the call holds alone and gives back (after waiting for
+// the stream, unless done() says it has) to at most four kept for later calls,
+// each of at most 256 MiB; batmap_release_scratch frees them.
+struct Arena;
+class Workspace {
+  public:
+    explicit Workspace(cudaStream_t st);
+    ~Workspace();
+    Workspace(const Workspace &) = delete;
+    Workspace &operator=(const Workspace &) = delete;
+    void *bytes(size_t count);  // nullptr for 0
+    void *host();               // PINNED bytes of pinned host memory, for what the call reads back
+    static constexpr size_t PINNED = 128 << 10;
+    void done() { synced_ = true; }
+
+  private:
+    Arena *arena_;
+    cudaStream_t st_;
+    bool synced_ = false;
+};
+template <typename T>
+struct WsBuf {
+    T *p;
+    size_t n;
+    WsBuf(Workspace &w, size_t count) : p(static_cast<T *>(w.bytes(count * sizeof(T)))), n(count) {}
+    size_t bytes() const { return n * sizeof(T); }
+};
+void release_arenas();
+
+// Events bracketing phases of a call on its stream (kept for later sets).
 struct PhaseEvents {
     static constexpr int N = 8;
     cudaEvent_t ev[N] = {};
     bool ok = false;
-    void create() {
-        if (ok) return;
-        for (int i = 0; i < N; i++) BM_CUDA(cudaEventCreate(&ev[i]));
-        ok = true;
-    }
+    void create();
     void record(int i, cudaStream_t st) { BM_CUDA(cudaEventRecord(ev[i], st)); }
     float ms(int a, int b) const {
         float t = 0.f;
@@ -119,10 +156,10 @@ struct PhaseEvents {
         }
         return t;
     }
-    ~PhaseEvents() {
-        if (ok)
-            for (int i = 0; i < N; i++) cudaEventDestroy(ev[i]);
-    }
+    PhaseEvents() = default;
+    PhaseEvents(const PhaseEvents &) = delete;
+    PhaseEvents &operator=(const PhaseEvents &) = delete;
+    ~PhaseEvents();
 };
 
 // ---- layout arithmetic (Sec. III-A) ----------------------------------------
@@ -211,18 +248,20 @@ struct batmap_set {
     bool mm_add = false;                  // its units add into zeroed supports
     uint32_t mm_count = 0, kblocks = 0;
     bm::BmBuf d_bits;                     // bit rows, original item order
-    bm::BmBuf d_mm;                       // queue counter and timeout flag (64 bytes), then the units
-    bm::DevBuf<uint32_t> d_line_off;      // [n] sorted
-    bm::DevBuf<uint32_t> d_wshift;        // [n] sorted
-    bm::DevBuf<uint32_t> d_order;         // [n]
-    bm::DevBuf<bm::WorkUnit> d_units;
-    bm::DevBuf<uint32_t> d_corr;          // [2 * n_corr] (i, j) original ids, i < j
-    bm::DevBuf<uint64_t> d_fail_off;      // [n+1] failed tids per item (CSR)
-    bm::DevBuf<uint32_t> d_fail_tid;      // [n_failed], sorted per item
+    bm::BmBuf d_mm;                       // queue counter, timeout flag, number of pairs (64 bytes); the units
+    bm::CacheBuf<uint32_t> d_meta;          // the per-item arrays of the build, one upload
+    struct DevPtr { uint32_t *p = nullptr; };
+    DevPtr d_line_off;                    // [n] sorted (in d_meta, as the next two)
+    DevPtr d_wshift;                      // [n] sorted
+    DevPtr d_order;                       // [n]
+    bm::CacheBuf<bm::WorkUnit> d_units;
+    bm::CacheBuf<uint32_t> d_corr;          // [2 * n_corr] (i, j) original ids, i < j
+    bm::CacheBuf<uint64_t> d_fail_off;      // [n+1] failed tids per item (CSR)
+    bm::CacheBuf<uint32_t> d_fail_tid;      // [n_failed], sorted per item
     // 3-of-4 sets (original item order): byte offsets, log2 r_i, own copy of pi_0..pi_3
-    bm::DevBuf<uint64_t> d_base;          // [n+1]
-    bm::DevBuf<uint32_t> d_rlog;          // [n]
-    bm::DevBuf<uint32_t> d_perm;          // [4 m] copy of the caller's table, if one was given
+    bm::CacheBuf<uint64_t> d_base;          // [n+1]
+    bm::CacheBuf<uint32_t> d_rlog;          // [n]
+    bm::CacheBuf<uint32_t> d_perm;          // [4 m] copy of the caller's table, if one was given
     bm::PermView perm{};                  // the set's pi_t (table view or computed)
 
     // timing of the most recent calls
@@ -230,9 +269,9 @@ struct batmap_set {
     batmap_timing timing{};
 
     // scratch reused across pair_support_all calls
-    bm::DevBuf<uint32_t> d_C;             // packed upper triangle when no d_full
-    bm::DevBuf<uint32_t> d_counters;      // work-queue counter
-    bm::DevBuf<bm::InstView> d_view;      // device copy of this set's InstView
-    bm::DevBuf<uint64_t> d_blocksums;     // compaction tile states
-    bm::DevBuf<uint64_t> d_total;         // compaction total
+    bm::CacheBuf<uint32_t> d_C;             // packed upper triangle when no d_full
+    bm::CacheBuf<uint32_t> d_counters;      // work-queue counter
+    bm::CacheBuf<bm::InstView> d_view;      // device copy of this set's InstView
+    bm::CacheBuf<uint64_t> d_blocksums;     // compaction tile states
+    bm::CacheBuf<uint64_t> d_total;         // compaction total
 };

@@ -56,6 +56,9 @@ inline unsigned grid_for(uint64_t work, unsigned tpb = 256) {
     return (unsigned)std::min<uint64_t>(std::max<uint64_t>(g, 1), 1u << 20);
 }
 
+// The CSR offsets (off.size() of them) to the host; synchronises the stream.
+void read_offsets(Workspace &ws, std::vector<uint64_t> &off, const uint64_t *d_offsets, cudaStream_t st);
+
 extern std::mutex g_scratch_mu;             // held for the duration of a build
 DevBuf<uint32_t> &scratch_table(uint64_t slots);
 

@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
             if (__any_sync(0xffffffffu, busy)) {
                 if (busy) {
                     if (!P.table) v = P.pass(P.key[idx % NT], v);
-                    if (v < P.m) {
+                    if (P.table || v < P.m) {
                         pos[idx] = (uint16_t)(v & rm);
                         code[idx] = (uint8_t)((v >> J.shift) + 1u);
                         busy = false;

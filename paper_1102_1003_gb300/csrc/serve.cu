@@ -427,6 +427,7 @@ static void intersect_list(const batmap_pool *pool, const uint32_t *qoff, const 
                            uint64_t *d_out_off, uint32_t *d_out, uint64_t cap, uint64_t *n_total, cudaStream_t st) {
     BM_REQUIRE(pool && qoff && n_total && d_out_off, BATMAP_ERR_ARG, "NULL argument");
     BM_REQUIRE(cap == 0 || d_out, BATMAP_ERR_ARG, "d_out is NULL with cap > 0");
+    Workspace ws(st);
     std::vector<QueryDesc> qs;
     std::vector<ProbeTask> tasks;
     if (nq) prepare_batch(pool, qoff, ids, 0, nq, &qs, &tasks);
@@ -434,10 +435,10 @@ static void intersect_list(const batmap_pool *pool, const uint32_t *qoff, const 
     std::vector<uint32_t> first(nq + 1, (uint32_t)nt);
     for (uint64_t t = nt; t-- > 0;) first[tasks[t].q] = (uint32_t)t;
     for (uint32_t q = nq; q-- > 0;) first[q] = std::min(first[q], first[q + 1]);
-    DevBuf<QueryDesc> d_q(std::max<uint64_t>(qs.size(), 1));
-    DevBuf<ProbeTask> d_t(std::max<uint64_t>(nt, 1));
-    DevBuf<uint64_t> d_toff(nt + 1), d_total(1);
-    DevBuf<uint32_t> d_first(nq + 1);
+    WsBuf<QueryDesc> d_q(ws, std::max<uint64_t>(qs.size(), 1));
+    WsBuf<ProbeTask> d_t(ws, std::max<uint64_t>(nt, 1));
+    WsBuf<uint64_t> d_toff(ws, nt + 1), d_total(ws, 1);
+    WsBuf<uint32_t> d_first(ws, nq + 1);
     if (nq) BM_CUDA(cudaMemcpyAsync(d_q.p, qs.data(), qs.size() * sizeof(QueryDesc), cudaMemcpyHostToDevice, st));
     if (nt) BM_CUDA(cudaMemcpyAsync(d_t.p, tasks.data(), nt * sizeof(ProbeTask), cudaMemcpyHostToDevice, st));
     BM_CUDA(cudaMemcpyAsync(d_first.p, first.data(), (nq + 1) * 4ull, cudaMemcpyHostToDevice, st));
@@ -457,6 +458,7 @@ static void intersect_list(const batmap_pool *pool, const uint32_t *qoff, const 
     uint64_t total = 0;
     BM_CUDA(cudaMemcpyAsync(&total, d_total.p, 8, cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaStreamSynchronize(st));
+    ws.done();
     *n_total = total;
     if (total > cap)
         throw Error{BATMAP_ERR_CAPACITY, "d_out too small: " + std::to_string(total) + " elements in the answers"};
@@ -473,23 +475,19 @@ struct Slot {
     uint64_t qcap = 0, tcap = 0;
     uint64_t q0 = 0, q1 = 0, work = 0;
     bool busy = false;
-    void init(uint64_t qc, uint64_t tc, bool own_stream, cudaStream_t shared) {
+    void init(uint64_t qc, uint64_t tc) {
         qcap = qc;
         tcap = tc;
-        if (own_stream) {
-            BM_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-        } else {
-            st = shared;
-        }
+        BM_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
         BM_CUDA(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
         BM_CUDA(cudaMallocHost(&h_q, qc * sizeof(QueryDesc)));
         BM_CUDA(cudaMallocHost(&h_t, tc * sizeof(ProbeTask)));
         d_q.alloc(qc);
         d_t.alloc(tc);
     }
-    void destroy(bool own_stream) {
+    void destroy() {
         if (done) cudaEventDestroy(done);
-        if (own_stream && st) cudaStreamDestroy(st);
+        if (st) cudaStreamDestroy(st);
         if (h_q) cudaFreeHost(h_q);
         if (h_t) cudaFreeHost(h_t);
         done = nullptr;
@@ -499,21 +497,25 @@ struct Slot {
     }
 };
 
+// Copies a batch's descriptors to the device and counts its answers (zeroed first).
+static void launch_probe(const batmap_pool *pool, const QueryDesc *qs, uint64_t nq, QueryDesc *d_q, const ProbeTask *tasks,
+                         uint64_t nt, ProbeTask *d_t, unsigned long long *d_counts, cudaStream_t st) {
+    BM_CUDA(cudaMemcpyAsync(d_q, qs, nq * sizeof(QueryDesc), cudaMemcpyHostToDevice, st));
+    if (nt) BM_CUDA(cudaMemcpyAsync(d_t, tasks, nt * sizeof(ProbeTask), cudaMemcpyHostToDevice, st));
+    BM_CUDA(cudaMemsetAsync(d_counts, 0, nq * sizeof(unsigned long long), st));
+    if (nt) {
+        const uint32_t warps_per_block = 8;
+        const uint64_t blocks = std::min<uint64_t>((nt + warps_per_block - 1) / warps_per_block, 4096);
+        k_probe<<<(unsigned)blocks, 32 * warps_per_block, 0, st>>>(pool->view, d_q, d_t, (uint32_t)nt, d_counts);
+        BM_CHECK_LAUNCH();
+    }
+}
+
 static void launch_batch(const batmap_pool *pool, Slot &S, const std::vector<QueryDesc> &qs,
                          const std::vector<ProbeTask> &tasks, unsigned long long *d_counts) {
     std::memcpy(S.h_q, qs.data(), qs.size() * sizeof(QueryDesc));
     if (!tasks.empty()) std::memcpy(S.h_t, tasks.data(), tasks.size() * sizeof(ProbeTask));
-    BM_CUDA(cudaMemcpyAsync(S.d_q.p, S.h_q, qs.size() * sizeof(QueryDesc), cudaMemcpyHostToDevice, S.st));
-    if (!tasks.empty())
-        BM_CUDA(cudaMemcpyAsync(S.d_t.p, S.h_t, tasks.size() * sizeof(ProbeTask), cudaMemcpyHostToDevice, S.st));
-    BM_CUDA(cudaMemsetAsync(d_counts + S.q0, 0, (S.q1 - S.q0) * sizeof(unsigned long long), S.st));
-    if (!tasks.empty()) {
-        const uint32_t warps_per_block = 8;
-        const uint64_t blocks = std::min<uint64_t>((tasks.size() + warps_per_block - 1) / warps_per_block, 4096);
-        k_probe<<<(unsigned)blocks, 32 * warps_per_block, 0, S.st>>>(pool->view, S.d_q.p, S.d_t.p,
-                                                                      (uint32_t)tasks.size(), d_counts + S.q0);
-        BM_CHECK_LAUNCH();
-    }
+    launch_probe(pool, S.h_q, qs.size(), S.d_q.p, S.h_t, tasks.size(), S.d_t.p, d_counts + S.q0, S.st);
     BM_CUDA(cudaEventRecord(S.done, S.st));
 }
 
@@ -524,19 +526,12 @@ static void intersect(const batmap_pool *pool, const uint32_t *qoff, const uint3
     std::vector<QueryDesc> qs;
     std::vector<ProbeTask> tasks;
     prepare_batch(pool, qoff, ids, 0, nq, &qs, &tasks);
-    Slot S;
-    S.init(nq, std::max<uint64_t>(tasks.size(), 1), false, st);
-    S.q0 = 0;
-    S.q1 = nq;
-    try {
-        launch_batch(pool, S, qs, tasks, d_counts);
-        BM_CUDA(cudaStreamSynchronize(st));
-    } catch (...) {
-        cudaStreamSynchronize(st);
-        S.destroy(false);
-        throw;
-    }
-    S.destroy(false);
+    Workspace ws(st);
+    WsBuf<QueryDesc> d_q(ws, nq);
+    WsBuf<ProbeTask> d_t(ws, tasks.size());
+    launch_probe(pool, qs.data(), nq, d_q.p, tasks.data(), tasks.size(), d_t.p, d_counts, st);
+    BM_CUDA(cudaStreamSynchronize(st));
+    ws.done();
 }
 
 // The continuous-batching request loop.  Queries arrive at h_arrival[q]
@@ -572,7 +567,7 @@ static void serve(const batmap_pool *pool, const uint32_t *qoff, const uint32_t 
     const uint64_t tcap = std::max<uint64_t>(max_tasks * 2, budget / TASK_ELEMS + (uint64_t)opt.max_batch);
     DevBuf<unsigned long long> d_counts(std::max<uint32_t>(nq, 1));
     std::vector<Slot> slots(opt.slots);
-    for (auto &s : slots) s.init(opt.max_batch, tcap, true, st);
+    for (auto &s : slots) s.init(opt.max_batch, tcap);
     std::vector<QueryDesc> qs;
     std::vector<ProbeTask> tasks;
     using clk = std::chrono::steady_clock;
@@ -647,13 +642,13 @@ static void serve(const batmap_pool *pool, const uint32_t *qoff, const uint32_t 
     } catch (...) {
         for (auto &s : slots) {
             if (s.st) cudaStreamSynchronize(s.st);
-            s.destroy(true);
+            s.destroy();
         }
         throw;
     }
     for (auto &s : slots) {
         cudaStreamSynchronize(s.st);
-        s.destroy(true);
+        s.destroy();
     }
 }
 

@@ -81,6 +81,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     std::lock_guard<std::mutex> scratch_lock(g_scratch_mu);
     const uint32_t m = S->m, n = S->n;
     cudaStream_t st = S->stream;
+    Workspace ws(st);
     const batmap_params &P = S->params;
     PhaseEvents &E = S->build_ev;
     E.create();
@@ -89,8 +90,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     std::vector<uint64_t> off(n + 1, 0);
     if (n) {
         BM_REQUIRE(d_offsets != nullptr, BATMAP_ERR_ARG, "d_offsets is NULL");
-        BM_CUDA(cudaMemcpyAsync(off.data(), d_offsets, (n + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
-        BM_CUDA(cudaStreamSynchronize(st));
+        read_offsets(ws, off, d_offsets, st);
     }
     BM_REQUIRE(off[0] == 0, BATMAP_ERR_ARG, "offsets[0] must be 0");
     for (uint32_t i = 0; i < n; i++)
@@ -143,8 +143,8 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
         }
     }
     const uint32_t nch = (uint32_t)ch_item.size();
-    DevBuf<uint32_t> d_ch_item(nch);
-    DevBuf<uint64_t> d_ch_start(nch);
+    WsBuf<uint32_t> d_ch_item(ws, nch);
+    WsBuf<uint64_t> d_ch_start(ws, nch);
     if (nch) {
         BM_CUDA(cudaMemcpyAsync(d_ch_item.p, ch_item.data(), nch * 4ull, cudaMemcpyHostToDevice, st));
         BM_CUDA(cudaMemcpyAsync(d_ch_start.p, ch_start.data(), nch * 8ull, cudaMemcpyHostToDevice, st));
@@ -155,7 +155,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     // has at least m / 16 (d = 3) or m / 6 (d = 4), and costs an AND and a popcount per 32
     // transactions, whatever the item's size.  tile, shape_mask or probe_log ask for the BatMap
     // kernels, as for pairs.
-    DevBuf<int> d_err(4);  // [0] a bad list or permutation, [2], [3] the bit rows' flags
+    WsBuf<int> d_err(ws, 4);  // [0] a bad list or permutation, [2], [3] the bit rows' flags
     BM_CUDA(cudaMemsetAsync(d_err.p, 0, 4 * sizeof(int), st));
     const BitsLayout BL = bits_row_major(m);
     S->kblocks = BL.kblocks;
@@ -163,7 +163,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     if (with_bits) enqueue_bits(d_offsets, d_tids, n, m, BL, S->d_bits.p, d_err.p + 2, P.validate != 0, st);
 
     if (P.validate) {
-        DevBuf<uint32_t> d_bits(d_perm ? (uint64_t)TABLES * ((m + 31) / 32) : 0);
+        WsBuf<uint32_t> d_bits(ws, d_perm ? (uint64_t)TABLES * ((m + 31) / 32) : 0);
         if (d_perm) BM_CUDA(cudaMemsetAsync(d_bits.p, 0, d_bits.bytes(), st));
         if (nch && !with_bits) {  // the bit rows' build checks every list
             k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_err.p);
@@ -184,9 +184,9 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     S->n_failed = 0;
     if (nch) {
         E.record(2, st);
-        DevBuf<uint64_t> bs(nch + 1), d_tot(1);
-        DevBuf<uint32_t> d_mask((uint64_t)nch * (CHUNK / 32)), d_queue(PLACE_QUEUES);
-        DevBuf<uint32_t> d_list(n), d_chunk0(n);
+        WsBuf<uint64_t> bs(ws, nch + 1), d_tot(ws, 1);
+        WsBuf<uint32_t> d_mask(ws, (uint64_t)nch * (CHUNK / 32)), d_queue(ws, PLACE_QUEUES);
+        WsBuf<uint32_t> d_list(ws, n), d_chunk0(ws, n);
         std::vector<PlaceItem> list(n);
         for (uint32_t i = 0; i < n; i++) list[i] = {i, rlog[i], off[i + 1] - off[i]};
         BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
@@ -210,7 +210,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
         BM_CUDA(cudaMemcpyAsync(&nfail, d_tot.p, 8, cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
         S->n_failed = nfail;
-        DevBuf<uint32_t> f_item(nfail);
+        WsBuf<uint32_t> f_item(ws, nfail);
         S->d_fail_tid.alloc(nfail);
         if (nfail) {
             k_failures<<<nch, TPB, 0, st>>>(v, d_mask.p, bs.p, f_item.p, S->d_fail_tid.p);
@@ -227,6 +227,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     }
     E.record(1, st);
     BM_CUDA(cudaStreamSynchronize(st));
+    ws.done();
     S->timing.build_ms = E.ms(0, 1);
     S->timing.place_ms = E.ms(2, 3);
     S->timing.finalize_ms = E.ms(3, 4);
@@ -1043,13 +1044,13 @@ static void launch_witness(const wit::View &V, uint32_t d, uint32_t k, const uin
 // the width-skewed candidates, the probe kernel takes them.  Records event 4
 // of E between the two.
 static void witness_routed5(const wit::View &V, uint32_t k, const uint32_t *d_items, uint64_t nq,
-                            const uint32_t *d_rlog, uint32_t *d_support, PhaseEvents &E, cudaStream_t st) {
+                            const uint32_t *d_rlog, uint32_t *d_support, PhaseEvents &E, Workspace &ws, cudaStream_t st) {
     using namespace wit;
     if (nq == 0) return;
     launch_witness(V, 4, k, d_items, nq, d_support, st, 1);
     E.record(4, st);
-    DevBuf<uint32_t> plist(nq);
-    DevBuf<unsigned long long> pcount(1);
+    WsBuf<uint32_t> plist(ws, nq);
+    WsBuf<unsigned long long> pcount(ws, 1);
     BM_CUDA(cudaMemsetAsync(pcount.p, 0, sizeof(unsigned long long), st));
     if (k == 3) k_route_probe_k<3, 5><<<grid_for(nq), 256, 0, st>>>(d_items, nq, d_rlog, plist.p, pcount.p);
     else k_route_probe_k<4, 5><<<grid_for(nq), 256, 0, st>>>(d_items, nq, d_rlog, plist.p, pcount.p);
@@ -1068,13 +1069,15 @@ void witness_support(batmap_set *S, uint32_t k, uint64_t nq, const uint32_t *d_i
     if (nq == 0) return;
     BM_REQUIRE(d_items && d_support, BATMAP_ERR_ARG, "NULL argument");
     {
-        DevBuf<int> err(1);
+        Workspace ws(st);
+        WsBuf<int> err(ws, 1);
         BM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
         k_check_ids<<<grid_for(nq * k), 256, 0, st>>>(d_items, nq * k, S->n, err.p);
         BM_CHECK_LAUNCH();
         int h = 0;
         BM_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
+        ws.done();
         BM_REQUIRE(h == 0, BATMAP_ERR_ARG, "item id >= n in a query");
     }
     if (S->d_bits.p) {
@@ -1100,48 +1103,49 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
     PhaseEvents &E = S->pairs_ev;
     E.create();
     E.record(0, st);
+    Workspace ws(st);
     const uint32_t n = S->n;
     uint64_t nc = 0, n_units = 0;
-    DevBuf<uint32_t> cand, sup;
-    DevBuf<uint2> units;
-    DevBuf<uint64_t> cnt;  // candidate offsets per frequent pair, [np + 1]
+    uint32_t *cand = nullptr, *sup = nullptr;
+    uint2 *units = nullptr;
+    uint64_t *cnt = nullptr;  // candidate offsets per frequent pair, [np + 1]
     if (np) {
-        DevBuf<int> err(1);
+        WsBuf<int> err(ws, 1);
         BM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
         k_check_pairs<<<grid_for(np), 256, 0, st>>>(d_pairs, np, n, err.p);
         BM_CHECK_LAUNCH();
-        DevBuf<uint64_t> row_off(n + 1), tot(1);
-        cnt.alloc(np + 1);
+        WsBuf<uint64_t> row_off(ws, n + 1), tot(ws, 1);
+        cnt = WsBuf<uint64_t>(ws, np + 1).p;
         k_rows<3><<<grid_for(n + 1), 256, 0, st>>>(d_pairs, np, n, row_off.p);
         BM_CHECK_LAUNCH();
         int h = 0;
         BM_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
         BM_REQUIRE(h == 0, BATMAP_ERR_ARG, "pairs must be (i, j, support) with i < j < n, lexicographic");
-        k_candidates<false><<<grid_for(32 * np), 256, 0, st>>>(d_pairs, np, row_off.p, cnt.p, nullptr);
+        k_candidates<false><<<grid_for(32 * np), 256, 0, st>>>(d_pairs, np, row_off.p, cnt, nullptr);
         BM_CHECK_LAUNCH();
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(cnt.p, np, tot.p, 1);  // cnt[np] = total
+        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(cnt, np, tot.p, 1);  // cnt[np] = total
         BM_CHECK_LAUNCH();
         BM_CUDA(cudaMemcpyAsync(&nc, tot.p, 8, cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
-        cand.alloc(3 * nc);
-        sup.alloc(nc);
+        cand = WsBuf<uint32_t>(ws, 3 * nc).p;
+        sup = WsBuf<uint32_t>(ws, nc).p;
         if (nc) {
-            k_candidates<true><<<grid_for(32 * np), 256, 0, st>>>(d_pairs, np, row_off.p, cnt.p, cand.p);
+            k_candidates<true><<<grid_for(32 * np), 256, 0, st>>>(d_pairs, np, row_off.p, cnt, cand);
             BM_CHECK_LAUNCH();
         }
         if (nc && grouped) {
             // work units of up to GROUP candidates sharing their frequent pair
-            DevBuf<uint64_t> uoff(np + 1), utot(1);
-            k_unit_counts<<<grid_for(np), 256, 0, st>>>(cnt.p, np, uoff.p);
+            WsBuf<uint64_t> uoff(ws, np + 1), utot(ws, 1);
+            k_unit_counts<<<grid_for(np), 256, 0, st>>>(cnt, np, uoff.p);
             BM_CHECK_LAUNCH();
             k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(uoff.p, np, utot.p, 1);
             BM_CHECK_LAUNCH();
             uint64_t nu = 0;
             BM_CUDA(cudaMemcpyAsync(&nu, utot.p, 8, cudaMemcpyDeviceToHost, st));
             BM_CUDA(cudaStreamSynchronize(st));
-            units.alloc(nu);
-            k_unit_fill<<<grid_for(np), 256, 0, st>>>(cnt.p, uoff.p, np, units.p);
+            units = WsBuf<uint2>(ws, nu).p;
+            k_unit_fill<<<grid_for(np), 256, 0, st>>>(cnt, uoff.p, np, units);
             BM_CHECK_LAUNCH();
             n_units = nu;
         }
@@ -1152,22 +1156,22 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
         const View V{reinterpret_cast<const uint32_t *>(S->d_bm.p), S->d_base.p, S->d_rlog.p, S->perm,
                      S->d_fail_off.p, S->d_fail_tid.p, S->m, S->n, S->shift};
         if (by_bits) {
-            enqueue_bits_support(S->d_bits.p, S->kblocks, 3, cand.p, nc, sup.p, st);
+            enqueue_bits_support(S->d_bits.p, S->kblocks, 3, cand, nc, sup, st);
         } else if (grouped) {
             const uint64_t wpb = WG_TPB / 32;
             const unsigned grid = (unsigned)std::min<uint64_t>((n_units + wpb - 1) / wpb, 152ull * 64);
-            k_witness_group<<<grid, WG_TPB, 0, st>>>(V, d_pairs, cnt.p, cand.p, units.p, n_units, sup.p);
+            k_witness_group<<<grid, WG_TPB, 0, st>>>(V, d_pairs, cnt, cand, units, n_units, sup);
             BM_CHECK_LAUNCH();
             E.record(4, st);
-            DevBuf<uint32_t> plist(nc);
-            DevBuf<unsigned long long> pcount(1);
+            WsBuf<uint32_t> plist(ws, nc);
+            WsBuf<unsigned long long> pcount(ws, 1);
             BM_CUDA(cudaMemsetAsync(pcount.p, 0, sizeof(unsigned long long), st));
-            k_route_probe<<<grid_for(nc), 256, 0, st>>>(cand.p, nc, S->d_rlog.p, plist.p, pcount.p);
+            k_route_probe<<<grid_for(nc), 256, 0, st>>>(cand, nc, S->d_rlog.p, plist.p, pcount.p);
             BM_CHECK_LAUNCH();
-            k_witness_probe<<<152 * 16, 256, 0, st>>>(V, cand.p, plist.p, pcount.p, sup.p);
+            k_witness_probe<<<152 * 16, 256, 0, st>>>(V, cand, plist.p, pcount.p, sup);
             BM_CHECK_LAUNCH();
         } else {
-            witness_routed5(V, 3, cand.p, nc, S->d_rlog.p, sup.p, E, st);  // one warp per candidate or probe
+            witness_routed5(V, 3, cand, nc, S->d_rlog.p, sup, E, ws, st);  // one warp per candidate or probe
         }
     }
     E.record(2, st);
@@ -1175,17 +1179,18 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
     if (nc) {
         const uint64_t per_block = (uint64_t)SCAN_TPB * TH_PER;
         const uint64_t nb = (nc + per_block - 1) / per_block;
-        DevBuf<uint64_t> bs(nb + 1), tot(1);
-        k_tuple_threshold<3, false><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand.p, sup.p, nc, s, bs.p, nullptr, 0);
+        WsBuf<uint64_t> bs(ws, nb + 1), tot(ws, 1);
+        k_tuple_threshold<3, false><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand, sup, nc, s, bs.p, nullptr, 0);
         BM_CHECK_LAUNCH();
         k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nb, tot.p, 1);
         BM_CHECK_LAUNCH();
-        k_tuple_threshold<3, true><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand.p, sup.p, nc, s, bs.p, d_out, cap);
+        k_tuple_threshold<3, true><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand, sup, nc, s, bs.p, d_out, cap);
         BM_CHECK_LAUNCH();
         BM_CUDA(cudaMemcpyAsync(&total, tot.p, 8, cudaMemcpyDeviceToHost, st));
     }
     E.record(3, st);
     BM_CUDA(cudaStreamSynchronize(st));
+    ws.done();
     S->timing.compare_ms = E.ms(1, 2);
     S->timing.compact_ms = E.ms(0, 1) + E.ms(2, 3);
     S->timing.pairs_ms = E.ms(0, 3);
@@ -1210,11 +1215,12 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
     PhaseEvents &E = S->pairs_ev;
     E.create();
     E.record(0, st);
+    Workspace ws(st);
     uint64_t nc = 0;
-    DevBuf<uint32_t> cand, sup;
+    uint32_t *cand = nullptr, *sup = nullptr;
     if (nt) {
-        DevBuf<int> err(1);
-        DevBuf<uint64_t> cnt(nt + 1), tot(1);
+        WsBuf<int> err(ws, 1);
+        WsBuf<uint64_t> cnt(ws, nt + 1), tot(ws, 1);
         BM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
         k_check_triples<<<grid_for(nt), 256, 0, st>>>(d_triples, nt, S->n, err.p);
         BM_CHECK_LAUNCH();
@@ -1222,7 +1228,7 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
         BM_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
         BM_REQUIRE(h == 0, BATMAP_ERR_ARG, "triples must be (a, b, c, support) with a < b < c < n, lexicographic");
-        DevBuf<uint64_t> row_off(S->n + 1);
+        WsBuf<uint64_t> row_off(ws, S->n + 1);
         k_rows<4><<<grid_for(S->n + 1), 256, 0, st>>>(d_triples, nt, S->n, row_off.p);
         BM_CHECK_LAUNCH();
         k_quad_candidates<false><<<grid_for(32 * nt), 256, 0, st>>>(d_triples, nt, row_off.p, cnt.p, nullptr);
@@ -1231,10 +1237,10 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
         BM_CHECK_LAUNCH();
         BM_CUDA(cudaMemcpyAsync(&nc, tot.p, 8, cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
-        cand.alloc(4 * nc);
-        sup.alloc(nc);
+        cand = WsBuf<uint32_t>(ws, 4 * nc).p;
+        sup = WsBuf<uint32_t>(ws, nc).p;
         if (nc) {
-            k_quad_candidates<true><<<grid_for(32 * nt), 256, 0, st>>>(d_triples, nt, row_off.p, cnt.p, cand.p);
+            k_quad_candidates<true><<<grid_for(32 * nt), 256, 0, st>>>(d_triples, nt, row_off.p, cnt.p, cand);
             BM_CHECK_LAUNCH();
         }
     }
@@ -1243,25 +1249,26 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
     if (nc) {
         const View V{reinterpret_cast<const uint32_t *>(S->d_bm.p), S->d_base.p, S->d_rlog.p, S->perm,
                      S->d_fail_off.p, S->d_fail_tid.p, S->m, S->n, S->shift};
-        if (S->d_bits.p) enqueue_bits_support(S->d_bits.p, S->kblocks, 4, cand.p, nc, sup.p, st);
-        else witness_routed5(V, 4, cand.p, nc, S->d_rlog.p, sup.p, E, st);
+        if (S->d_bits.p) enqueue_bits_support(S->d_bits.p, S->kblocks, 4, cand, nc, sup, st);
+        else witness_routed5(V, 4, cand, nc, S->d_rlog.p, sup, E, ws, st);
     }
     E.record(2, st);
     uint64_t total = 0;
     if (nc) {
         const uint64_t per_block = (uint64_t)SCAN_TPB * TH_PER;
         const uint64_t nb = (nc + per_block - 1) / per_block;
-        DevBuf<uint64_t> bs(nb + 1), tot(1);
-        k_tuple_threshold<4, false><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand.p, sup.p, nc, s, bs.p, nullptr, 0);
+        WsBuf<uint64_t> bs(ws, nb + 1), tot(ws, 1);
+        k_tuple_threshold<4, false><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand, sup, nc, s, bs.p, nullptr, 0);
         BM_CHECK_LAUNCH();
         k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nb, tot.p, 1);
         BM_CHECK_LAUNCH();
-        k_tuple_threshold<4, true><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand.p, sup.p, nc, s, bs.p, d_out, cap);
+        k_tuple_threshold<4, true><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand, sup, nc, s, bs.p, d_out, cap);
         BM_CHECK_LAUNCH();
         BM_CUDA(cudaMemcpyAsync(&total, tot.p, 8, cudaMemcpyDeviceToHost, st));
     }
     E.record(3, st);
     BM_CUDA(cudaStreamSynchronize(st));
+    ws.done();
     S->timing.compare_ms = E.ms(1, 2);
     const bool split = nc > 0 && !S->d_bits.p;  // event 4 sits between the scan and the probe kernels
     S->timing.scan_ms = split ? E.ms(1, 4) : 0.f;

@@ -9,8 +9,8 @@
 //     rows of a tile are one contiguous bulk copy per block;
 //   * a CTA computes 256 rows x 240 columns as two 128 x 240 tiles that share
 //     their B operand; per block of 256 transactions one bulk copy each brings
-//     the bits of the A and the B rows (15.5 KiB, 2-stage ring), sixteen
-//     expander warps turn them into e2m1 {0, 1} nibbles (1.0 = 0x2) in the
+//     the bits of the A and the B rows (15.5 KiB, 2-stage ring), two groups of
+//     eight expander warps, a block each in turn, turn them into e2m1 {0, 1} nibbles (1.0 = 0x2) in the
 //     128-byte-swizzled layout the MMA reads (62 KiB, 3-stage ring) and publish
 //     each stage after a proxy fence;
 //   * one thread issues tcgen05.mma.cta_group::1.kind::mxf4 (M = 128, N = 240,
@@ -25,10 +25,14 @@
 // accumulator represents exactly; partial sums of a split K are added as
 // integers.  INT8 MMA (kind::i8) is not available on sm_103a.
 //
-// What bounds it: shared-memory bandwidth (128 B/clk/SM).  A 128 x 240 x 64
-// MMA reads 11.5 KiB of operands, and the expanders write 31 KiB for two of
-// them.  With e4m3 operands (kind::f8f6f4, K = 32) the same bytes carry half
-// the K.
+// What bounds it: the MMA pipe, 173 clk per 128 x 240 x 64 with stale operands
+// (7.1 PFLOP/s), which the nibble stores slow to 217 (5.7): m = 2^22, n = 8,192
+// takes 54.4 ms, 43.3 without the stores.  Pairs of CTAs (cta_group::2), which
+// expand and read each B row once for two, were no faster (54.5 ms): the bytes
+// through shared memory (105 of 128 per clk here, 76 there) are not what counts.
+// One group of sixteen warps, a row per thread: 54.7 ms, and 0.36 instead of
+// 0.34 ms on short K (m = 25,000, n = 8,000).  e4m3 operands (kind::f8f6f4,
+// K = 32): 92 ms.
 //
 // Every mbarrier wait is bounded; on timeout the kernel records an error
 // flag, stops issuing work, waits (bounded) for what it issued, frees its
@@ -64,12 +68,17 @@ constexpr uint32_t BITS_STAGE = ROWS * BIT_ROW;    // 15.5 KiB
 constexpr int MMA_PER_STAGE = BITS_K / 64;         // K = 64 per MMA: 32 bytes of a row
 constexpr uint32_t TMEM_COLS = 512;                // accumulators at 0 and ACC1, scales at SFA, SFB
 constexpr uint32_t SFA = 240, SFB = 248, ACC1 = 256;
-constexpr int XW = 16;                             // expander warps 2 .. 17
-constexpr int THREADS = 64 + 32 * XW;              // warp 0 copies, warp 1 MMA
+constexpr int NG = 2, RPT = 2;                     // expander groups, a step each in turn; rows per thread
+constexpr int XW = (ROWS + 32 * RPT - 1) / (32 * RPT);  // warps of a group
+constexpr int EW = NG * XW;                        // warps 2 .. 17: expanders, then the epilogue
+constexpr int THREADS = 64 + 32 * EW;              // warp 0 copies, warp 1 MMA
 constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + (size_t)SB * BITS_STAGE + 1024 /*align*/ + 256;
 static_assert(SMEM <= 232448, "shared memory of one CTA");
 static_assert(A_BYTES % 1024 == 0 && STAGE_BYTES % 1024 == 0, "swizzle atoms");
-static_assert(XW * 32 * 33 * 4 <= STAGES * STAGE_BYTES, "epilogue staging fits the ring");
+static_assert(EW * 32 * 33 * 4 <= STAGES * STAGE_BYTES && EW % 4 == 0, "epilogue staging fits the ring");
+// a group waits for every use of its bits stages, a parity at a time; of the nibble stages its waits
+// are at most NG <= STAGES steps apart, so a parity never stands for an older use
+static_assert(SB % NG == 0 && NG <= STAGES, "barrier phases");
 constexpr uint32_t SPIN_LIMIT = 1u << 26;          // bounded waits (tens of ms per wait)
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -257,12 +266,12 @@ k_contract(const MmView *__restrict__ views, const MmView one, const MmUnit *__r
             }
             umma_commit(smem_addr(&bars[ACC]));  // accumulators ready (or nothing issued)
         } else if (warp >= 2) {
-            // expanders: thread t owns row t (A0 0..127, A1 128..255, B 256..495); row r of a stage
-            // starts at r * 128, 16-byte chunk c at c ^ (r & 7)
-            const uint32_t t = (uint32_t)threadIdx.x - 64;
-            const bool mine = t < (uint32_t)ROWS && (half1 || t < (uint32_t)BM || t >= 2u * BM);
+            // expanders: a thread owns rows t0 + 32 XW r (A0 0..127, A1 128..255, B 256..495); row r of a
+            // stage starts at r * 128, 16-byte chunk c at c ^ (r & 7)
+            const uint32_t grp = (uint32_t)(warp - 2) / XW, t0 = (uint32_t)((warp - 2) % XW) * 32u + lane;
             for (uint32_t it = 0; it < nk; it++) {
                 const uint32_t g = step0 + it, sb = g % SB, st = g % STAGES;
+                if (g % NG != grp) continue;
                 bool ok = !s_abort && mbar_wait(smem_addr(&bars[BF + sb]), (g / SB) & 1, spin);
                 if (ok && g >= (uint32_t)STAGES)
                     ok = mbar_wait(smem_addr(&bars[YE + st]), ((g / STAGES) - 1) & 1, spin);
@@ -271,7 +280,10 @@ k_contract(const MmView *__restrict__ views, const MmView one, const MmUnit *__r
                     s_abort = 1;
                     break;
                 }
-                if (mine) {
+#pragma unroll
+                for (int r = 0; r < RPT; r++) {
+                    const uint32_t t = t0 + (uint32_t)(32 * XW * r);
+                    if (t >= (uint32_t)ROWS || (!half1 && t >= (uint32_t)BM && t < 2u * BM)) continue;
                     const uint4 *src = reinterpret_cast<const uint4 *>(bits + sb * BITS_STAGE + t * BIT_ROW);
                     uint8_t *row = smem + st * STAGE_BYTES + t * ROW_BYTES;
                     const uint4 w0 = src[0], w1 = src[1];
@@ -301,7 +313,7 @@ k_contract(const MmView *__restrict__ views, const MmView one, const MmUnit *__r
                 uint32_t *stg = reinterpret_cast<uint32_t *>(smem) + (warp - 2) * (32 * 33);  // the MMAs are done
                 const uint64_t nn = V.n;
 #pragma unroll 1
-                for (uint32_t p = gq; p < 16; p += XW / 4) {
+                for (uint32_t p = gq; p < 16; p += EW / 4) {
                     const uint32_t h = p >> 3, c0 = (p & 7u) * 32u;
                     if (h && !half1) break;
                     const uint32_t gi0 = U.r0 + h * BM + q * 32u, gj = U.c0 + c0 + (uint32_t)lane;
@@ -363,7 +375,7 @@ k_contract(const MmView *__restrict__ views, const MmView one, const MmUnit *__r
 // ---- units -----------------------------------------------------------------------
 
 // Seconds of one K block of a 256 x 240 unit and of a unit's fill and epilogue.
-constexpr double MM_STEP_S = 0.75e-6, MM_UNIT_S = 8e-6, MM_LAUNCH_S = 10e-6;
+constexpr double MM_STEP_S = 0.84e-6, MM_UNIT_S = 8e-6, MM_LAUNCH_S = 10e-6;
 
 // Tiles holding a reported pair: row blocks of 256 from 0, column blocks of 240 from the first
 // column (cross: family B).

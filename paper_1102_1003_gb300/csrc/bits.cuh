@@ -70,7 +70,8 @@ void launch_contract(const MmView *d_views, const MmView &one, const MmUnit *d_u
 
 // Decides whether a set's pair supports come from its bit rows; if so, allocates
 // them and enqueues their build (d_flags as in enqueue_bits) and the units.
-void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids, int *d_flags, bool sorted_only);
+void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids, int *d_flags, bool sorted_only,
+                   cudaStream_t st);
 // Supports of all pairs of a set planned that way into C.
 void enqueue_contract(batmap_set *S, uint32_t *C, cudaStream_t st);
 MmView contract_view(const batmap_set *S, uint32_t *C);

@@ -397,6 +397,35 @@ void release_arenas() {
     g_arenas.clear();
 }
 
+// ---- side stream ----
+
+namespace {
+cudaStream_t g_side = nullptr;  // created at the first build, kept
+cudaEvent_t g_fork = nullptr, g_join = nullptr;
+}  // namespace
+
+SideStream::SideStream(cudaStream_t st) : st_(st) {
+    if (!g_side) {
+        BM_CUDA(cudaEventCreateWithFlags(&g_fork, cudaEventDisableTiming));
+        BM_CUDA(cudaEventCreateWithFlags(&g_join, cudaEventDisableTiming));
+        BM_CUDA(cudaStreamCreateWithFlags(&g_side, cudaStreamNonBlocking));
+    }
+    side_ = g_side;
+    BM_CUDA(cudaEventRecord(g_fork, st_));
+    BM_CUDA(cudaStreamWaitEvent(side_, g_fork, 0));
+}
+
+void SideStream::join() {
+    if (joined_) return;
+    joined_ = true;
+    BM_CUDA(cudaEventRecord(g_join, side_));
+    BM_CUDA(cudaStreamWaitEvent(st_, g_join, 0));
+}
+
+SideStream::~SideStream() {
+    if (!joined_) cudaStreamSynchronize(side_);  // an error on the way: nothing may outlive the call's memory
+}
+
 // The CSR offsets to the host (synchronises).
 void read_offsets(Workspace &ws, std::vector<uint64_t> &off, const uint64_t *d_offsets, cudaStream_t st) {
     const size_t bytes = off.size() * sizeof(uint64_t);
@@ -532,19 +561,17 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         k_chunks<<<n, 64, 0, st>>>(d_offsets, d_chunk0, d_ch_item.p, d_ch_start.p);
         BM_CHECK_LAUNCH();
     };
-    // what the host reads back: flags ([0] a bad list or permutation, [2], [3] the bit rows'), failed
-    // insertions, correction entries
-    struct Stat {
-        int err[4];
-        unsigned long long nfail, ncorr;
-    };
-    WsBuf<Stat> d_stat(ws, 1);
-    Stat *stat = static_cast<Stat *>(ws.host());
-    BM_CUDA(cudaMemsetAsync(d_stat.p, 0, sizeof(Stat), st));
+    WsBuf<BuildStat> d_stat(ws, 1);
+    BuildStat *stat = static_cast<BuildStat *>(ws.host());
+    BM_CUDA(cudaMemsetAsync(d_stat.p, 0, sizeof(BuildStat), st));
 
     // ---- bit rows (where the pair supports come from them) and validation; the placement is safe on
     // lists and permutations that are refused behind it ----
-    plan_contract(S, d_offsets, d_tids, d_stat.p->err + 2, P.validate != 0);
+    WsBuf<uint64_t> bs(ws, nch + 1);  // failed insertions per chunk
+    WsBuf<uint32_t> d_mask(ws, (uint64_t)nch * (CHUNK / 32));
+    BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
+    SideStream side(st);  // bit rows and the placement in shared memory, beside the placement in L2
+    plan_contract(S, d_offsets, d_tids, d_stat.p->err + 2, P.validate != 0, side.side());
     if (P.validate && !S->contract) {  // (the bit rows' build checks every list)
         make_chunks();
         k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_stat.p->err);
@@ -560,9 +587,6 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     // ---- placement and bytes ----
     {
         E.record(2, st);
-        WsBuf<uint64_t> bs(ws, nch + 1);
-        WsBuf<uint32_t> d_mask(ws, (uint64_t)nch * (CHUNK / 32));
-        BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
         std::vector<PlaceItem> list(n);
         for (uint32_t i = 0; i < n; i++) list[i] = {i, rlog[i], off[i + 1] - off[i]};
         WsBuf<uint32_t> d_list(ws, n), d_queue(ws, PLACE_QUEUES);
@@ -577,7 +601,8 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         J.fails = bs.p;
         J.mask = d_mask.p;
         J.queue = d_queue.p;
-        enqueue_place(3, J, PV, std::move(list), d_list.p, st);
+        enqueue_place(3, J, PV, std::move(list), d_list.p, st, side.side());
+        side.join();
         E.record(3, st);
         // failed insertions, ordered by (item, tid): counted and marked by the placement
         k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, reinterpret_cast<uint64_t *>(&d_stat.p->nfail), 1);
@@ -586,13 +611,9 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         if (!S->skip_schedule && !S->contract) build_schedule(S);
         E.record(4, st);
         E.record(1, st);
-        BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(Stat), cudaMemcpyDeviceToHost, st));
+        BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(BuildStat), cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
-        if (P.validate) {
-            BM_REQUIRE(stat->err[0] != 1 && !stat->err[2] && !stat->err[3], BATMAP_ERR_ARG,
-                       "tids must be strictly increasing per item and < m");
-            BM_REQUIRE(stat->err[0] != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
-        }
+        if (P.validate) stat->check();
         const uint64_t nfail = stat->nfail;
         S->n_failed = nfail;
         WsBuf<uint32_t> f_item(ws, nfail);
@@ -643,7 +664,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
                                                        nullptr);
             BM_CHECK_LAUNCH();
             if (!S->contract) {
-                BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(Stat), cudaMemcpyDeviceToHost, st));
+                BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(BuildStat), cudaMemcpyDeviceToHost, st));
                 BM_CUDA(cudaStreamSynchronize(st));
                 if (stat->ncorr) {
                     S->d_corr.alloc(2 * stat->ncorr);
@@ -657,7 +678,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         if (nfail) {
             E.record(4, st);
             E.record(1, st);
-            BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(Stat), cudaMemcpyDeviceToHost, st));
+            BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(BuildStat), cudaMemcpyDeviceToHost, st));
             BM_CUDA(cudaStreamSynchronize(st));
             S->n_corr = stat->ncorr;
         }

@@ -473,7 +473,8 @@ void launch_contract(const MmView *d_views, const MmView &one, const MmUnit *d_u
 // where they would take more than half of the free memory.
 constexpr double SCAN_WORD_PAIRS_PER_S = 7e12, SCAN_MIN_S = 40e-6, BITS_BYTES_PER_S = 4e12;
 
-void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids, int *d_flags, bool sorted_only) {
+void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids, int *d_flags, bool sorted_only,
+                   cudaStream_t st) {
     const batmap_params &P = S->params;
     S->contract = false;
     if (S->skip_schedule || P.tile || P.shape_mask || P.probe_log || !S->npairs() || !S->n_elements) return;
@@ -488,8 +489,8 @@ void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids,
     S->kblocks = L.kblocks;
     S->d_mm.alloc(64 + units.size() * sizeof(MmUnit));
     BM_CUDA(cudaMemcpyAsync(S->d_mm.p + 64, units.data(), units.size() * sizeof(MmUnit), cudaMemcpyHostToDevice,
-                            S->stream));
-    enqueue_bits(d_off, d_tids, S->n, S->m, L, S->d_bits.p, d_flags, sorted_only, S->stream);
+                            st));
+    enqueue_bits(d_off, d_tids, S->n, S->m, L, S->d_bits.p, d_flags, sorted_only, st);
     S->contract = true;
 }
 

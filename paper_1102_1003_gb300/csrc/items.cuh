@@ -59,6 +59,36 @@ inline unsigned grid_for(uint64_t work, unsigned tpb = 256) {
 // The CSR offsets (off.size() of them) to the host; synchronises the stream.
 void read_offsets(Workspace &ws, std::vector<uint64_t> &off, const uint64_t *d_offsets, cudaStream_t st);
 
+// What a build reads back: flags ([0] 1: a bad list, 2: a bad permutation; [2],
+// [3]: the bit rows' flags), failed insertions, correction entries.
+struct BuildStat {
+    int err[4];
+    unsigned long long nfail, ncorr;
+    void check() const {
+        BM_REQUIRE(err[0] != 1 && !err[2] && !err[3], BATMAP_ERR_ARG, "tids must be strictly increasing per item and < m");
+        BM_REQUIRE(err[0] != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
+    }
+};
+
+// Chunk b: elements [ch_start[b], + CHUNK) of item ch_item[b] (a block per item).
+__global__ void k_chunks(const uint64_t *off, const uint32_t *chunk0, uint32_t *ch_item, uint64_t *ch_start);
+
+// A second stream beside the call's, for the parts of a build that do not wait
+// on one another (used under g_scratch_mu).  Work enqueued on side() comes after
+// what `st` held at the fork; join() (or the end of the scope) makes `st` wait
+// for it.
+class SideStream {
+  public:
+    explicit SideStream(cudaStream_t st);
+    ~SideStream();
+    cudaStream_t side() const { return side_; }
+    void join();
+
+  private:
+    cudaStream_t st_, side_;
+    bool joined_ = false;
+};
+
 extern std::mutex g_scratch_mu;             // held for the duration of a build
 DevBuf<uint32_t> &scratch_table(uint64_t slots);
 

@@ -475,7 +475,7 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
 
 template <int NT>
 static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceItem> &list, uint32_t *d_list,
-                      cudaStream_t st) {
+                      cudaStream_t st, cudaStream_t side) {
     static const bool ready = [] {
         BM_CUDA(cudaFuncSetAttribute(k_place_small<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024));
         return true;
@@ -491,7 +491,7 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
     });
     std::vector<uint32_t> ids;
     for (const PlaceItem &I : list) ids.push_back(I.item);
-    BM_CUDA(cudaMemcpyAsync(d_list, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, st));
+    BM_CUDA(cudaMemcpyAsync(d_list, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, side));
     if (mid != list.begin()) place_large<NT>(job, P, std::vector<PlaceItem>(list.begin(), mid), st);
     uint32_t launch = 0;
     for (size_t k = mid - list.begin(); k < list.size();) {
@@ -507,7 +507,7 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
         // four elements a thread where the items fill their range
         const uint32_t tpb = std::min(1024u, std::max(128u, (1u << J.rlog) / 8u));
         const uint32_t fit = std::max(1u, std::min(2048u / tpb, 226u * 1024u / (smem + 1024u)));
-        k_place_small<NT><<<std::min(J.count, (uint32_t)device_sms() * fit), tpb, smem, st>>>(J, P, cap);
+        k_place_small<NT><<<std::min(J.count, (uint32_t)device_sms() * fit), tpb, smem, side>>>(J, P, cap);
         BM_CHECK_LAUNCH();
         k = e;
     }
@@ -516,12 +516,12 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
 }  // namespace place
 
 void enqueue_place(uint32_t tables, const PlaceJob &job, const PermView &P, std::vector<PlaceItem> list,
-                   uint32_t *d_list, cudaStream_t st) {
+                   uint32_t *d_list, cudaStream_t st, cudaStream_t side) {
     if (list.empty()) return;
-    BM_CUDA(cudaMemsetAsync(job.queue, 0, PLACE_QUEUES * sizeof(uint32_t), st));
-    if (tables == 3) place::place_all<3>(job, P, list, d_list, st);
-    if (tables == 4) place::place_all<4>(job, P, list, d_list, st);
-    if (tables == 5) place::place_all<5>(job, P, list, d_list, st);
+    BM_CUDA(cudaMemsetAsync(job.queue, 0, PLACE_QUEUES * sizeof(uint32_t), side));
+    if (tables == 3) place::place_all<3>(job, P, list, d_list, st, side);
+    if (tables == 4) place::place_all<4>(job, P, list, d_list, st, side);
+    if (tables == 5) place::place_all<5>(job, P, list, d_list, st, side);
 }
 
 __global__ void k_failures(ItemView v, const uint32_t *mask, const uint64_t *offsets, uint32_t *f_item, uint32_t *f_tid) {

@@ -132,65 +132,55 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     if (S->bytes && !T) BM_CUDA(cudaMemsetAsync(S->d_bm.p, 0, S->bytes, st));
     S->d_fail_off.alloc(n + 1);
 
-    std::vector<uint32_t> ch_item;
-    std::vector<uint64_t> ch_start;
+    uint32_t nch = 0;  // chunk b: CHUNK elements of one item
     std::vector<uint32_t> chunk0(n);
     for (uint32_t i = 0; i < n; i++) {
-        chunk0[i] = (uint32_t)ch_item.size();
-        for (uint64_t s0 = off[i]; s0 < off[i + 1]; s0 += CHUNK) {
-            ch_item.push_back(i);
-            ch_start.push_back(s0);
-        }
+        chunk0[i] = nch;
+        nch += (uint32_t)((off[i + 1] - off[i] + CHUNK - 1) / CHUNK);
     }
-    const uint32_t nch = (uint32_t)ch_item.size();
-    WsBuf<uint32_t> d_ch_item(ws, nch);
-    WsBuf<uint64_t> d_ch_start(ws, nch);
-    if (nch) {
-        BM_CUDA(cudaMemcpyAsync(d_ch_item.p, ch_item.data(), nch * 4ull, cudaMemcpyHostToDevice, st));
-        BM_CUDA(cudaMemcpyAsync(d_ch_start.p, ch_start.data(), nch * 8ull, cudaMemcpyHostToDevice, st));
-    }
+    WsBuf<uint32_t> d_ch_item(ws, nch), d_chunk0(ws, n);
+    WsBuf<uint64_t> d_ch_start(ws, nch), bs(ws, nch + 1);
+    WsBuf<uint32_t> d_mask(ws, (uint64_t)nch * (CHUNK / 32));
+    WsBuf<BuildStat> d_stat(ws, 1);
+    BuildStat *stat = static_cast<BuildStat *>(ws.host());
+    BM_CUDA(cudaMemsetAsync(d_stat.p, 0, sizeof(BuildStat), st));
+    BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
+    BM_CUDA(cudaMemsetAsync(S->d_fail_off.p, 0, (n + 1) * sizeof(uint64_t), st));
+    if (n) BM_CUDA(cudaMemcpyAsync(d_chunk0.p, chunk0.data(), n * 4ull, cudaMemcpyHostToDevice, st));
     ItemView v{d_offsets, d_tids, S->d_base.p, S->d_rlog.p, d_ch_item.p, d_ch_start.p};
+    auto make_chunks = [&] {
+        k_chunks<<<n, 64, 0, st>>>(d_offsets, d_chunk0.p, d_ch_item.p, d_ch_start.p);
+        BM_CHECK_LAUNCH();
+    };
 
     // bit rows for the k-way supports, in the items' order: a row is m / 8 bytes where the BatMap
     // has at least m / 16 (d = 3) or m / 6 (d = 4), and costs an AND and a popcount per 32
     // transactions, whatever the item's size.  tile, shape_mask or probe_log ask for the BatMap
-    // kernels, as for pairs.
-    WsBuf<int> d_err(ws, 4);  // [0] a bad list or permutation, [2], [3] the bit rows' flags
-    BM_CUDA(cudaMemsetAsync(d_err.p, 0, 4 * sizeof(int), st));
+    // kernels, as for pairs.  They and the placement in shared memory run beside the placement in
+    // L2, which is safe on lists and permutations that are refused behind it.
+    SideStream side(st);
     const BitsLayout BL = bits_row_major(m);
     S->kblocks = BL.kblocks;
     const bool with_bits = T && !P.tile && !P.shape_mask && !P.probe_log && take_bits(&S->d_bits, BL.row_stride * n);
-    if (with_bits) enqueue_bits(d_offsets, d_tids, n, m, BL, S->d_bits.p, d_err.p + 2, P.validate != 0, st);
-
-    if (P.validate) {
-        WsBuf<uint32_t> d_bits(ws, d_perm ? (uint64_t)TABLES * ((m + 31) / 32) : 0);
-        if (d_perm) BM_CUDA(cudaMemsetAsync(d_bits.p, 0, d_bits.bytes(), st));
-        if (nch && !with_bits) {  // the bit rows' build checks every list
-            k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_err.p);
-            BM_CHECK_LAUNCH();
-        }
-        if (d_perm) {  // computed permutations are bijections by construction
-            k_validate_perm<<<grid_for((uint64_t)TABLES * m), 256, 0, st>>>(d_perm, m, TABLES, d_bits.p, d_err.p);
-            BM_CHECK_LAUNCH();
-        }
-        int err[4] = {0, 0, 0, 0};
-        BM_CUDA(cudaMemcpyAsync(err, d_err.p, sizeof(err), cudaMemcpyDeviceToHost, st));
-        BM_CUDA(cudaStreamSynchronize(st));
-        BM_REQUIRE(err[0] != 1 && !err[2] && !err[3], BATMAP_ERR_ARG,
-                   "tids must be strictly increasing per item and < m");
-        BM_REQUIRE(err[0] != 2, BATMAP_ERR_ARG, "each permutation row must be a bijection of [0, m)");
+    if (with_bits) enqueue_bits(d_offsets, d_tids, n, m, BL, S->d_bits.p, d_stat.p->err + 2, P.validate != 0, side.side());
+    if (P.validate && nch && !with_bits) {  // (the bit rows' build checks every list)
+        make_chunks();
+        k_validate_tids<<<nch, TPB, 0, st>>>(v, m, d_stat.p->err);
+        BM_CHECK_LAUNCH();
+    }
+    if (P.validate && d_perm) {  // computed permutations are bijections by construction
+        WsBuf<uint32_t> d_bits(ws, (uint64_t)TABLES * ((m + 31) / 32));
+        BM_CUDA(cudaMemsetAsync(d_bits.p, 0, d_bits.bytes(), st));
+        k_validate_perm<<<grid_for((uint64_t)TABLES * m), 256, 0, st>>>(d_perm, m, TABLES, d_bits.p, d_stat.p->err);
+        BM_CHECK_LAUNCH();
     }
 
     S->n_failed = 0;
+    E.record(2, st);
     if (nch) {
-        E.record(2, st);
-        WsBuf<uint64_t> bs(ws, nch + 1), d_tot(ws, 1);
-        WsBuf<uint32_t> d_mask(ws, (uint64_t)nch * (CHUNK / 32)), d_queue(ws, PLACE_QUEUES);
-        WsBuf<uint32_t> d_list(ws, n), d_chunk0(ws, n);
         std::vector<PlaceItem> list(n);
         for (uint32_t i = 0; i < n; i++) list[i] = {i, rlog[i], off[i + 1] - off[i]};
-        BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
-        BM_CUDA(cudaMemcpyAsync(d_chunk0.p, chunk0.data(), n * 4ull, cudaMemcpyHostToDevice, st));
+        WsBuf<uint32_t> d_list(ws, n), d_queue(ws, PLACE_QUEUES);
         PlaceJob J{};
         J.off = d_offsets;
         J.tids = d_tids;
@@ -202,31 +192,33 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
         J.fails = bs.p;
         J.mask = d_mask.p;
         J.queue = d_queue.p;
-        enqueue_place(NT, J, PV, std::move(list), d_list.p, st);
-        E.record(3, st);
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, d_tot.p, 1);
+        enqueue_place(NT, J, PV, std::move(list), d_list.p, st, side.side());
+    }
+    side.join();
+    E.record(3, st);
+    if (nch) {
+        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, reinterpret_cast<uint64_t *>(&d_stat.p->nfail), 1);
         BM_CHECK_LAUNCH();
-        uint64_t nfail = 0;
-        BM_CUDA(cudaMemcpyAsync(&nfail, d_tot.p, 8, cudaMemcpyDeviceToHost, st));
-        BM_CUDA(cudaStreamSynchronize(st));
+    }
+    E.record(4, st);
+    E.record(1, st);
+    BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(BuildStat), cudaMemcpyDeviceToHost, st));
+    BM_CUDA(cudaStreamSynchronize(st));
+    if (P.validate) stat->check();
+    const uint64_t nfail = stat->nfail;
+    if (nfail) {
         S->n_failed = nfail;
         WsBuf<uint32_t> f_item(ws, nfail);
         S->d_fail_tid.alloc(nfail);
-        if (nfail) {
-            k_failures<<<nch, TPB, 0, st>>>(v, d_mask.p, bs.p, f_item.p, S->d_fail_tid.p);
-            BM_CHECK_LAUNCH();
-        }
+        make_chunks();
+        k_failures<<<nch, TPB, 0, st>>>(v, d_mask.p, bs.p, f_item.p, S->d_fail_tid.p);
+        BM_CHECK_LAUNCH();
         k_fail_offsets<<<(n + 1 + 255) / 256, 256, 0, st>>>(f_item.p, nfail, n, S->d_fail_off.p);
         BM_CHECK_LAUNCH();
         E.record(4, st);
-    } else {
-        BM_CUDA(cudaMemsetAsync(S->d_fail_off.p, 0, (n + 1) * sizeof(uint64_t), st));
-        E.record(2, st);
-        E.record(3, st);
-        E.record(4, st);
+        E.record(1, st);
+        BM_CUDA(cudaStreamSynchronize(st));
     }
-    E.record(1, st);
-    BM_CUDA(cudaStreamSynchronize(st));
     ws.done();
     S->timing.build_ms = E.ms(0, 1);
     S->timing.place_ms = E.ms(2, 3);

@@ -12,6 +12,7 @@
 
 #include "bits.cuh"
 #include "common.cuh"
+#include "scan.cuh"
 #include "compare.cuh"
 
 namespace bm {
@@ -19,7 +20,6 @@ namespace bm {
 void enqueue_correct_compact(batmap_set *S, uint32_t *C, uint32_t s, uint32_t *d_pairs, uint64_t cap,
                              uint64_t *d_total, cudaStream_t st);
 void prepare_compaction(batmap_set *S);
-void check_total(uint64_t total);
 
 struct BatchPlan {
     std::vector<uint64_t> key;

@@ -605,8 +605,8 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         side.join();
         E.record(3, st);
         // failed insertions, ordered by (item, tid): counted and marked by the placement
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, reinterpret_cast<uint64_t *>(&d_stat.p->nfail), 1);
-        BM_CHECK_LAUNCH();
+        WsBuf<uint64_t> scan_state(ws, scan_states(nch));
+        scan_with_tail(bs.p, nch, reinterpret_cast<uint64_t *>(&d_stat.p->nfail), scan_state.p, st);
         BM_CUDA(cudaMemsetAsync(S->d_fail_off.p, 0, (n + 1) * sizeof(uint64_t), st));
         if (!S->skip_schedule && !S->contract) build_schedule(S);
         E.record(4, st);
@@ -614,6 +614,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(BuildStat), cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
         if (P.validate) stat->check();
+        check_total(stat->nfail);
         const uint64_t nfail = stat->nfail;
         S->n_failed = nfail;
         WsBuf<uint32_t> f_item(ws, nfail);

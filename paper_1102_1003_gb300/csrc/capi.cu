@@ -8,6 +8,7 @@
 
 #include "bits.cuh"
 #include "common.cuh"
+#include "scan.cuh"
 #include "compare.cuh"
 
 namespace bm {
@@ -28,7 +29,6 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
                          uint64_t cap, uint64_t *n_out, uint64_t *n_cand, cudaStream_t st);
 void enqueue_correct_compact(batmap_set *S, uint32_t *C, uint32_t s, uint32_t *d_pairs, uint64_t cap,
                              uint64_t *d_total, cudaStream_t st);
-void check_total(uint64_t total);
 void run_batch(batmap_set *const *sets, const uint32_t *s, uint32_t k, batmap_out *outs, cudaStream_t st);
 void autotune(batmap_set *const *sets, uint32_t k, double *eff_out, cudaStream_t st);
 void release_scratch();

@@ -23,8 +23,6 @@ constexpr int CTPB = SCAN_TPB;
 constexpr int CQ = 4;                                // 16-byte loads per thread
 constexpr uint32_t CCHUNK = CTPB * 4 * CQ;           // 4,096 supports per tile
 constexpr uint32_t CSTAGE = CCHUNK / 2;              // triples staged at a time
-constexpr uint64_t STATE_SUM = 1ull << 62, STATE_PREFIX = 2ull << 62, STATE_VALUE = STATE_SUM - 1;
-constexpr uint32_t LOOKBACK_SPINS = 1u << 24;
 
 __global__ void k_apply_corrections(const uint32_t *__restrict__ corr, uint64_t ncorr, uint64_t n,
                                     uint32_t n_a, uint32_t *__restrict__ C) {
@@ -48,30 +46,6 @@ __device__ __forceinline__ uint32_t row_of(uint64_t L, uint64_t n, uint32_t n_a,
         if (row_start(mid, n, n_a) <= L) lo = mid; else hi = mid - 1;
     }
     return lo;
-}
-
-// Sum of the tiles before `tile` by the first warp (all lanes): looks back 32
-// states at a time.  ~0 if a predecessor's state did not come (bounded; the
-// predecessors run, as tiles are handed out in order).
-__device__ __forceinline__ uint64_t look_back(uint64_t *state, uint64_t tile, uint32_t lane) {
-    uint64_t sum = 0;
-    for (int64_t last = (int64_t)tile - 1; last >= 0; last -= 32) {
-        const int64_t at = last - lane;
-        uint64_t v = at < 0 ? STATE_PREFIX : 0;
-        for (uint32_t it = 0; !(v >> 62); it++) {
-            if (it == LOOKBACK_SPINS) break;
-            v = *(volatile uint64_t *)&state[at];
-        }
-        if (!__all_sync(0xffffffffu, (v >> 62) != 0)) return ~0ull;
-        const uint32_t done = __ballot_sync(0xffffffffu, (v >> 62) == 2);
-        const uint32_t upto = done ? __ffs(done) - 1 : 31;  // lanes behind a prefix do not count
-        uint64_t x = lane <= upto ? v & STATE_VALUE : 0;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
-        sum += x;
-        if (done) break;
-    }
-    return sum;
 }
 
 // state: one zeroed word per tile, then the zeroed tile counter.  *total <- the

@@ -54,7 +54,6 @@ namespace bm {
 
 void enqueue_threshold(const uint32_t *C, uint64_t n, uint32_t s, uint32_t *d_pairs, uint64_t cap,
                        DevBuf<uint64_t> *state, uint64_t *d_total, cudaStream_t st);
-void check_total(uint64_t total);
 
 namespace dense {
 

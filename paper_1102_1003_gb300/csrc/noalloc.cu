@@ -16,6 +16,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "scan.cuh"
 
 namespace bm {
 
@@ -23,7 +24,6 @@ namespace bm {
 uint64_t threshold_blocks(uint64_t n);
 void enqueue_threshold_into(const uint32_t *C, uint64_t n, uint32_t s, uint32_t *d_pairs, uint64_t cap,
                             uint64_t *state, uint64_t *d_total, cudaStream_t st);
-void check_total(uint64_t total);
 
 // Capacity of the fixed scratch: one 64-bit state per tile of 4096 pairs.
 constexpr uint64_t NOALLOC_BLOCK_PAIRS = 4096;

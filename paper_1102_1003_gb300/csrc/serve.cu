@@ -447,8 +447,8 @@ static void intersect_list(const batmap_pool *pool, const uint32_t *qoff, const 
         k_probe_count<<<blocks, 256, 0, st>>>(pool->view, d_q.p, d_t.p, (uint32_t)nt, d_toff.p);
         BM_CHECK_LAUNCH();
     }
-    k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(d_toff.p, nt, d_total.p, 1);
-    BM_CHECK_LAUNCH();
+    WsBuf<uint64_t> scan_state(ws, scan_states(nt));
+    scan_with_tail(d_toff.p, nt, d_total.p, scan_state.p, st);
     k_query_offsets<<<(nq + 1 + 255) / 256, 256, 0, st>>>(d_toff.p, d_first.p, nq, d_out_off);
     BM_CHECK_LAUNCH();
     if (nt && cap) {
@@ -459,6 +459,7 @@ static void intersect_list(const batmap_pool *pool, const uint32_t *qoff, const 
     BM_CUDA(cudaMemcpyAsync(&total, d_total.p, 8, cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaStreamSynchronize(st));
     ws.done();
+    check_total(total);
     *n_total = total;
     if (total > cap)
         throw Error{BATMAP_ERR_CAPACITY, "d_out too small: " + std::to_string(total) + " elements in the answers"};

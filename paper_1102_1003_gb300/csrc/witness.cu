@@ -197,14 +197,15 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     side.join();
     E.record(3, st);
     if (nch) {
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nch, reinterpret_cast<uint64_t *>(&d_stat.p->nfail), 1);
-        BM_CHECK_LAUNCH();
+        WsBuf<uint64_t> scan_state(ws, scan_states(nch));
+        scan_with_tail(bs.p, nch, reinterpret_cast<uint64_t *>(&d_stat.p->nfail), scan_state.p, st);
     }
     E.record(4, st);
     E.record(1, st);
     BM_CUDA(cudaMemcpyAsync(stat, d_stat.p, sizeof(BuildStat), cudaMemcpyDeviceToHost, st));
     BM_CUDA(cudaStreamSynchronize(st));
     if (P.validate) stat->check();
+    check_total(stat->nfail);
     const uint64_t nfail = stat->nfail;
     if (nfail) {
         S->n_failed = nfail;
@@ -1116,10 +1117,11 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
         BM_REQUIRE(h == 0, BATMAP_ERR_ARG, "pairs must be (i, j, support) with i < j < n, lexicographic");
         k_candidates<false><<<grid_for(32 * np), 256, 0, st>>>(d_pairs, np, row_off.p, cnt, nullptr);
         BM_CHECK_LAUNCH();
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(cnt, np, tot.p, 1);  // cnt[np] = total
-        BM_CHECK_LAUNCH();
+        WsBuf<uint64_t> tot_state(ws, scan_states(np));
+        scan_with_tail(cnt, np, tot.p, tot_state.p, st);  // cnt[np] = total
         BM_CUDA(cudaMemcpyAsync(&nc, tot.p, 8, cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
+        check_total(nc);
         cand = WsBuf<uint32_t>(ws, 3 * nc).p;
         sup = WsBuf<uint32_t>(ws, nc).p;
         if (nc) {
@@ -1131,11 +1133,12 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
             WsBuf<uint64_t> uoff(ws, np + 1), utot(ws, 1);
             k_unit_counts<<<grid_for(np), 256, 0, st>>>(cnt, np, uoff.p);
             BM_CHECK_LAUNCH();
-            k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(uoff.p, np, utot.p, 1);
-            BM_CHECK_LAUNCH();
+            WsBuf<uint64_t> utot_state(ws, scan_states(np));
+        scan_with_tail(uoff.p, np, utot.p, utot_state.p, st);
             uint64_t nu = 0;
             BM_CUDA(cudaMemcpyAsync(&nu, utot.p, 8, cudaMemcpyDeviceToHost, st));
             BM_CUDA(cudaStreamSynchronize(st));
+            check_total(nu);
             units = WsBuf<uint2>(ws, nu).p;
             k_unit_fill<<<grid_for(np), 256, 0, st>>>(cnt, uoff.p, np, units);
             BM_CHECK_LAUNCH();
@@ -1174,8 +1177,8 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
         WsBuf<uint64_t> bs(ws, nb + 1), tot(ws, 1);
         k_tuple_threshold<3, false><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand, sup, nc, s, bs.p, nullptr, 0);
         BM_CHECK_LAUNCH();
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nb, tot.p, 1);
-        BM_CHECK_LAUNCH();
+        WsBuf<uint64_t> tot_state(ws, scan_states(nb));
+        scan_with_tail(bs.p, nb, tot.p, tot_state.p, st);
         k_tuple_threshold<3, true><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand, sup, nc, s, bs.p, d_out, cap);
         BM_CHECK_LAUNCH();
         BM_CUDA(cudaMemcpyAsync(&total, tot.p, 8, cudaMemcpyDeviceToHost, st));
@@ -1189,6 +1192,7 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
     const bool split = nc > 0 && !by_bits;  // event 4 sits between the scan and the probe kernels
     S->timing.scan_ms = split ? E.ms(1, 4) : 0.f;
     S->timing.probe_ms = split ? E.ms(4, 2) : 0.f;
+    check_total(total);
     *n_out = total;
     if (total > cap)
         throw Error{BATMAP_ERR_CAPACITY, "d_out too small: " + std::to_string(total) + " triples qualify"};
@@ -1225,10 +1229,11 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
         BM_CHECK_LAUNCH();
         k_quad_candidates<false><<<grid_for(32 * nt), 256, 0, st>>>(d_triples, nt, row_off.p, cnt.p, nullptr);
         BM_CHECK_LAUNCH();
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(cnt.p, nt, tot.p, 1);
-        BM_CHECK_LAUNCH();
+        WsBuf<uint64_t> tot_state(ws, scan_states(nt));
+        scan_with_tail(cnt.p, nt, tot.p, tot_state.p, st);
         BM_CUDA(cudaMemcpyAsync(&nc, tot.p, 8, cudaMemcpyDeviceToHost, st));
         BM_CUDA(cudaStreamSynchronize(st));
+        check_total(nc);
         cand = WsBuf<uint32_t>(ws, 4 * nc).p;
         sup = WsBuf<uint32_t>(ws, nc).p;
         if (nc) {
@@ -1252,8 +1257,8 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
         WsBuf<uint64_t> bs(ws, nb + 1), tot(ws, 1);
         k_tuple_threshold<4, false><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand, sup, nc, s, bs.p, nullptr, 0);
         BM_CHECK_LAUNCH();
-        k_scan_single_block<<<1, SCAN_TPB, 0, st>>>(bs.p, nb, tot.p, 1);
-        BM_CHECK_LAUNCH();
+        WsBuf<uint64_t> tot_state(ws, scan_states(nb));
+        scan_with_tail(bs.p, nb, tot.p, tot_state.p, st);
         k_tuple_threshold<4, true><<<(unsigned)nb, SCAN_TPB, 0, st>>>(cand, sup, nc, s, bs.p, d_out, cap);
         BM_CHECK_LAUNCH();
         BM_CUDA(cudaMemcpyAsync(&total, tot.p, 8, cudaMemcpyDeviceToHost, st));
@@ -1267,6 +1272,7 @@ void frequent_quadruples(batmap_set *S, uint32_t s, const uint32_t *d_triples, u
     S->timing.probe_ms = split ? E.ms(4, 2) : 0.f;
     S->timing.compact_ms = E.ms(0, 1) + E.ms(2, 3);
     S->timing.pairs_ms = E.ms(0, 3);
+    check_total(total);
     *n_out = total;
     if (total > cap)
         throw Error{BATMAP_ERR_CAPACITY, "d_out too small: " + std::to_string(total) + " quadruples qualify"};

@@ -400,7 +400,7 @@ void release_arenas() {
 // ---- side stream ----
 
 namespace {
-cudaStream_t g_side = nullptr;  // created at the first build, kept
+cudaStream_t g_side = nullptr, g_more[SideStream::MORE];  // created at the first build, kept
 cudaEvent_t g_fork = nullptr, g_join = nullptr;
 }  // namespace
 
@@ -408,6 +408,7 @@ SideStream::SideStream(cudaStream_t st) : st_(st) {
     if (!g_side) {
         BM_CUDA(cudaEventCreateWithFlags(&g_fork, cudaEventDisableTiming));
         BM_CUDA(cudaEventCreateWithFlags(&g_join, cudaEventDisableTiming));
+        for (cudaStream_t &s : g_more) BM_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
         BM_CUDA(cudaStreamCreateWithFlags(&g_side, cudaStreamNonBlocking));
     }
     side_ = g_side;
@@ -415,15 +416,28 @@ SideStream::SideStream(cudaStream_t st) : st_(st) {
     BM_CUDA(cudaStreamWaitEvent(side_, g_fork, 0));
 }
 
+cudaStream_t SideStream::more(uint32_t i) {
+    BM_CUDA(cudaEventRecord(g_fork, st_));
+    BM_CUDA(cudaStreamWaitEvent(g_more[i], g_fork, 0));
+    used_ = i + 1;
+    return g_more[i];
+}
+
 void SideStream::join() {
     if (joined_) return;
-    joined_ = true;
     BM_CUDA(cudaEventRecord(g_join, side_));
     BM_CUDA(cudaStreamWaitEvent(st_, g_join, 0));
+    for (uint32_t i = 0; i < used_; i++) {
+        BM_CUDA(cudaEventRecord(g_join, g_more[i]));
+        BM_CUDA(cudaStreamWaitEvent(st_, g_join, 0));
+    }
+    joined_ = true;
 }
 
 SideStream::~SideStream() {
-    if (!joined_) cudaStreamSynchronize(side_);  // an error on the way: nothing may outlive the call's memory
+    if (joined_) return;  // an error on the way: nothing may outlive the call's memory
+    cudaStreamSynchronize(side_);
+    for (uint32_t i = 0; i < used_; i++) cudaStreamSynchronize(g_more[i]);
 }
 
 // The CSR offsets to the host (synchronises).
@@ -601,7 +615,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         J.fails = bs.p;
         J.mask = d_mask.p;
         J.queue = d_queue.p;
-        enqueue_place(3, J, PV, std::move(list), d_list.p, st, side.side());
+        enqueue_place(3, J, PV, std::move(list), d_list.p, side);
         side.join();
         E.record(3, st);
         // failed insertions, ordered by (item, tid): counted and marked by the placement

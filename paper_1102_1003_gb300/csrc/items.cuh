@@ -81,11 +81,15 @@ class SideStream {
   public:
     explicit SideStream(cudaStream_t st);
     ~SideStream();
+    cudaStream_t main() const { return st_; }
     cudaStream_t side() const { return side_; }
+    static constexpr uint32_t MORE = 1;
+    cudaStream_t more(uint32_t i);  // i < MORE: another, behind what the caller's stream holds now (called in order)
     void join();
 
   private:
     cudaStream_t st_, side_;
+    uint32_t used_ = 0;
     bool joined_ = false;
 };
 

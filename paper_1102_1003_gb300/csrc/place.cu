@@ -18,8 +18,9 @@
 //   - up to 8,192 slots per table (k_place_small): in the shared memory of one
 //     CTA, beside the item's slots in every table, computed once;
 //   - above (k_place_large): in L2.  Items go in batches, alternately through
-//     two regions of PLACE_L2_BYTES in all; a launch inserts one batch and forms
-//     the bytes of the batch before, so that long chains do not hold the chip
+//     two regions of PLACE_L2_BYTES in all (or two sequences of batches, two
+//     regions each); a launch inserts one batch and forms the bytes of the one
+//     before, so that long chains do not hold the chip
 //     up.  Bytes are formed slot by slot from a coalesced pass over the table:
 //     one load in another table per copy tells which tables hold the element (no
 //     byte is stored at random).  Entries carry an epoch above the tid, so a
@@ -38,6 +39,9 @@ namespace place {
 constexpr uint32_t SMALL_RLOG = 13;
 static_assert(SMALL_RLOG < PLACE_QUEUES, "a queue per width in shared memory");
 constexpr uint64_t PLACE_L2_BYTES = 96ull << 20;
+constexpr uint32_t SEQS = 2;
+constexpr uint64_t SEQ_REGION = 22ull << 20;
+static_assert(SEQS <= 1 + SideStream::MORE, "a stream for each");
 constexpr int LTPB = 128;
 constexpr uint32_t SUBS = LTPB / 32;                       // a warp per part of a CTA's task
 constexpr uint32_t A_SUB = 256, A_ELEMS = SUBS * A_SUB;    // elements of a warp's, a CTA's insertions
@@ -391,7 +395,8 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
 
 // The large items in order of the list (widest first): batches, places and tasks.
 template <int NT>
-static void place_large(const PlaceJob &job, const PermView &P, const std::vector<PlaceItem> &list, cudaStream_t st) {
+static void place_large(const PlaceJob &job, const PermView &P, const std::vector<PlaceItem> &list, SideStream &streams) {
+    cudaStream_t st = streams.main();
     uint32_t tbits = 1;
     while (tbits < 30 && (1ull << tbits) < P.m) tbits++;
     // the bits of pi_t(x) that its position does not give go along in the entry where there is room
@@ -401,7 +406,15 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     if (!known) hbits = 0;
     const uint32_t epochs = (1u << (32 - tbits - hbits)) - 1u;
     const uint64_t widest = (uint64_t)NT << list[0].rlog;  // words
-    const uint64_t region = std::max<uint64_t>(widest, PLACE_L2_BYTES / 4 / 2) / 64 * 64;  // (16-byte loads)
+    uint64_t total = 0;
+    for (const PlaceItem &I : list) total += (uint64_t)NT << I.rlog;
+    // Two sequences of launches where there are batches for both and room for their regions: the end of
+    // one's launch, a few long chains of exchanges, runs beside the body of the other's.  m = 2^22, 5%,
+    // n = 2,048 (6.3 MB an item): one sequence 21.0 ms, two with 4 items a region 19.4, with 3 items
+    // 17.9 (75 MB in use), three with 2 items 17.9; zipf m = 1 M, n = 2,000 (up to 25 MB) 2.2 and 2.0 ms.
+    const uint64_t part = std::max<uint64_t>(widest, SEQ_REGION / 4);
+    const uint32_t seqs = 2 * SEQS * part <= PLACE_L2_BYTES / 4 && total >= 2 * SEQS * part ? SEQS : 1;
+    const uint64_t region = (seqs > 1 ? part : std::max<uint64_t>(widest, PLACE_L2_BYTES / 4 / 2)) / 64 * 64;  // (16-byte loads)
     static const bool ready = [] {
         BM_CUDA(cudaFuncSetAttribute(k_place_large<NT, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LARGE_SMEM));
         BM_CUDA(cudaFuncSetAttribute(k_place_large<NT, uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LARGE_SMEM));
@@ -419,27 +432,27 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
         }
         const uint32_t b = (uint32_t)first.size() - 1;
         LargeItem &I = items[q];
-        I.table = (b & 1u) * region + fill;
+        I.table = b % (2 * seqs) * region + fill;
         I.item = list[q].item;
         I.rlog = list[q].rlog;
-        I.epoch = 1 + (b >> 1) % epochs;
+        I.epoch = 1 + b / (2 * seqs) % epochs;
         I.na = (uint32_t)((list[q].size + A_ELEMS - 1) / A_ELEMS);
         I.nb = (uint32_t)((words + B_SLOTS - 1) / B_SLOTS);
         fill += words;
     }
     const uint32_t nb = (uint32_t)first.size();
     first.push_back(list.size());
-    std::vector<uint64_t> start;  // first task of each launch
+    std::vector<uint64_t> start;  // first task of each launch: the insertions of batch b, the bytes of the one before in its sequence
     uint64_t pos = 0;
-    for (uint32_t b = 0; b <= nb; b++) {
+    for (uint32_t b = 0; b < nb + seqs; b++) {
         start.push_back(pos);
         if (b < nb)
             for (size_t q = first[b]; q < first[b + 1]; q++) {
                 items[q].first_a = (uint32_t)pos;
                 pos += items[q].na;
             }
-        if (b)
-            for (size_t q = first[b - 1]; q < first[b]; q++) {
+        if (b >= seqs && b - seqs < nb)
+            for (size_t q = first[b - seqs]; q < first[b - seqs + 1]; q++) {
                 items[q].first_b = (uint32_t)pos;
                 pos += items[q].nb;
             }
@@ -449,7 +462,7 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     // scratch words: drops (zeroed) | items | tasks | the regions
     auto up = [](uint64_t w) { return (w + 63) / 64 * 64; };
     const uint64_t o_items = up(items.size()), o_tasks = o_items + up(items.size() * sizeof(LargeItem) / 4),
-                   o_reg = o_tasks + up(pos * sizeof(LargeTask) / 4), regions = std::min<uint64_t>(nb, 2);
+                   o_reg = o_tasks + up(pos * sizeof(LargeTask) / 4), regions = std::min<uint64_t>(nb, 2 * seqs);
     uint32_t *w = scratch_table(o_reg + regions * region).p;
     BM_CUDA(cudaMemsetAsync(w, 0, o_items * 4, st));
     BM_CUDA(cudaMemcpyAsync(w + o_items, items.data(), items.size() * sizeof(LargeItem), cudaMemcpyHostToDevice, st));
@@ -457,10 +470,13 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     LargeTask *d_tasks = reinterpret_cast<LargeTask *>(w + o_tasks);
     k_large_tasks<<<(unsigned)items.size(), 128, 0, st>>>(d_items, d_tasks);
     BM_CHECK_LAUNCH();
-    for (uint32_t b = 0; b <= nb; b++) {
+    cudaStream_t seq[SEQS] = {st};
+    for (uint32_t c = 1; c < seqs; c++) seq[c] = streams.more(c - 1);
+    for (uint32_t b = 0; b < nb + seqs; b++) {
+        st = seq[b % seqs];
         // a region's first use, or all epochs used: clear it
-        if (b < nb && (b >> 1) % epochs == 0)
-            BM_CUDA(cudaMemsetAsync(w + o_reg + (b & 1u) * region, 0, region * 4, st));
+        if (b < nb && b / (2 * seqs) % epochs == 0)
+            BM_CUDA(cudaMemsetAsync(w + o_reg + b % (2 * seqs) * region, 0, region * 4, st));
         const unsigned grid = (unsigned)(start[b + 1] - start[b]);
         if (!grid) continue;
         if (list[0].rlog <= SLOT32_RLOG)
@@ -475,7 +491,8 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
 
 template <int NT>
 static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceItem> &list, uint32_t *d_list,
-                      cudaStream_t st, cudaStream_t side) {
+                      SideStream &streams) {
+    cudaStream_t side = streams.side();
     static const bool ready = [] {
         BM_CUDA(cudaFuncSetAttribute(k_place_small<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024));
         return true;
@@ -492,7 +509,7 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
     std::vector<uint32_t> ids;
     for (const PlaceItem &I : list) ids.push_back(I.item);
     BM_CUDA(cudaMemcpyAsync(d_list, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, side));
-    if (mid != list.begin()) place_large<NT>(job, P, std::vector<PlaceItem>(list.begin(), mid), st);
+    if (mid != list.begin()) place_large<NT>(job, P, std::vector<PlaceItem>(list.begin(), mid), streams);
     uint32_t launch = 0;
     for (size_t k = mid - list.begin(); k < list.size();) {
         size_t e = k;
@@ -516,12 +533,12 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
 }  // namespace place
 
 void enqueue_place(uint32_t tables, const PlaceJob &job, const PermView &P, std::vector<PlaceItem> list,
-                   uint32_t *d_list, cudaStream_t st, cudaStream_t side) {
+                   uint32_t *d_list, SideStream &streams) {
     if (list.empty()) return;
-    BM_CUDA(cudaMemsetAsync(job.queue, 0, PLACE_QUEUES * sizeof(uint32_t), side));
-    if (tables == 3) place::place_all<3>(job, P, list, d_list, st, side);
-    if (tables == 4) place::place_all<4>(job, P, list, d_list, st, side);
-    if (tables == 5) place::place_all<5>(job, P, list, d_list, st, side);
+    BM_CUDA(cudaMemsetAsync(job.queue, 0, PLACE_QUEUES * sizeof(uint32_t), streams.side()));
+    if (tables == 3) place::place_all<3>(job, P, list, d_list, streams);
+    if (tables == 4) place::place_all<4>(job, P, list, d_list, streams);
+    if (tables == 5) place::place_all<5>(job, P, list, d_list, streams);
 }
 
 __global__ void k_failures(ItemView v, const uint32_t *mask, const uint64_t *offsets, uint32_t *f_item, uint32_t *f_tid) {

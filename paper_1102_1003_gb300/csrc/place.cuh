@@ -20,15 +20,15 @@ struct PlaceJob {
 };
 
 // Places all items of the list (ids, any order; d_list: room for as many ids on
-// the device); tables: d + 1 (3, 4 or 5).  The wide ones go on `st`, the others on
-// `side`, which the caller joins.
+// the device); tables: d + 1 (3, 4 or 5).  The wide ones go on the caller's stream and
+// another, the rest on the side stream; the caller joins them.
 struct PlaceItem {
     uint32_t item, rlog;
     uint64_t size;
 };
 constexpr uint32_t PLACE_QUEUES = 64;
 void enqueue_place(uint32_t tables, const PlaceJob &job, const PermView &P, std::vector<PlaceItem> list,
-                   uint32_t *d_list, cudaStream_t st, cudaStream_t side);
+                   uint32_t *d_list, SideStream &streams);
 
 // F_i of every chunk with failures, in (item, tid) order: offsets[b] = first
 // entry of chunk b (exclusive scan of the counts, with the total behind it).

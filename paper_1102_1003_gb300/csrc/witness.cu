@@ -192,7 +192,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
         J.fails = bs.p;
         J.mask = d_mask.p;
         J.queue = d_queue.p;
-        enqueue_place(NT, J, PV, std::move(list), d_list.p, st, side.side());
+        enqueue_place(NT, J, PV, std::move(list), d_list.p, side);
     }
     side.join();
     E.record(3, st);

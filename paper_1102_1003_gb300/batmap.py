@@ -590,7 +590,7 @@ def intersect_query(pool: BatMapPool, queries, counts=None, stream=None):
 
 def intersect_query_list(pool: BatMapPool, queries, stream=None):
     """Elements of each query's intersection; returns (offsets int64 [nq+1], elements int32),
-    both cuda tensors.  Sizes the output with a first counting call."""
+    both cuda tensors.  Longer answers than the first call has room for take a second one."""
     import torch
     L = load_library()
     qoff, ids = _queries_csr(queries)
@@ -598,12 +598,14 @@ def intersect_query_list(pool: BatMapPool, queries, stream=None):
     off = torch.zeros(nq + 1, dtype=torch.int64, device="cuda")
     total = ctypes.c_uint64(0)
     st = _stream_handle(stream)
-    rc = L.intersect_query_list(pool.handle, qoff.ctypes.data, ids.ctypes.data, nq, _ptr(off), None, 0,
-                                ctypes.byref(total), st)
+    out = torch.empty(1 << 16, dtype=torch.int32, device="cuda")
+    rc = L.intersect_query_list(pool.handle, qoff.ctypes.data, ids.ctypes.data, nq, _ptr(off), _ptr(out),
+                                out.numel(), ctypes.byref(total), st)
     _check(rc, allow=(BATMAP_ERR_CAPACITY,))
-    out = torch.empty(max(int(total.value), 1), dtype=torch.int32, device="cuda")
-    _check(L.intersect_query_list(pool.handle, qoff.ctypes.data, ids.ctypes.data, nq, _ptr(off), _ptr(out),
-                                  out.numel(), ctypes.byref(total), st))
+    if int(total.value) > out.numel():
+        out = torch.empty(int(total.value), dtype=torch.int32, device="cuda")
+        _check(L.intersect_query_list(pool.handle, qoff.ctypes.data, ids.ctypes.data, nq, _ptr(off), _ptr(out),
+                                      out.numel(), ctypes.byref(total), st))
     return off, out[:int(total.value)]
 
 

@@ -584,6 +584,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     WsBuf<uint64_t> bs(ws, nch + 1);  // failed insertions per chunk
     WsBuf<uint32_t> d_mask(ws, (uint64_t)nch * (CHUNK / 32));
     BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
+    const PermView place_perm = place_perms(PV, 3, off[n], ws, st);
     SideStream side(st);  // bit rows and the placement in shared memory, beside the placement in L2
     plan_contract(S, d_offsets, d_tids, d_stat.p->err + 2, P.validate != 0, side.side());
     if (P.validate && !S->contract) {  // (the bit rows' build checks every list)
@@ -615,7 +616,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         J.fails = bs.p;
         J.mask = d_mask.p;
         J.queue = d_queue.p;
-        enqueue_place(3, J, PV, std::move(list), d_list.p, side);
+        enqueue_place(3, J, place_perm, std::move(list), d_list.p, side);
         side.join();
         E.record(3, st);
         // failed insertions, ordered by (item, tid): counted and marked by the placement

@@ -532,6 +532,28 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
 
 }  // namespace place
 
+__global__ void k_perm_table(const __grid_constant__ PermView P, uint32_t tables, uint32_t *__restrict__ out) {
+    const uint64_t total = (uint64_t)tables * P.m;
+    for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < total; k += (uint64_t)gridDim.x * blockDim.x)
+        out[k] = place::pi_of(P, (uint32_t)(k / P.m), (uint32_t)(k % P.m));
+}
+
+// A pass of the network is about 50 instructions.  Where 2^b is near m a warp takes one or
+// two of them, 450 to 800 G/s; at 2^b = 2.6 m its slowest lane takes eight or nine, 100 G/s,
+// against 272 G/s loads in L2.  So from 2^b = 1.5 m on, where the table stays small beside
+// the batches in L2 and is read far more often than it is long.  n = 8,000, m = 25,000
+// (2^16): 1474 -> 1200 us with the supports; triples and quadruples of n = 1,000,
+// m = 100,000 (2^18): 2168 -> 1824 and 3367 -> 2683 us.
+PermView place_perms(const PermView &P, uint32_t tables, uint64_t total, Workspace &ws, cudaStream_t st) {
+    if (P.table || 2 * (1ull << (2 * P.half)) < 3ull * P.m || 4ull * tables * P.m > (16u << 20) || total < 16ull * P.m) return P;
+    PermView T = P;
+    WsBuf<uint32_t> table(ws, (uint64_t)tables * P.m);
+    k_perm_table<<<(unsigned)std::min<uint64_t>(((uint64_t)tables * P.m + 255) / 256, 4096), 256, 0, st>>>(P, tables, table.p);
+    BM_CHECK_LAUNCH();
+    T.table = table.p;
+    return T;
+}
+
 void enqueue_place(uint32_t tables, const PlaceJob &job, const PermView &P, std::vector<PlaceItem> list,
                    uint32_t *d_list, SideStream &streams) {
     if (list.empty()) return;

@@ -30,6 +30,10 @@ constexpr uint32_t PLACE_QUEUES = 64;
 void enqueue_place(uint32_t tables, const PlaceJob &job, const PermView &P, std::vector<PlaceItem> list,
                    uint32_t *d_list, SideStream &streams);
 
+// The permutations that the placement of `total` elements reads: a table in ws, written on
+// st, where computing them by cycle walking costs more, else P.
+PermView place_perms(const PermView &P, uint32_t tables, uint64_t total, Workspace &ws, cudaStream_t st);
+
 // F_i of every chunk with failures, in (item, tid) order: offsets[b] = first
 // entry of chunk b (exclusive scan of the counts, with the total behind it).
 __global__ void k_failures(ItemView v, const uint32_t *mask, const uint64_t *offsets, uint32_t *f_item, uint32_t *f_tid);

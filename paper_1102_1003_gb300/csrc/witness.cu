@@ -158,6 +158,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     // transactions, whatever the item's size.  tile, shape_mask or probe_log ask for the BatMap
     // kernels, as for pairs.  They and the placement in shared memory run beside the placement in
     // L2, which is safe on lists and permutations that are refused behind it.
+    const PermView place_perm = place_perms(PV, NT, T, ws, st);
     SideStream side(st);
     const BitsLayout BL = bits_row_major(m);
     S->kblocks = BL.kblocks;
@@ -192,7 +193,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
         J.fails = bs.p;
         J.mask = d_mask.p;
         J.queue = d_queue.p;
-        enqueue_place(NT, J, PV, std::move(list), d_list.p, side);
+        enqueue_place(NT, J, place_perm, std::move(list), d_list.p, side);
     }
     side.join();
     E.record(3, st);

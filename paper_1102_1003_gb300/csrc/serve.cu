@@ -12,12 +12,12 @@
 // a binary search of the set's failed insertions; a set without a BatMap is
 // searched in two levels: a sampled index of every IDX_STRIDE-th tid of each
 // set (1/64 of the tidlists, small enough that its upper levels stay in L2)
-// narrows the search to one block of IDX_STRIDE tids (256 contiguous bytes),
-// so a membership test takes about two dependent DRAM reads instead of one per
-// level of a binary search over the whole tidlist.
+// narrows the search to one block of IDX_STRIDE tids (256 contiguous bytes).
+// Where the other set is not much larger than the smallest one, its tids between
+// a task's first and last element are read once instead, whichever form it has.
 //
-// Work is cut into tasks of up to 1024 elements of the smallest set; one warp
-// runs a task and adds its count with one atomic.
+// Work is cut into tasks of up to 512 elements of the smallest set; one warp
+// runs a task.
 #include <algorithm>
 #include <chrono>
 #include <memory>
@@ -32,7 +32,7 @@ namespace bm {
 
 void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids, const uint32_t *d_perm);
 
-constexpr uint32_t TASK_ELEMS = 1024;
+constexpr uint32_t TASK_ELEMS = 512;
 constexpr uint32_t MAX_K = 8;
 constexpr uint32_t IDX_STRIDE = 64;  // tids per block of the sampled index
 
@@ -61,6 +61,179 @@ struct PoolView {
     const uint32_t *idx;      // entry j of set c = tid IDX_STRIDE * j of set c
 };
 
+// ---- one task: the elements of a range of the smallest set that all others hold ----
+// A warp keeps the task's elements in shared memory and one bit per element in
+// registers: bit j of a lane's word is element 32 j + lane.
+//
+// Against one more set, whose tids between the task's first and last element
+// ("window") are found by two 32-way searches of the sampled index:
+// stream: the window goes through shared memory once, PART tids at a time with the
+//   next on their way; the elements up to a chunk's last tid are searched in it,
+//   four of a lane at once.  Where the window has up to STREAM tids per element.
+// search: each element by itself, four of a lane at once: a sample of the window's
+//   index entries in shared memory, then at most the block of IDX_STRIDE tids.
+// bytes: sets with a BatMap, two byte probes and the failed insertions.
+// Bound: instruction issue (56% of it at 24% occupancy) and the latency of a task's
+// first reads.  4096 queries over 4000 sets of 10..10^6 tids (51 M elements, 0.6 GB of
+// windows), a call: 1200 us with one element at a time, its 20 dependent reads 32
+// times in a row; 610 us; 540 us with shorter tasks in smaller blocks (here).  STREAM 4,
+// 8, 16, 32, 64: 803, 691, 629, 610, 620 us.  The lists of 256: 874 -> 245 us, as the
+// write pass probed again and the binding called twice.
+constexpr uint32_t PROBE_WARPS = 2, WIN = 512, PART = 512;
+constexpr uint32_t STREAM = 32;
+
+struct ProbeShared {
+    uint32_t x[TASK_ELEMS + 4];  // from a 16-byte boundary of the set on
+    union {
+        uint32_t chunk[2][PART];  // stream
+        uint32_t win[WIN];         // search
+    };
+};
+
+// 16-byte asynchronous copies of p's `quads` quads by a warp, one group.
+__device__ __forceinline__ void copy_quads(uint32_t *to, const uint32_t *from, uint32_t quads, uint32_t lane) {
+    for (uint32_t q = lane; q < quads; q += 32)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to + 4 * q)),
+                     "l"(from + 4 * q)
+                     : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void copies_wait() {  // all but the last N groups are there
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+    __syncwarp();
+}
+
+// Numbers of entries <= v0 and <= v1 of the ascending a[0..n), by a warp.
+__device__ __forceinline__ void count_le(const uint32_t *__restrict__ a, uint32_t n, uint32_t v0, uint32_t v1,
+                                         uint32_t lane, uint32_t &c0, uint32_t &c1) {
+    uint32_t lo[2] = {0, 0}, hi[2] = {n, n};
+    const uint32_t v[2] = {v0, v1};
+    while (hi[0] - lo[0] || hi[1] - lo[1]) {
+        uint32_t x[2], at[2];
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const uint32_t span = hi[q] - lo[q];
+            at[q] = span > 32 ? (uint32_t)((uint64_t)span * (lane + 1) / 33) : lane;  // ascending, < span (or no lane)
+            x[q] = at[q] < span ? __ldg(&a[lo[q] + at[q]]) : 0xffffffffu;
+        }
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const uint32_t span = hi[q] - lo[q];
+            const uint32_t c = __popc(__ballot_sync(0xffffffffu, at[q] < span && x[q] <= v[q]));
+            const uint32_t below = __shfl_sync(0xffffffffu, at[q], c ? c - 1 : 0);
+            const uint32_t above = __shfl_sync(0xffffffffu, at[q], c < 32 ? c : 31);
+            if (!span) continue;
+            if (c < 32 && above < span) hi[q] = lo[q] + above;
+            if (c) lo[q] += below + 1;
+        }
+    }
+    c0 = lo[0];
+    c1 = lo[1];
+}
+
+// x: the task's n elements, of which [from, to) of the tids may hold some.
+__device__ __forceinline__ uint32_t stream_members(const PoolView &P, ProbeShared &S, const uint32_t *x, uint32_t n,
+                                                   uint32_t alive, uint64_t from, uint64_t to, uint32_t lane) {
+    const uint32_t rows = (n + 31) / 32, top = x[n - 1];
+    uint32_t kept = 0, row = 0, skip = (uint32_t)(from & 3);
+    int32_t past = -1;  // (tids are below 2^30) the last tid of the chunk before
+    // chunks lie on 16-byte boundaries (the tids have room up to a multiple of 4)
+    const uint32_t *p = P.tids + (from - skip);
+    uint64_t left = to - (from - skip);
+    auto quads = [](uint64_t tids) { return (uint32_t)(min(tids, (uint64_t)PART) + 3) / 4; };
+    copy_quads(S.chunk[0], p, quads(left), lane);
+    for (uint32_t c = 0; left; c ^= 1) {
+        const uint32_t len = (uint32_t)min(left, (uint64_t)PART);
+        left -= len;
+        p += PART;
+        copy_quads(S.chunk[c ^ 1], p, left ? quads(left) : 0, lane);
+        copies_wait<1>();
+        const uint32_t *s = S.chunk[c] + skip, count = len - skip, last = s[count - 1];
+        skip = 0;
+        const uint32_t upto = __popc(__ballot_sync(0xffffffffu, lane < rows && x[min(32 * lane, n - 1)] <= last));
+        const uint32_t p2 = 1u << (31 - __clz(count));
+        for (uint32_t j = row; j < upto; j += 4) {
+            uint32_t v[4], at[4], want = 0;
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                v[u] = x[min(32 * (j + u) + lane, n - 1)];
+                at[u] = 0;
+                if (j + u < upto && v[u] <= last && (int32_t)v[u] > past) want |= 1u << u;
+            }
+            want &= alive >> j;  // (no bits from n on)
+            if (!__any_sync(0xffffffffu, want)) continue;
+            for (uint32_t step = p2; step; step >>= 1)
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    if (at[u] + step < count && s[at[u] + step] <= v[u]) at[u] += step;
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if ((want >> u & 1u) && s[at[u]] == v[u]) kept |= 1u << (j + u);
+        }
+        __syncwarp();
+        if (last >= top) break;
+        past = (int32_t)last;
+        row = upto ? upto - 1 : 0;
+    }
+    copies_wait<0>();
+    return kept;
+}
+
+// from, win: the index entries that elements may follow (entry from - 1, if any, is <= all).
+__device__ __forceinline__ uint32_t search_members(const PoolView &P, ProbeShared &S, const uint32_t *xs, uint32_t alive, uint32_t c,
+                                                   uint32_t from, uint32_t win, uint32_t lane) {
+    const uint64_t b = P.off[c];
+    const uint32_t size = (uint32_t)(P.off[c + 1] - b);  // <= 2^30
+    const uint32_t *idx = P.idx + P.idx_off[c] + from, *tids = P.tids + b;
+    const uint32_t every = win > WIN ? (win + WIN - 1) / WIN : 1, ns = win / every;  // samples, <= WIN
+    for (uint32_t i = lane; i < ns; i += 32) S.win[i] = __ldg(&idx[(i + 1) * every - 1]);
+    __syncwarp();
+    const uint32_t s2 = ns ? 1u << (31 - __clz(ns)) : 0, e2 = every > 1 ? 1u << (31 - __clz(every - 1)) : 0;
+    uint32_t kept = 0;
+    for (uint32_t left = alive; __any_sync(0xffffffffu, left != 0);) {
+        uint32_t bit[4], x[4], lo[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            bit[u] = left & (0u - left);
+            left &= left - 1;
+            x[u] = bit[u] ? xs[32 * (__ffs(bit[u]) - 1) + lane] : 0;
+            lo[u] = 0;
+        }
+        for (uint32_t step = s2; step; step >>= 1)  // samples <= x
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (lo[u] + step <= ns && S.win[lo[u] + step - 1] <= x[u]) lo[u] += step;
+#pragma unroll
+        for (int u = 0; u < 4; u++) lo[u] *= every;
+        uint32_t end[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) end[u] = min(win, lo[u] + every - 1);
+        for (uint32_t step = e2; step; step >>= 1)  // entries of the window <= x
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (bit[u] && lo[u] + step <= end[u] && __ldg(&idx[lo[u] + step - 1]) <= x[u]) lo[u] += step;
+        uint32_t at[4], top[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {  // the block of tids whose first is the last entry <= x
+            const uint32_t e = from + lo[u];
+            if (!e) bit[u] = 0;  // below the set's first tid
+            at[u] = e ? IDX_STRIDE * (e - 1) : 0;
+            top[u] = min(size, at[u] + IDX_STRIDE);
+        }
+#pragma unroll
+        for (uint32_t step = IDX_STRIDE / 2; step; step >>= 1)
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (bit[u] && at[u] + step < top[u] && __ldg(&tids[at[u] + step]) <= x[u]) at[u] += step;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (bit[u] && __ldg(&tids[at[u]]) == x[u]) kept |= bit[u];
+    }
+    __syncwarp();
+    return kept;
+}
+
 __device__ __forceinline__ bool bsearch_u32(const uint32_t *a, uint64_t lo, uint64_t hi, uint32_t x) {
     while (lo < hi) {
         const uint64_t mid = (lo + hi) >> 1;
@@ -71,107 +244,105 @@ __device__ __forceinline__ bool bsearch_u32(const uint32_t *a, uint64_t lo, uint
     return false;
 }
 
-// x in set c's sorted tidlist: the last index entry <= x names the block of
-// IDX_STRIDE tids that can hold x; that block is binary-searched.
-__device__ __forceinline__ bool tidlist_member(const PoolView &P, uint32_t c, uint32_t x) {
-    const uint64_t i0 = P.idx_off[c];
-    uint64_t lo = i0, hi = P.idx_off[c + 1];
-    while (lo < hi) {  // first entry > x
-        const uint64_t mid = (lo + hi) >> 1;
-        const uint32_t v = P.idx[mid];
-        if (v == x) return true;
-        if (v < x) lo = mid + 1; else hi = mid;
-    }
-    if (lo == i0) return false;  // x below the set's first tid
-    const uint64_t s0 = P.off[c], first = s0 + (uint64_t)IDX_STRIDE * (lo - 1 - i0);
-    const uint64_t end = min(P.off[c + 1], first + IDX_STRIDE);
-    return bsearch_u32(P.tids, first + 1, end, x);  // the block's first tid is the entry, != x
-}
-
-__device__ __forceinline__ bool member(const PoolView &P, uint32_t c, uint32_t x) {
-    const int32_t b = P.bm_index[c];
-    if (b < 0) return tidlist_member(P, c, x);
-    const uint64_t base = P.bm_base[b];
+__device__ __forceinline__ uint32_t byte_members(const PoolView &P, const uint32_t *xs, uint32_t alive, uint32_t b,
+                                                 uint32_t lane) {
+    const uint8_t *bm = P.bm + P.bm_base[b];
     const uint32_t r = 1u << P.bm_rlog[b];
+    const uint64_t f0 = P.f_off[b], f1 = P.f_off[b + 1];
+    uint32_t kept = 0;
+    for (uint32_t left = alive; left;) {
+        uint32_t bit[4], x[4], want[4][2], got[4][2];
 #pragma unroll
-    for (uint32_t t = 0; t < 2; t++) {
-        const uint32_t pi = P.perm(t, x);
-        const uint8_t byte = P.bm[base + slot_of(t, pi, r, P.shift)];
-        if ((uint32_t)(byte & 0x7F) == (pi >> P.shift) + 1u) return true;
-    }
-    return bsearch_u32(P.f_tid, P.f_off[b], P.f_off[b + 1], x);
-}
-
-__global__ void k_probe(PoolView P, const QueryDesc *__restrict__ qs, const ProbeTask *__restrict__ tasks,
-                        uint32_t ntasks, unsigned long long *__restrict__ counts) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < ntasks; w += warps) {
-        const ProbeTask tk = tasks[w];
-        const QueryDesc &Q = qs[tk.q];
-        const uint32_t a = Q.ids[0];
-        const uint64_t a0 = P.off[a];
-        uint32_t cnt = 0;
-        for (uint32_t i = tk.begin + lane; i < tk.end; i += 32) {
-            const uint32_t x = P.tids[a0 + i];
-            bool in_all = true;
-            for (uint32_t t = 1; t < Q.k && in_all; t++) in_all = member(P, Q.ids[t], x);
-            cnt += in_all ? 1u : 0u;
+        for (int u = 0; u < 4; u++) {
+            bit[u] = left & (0u - left);
+            left &= left - 1;
+            x[u] = bit[u] ? xs[32 * (__ffs(bit[u]) - 1) + lane] : 0;
+#pragma unroll
+            for (uint32_t t = 0; t < 2; t++) {
+                const uint32_t pi = P.perm(t, x[u]);
+                want[u][t] = (pi >> P.shift) + 1u;
+                got[u][t] = bit[u] ? __ldg(&bm[slot_of(t, pi, r, P.shift)]) & 0x7Fu : 0;
+            }
         }
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, d);
-        if (lane == 0 && cnt) atomicAdd(&counts[tk.q], (unsigned long long)cnt);
+        for (int u = 0; u < 4; u++)
+            if (bit[u] && (got[u][0] == want[u][0] || got[u][1] == want[u][1] || bsearch_u32(P.f_tid, f0, f1, x[u]))) kept |= bit[u];
     }
+    __syncwarp();
+    return kept;
 }
 
-// Materialised answers: the count pass stores one count per task; after an
-// exclusive scan over tasks the write pass lists each task's matches in
-// element order (a warp ballot ranks them), so every answer is ascending.
-__global__ void k_probe_count(PoolView P, const QueryDesc *__restrict__ qs, const ProbeTask *__restrict__ tasks,
-                              uint32_t ntasks, uint64_t *__restrict__ task_counts) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < ntasks; w += warps) {
-        const ProbeTask tk = tasks[w];
-        const QueryDesc &Q = qs[tk.q];
-        const uint64_t a0 = P.off[Q.ids[0]];
-        uint32_t cnt = 0;
-        for (uint32_t i = tk.begin + lane; i < tk.end; i += 32) {
-            const uint32_t x = P.tids[a0 + i];
-            bool in_all = true;
-            for (uint32_t t = 1; t < Q.k && in_all; t++) in_all = member(P, Q.ids[t], x);
-            cnt += in_all ? 1u : 0u;
-        }
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, d);
-        if (lane == 0) task_counts[w] = cnt;
+__device__ __forceinline__ uint32_t probe_task(const PoolView &P, const QueryDesc &Q, const ProbeTask &tk, ProbeShared &S,
+                                               uint32_t lane) {
+    const uint32_t n = tk.end - tk.begin, mine = n > lane ? (n - lane + 31) / 32 : 0;
+    uint32_t alive = mine == 32 ? 0xffffffffu : (1u << mine) - 1;
+    if (Q.k == 1) return alive;
+    const uint64_t a0 = P.off[Q.ids[0]] + tk.begin;
+    const uint32_t skip = (uint32_t)(a0 & 3), *x = S.x + skip;
+    copy_quads(S.x, P.tids + (a0 - skip), (n + skip + 3) / 4, lane);
+    const uint32_t first = __ldg(&P.tids[a0]), last = __ldg(&P.tids[a0 + n - 1]);
+    bool there = false;
+    for (uint32_t t = 1; t < Q.k; t++) {
+        const uint32_t todo = __reduce_add_sync(0xffffffffu, __popc(alive));
+        if (!todo) break;
+        const uint32_t c = Q.ids[t];
+        const uint64_t b = P.off[c], i0 = P.idx_off[c];
+        uint32_t c0, c1;
+        count_le(P.idx + i0, (uint32_t)(P.idx_off[c + 1] - i0), first, last, lane, c0, c1);
+        const uint64_t from = b + (uint64_t)IDX_STRIDE * (c0 ? c0 - 1 : 0), to = min(P.off[c + 1], b + (uint64_t)IDX_STRIDE * c1);
+        const int32_t bm = P.bm_index[c];
+        if (!there) copies_wait<0>();
+        there = true;
+        if (to <= from) return 0;  // all are below its first tid
+        if (to - from <= (uint64_t)STREAM * todo) alive = stream_members(P, S, x, n, alive, from, to, lane);
+        else if (bm >= 0) alive = byte_members(P, x, alive, (uint32_t)bm, lane);
+        else alive = search_members(P, S, x, alive, c, c0, c1 - c0, lane);
     }
+    return alive;
+}
+
+// The tasks of each query, a block each.
+__global__ void k_query_tasks(const uint64_t *__restrict__ off, const QueryDesc *__restrict__ qs,
+                              const uint32_t *__restrict__ first, uint32_t elems, ProbeTask *__restrict__ tasks) {
+    const uint32_t q = blockIdx.x, t0 = first[q], n = first[q + 1] - t0, a = qs[q].ids[0];
+    const uint32_t size = (uint32_t)(off[a + 1] - off[a]);
+    for (uint32_t k = threadIdx.x; k < n; k += blockDim.x) tasks[t0 + k] = {q, k * elems, min(size, (k + 1) * elems)};
+}
+
+// One warp a task.  Counts: added to the query's.  Lists (masks not NULL): the
+// task's count and its words, which the write pass after an exclusive scan over
+// tasks ranks in element order, so every answer is ascending.
+__global__ void __launch_bounds__(32 * PROBE_WARPS)
+k_probe(PoolView P, const QueryDesc *__restrict__ qs, const ProbeTask *__restrict__ tasks, uint32_t ntasks,
+        unsigned long long *__restrict__ counts, uint64_t *__restrict__ task_counts, uint32_t *__restrict__ masks) {
+    __shared__ __align__(16) ProbeShared shared[PROBE_WARPS];
+    const uint32_t lane = threadIdx.x & 31, w = blockIdx.x * PROBE_WARPS + (threadIdx.x >> 5);
+    if (w >= ntasks) return;
+    const ProbeTask tk = tasks[w];
+    const uint32_t alive = probe_task(P, qs[tk.q], tk, shared[threadIdx.x >> 5], lane);
+    const uint32_t cnt = __reduce_add_sync(0xffffffffu, __popc(alive));
+    if (masks) masks[32ull * w + lane] = alive;
+    if (lane) return;
+    if (task_counts) task_counts[w] = cnt;
+    else if (cnt) atomicAdd(&counts[tk.q], (unsigned long long)cnt);
 }
 
 __global__ void k_probe_write(PoolView P, const QueryDesc *__restrict__ qs, const ProbeTask *__restrict__ tasks,
-                              uint32_t ntasks, const uint64_t *__restrict__ task_off, uint32_t *__restrict__ out,
-                              uint64_t cap) {
+                              uint32_t ntasks, const uint64_t *__restrict__ task_off, const uint32_t *__restrict__ masks,
+                              uint32_t *__restrict__ out, uint64_t cap) {
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < ntasks; w += warps) {
-        const ProbeTask tk = tasks[w];
-        const QueryDesc &Q = qs[tk.q];
-        const uint64_t a0 = P.off[Q.ids[0]];
-        uint64_t running = task_off[w];
-        for (uint32_t base = tk.begin; base < tk.end; base += 32) {
-            const uint32_t i = base + lane;
-            bool in_all = false;
-            uint32_t x = 0;
-            if (i < tk.end) {
-                x = P.tids[a0 + i];
-                in_all = true;
-                for (uint32_t t = 1; t < Q.k && in_all; t++) in_all = member(P, Q.ids[t], x);
-            }
-            const uint32_t mask = __ballot_sync(0xffffffffu, in_all);
-            const uint64_t pos = running + __popc(mask & ((1u << lane) - 1u));
-            if (in_all && pos < cap) out[pos] = x;
-            running += __popc(mask);
-        }
+    const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= ntasks) return;
+    const uint32_t mine = masks[32ull * w + lane];
+    if (!__any_sync(0xffffffffu, mine != 0)) return;
+    const ProbeTask tk = tasks[w];
+    const uint32_t *a = P.tids + P.off[qs[tk.q].ids[0]] + tk.begin;
+    uint64_t running = task_off[w];
+    for (uint32_t j = 0; j < 32; j++) {
+        const uint32_t mask = __ballot_sync(0xffffffffu, mine >> j & 1u);
+        const uint64_t pos = running + __popc(mask & ((1u << lane) - 1u));
+        if ((mine >> j & 1u) && pos < cap) out[pos] = a[32 * j + lane];
+        running += __popc(mask);
     }
 }
 
@@ -246,7 +417,7 @@ static void pool_create(const batmap_params *p, uint32_t m, uint32_t n, const ui
     }
     const uint64_t T = pool->h_off[n];
     pool->d_off.alloc(n + 1);
-    pool->d_tids.alloc(T);
+    pool->d_tids.alloc((T + 3) / 4 * 4);  // read 16 bytes at a time
     if (d_perm) pool->d_perm.alloc(3ull * m);  // computed permutations need no table
     if (n) BM_CUDA(cudaMemcpyAsync(pool->d_off.p, d_offsets, (n + 1) * 8ull, cudaMemcpyDeviceToDevice, st));
     if (T) BM_CUDA(cudaMemcpyAsync(pool->d_tids.p, d_tids, T * 4ull, cudaMemcpyDeviceToDevice, st));
@@ -386,16 +557,26 @@ static void pool_create(const batmap_params *p, uint32_t m, uint32_t n, const ui
     *out = pool.release();
 }
 
-// Host-side preparation of one batch: descriptors with the smallest set first,
-// and the element tasks.  Returns the number of tasks.
-static uint64_t prepare_batch(const batmap_pool *pool, const uint32_t *qoff, const uint32_t *ids, uint64_t q0,
-                              uint64_t q1, std::vector<QueryDesc> *qs, std::vector<ProbeTask> *tasks) {
-    qs->resize(q1 - q0);
-    tasks->clear();
+// A batch of queries on the host: descriptors with the smallest set first, and the
+// first task of each (one more: the number of tasks), tasks of `elems` elements.
+struct Batch {
+    std::vector<QueryDesc> qs;
+    std::vector<uint32_t> first;
+    uint32_t elems = 0;
+    uint64_t tasks() const { return first.empty() ? 0 : first.back(); }
+};
+
+// elems 0: chosen by the work.
+static void prepare_batch(const batmap_pool *pool, const uint32_t *qoff, const uint32_t *ids, uint64_t q0, uint64_t q1,
+                          Batch &B, uint32_t elems) {
+    B.qs.resize(q1 - q0);
+    B.first.resize(q1 - q0 + 1);
+    auto size_of = [&](uint32_t c) { return pool->h_off[c + 1] - pool->h_off[c]; };
+    uint64_t total = 0;
     for (uint64_t q = q0; q < q1; q++) {
         const uint32_t k = qoff[q + 1] - qoff[q];
         BM_REQUIRE(k >= 1 && k <= MAX_K, BATMAP_ERR_ARG, "each query names 1..8 sets");
-        QueryDesc &d = (*qs)[q - q0];
+        QueryDesc &d = B.qs[q - q0];
         d.k = k;
         for (uint32_t t = 0; t < k; t++) {
             const uint32_t c = ids[qoff[q] + t];
@@ -403,15 +584,25 @@ static uint64_t prepare_batch(const batmap_pool *pool, const uint32_t *qoff, con
             d.ids[t] = c;
         }
         std::sort(d.ids, d.ids + k, [&](uint32_t a, uint32_t b) {
-            const uint64_t sa = pool->h_off[a + 1] - pool->h_off[a], sb = pool->h_off[b + 1] - pool->h_off[b];
+            const uint64_t sa = size_of(a), sb = size_of(b);
             return sa < sb || (sa == sb && a < b);
         });
-        const uint32_t small = (uint32_t)(pool->h_off[d.ids[0] + 1] - pool->h_off[d.ids[0]]);
-        for (uint32_t b = 0; b < small; b += TASK_ELEMS)
-            tasks->push_back({(uint32_t)(q - q0), b, std::min(small, b + TASK_ELEMS)});
+        total += size_of(d.ids[0]);
     }
-    return tasks->size();
+    // Small batches: shorter tasks until there are some for every warp that the chip holds.
+    if (!elems)
+        for (elems = TASK_ELEMS; elems > 128 && total / elems < 8192;) elems /= 2;
+    B.elems = elems;
+    uint64_t nt = 0;
+    for (uint64_t q = 0; q < q1 - q0; q++) {
+        B.first[q] = (uint32_t)nt;
+        nt += (size_of(B.qs[q].ids[0]) + elems - 1) / elems;
+    }
+    BM_REQUIRE(nt < (1ull << 32), BATMAP_ERR_ARG, "too much work in one call");
+    B.first[q1 - q0] = (uint32_t)nt;
 }
+
+static unsigned probe_blocks(uint64_t tasks) { return (unsigned)((tasks + PROBE_WARPS - 1) / PROBE_WARPS); }
 
 static uint64_t query_work(const batmap_pool *pool, const uint32_t *qoff, const uint32_t *ids, uint64_t q) {
     uint64_t small = UINT64_MAX;
@@ -422,29 +613,35 @@ static uint64_t query_work(const batmap_pool *pool, const uint32_t *qoff, const 
     return (small == UINT64_MAX ? 0 : small) * (qoff[q + 1] - qoff[q]) + 1;
 }
 
+// The descriptors and tasks of a batch on the device.
+static void upload_batch(const batmap_pool *pool, const QueryDesc *qs, uint64_t nq, QueryDesc *d_q, const uint32_t *first,
+                         uint32_t *d_first, uint32_t elems, ProbeTask *d_t, cudaStream_t st) {
+    BM_CUDA(cudaMemcpyAsync(d_first, first, (nq + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
+    if (!nq) return;
+    BM_CUDA(cudaMemcpyAsync(d_q, qs, nq * sizeof(QueryDesc), cudaMemcpyHostToDevice, st));
+    if (!first[nq]) return;
+    k_query_tasks<<<(unsigned)nq, 64, 0, st>>>(pool->view.off, d_q, d_first, elems, d_t);
+    BM_CHECK_LAUNCH();
+}
+
 // Answers as element lists: out_off[q] .. out_off[q+1] in out (ascending).
 static void intersect_list(const batmap_pool *pool, const uint32_t *qoff, const uint32_t *ids, uint32_t nq,
                            uint64_t *d_out_off, uint32_t *d_out, uint64_t cap, uint64_t *n_total, cudaStream_t st) {
     BM_REQUIRE(pool && qoff && n_total && d_out_off, BATMAP_ERR_ARG, "NULL argument");
     BM_REQUIRE(cap == 0 || d_out, BATMAP_ERR_ARG, "d_out is NULL with cap > 0");
     Workspace ws(st);
-    std::vector<QueryDesc> qs;
-    std::vector<ProbeTask> tasks;
-    if (nq) prepare_batch(pool, qoff, ids, 0, nq, &qs, &tasks);
-    const uint64_t nt = tasks.size();
-    std::vector<uint32_t> first(nq + 1, (uint32_t)nt);
-    for (uint64_t t = nt; t-- > 0;) first[tasks[t].q] = (uint32_t)t;
-    for (uint32_t q = nq; q-- > 0;) first[q] = std::min(first[q], first[q + 1]);
-    WsBuf<QueryDesc> d_q(ws, std::max<uint64_t>(qs.size(), 1));
+    Batch B;
+    prepare_batch(pool, qoff, ids, 0, nq, B, 0);
+    const uint64_t nt = B.tasks();
+    WsBuf<QueryDesc> d_q(ws, std::max<uint64_t>(nq, 1));
     WsBuf<ProbeTask> d_t(ws, std::max<uint64_t>(nt, 1));
     WsBuf<uint64_t> d_toff(ws, nt + 1), d_total(ws, 1);
     WsBuf<uint32_t> d_first(ws, nq + 1);
-    if (nq) BM_CUDA(cudaMemcpyAsync(d_q.p, qs.data(), qs.size() * sizeof(QueryDesc), cudaMemcpyHostToDevice, st));
-    if (nt) BM_CUDA(cudaMemcpyAsync(d_t.p, tasks.data(), nt * sizeof(ProbeTask), cudaMemcpyHostToDevice, st));
-    BM_CUDA(cudaMemcpyAsync(d_first.p, first.data(), (nq + 1) * 4ull, cudaMemcpyHostToDevice, st));
-    const unsigned blocks = (unsigned)std::min<uint64_t>((nt + 7) / 8, 4096);
+    upload_batch(pool, B.qs.data(), nq, d_q.p, B.first.data(), d_first.p, B.elems, d_t.p, st);
+    WsBuf<uint32_t> d_masks(ws, cap ? 32 * nt : 0);
     if (nt) {
-        k_probe_count<<<blocks, 256, 0, st>>>(pool->view, d_q.p, d_t.p, (uint32_t)nt, d_toff.p);
+        k_probe<<<probe_blocks(nt), 32 * PROBE_WARPS, 0, st>>>(pool->view, d_q.p, d_t.p, (uint32_t)nt, nullptr, d_toff.p,
+                                                               cap ? d_masks.p : nullptr);
         BM_CHECK_LAUNCH();
     }
     WsBuf<uint64_t> scan_state(ws, scan_states(nt));
@@ -452,7 +649,8 @@ static void intersect_list(const batmap_pool *pool, const uint32_t *qoff, const 
     k_query_offsets<<<(nq + 1 + 255) / 256, 256, 0, st>>>(d_toff.p, d_first.p, nq, d_out_off);
     BM_CHECK_LAUNCH();
     if (nt && cap) {
-        k_probe_write<<<blocks, 256, 0, st>>>(pool->view, d_q.p, d_t.p, (uint32_t)nt, d_toff.p, d_out, cap);
+        k_probe_write<<<(unsigned)((nt + 7) / 8), 256, 0, st>>>(pool->view, d_q.p, d_t.p, (uint32_t)nt, d_toff.p, d_masks.p,
+                                                                d_out, cap);
         BM_CHECK_LAUNCH();
     }
     uint64_t total = 0;
@@ -470,8 +668,9 @@ struct Slot {
     cudaStream_t st = nullptr;
     cudaEvent_t done = nullptr;
     QueryDesc *h_q = nullptr;
-    ProbeTask *h_t = nullptr;
+    uint32_t *h_first = nullptr;
     DevBuf<QueryDesc> d_q;
+    DevBuf<uint32_t> d_first;
     DevBuf<ProbeTask> d_t;
     uint64_t qcap = 0, tcap = 0;
     uint64_t q0 = 0, q1 = 0, work = 0;
@@ -482,41 +681,39 @@ struct Slot {
         BM_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
         BM_CUDA(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
         BM_CUDA(cudaMallocHost(&h_q, qc * sizeof(QueryDesc)));
-        BM_CUDA(cudaMallocHost(&h_t, tc * sizeof(ProbeTask)));
+        BM_CUDA(cudaMallocHost(&h_first, (qc + 1) * sizeof(uint32_t)));
         d_q.alloc(qc);
+        d_first.alloc(qc + 1);
         d_t.alloc(tc);
     }
     void destroy() {
         if (done) cudaEventDestroy(done);
         if (st) cudaStreamDestroy(st);
         if (h_q) cudaFreeHost(h_q);
-        if (h_t) cudaFreeHost(h_t);
+        if (h_first) cudaFreeHost(h_first);
         done = nullptr;
         st = nullptr;
         h_q = nullptr;
-        h_t = nullptr;
+        h_first = nullptr;
     }
 };
 
-// Copies a batch's descriptors to the device and counts its answers (zeroed first).
-static void launch_probe(const batmap_pool *pool, const QueryDesc *qs, uint64_t nq, QueryDesc *d_q, const ProbeTask *tasks,
-                         uint64_t nt, ProbeTask *d_t, unsigned long long *d_counts, cudaStream_t st) {
-    BM_CUDA(cudaMemcpyAsync(d_q, qs, nq * sizeof(QueryDesc), cudaMemcpyHostToDevice, st));
-    if (nt) BM_CUDA(cudaMemcpyAsync(d_t, tasks, nt * sizeof(ProbeTask), cudaMemcpyHostToDevice, st));
+// Uploads a batch and counts its answers (zeroed first).
+static void launch_probe(const batmap_pool *pool, const QueryDesc *qs, uint64_t nq, QueryDesc *d_q, const uint32_t *first,
+                         uint32_t *d_first, uint32_t elems, ProbeTask *d_t, unsigned long long *d_counts, cudaStream_t st) {
+    const uint64_t nt = first[nq];
+    upload_batch(pool, qs, nq, d_q, first, d_first, elems, d_t, st);
     BM_CUDA(cudaMemsetAsync(d_counts, 0, nq * sizeof(unsigned long long), st));
     if (nt) {
-        const uint32_t warps_per_block = 8;
-        const uint64_t blocks = std::min<uint64_t>((nt + warps_per_block - 1) / warps_per_block, 4096);
-        k_probe<<<(unsigned)blocks, 32 * warps_per_block, 0, st>>>(pool->view, d_q, d_t, (uint32_t)nt, d_counts);
+        k_probe<<<probe_blocks(nt), 32 * PROBE_WARPS, 0, st>>>(pool->view, d_q, d_t, (uint32_t)nt, d_counts, nullptr, nullptr);
         BM_CHECK_LAUNCH();
     }
 }
 
-static void launch_batch(const batmap_pool *pool, Slot &S, const std::vector<QueryDesc> &qs,
-                         const std::vector<ProbeTask> &tasks, unsigned long long *d_counts) {
-    std::memcpy(S.h_q, qs.data(), qs.size() * sizeof(QueryDesc));
-    if (!tasks.empty()) std::memcpy(S.h_t, tasks.data(), tasks.size() * sizeof(ProbeTask));
-    launch_probe(pool, S.h_q, qs.size(), S.d_q.p, S.h_t, tasks.size(), S.d_t.p, d_counts + S.q0, S.st);
+static void launch_batch(const batmap_pool *pool, Slot &S, const Batch &B, unsigned long long *d_counts) {
+    std::memcpy(S.h_q, B.qs.data(), B.qs.size() * sizeof(QueryDesc));
+    std::memcpy(S.h_first, B.first.data(), B.first.size() * sizeof(uint32_t));
+    launch_probe(pool, S.h_q, B.qs.size(), S.d_q.p, S.h_first, S.d_first.p, B.elems, S.d_t.p, d_counts + S.q0, S.st);
     BM_CUDA(cudaEventRecord(S.done, S.st));
 }
 
@@ -524,13 +721,13 @@ static void intersect(const batmap_pool *pool, const uint32_t *qoff, const uint3
                       unsigned long long *d_counts, cudaStream_t st) {
     BM_REQUIRE(pool && qoff && (nq == 0 || ids) && (nq == 0 || d_counts), BATMAP_ERR_ARG, "NULL argument");
     if (!nq) return;
-    std::vector<QueryDesc> qs;
-    std::vector<ProbeTask> tasks;
-    prepare_batch(pool, qoff, ids, 0, nq, &qs, &tasks);
+    Batch B;
+    prepare_batch(pool, qoff, ids, 0, nq, B, 0);
     Workspace ws(st);
     WsBuf<QueryDesc> d_q(ws, nq);
-    WsBuf<ProbeTask> d_t(ws, tasks.size());
-    launch_probe(pool, qs.data(), nq, d_q.p, tasks.data(), tasks.size(), d_t.p, d_counts, st);
+    WsBuf<uint32_t> d_first(ws, nq + 1);
+    WsBuf<ProbeTask> d_t(ws, B.tasks());
+    launch_probe(pool, B.qs.data(), nq, d_q.p, B.first.data(), d_first.p, B.elems, d_t.p, d_counts, st);
     BM_CUDA(cudaStreamSynchronize(st));
     ws.done();
 }
@@ -569,8 +766,7 @@ static void serve(const batmap_pool *pool, const uint32_t *qoff, const uint32_t 
     DevBuf<unsigned long long> d_counts(std::max<uint32_t>(nq, 1));
     std::vector<Slot> slots(opt.slots);
     for (auto &s : slots) s.init(opt.max_batch, tcap);
-    std::vector<QueryDesc> qs;
-    std::vector<ProbeTask> tasks;
+    Batch B;
     using clk = std::chrono::steady_clock;
     const auto t0 = clk::now();
     auto now_s = [&] { return std::chrono::duration<double>(clk::now() - t0).count(); };
@@ -600,17 +796,17 @@ static void serve(const batmap_pool *pool, const uint32_t *qoff, const uint32_t 
                                    : inflight_work + w + work[q1] <= budget))
                     w += work[q1++];
                 if (q1 == next) break;  // budget full: wait for completions
-                prepare_batch(pool, qoff, ids, next, q1, &qs, &tasks);
-                if (tasks.size() > s.tcap) {  // admit fewer queries
+                prepare_batch(pool, qoff, ids, next, q1, B, TASK_ELEMS);
+                if (B.tasks() > s.tcap) {  // admit fewer queries
                     q1 = next + 1;
-                    prepare_batch(pool, qoff, ids, next, q1, &qs, &tasks);
-                    BM_REQUIRE(tasks.size() <= s.tcap, BATMAP_ERR_INTERNAL, "task capacity");
+                    prepare_batch(pool, qoff, ids, next, q1, B, TASK_ELEMS);
+                    BM_REQUIRE(B.tasks() <= s.tcap, BATMAP_ERR_INTERNAL, "task capacity");
                     w = work[next];
                 }
                 s.q0 = next;
                 s.q1 = q1;
                 s.work = w;
-                launch_batch(pool, s, qs, tasks, d_counts.p);
+                launch_batch(pool, s, B, d_counts.p);
                 s.busy = true;
                 inflight++;
                 inflight_work += w;

@@ -20,42 +20,44 @@ constexpr uint32_t CHUNK_KB = 64;                    // blocks per warp
 constexpr uint32_t CHUNK_BITS = CHUNK_KB * BITS_K;   // 16,384
 constexpr int BW = 8;                                // warps per CTA
 
+// A longer list repeats tids; it is reported as not sorted without a look at it.  So
+// places and searches take 32 bits.
+constexpr uint32_t MAX_LIST = 1u << 30;
+
 // One round of a 32-way search for the first index in [lo, hi) whose value is
 // >= v, by the whole warp.  The result of all rounds is a function of the list
 // and v alone, so neighbouring chunks agree on their border even when the list
 // is not sorted.
-__device__ __forceinline__ void search_round(const uint32_t *__restrict__ a, uint64_t &lo, uint64_t &hi, uint32_t v,
+__device__ __forceinline__ void search_round(const uint32_t *__restrict__ a, uint32_t &lo, uint32_t &hi, uint32_t v,
                                              uint32_t lane) {
     if (lo >= hi) return;  // done (warp-uniform): a further round could move the result of an unsorted list
-    const uint64_t step = (hi - lo + 31) >> 5;
-    const uint64_t p = lo + lane * step + (step - 1);
+    const uint32_t step = (hi - lo + 31) >> 5;  // (hi <= MAX_LIST: no overflow below)
+    const uint32_t p = lo + lane * step + (step - 1);
     const bool below = p < hi && __ldg(&a[p]) < v;
     const uint32_t c = __popc(__ballot_sync(0xffffffffu, below));
-    const uint64_t top = lo + c * step + (step - 1);  // the first probe not below, if c < 32
+    const uint32_t top = lo + c * step + (step - 1);  // the first probe not below, if c < 32
     lo = min(lo + c * step, hi);
     if (c < 32) hi = min(hi, top);
 }
 
-// BLOCK tids of one list from place f on, four per lane and 16-byte load; place f
-// stands for element f - skew, which starts a 16-byte boundary.  Places before
-// `begin` hold `before` (the predecessor of the first), those from `end` on 0.
+// BLOCK tids from place f of r, a 16-byte boundary, four per lane and load.  Places
+// before `begin` hold `before` (the predecessor of the first), those from `end` on 0.
 constexpr int BQ = 2;                  // loads in flight per lane and block
 constexpr uint32_t BLOCK = 128 * BQ;
 struct TidBlock {
     uint32_t x[BQ][4];
 };
-__device__ __forceinline__ void load_block(TidBlock &B, const uint32_t *__restrict__ a, uint64_t f, uint32_t skew,
-                                           uint64_t begin, uint64_t end, uint32_t before, uint32_t lane) {
+__device__ __forceinline__ void load_block(TidBlock &B, const uint32_t *__restrict__ r, uint32_t f, uint32_t begin,
+                                           uint32_t end, uint32_t before, uint32_t lane) {
 #pragma unroll
     for (int q = 0; q < BQ; q++) {
-        const uint64_t i = f + 128u * q + 4u * lane;
+        const uint32_t i = f + 128u * q + 4u * lane;
         if (i >= begin && i + 4 <= end) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(a + (i - skew)));
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(r + i));
             B.x[q][0] = v.x; B.x[q][1] = v.y; B.x[q][2] = v.z; B.x[q][3] = v.w;
         } else {
 #pragma unroll
-            for (int j = 0; j < 4; j++)
-                B.x[q][j] = i + j < begin ? before : i + j < end ? __ldg(&a[i + j - skew]) : 0;
+            for (int j = 0; j < 4; j++) B.x[q][j] = i + j < begin ? before : i + j < end ? __ldg(&r[i + j]) : 0;
         }
     }
 }
@@ -72,23 +74,26 @@ k_bits(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tids, uint
     bool bad_tid = false, unsorted = false;
     // neighbouring warps: neighbouring items of the same chunks, whose 32-byte pieces share lines
     for (uint64_t w = blockIdx.x * (uint64_t)BW + (threadIdx.x >> 5); w < tasks; w += warps) {
-        const uint32_t item = (uint32_t)(w % n), c0 = (uint32_t)(w / n) * run, c1 = min(c0 + run, nchunk);
-        const uint64_t b = off[item], size = off[item + 1] - b;
+        const uint32_t at = tasks >> 32 ? (uint32_t)(w / n) : (uint32_t)w / n, item = (uint32_t)(w - (uint64_t)at * n);
+        const uint32_t c0 = at * run, c1 = min(c0 + run, nchunk);
+        const uint64_t b = off[item], long_size = off[item + 1] - b;
+        const uint32_t size = long_size <= MAX_LIST ? (uint32_t)long_size : 0;
         const uint32_t *a = tids + b;
         const uint32_t first = c0 * CHUNK_BITS, past = c1 * CHUNK_BITS;  // m <= 2^30: no overflow
-        uint64_t e0 = 0, h0 = c0 ? size : 0, e1 = c1 == nchunk ? size : 0, h1 = size;
+        uint32_t e0 = 0, h0 = c0 ? size : 0, e1 = c1 == nchunk ? size : 0, h1 = size;
         while (e0 < h0 || e1 < h1) {
             search_round(a, e0, h0, first, lane);
             search_round(a, e1, h1, past, lane);
         }
-        unsorted |= e1 < e0;
-        const uint32_t skew = (uint32_t)(reinterpret_cast<uintptr_t>(a + e0) >> 2) & 3u;
-        const uint64_t begin = e0 + skew, end = e1 + skew;  // places of the run's elements
-        uint32_t carry = e0 ? __ldg(&a[e0 - 1]) : 0;         // predecessor of the block's first tid
-        uint64_t f = e0;                                     // the block in hand; the one behind it is on its way
+        unsorted |= e1 < e0 || size != long_size;
+        // places: from the 16-byte boundary at or before the run's first tid
+        const uint32_t begin = (uint32_t)(reinterpret_cast<uintptr_t>(a + e0) >> 2) & 3u, end = begin + (e1 > e0 ? e1 - e0 : 0);
+        const uint32_t *r = a + e0 - begin;
+        uint32_t carry = e0 ? __ldg(&a[e0 - 1]) : 0;  // predecessor of the block's first tid
+        uint32_t f = 0;                               // the block in hand; the one behind it is on its way
         TidBlock B, N;
-        load_block(B, a, f, skew, begin, end, carry, lane);
-        load_block(N, a, f + BLOCK, skew, begin, end, carry, lane);
+        load_block(B, r, f, begin, end, carry, lane);
+        load_block(N, r, f + BLOCK, begin, end, carry, lane);
         uint32_t b0 = 0;       // the block's first tid (carry: its last)
         bool fresh = true, plain = false;
         for (uint32_t c = c0; c < c1; c++) {
@@ -102,7 +107,7 @@ k_bits(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tids, uint
                     const uint32_t last = __shfl_sync(0xffffffffu, B.x[BQ - 1][3], 31);
                     b0 = __shfl_sync(0xffffffffu, B.x[0][0], 0);
                     plain = f >= begin && f + BLOCK <= end && b0 >= first && last < past && last < m &&
-                            (f == 0 || carry < b0);
+                            ((f == 0 && e0 == 0) || carry < b0);
                     bool ok = true;
 #pragma unroll
                     for (int q = 0; q < BQ; q++) {
@@ -116,7 +121,7 @@ k_bits(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tids, uint
                     if (!plain) {  // place by place
 #pragma unroll
                         for (int q = 0; q < BQ; q++) {
-                            const uint64_t i = f + 128u * q + 4u * lane;
+                            const uint32_t i = f + 128u * q + 4u * lane;
                             uint32_t prev = __shfl_up_sync(0xffffffffu, B.x[q][3], 1);
                             if (lane == 0) prev = carry;
 #pragma unroll
@@ -124,7 +129,7 @@ k_bits(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tids, uint
                                 const uint32_t y = B.x[q][j];
                                 if (i + j >= begin && i + j < end) {
                                     // (the list's first tid has no predecessor)
-                                    unsorted |= (i + j != skew && !(prev < y)) || y < first || y >= past;
+                                    unsorted |= ((e0 || i + j != begin) && !(prev < y)) || y < first || y >= past;
                                     bad_tid |= y >= m;
                                 }
                                 prev = y;
@@ -136,7 +141,7 @@ k_bits(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tids, uint
                 }
 #pragma unroll
                 for (int q = 0; q < BQ; q++) {
-                    const uint64_t i = f + 128u * q + 4u * lane;
+                    const uint32_t i = f + 128u * q + 4u * lane;
                     uint32_t word = 0, mask = 0;  // bits of one word are set together
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
@@ -158,7 +163,7 @@ k_bits(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tids, uint
                 if (!fresh) break;
                 f += BLOCK;
                 B = N;
-                load_block(N, a, f + BLOCK, skew, begin, end, carry, lane);
+                load_block(N, r, f + BLOCK, begin, end, carry, lane);
             }
             __syncwarp();
             uint8_t *row = out + item * L.row_stride;

@@ -11,7 +11,8 @@
 // Bound: HBM, 4 bytes read per pair and 12 written per frequent pair.  Before,
 // a count pass, a scan and a write pass that ranked 256 supports at a time and
 // searched each one's row: 598 us for 32 M pairs of n = 8,000, all frequent
-// (512 MB: 76 us at the copy rate).
+// (512 MB: 76 us at the copy rate); this one 218 us with 72 registers, three blocks
+// per SM that wait at their barriers, and about 175 with 48 and 32-bit row borders.
 #include <algorithm>
 
 #include "common.cuh"
@@ -50,7 +51,7 @@ __device__ __forceinline__ uint32_t row_of(uint64_t L, uint64_t n, uint32_t n_a,
 
 // state: one zeroed word per tile, then the zeroed tile counter.  *total <- the
 // number of qualifying pairs (~0: a bounded wait gave up).  out may be NULL.
-__global__ void __launch_bounds__(CTPB) k_threshold(const uint32_t *__restrict__ C, uint64_t npairs, uint64_t n,
+__global__ void __launch_bounds__(CTPB, 5) k_threshold(const uint32_t *__restrict__ C, uint64_t npairs, uint64_t n,
                                                     uint32_t n_a, uint32_t s, uint64_t *__restrict__ state,
                                                     uint64_t tiles, uint32_t *__restrict__ out, uint64_t cap,
                                                     uint64_t *__restrict__ total) {
@@ -110,20 +111,23 @@ __global__ void __launch_bounds__(CTPB) k_threshold(const uint32_t *__restrict__
             const uint32_t bits = (keep >> (4 * q)) & 15u;
             if (bits && rank < p0 + CSTAGE && rank + 4 > p0) {
                 const uint64_t L = base + 1024u * q + 4u * threadIdx.x;
+                const uint32_t p = 1024u * q + 4u * threadIdx.x;  // its place in the tile
                 uint32_t i = row_of(L, n, n_a, r0, r1);
-                uint64_t next = row_start(i + 1ull, n, n_a), here = row_start(i, n, n_a);
+                // starts of its row (modulo 2^32) and of the next, from the tile's first place on
+                uint32_t here = (uint32_t)(row_start(i, n, n_a) - base);
+                uint32_t next = i < r1 ? (uint32_t)(row_start(i + 1ull, n, n_a) - base) : CCHUNK;
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    while (L + j >= next && i < r1) {
+                    while (p + j >= next && i < r1) {
                         i++;
                         here = next;
-                        next = row_start(i + 1ull, n, n_a);
+                        next = i < r1 ? (uint32_t)(row_start(i + 1ull, n, n_a) - base) : CCHUNK;
                     }
                     if ((bits >> j) & 1u) {
                         if (rank >= p0 && rank < p0 + CSTAGE) {
                             uint32_t *o = s_out + 3 * (rank - p0);
                             o[0] = i;
-                            o[1] = (uint32_t)(L + j - here) + (n_a ? 0 : i + 1);  // B items count from 0
+                            o[1] = p + j - here + (n_a ? 0 : i + 1);  // B items count from 0
                             o[2] = v[q][j];
                         }
                         rank++;

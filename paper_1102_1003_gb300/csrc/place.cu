@@ -28,6 +28,7 @@
 // Before, one launch placed all items through one table in DRAM (25.8 GB at
 // m = 2^22, n = 4,096, 5%) and another looked every element up in it.
 #include <algorithm>
+#include <type_traits>
 
 #include "compare.cuh"
 #include "place.cuh"
@@ -72,13 +73,18 @@ __device__ __forceinline__ Slot slot_of_h(uint32_t t, uint32_t h, uint32_t shift
 }
 constexpr uint32_t SLOT32_RLOG = 28;
 
+// Cycle walking with the round keys of a table.
+__device__ __forceinline__ uint32_t pi_by(const PermView &P, const uint4 &k, uint32_t x) {
+    uint32_t v = P.pass(k, x);
+    while (v >= P.m) v = P.pass(k, v);
+    return v;
+}
+
 // pi_t(x), the round keys of table t read by index from the kernel's parameters.
 __device__ __forceinline__ uint32_t pi_of(const PermView &P, uint32_t t, uint32_t x) {
     if (P.table) return __ldg(&P.table[(uint64_t)t * P.m + x]);
     const uint4 k = P.key[t];
-    uint32_t v = P.pass(k, x);
-    while (v >= P.m) v = P.pass(k, v);
-    return v;
+    return pi_by(P, k, x);
 }
 
 // Records the failures of 32 consecutive elements, the w-th of the item.
@@ -117,35 +123,48 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
         const uint32_t size = (uint32_t)(J.off[item + 1] - e0);  // <= cap, <= slots
         for (uint32_t e = threadIdx.x; e < size; e += tpb) table[e] = J.tids[e0 + e];
         __syncthreads();
-        // pi_t(x): cycle walking takes 1 to 4 passes on average, the longest of 32 lanes far more, so
-        // a lane that is done takes the warp's next (element, table)
-        const uint32_t total = NT * size;
-        uint32_t taken = 0, idx = 0, v = 0;
-        bool busy = false;
-        for (;;) {
-            const uint32_t idle = __ballot_sync(0xffffffffu, !busy);
-            if (!busy) {
-                const uint32_t k = taken + __popc(idle & ((1u << lane) - 1u));
-                idx = ((k >> 5) * warps + warp) * 32u + (k & 31u);
-                if (idx < total) {
-                    v = table[idx / NT];
-                    busy = v < P.m;  // else rejected by validation
-                    if (!busy) code[idx] = 0, pos[idx] = 0;
-                    else if (P.table) v = __ldg(&P.table[(uint64_t)(idx % NT) * P.m + v]);
+        if (P.table) {
+            for (uint32_t e = threadIdx.x; e < size; e += tpb) {
+                const uint32_t x = table[e];
+                uint32_t v[NT];
+#pragma unroll
+                for (uint32_t t = 0; t < NT; t++) v[t] = x < P.m ? __ldg(&P.table[(uint64_t)t * P.m + x]) : 0;
+#pragma unroll
+                for (uint32_t t = 0; t < NT; t++) {
+                    pos[e * NT + t] = (uint16_t)(v[t] & rm);
+                    code[e * NT + t] = x < P.m ? (uint8_t)((v[t] >> J.shift) + 1u) : 0;  // else rejected by validation
                 }
             }
-            taken += __popc(idle);
-            if (__any_sync(0xffffffffu, busy)) {
-                if (busy) {
-                    if (!P.table) v = P.pass(P.key[idx % NT], v);
-                    if (P.table || v < P.m) {
-                        pos[idx] = (uint16_t)(v & rm);
-                        code[idx] = (uint8_t)((v >> J.shift) + 1u);
-                        busy = false;
+        } else {
+            // pi_t(x): cycle walking takes 1 to 4 passes on average, the longest of 32 lanes far more, so
+            // a lane that is done takes the warp's next (element, table)
+            const uint32_t total = NT * size;
+            uint32_t taken = 0, idx = 0, v = 0;
+            bool busy = false;
+            for (;;) {
+                const uint32_t idle = __ballot_sync(0xffffffffu, !busy);
+                if (!busy) {
+                    const uint32_t k = taken + __popc(idle & ((1u << lane) - 1u));
+                    idx = ((k >> 5) * warps + warp) * 32u + (k & 31u);
+                    if (idx < total) {
+                        v = table[idx / NT];
+                        busy = v < P.m;  // else rejected by validation
+                        if (!busy) code[idx] = 0, pos[idx] = 0;
                     }
                 }
-            } else if (((taken >> 5) * warps + warp) * 32u >= total) {
-                break;
+                taken += __popc(idle);
+                if (__any_sync(0xffffffffu, busy)) {
+                    if (busy) {
+                        v = P.pass(P.key[idx % NT], v);
+                        if (v < P.m) {
+                            pos[idx] = (uint16_t)(v & rm);
+                            code[idx] = (uint8_t)((v >> J.shift) + 1u);
+                            busy = false;
+                        }
+                    }
+                } else if (((taken >> 5) * warps + warp) * 32u >= total) {
+                    break;
+                }
             }
         }
         __syncthreads();
@@ -301,7 +320,77 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
         // L1 may hold lines of an earlier use of the region: loads go to L2
         const bool lossy = drops[T.q] != 0;
         const uint64_t slots = (uint64_t)NT << rlog, s0 = (uint64_t)T.k * B_SLOTS + sub * B_SUB;
+        const uint32_t low = (1u << J.shift) - 1u;
         uint32_t *out = reinterpret_cast<uint32_t *>(J.out + J.base[I.item]);
+        // The entries of a pass: each looks into the next table.  `same`: all lie in one table, t0,
+        // at positions h0 on; its next one's keys are read once and no slot is taken apart.
+        auto entries = [&](auto one, Slot s, uint32_t used) {
+            constexpr bool ONE = decltype(one)::value;
+            const Slot seg0 = s >> J.shift;
+            const uint32_t t0 = ONE ? (uint32_t)(seg0 % NT) : 0, h0 = ONE ? ((uint32_t)(seg0 / NT) << J.shift) | ((uint32_t)s & low) : 0;
+            const uint32_t next0 = t0 + 1 == NT ? 0 : t0 + 1;
+            const uint4 key = P.key[next0];
+            const uint32_t *row = P.table + (uint64_t)next0 * P.m;
+            for (uint32_t k0 = 0; k0 < used; k0 += 64) {
+                // two entries a lane: their looks together
+                uint2 c[2];
+                uint32_t t[2], h[2], y[2];
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const uint32_t k = k0 + 32u * u + lane;
+                    y[u] = 0;
+                    if (k >= used) continue;
+                    c[u] = list[k];
+                    t[u] = t0;
+                    h[u] = h0 + c[u].y;
+                    uint32_t next = next0, pi;
+                    const uint32_t x = c[u].x & tidmask;
+                    if (!ONE) {
+                        const Slot at = s + c[u].y, seg = at >> J.shift;
+                        t[u] = (uint32_t)(seg % NT);
+                        h[u] = ((uint32_t)(seg / NT) << J.shift) | ((uint32_t)at & low);
+                        next = t[u] + 1 == NT ? 0 : t[u] + 1;
+                        pi = pi_of(P, next, x);
+                    } else {
+                        pi = P.table ? __ldg(&row[x]) : pi_by(P, key, x);
+                    }
+                    y[u] = __ldcg(&table[slot_of_h<NT, Slot>(next, pi & rm, J.shift)]);
+                }
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    if (k0 + 32u * u + lane >= used) continue;
+                    const uint32_t w = c[u].x, x = w & tidmask;
+                    const bool here = ((y[u] ^ w) & same) == 0;
+                    uint32_t has;
+                    bool whole = true;
+                    if (NT == 3 && !lossy) {  // in the next table or the one after
+                        const uint32_t at = t[u] + (here ? 1 : 2);
+                        has = 1u << t[u] | 1u << (at >= NT ? at - NT : at);
+                    } else {
+                        // the tables that hold x: t and, of the others, all but one; without lost copies the
+                        // last need not be looked at
+                        uint32_t at = t[u] + 1 == NT ? 0 : t[u] + 1, found = here ? 2 : 1;
+                        has = 1u << t[u] | (here ? 1u << at : 0u);
+                        for (uint32_t o = 2; o < NT; o++) {
+                            at = at + 1 == NT ? 0 : at + 1;
+                            if (!lossy && (found < o || o + 1 == NT)) {  // the missing table is known, or left to the last
+                                if (found == NT - 1) break;
+                                has |= 1u << at;
+                                found++;
+                            } else if (((__ldcg(&table[slot_of_h<NT, Slot>(at, pi_of(P, at, x) & rm, J.shift)]) ^ w) & same) == 0) {
+                                has |= 1u << at;
+                                found++;
+                            }
+                        }
+                        whole = found == NT - 1;
+                    }
+                    if (whole) {
+                        const uint32_t pi = known ? (((w >> tbits) & ((1u << hbits) - 1u)) << rlog) | h[u] : pi_of(P, t[u], x);
+                        bytes[c[u].y] = (uint8_t)byte_of<NT>(has, t[u], (pi >> J.shift) + 1u);
+                    }
+                }
+            }
+        };
         for (uint64_t s = s0; s < min(slots, s0 + B_SUB); s += B_PASS) {
             // the used slots of the pass, packed: few of a table's slots are used, and each costs a
             // permutation and a load
@@ -321,50 +410,8 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
                 }
             }
             __syncwarp();
-            for (uint32_t k0 = 0; k0 < used; k0 += 64) {
-                // two entries a lane: their looks into the next table together
-                uint2 c[2];
-                uint32_t t[2], h[2], y[2];
-#pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    const uint32_t k = k0 + 32u * u + lane;
-                    y[u] = 0;
-                    if (k >= used) continue;
-                    c[u] = list[k];
-                    const uint64_t at = s + c[u].y, seg = at >> J.shift;
-                    t[u] = (uint32_t)(seg % NT);
-                    h[u] = ((uint32_t)(seg / NT) << J.shift) | ((uint32_t)at & ((1u << J.shift) - 1u));
-                    const uint32_t next = t[u] + 1 == NT ? 0 : t[u] + 1;
-                    y[u] = __ldcg(&table[slot_of_h<NT, Slot>(next, pi_of(P, next, c[u].x & tidmask) & rm, J.shift)]);
-                }
-#pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    if (k0 + 32u * u + lane >= used) continue;
-                    const uint32_t w = c[u].x, x = w & tidmask;
-                    // the tables that hold x: t and, of the others, all but one; without lost copies the
-                    // last need not be looked at
-                    uint32_t at = t[u] + 1 == NT ? 0 : t[u] + 1, has = 1u << t[u], found = 1;
-                    if (((y[u] ^ w) & same) == 0) {
-                        has |= 1u << at;
-                        found = 2;
-                    }
-                    for (uint32_t o = 2; o < NT; o++) {
-                        at = at + 1 == NT ? 0 : at + 1;
-                        if (!lossy && (found < o || o + 1 == NT)) {  // the missing table is known, or left to the last
-                            if (found == NT - 1) break;
-                            has |= 1u << at;
-                            found++;
-                        } else if (((__ldcg(&table[slot_of_h<NT, Slot>(at, pi_of(P, at, x) & rm, J.shift)]) ^ w) & same) == 0) {
-                            has |= 1u << at;
-                            found++;
-                        }
-                    }
-                    if (found == NT - 1) {
-                        const uint32_t pi = known ? (((w >> tbits) & ((1u << hbits) - 1u)) << rlog) | h[u] : pi_of(P, t[u], x);
-                        bytes[c[u].y] = (uint8_t)byte_of<NT>(has, t[u], (pi >> J.shift) + 1u);
-                    }
-                }
-            }
+            if (1u << J.shift >= B_PASS) entries(std::true_type{}, (Slot)s, used);  // (passes and tables' blocks are powers of two)
+            else entries(std::false_type{}, (Slot)s, used);
             __syncwarp();
 #pragma unroll
             for (uint32_t i = 0; i < B_PASS / 128; i++) {

@@ -569,7 +569,7 @@ def batch_record(args, steps, warmup, small=False, instances=64, autotune=True):
         results[name]["compare_equiv_lane_op_frac"] = OPS_PER_WORD_PAIR * wp / t / 1e12 / alu_peak
     results["compare_equiv_definition"] = (
         "4 x sum over all pairs of max(|B_i|,|B_j|)/4 word pairs (the scan's work for every pair, "
-        "probe-routed pairs included) / compare time / lane-op peak")
+        "probe-routed pairs included) / compare time / lane-op peak; far above 1 where bit rows answer")
     results["probe_routed_share"] = sum(b.info["probe_word_pairs"] for b in sets) / wp
     # batched and plain give identical outputs; a sampled oracle check per instance
     batch_pairs = [b[:k].cpu().numpy().copy() for b, k in zip(bufs, n_out)]
@@ -736,7 +736,7 @@ def run_cross(args):
             "roofline": roofline,
             "phases_ms": {p: statistics.mean(t[p] for t in phases)
                           for p in ("build_ms", "compare_ms", "scan_ms", "probe_ms", "compact_ms")},
-            "probe_routed_share": info["probe_word_pairs"] / max(info["word_pairs"], 1.0),
+            "probe_routed_share": info["probe_word_pairs"] / max(info["word_pairs"], 1.0) if scan_s else 0.0,
             "nonempty_pairs": n_out, "failed_insertions": info["n_failed"], "gpu_launches": int(launches),
             "parity_sample": {"pairs": int(ia.size), "exact": bool(np.array_equal(got, ref))},
             "clocks": clocks}

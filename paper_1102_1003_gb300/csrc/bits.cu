@@ -18,7 +18,7 @@ namespace bm {
 
 constexpr uint32_t CHUNK_KB = 64;                    // blocks per warp
 constexpr uint32_t CHUNK_BITS = CHUNK_KB * BITS_K;   // 16,384
-constexpr int BW = 8;                                // warps per CTA
+constexpr int BW = 1;                                // warps per CTA: none waits for a neighbour with a longer list
 
 // A longer list repeats tids; it is reported as not sorted without a look at it.  So
 // places and searches take 32 bits.
@@ -243,7 +243,7 @@ bool take_bits(BmBuf *buf, uint64_t bytes) {
 // ones, from L1; popcount issues at 16 per clock and SM, so 511,714 triples of
 // 3,128 words take at least 0.32 ms, and their rows 6.4 GB of L2 reads.
 template <int K, int G, int W>
-__global__ void __launch_bounds__(256) k_bits_support(const uint4 *__restrict__ bits, uint32_t chunks,
+__global__ void __launch_bounds__(256, 4) k_bits_support(const uint4 *__restrict__ bits, uint32_t chunks,
                                                       const uint32_t *__restrict__ items, uint64_t nq,
                                                       uint32_t *__restrict__ out) {
     const uint32_t t = threadIdx.x % (32 * W);

@@ -38,6 +38,8 @@ namespace bm {
 namespace place {
 
 constexpr uint32_t SMALL_RLOG = 13;
+constexpr uint32_t FIRST_MOVES = 16;  // of a chain before it waits for the others
+static_assert(5u << SMALL_RLOG <= 1u << 16, "a slot of the widest table in 16 bits");
 static_assert(SMALL_RLOG < PLACE_QUEUES, "a queue per width in shared memory");
 constexpr uint64_t PLACE_L2_BYTES = 96ull << 20;
 constexpr uint32_t SEQS = 2;
@@ -99,23 +101,24 @@ __device__ __forceinline__ void record(const PlaceJob &J, uint32_t item, uint32_
 
 // One CTA per item, items from a queue.  Dynamic shared memory: NT 2^rlog
 // entries (first the tids, then element indices, then the item's bytes); per
-// element and table its position h_t = pi_t mod r (16 bits) and code (8 bits, 0:
+// element and table its slot (16 bits: at most 5 * 8,192 slots) and code (8 bits, 0:
 // not a tid); per element the tables that hold it (8 bits).  Each pi_t(x) is
-// computed once: chains and bytes read positions and codes.
+// computed once: chains and bytes read slots and codes.
 template <int NT>
 __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ PlaceJob J,
                                                       const __grid_constant__ PermView P, uint32_t cap) {
     extern __shared__ __align__(16) uint32_t table[];
-    __shared__ uint32_t s_item;
+    __shared__ uint32_t s_item, s_late;
     const uint32_t slots = (uint32_t)NT << J.rlog, rm = (1u << J.rlog) - 1u;
     uint8_t *bytes = reinterpret_cast<uint8_t *>(table);
-    uint16_t *pos = reinterpret_cast<uint16_t *>(table + slots);  // [cap][NT]
-    uint8_t *code = reinterpret_cast<uint8_t *>(pos + NT * cap);  // [cap][NT]
-    uint8_t *held = code + NT * cap;                              // [cap]
+    uint16_t *slot = reinterpret_cast<uint16_t *>(table + slots);  // [cap][NT]
+    uint8_t *code = reinterpret_cast<uint8_t *>(slot + NT * cap);  // [cap][NT]
+    uint8_t *held = code + NT * cap;                               // [cap]
+    uint32_t *late = reinterpret_cast<uint32_t *>(held);           // [cap / 4], before held is written
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tpb = blockDim.x, warps = tpb / 32;
     uint4 *t4 = reinterpret_cast<uint4 *>(table);
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(J.queue, 1u);
+        if (threadIdx.x == 0) s_item = atomicAdd(J.queue, 1u), s_late = 0;
         __syncthreads();
         if (s_item >= J.count) break;
         const uint32_t item = J.items[s_item];
@@ -131,7 +134,7 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
                 for (uint32_t t = 0; t < NT; t++) v[t] = x < P.m ? __ldg(&P.table[(uint64_t)t * P.m + x]) : 0;
 #pragma unroll
                 for (uint32_t t = 0; t < NT; t++) {
-                    pos[e * NT + t] = (uint16_t)(v[t] & rm);
+                    slot[e * NT + t] = (uint16_t)slot_of_h<NT, uint32_t>(t, v[t] & rm, J.shift);
                     code[e * NT + t] = x < P.m ? (uint8_t)((v[t] >> J.shift) + 1u) : 0;  // else rejected by validation
                 }
             }
@@ -149,7 +152,7 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
                     if (idx < total) {
                         v = table[idx / NT];
                         busy = v < P.m;  // else rejected by validation
-                        if (!busy) code[idx] = 0, pos[idx] = 0;
+                        if (!busy) code[idx] = 0, slot[idx] = 0;
                     }
                 }
                 taken += __popc(idle);
@@ -157,7 +160,7 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
                     if (busy) {
                         v = P.pass(P.key[idx % NT], v);
                         if (v < P.m) {
-                            pos[idx] = (uint16_t)(v & rm);
+                            slot[idx] = (uint16_t)slot_of_h<NT, uint32_t>(idx % NT, v & rm, J.shift);
                             code[idx] = (uint8_t)((v >> J.shift) + 1u);
                             busy = false;
                         }
@@ -170,16 +173,34 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
         __syncthreads();
         for (uint32_t k = threadIdx.x; k < slots / 4; k += tpb) t4[k] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
         __syncthreads();
+        // the chain of copy (e, t) goes on; true: it ended in an empty slot
+        auto walk = [&](uint32_t &e, uint32_t &t, uint32_t moves) {
+            for (uint32_t mv = 0; mv < moves; mv++) {
+                e = atomicExch(&table[slot[e * NT + t]], e);
+                if (e == EMPTY) return true;
+                t = t + 1 == NT ? 0 : t + 1;  // the same element: another of its copies, go on
+            }
+            return false;
+        };
+        // Few chains are long, and those of elements that cannot be placed take all their moves: they wait
+        // in a list until the rest is in, then go side by side and not one after another (3-of-4 and 4-of-5
+        // sets of n = 1,000, m = 100,000: launches of 120 us each, passes 1833 -> 1553 and 2631 -> 2412 us
+        // with the next rule for those in L2).
+        const uint32_t soon = min(J.max_moves, FIRST_MOVES), rest = J.max_moves - soon;
         for (uint32_t c = 0; c < NT - 1; c++)
             for (uint32_t k = threadIdx.x; k < size; k += tpb) {
                 if (!code[k * NT]) continue;
                 uint32_t e = k, t = c;
-                for (uint32_t mv = 0; mv < J.max_moves; mv++) {
-                    e = atomicExch(&table[slot_of_h<NT, uint32_t>(t, pos[e * NT + t], J.shift)], e);
-                    if (e == EMPTY) break;
-                    t = t + 1 == NT ? 0 : t + 1;  // the same element: another of its copies, go on
-                }
+                if (walk(e, t, soon) || !rest) continue;
+                const uint32_t at = atomicAdd(&s_late, 1u);
+                if (at < cap / 4) late[at] = e | t << 16;
+                else walk(e, t, rest);
             }
+        __syncthreads();
+        for (uint32_t k = threadIdx.x; k < min(s_late, cap / 4); k += tpb) {
+            uint32_t e = late[k] & 0xFFFFu, t = late[k] >> 16;
+            walk(e, t, rest);
+        }
         __syncthreads();
         for (uint32_t e = threadIdx.x; e < (size + 31u) / 32u * 32u; e += tpb) {
             bool failed = false;
@@ -187,7 +208,7 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
                 uint32_t has = 0;
 #pragma unroll
                 for (uint32_t t = 0; t < NT; t++)
-                    has |= (table[slot_of_h<NT, uint32_t>(t, pos[e * NT + t], J.shift)] == e ? 1u : 0u) << t;
+                    has |= (table[slot[e * NT + t]] == e ? 1u : 0u) << t;
                 const bool valid = code[e * NT] != 0, whole = valid && __popc(has) == NT - 1;
                 failed = valid && !whole;
                 held[e] = whole ? (uint8_t)has : 0;
@@ -202,7 +223,7 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
 #pragma unroll
             for (uint32_t t = 0; t < NT; t++)
                 if ((has >> t) & 1u)
-                    bytes[slot_of_h<NT, uint32_t>(t, pos[e * NT + t], J.shift)] = (uint8_t)byte_of<NT>(has, t, code[e * NT + t]);
+                    bytes[slot[e * NT + t]] = (uint8_t)byte_of<NT>(has, t, code[e * NT + t]);
         }
         __syncthreads();
         uint4 *out = reinterpret_cast<uint4 *>(J.out + J.base[item]);
@@ -460,8 +481,11 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     // n = 2,048 (6.3 MB an item): one sequence 21.0 ms, two with 4 items a region 19.4, with 3 items
     // 17.9 (75 MB in use), three with 2 items 17.9; zipf m = 1 M, n = 2,000 (up to 25 MB) 2.2 and 2.0 ms.
     const uint64_t part = std::max<uint64_t>(widest, SEQ_REGION / 4);
-    const uint32_t seqs = 2 * SEQS * part <= PLACE_L2_BYTES / 4 && total >= 2 * SEQS * part ? SEQS : 1;
-    const uint64_t region = (seqs > 1 ? part : std::max<uint64_t>(widest, PLACE_L2_BYTES / 4 / 2)) / 64 * 64;  // (16-byte loads)
+    // Everything in one batch where it fits: insertions, then bytes (two batches of the above triples' sets
+    // took three launches, each as long as its longest chains).
+    const bool once = total <= PLACE_L2_BYTES / 4;
+    const uint32_t seqs = !once && 2 * SEQS * part <= PLACE_L2_BYTES / 4 && total >= 2 * SEQS * part ? SEQS : 1;
+    const uint64_t region = once ? total : (seqs > 1 ? part : std::max<uint64_t>(widest, PLACE_L2_BYTES / 4 / 2)) / 64 * 64;  // (16-byte loads)
     static const bool ready = [] {
         BM_CUDA(cudaFuncSetAttribute(k_place_large<NT, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LARGE_SMEM));
         BM_CUDA(cudaFuncSetAttribute(k_place_large<NT, uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LARGE_SMEM));
@@ -556,8 +580,9 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
     std::vector<uint32_t> ids;
     for (const PlaceItem &I : list) ids.push_back(I.item);
     BM_CUDA(cudaMemcpyAsync(d_list, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, side));
-    if (mid != list.begin()) place_large<NT>(job, P, std::vector<PlaceItem>(list.begin(), mid), streams);
+    // (widths side by side on streams of their own: triples 2% slower, quadruples 10%)
     uint32_t launch = 0;
+    if (mid != list.begin()) place_large<NT>(job, P, std::vector<PlaceItem>(list.begin(), mid), streams);
     for (size_t k = mid - list.begin(); k < list.size();) {
         size_t e = k;
         uint64_t most = 0;

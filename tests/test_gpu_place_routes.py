@@ -58,3 +58,16 @@ def test_table_of_computed_permutations(d, m, size, less):
         r, at = int(lay["range"][i]), int(lay["byte_offset"][i])
         failed = lay["fail_tids"][int(lay["fail_offsets"][i]):int(lay["fail_offsets"][i + 1])]
         assert list(R.check_layout(lay["bytes"][at:at + (d + 1) * r], inst.tidlist(i), failed, perms, r, r0, s, d)) == []
+
+
+# elements that cannot be placed: none, some, and more chains than the list of long ones holds
+@pytest.mark.parametrize("load", [(2, 1), (1, 1), (1, 2)])
+@pytest.mark.parametrize("max_loop", [5, 6, 32])  # 15, 18 and 96 moves, 16 before a chain waits
+@pytest.mark.parametrize("m", [60_000, 4_096])
+def test_long_chains_in_shared_memory(load, max_loop, m):
+    import paper_1102_1003_gb300 as pkg
+    inst = _items(m, [0, 1, 33, 1_000, 2_047, 4_000, 4_096, 4_096], seed=max_loop)
+    off, tids, _ = device_inputs(inst, 5)
+    b = pkg.batmap_build(m, off, tids, params=seeded_params(5, pkg.batmap_default_params(
+        load_num=load[0], load_den=load[1], max_loop=max_loop)))
+    assert layout_errors(inst, b, 5, *load) == []

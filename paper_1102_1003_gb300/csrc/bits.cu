@@ -16,8 +16,6 @@
 
 namespace bm {
 
-constexpr uint32_t CHUNK_KB = 64;                    // blocks per warp
-constexpr uint32_t CHUNK_BITS = CHUNK_KB * BITS_K;   // 16,384
 constexpr int BW = 1;                                // warps per CTA: none waits for a neighbour with a longer list
 
 // A longer list repeats tids; it is reported as not sorted without a look at it.  So
@@ -62,9 +60,11 @@ __device__ __forceinline__ void load_block(TidBlock &B, const uint32_t *__restri
     }
 }
 
+template <uint32_t CHUNK_KB>
 __global__ void __launch_bounds__(32 * BW)
 k_bits(const uint64_t *__restrict__ off, const uint32_t *__restrict__ tids, uint32_t n, uint32_t m, BitsLayout L,
        uint32_t run, uint8_t *__restrict__ out, int *__restrict__ flags) {
+    constexpr uint32_t CHUNK_BITS = CHUNK_KB * BITS_K;
     __shared__ __align__(16) uint32_t s_bits[BW][CHUNK_BITS / 32];
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t *bits = s_bits[threadIdx.x >> 5];
@@ -200,16 +200,32 @@ __global__ void k_bits_unsorted(const uint64_t *__restrict__ off, const uint32_t
     }
 }
 
+// Blocks per chunk.  Fewer chunks than FEW_TASKS (two warps for each that the chip holds): a quarter of that, as
+// the time is that of a full list's chunk (triples of n = 1,000, m = 100,000
+// with full lists: the pass 1572 -> 1542 us).
+constexpr uint32_t CHUNK_KB = 64;
+constexpr uint64_t FEW_TASKS = 152 * 32 * 2;
+
+template <uint32_t KB>
+static void launch_bits(const uint64_t *d_off, const uint32_t *d_tids, uint32_t n, uint32_t m, const BitsLayout &L,
+                        uint32_t run, uint8_t *d_bits, int *d_flags, cudaStream_t st) {
+    const uint32_t nchunk = (L.kblocks + KB - 1) / KB;
+    const uint64_t tasks = (uint64_t)n * ((nchunk + run - 1) / run);
+    const unsigned grid = (unsigned)std::min<uint64_t>((tasks + BW - 1) / BW, 1u << 20);
+    k_bits<KB><<<grid, 32 * BW, 0, st>>>(d_off, d_tids, n, m, L, run, d_bits, d_flags);
+}
+
 void enqueue_bits(const uint64_t *d_off, const uint32_t *d_tids, uint32_t n, uint32_t m, const BitsLayout &L,
                   uint8_t *d_bits, int *d_flags, bool sorted_only, cudaStream_t st) {
     if (!n) return;
     const uint32_t nchunk = (L.kblocks + CHUNK_KB - 1) / CHUNK_KB;
-    // chunks per warp: about 200,000 warps (many rounds of the chip) before a warp takes several,
-    // which saves it their searches
-    const uint32_t run = (uint32_t)std::min<uint64_t>(16, std::max<uint64_t>(1, (uint64_t)n * nchunk / 200000));
-    const uint64_t tasks = (uint64_t)n * ((nchunk + run - 1) / run);
-    const unsigned grid = (unsigned)std::min<uint64_t>((tasks + BW - 1) / BW, 1u << 20);
-    k_bits<<<grid, 32 * BW, 0, st>>>(d_off, d_tids, n, m, L, run, d_bits, d_flags);
+    if ((uint64_t)n * nchunk < FEW_TASKS)
+        launch_bits<CHUNK_KB / 4>(d_off, d_tids, n, m, L, 1, d_bits, d_flags, st);
+    else  // chunks per warp: about 200,000 warps (many rounds of the chip) before a warp takes several,
+          // which saves it their searches
+        launch_bits<CHUNK_KB>(d_off, d_tids, n, m, L,
+                              (uint32_t)std::min<uint64_t>(16, std::max<uint64_t>(1, (uint64_t)n * nchunk / 200000)), d_bits,
+                              d_flags, st);
     BM_CHECK_LAUNCH();
     if (!sorted_only) {
         k_bits_unsorted<<<dim3(8, std::min<uint32_t>(n, 128u)), 256, 0, st>>>(d_off, d_tids, n, m, L, d_bits, d_flags);

@@ -12,7 +12,8 @@
 // a count pass, a scan and a write pass that ranked 256 supports at a time and
 // searched each one's row: 598 us for 32 M pairs of n = 8,000, all frequent
 // (512 MB: 76 us at the copy rate); this one 218 us with 72 registers, three blocks
-// per SM that wait at their barriers, and about 175 with 48 and 32-bit row borders.
+// per SM that wait at their barriers, 177 with 48 and 32-bit row borders, 167 with a
+// stage of each warp's own, behind no barrier but those of the count.
 #include <algorithm>
 
 #include "common.cuh"
@@ -23,7 +24,8 @@ namespace bm {
 constexpr int CTPB = SCAN_TPB;
 constexpr int CQ = 4;                                // 16-byte loads per thread
 constexpr uint32_t CCHUNK = CTPB * 4 * CQ;           // 4,096 supports per tile
-constexpr uint32_t CSTAGE = CCHUNK / 2;              // triples staged at a time
+constexpr uint32_t CWARPS = CTPB / 32;
+constexpr uint32_t CSTAGE = 128;                     // triples that a warp stages at a time
 
 __global__ void k_apply_corrections(const uint32_t *__restrict__ corr, uint64_t ncorr, uint64_t n,
                                     uint32_t n_a, uint32_t *__restrict__ C) {
@@ -55,10 +57,10 @@ __global__ void __launch_bounds__(CTPB, 5) k_threshold(const uint32_t *__restric
                                                     uint32_t n_a, uint32_t s, uint64_t *__restrict__ state,
                                                     uint64_t tiles, uint32_t *__restrict__ out, uint64_t cap,
                                                     uint64_t *__restrict__ total) {
-    __shared__ uint32_t s_out[3 * CSTAGE];
+    __shared__ uint32_t s_out[CWARPS][3 * CSTAGE];
     __shared__ uint64_t s_tile, s_before;
-    __shared__ uint32_t s_rows[2];
-    const uint32_t lane = threadIdx.x & 31u;
+    __shared__ uint32_t s_rows[2], s_count[CWARPS];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) s_tile = atomicAdd((unsigned long long *)&state[tiles], 1ull);
     __syncthreads();
     const uint64_t tile = s_tile, base = tile * CCHUNK;
@@ -66,14 +68,15 @@ __global__ void __launch_bounds__(CTPB, 5) k_threshold(const uint32_t *__restric
         const uint64_t L = threadIdx.x == 32 ? base : min(base + CCHUNK, npairs) - 1;
         s_rows[threadIdx.x - 32] = row_of(L, n, n_a, 0, n_a ? n_a - 1 : (uint32_t)n - 2);
     }
-    // thread t holds the supports base + 1024 q + 4 t + j
+    // a lane holds the supports base + place + 128 q + j
+    const uint32_t place = CSTAGE * CQ * warp + 4u * lane;
     uint32_t v[CQ][4];
-    uint64_t packed = 0;  // per q, the thread's number of qualifying supports (16 bits each)
+    uint64_t packed = 0;  // per q, the lane's number of qualifying supports (16 bits each)
     const bool vec = (reinterpret_cast<uintptr_t>(C) & 15u) == 0;
     uint32_t keep = 0;
 #pragma unroll
     for (int q = 0; q < CQ; q++) {
-        const uint64_t L = base + 1024u * q + 4u * threadIdx.x;
+        const uint64_t L = base + place + CSTAGE * q;
         if (vec && L + 4 <= npairs) {
             const uint4 x = __ldg(reinterpret_cast<const uint4 *>(C + L));
             v[q][0] = x.x; v[q][1] = x.y; v[q][2] = x.z; v[q][3] = x.w;
@@ -85,9 +88,23 @@ __global__ void __launch_bounds__(CTPB, 5) k_threshold(const uint32_t *__restric
         for (int j = 0; j < 4; j++) keep |= (v[q][j] >= s && L + j < npairs ? 1u : 0u) << (4 * q + j);
         packed |= (uint64_t)__popc((keep >> (4 * q)) & 15u) << (16 * q);
     }
-    uint64_t sums;
-    const uint64_t pre = block_exclusive_scan(packed, &sums);  // four 16-bit scans (<= 1024 each)
-    const uint32_t count = (uint32_t)((sums & 0xFFFF) + ((sums >> 16) & 0xFFFF) + ((sums >> 32) & 0xFFFF) + (sums >> 48));
+    uint64_t pre = packed;  // four 16-bit scans over the warp (<= 128 each)
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xffffffffu, pre, d);
+        if (lane >= (uint32_t)d) pre += y;
+    }
+    const uint64_t sums = __shfl_sync(0xffffffffu, pre, 31);
+    pre -= packed;
+    if (lane == 0)
+        s_count[warp] = (uint32_t)((sums & 0xFFFF) + ((sums >> 16) & 0xFFFF) + ((sums >> 32) & 0xFFFF) + (sums >> 48));
+    __syncthreads();
+    uint32_t count = 0, ahead = 0;  // the tile's, and those of the warps before
+#pragma unroll
+    for (uint32_t w = 0; w < CWARPS; w++) {
+        ahead += w < warp ? s_count[w] : 0;
+        count += s_count[w];
+    }
     if (threadIdx.x < 32) {
         if (lane == 0 && tile)
             *(volatile uint64_t *)&state[tile] = STATE_SUM | count;
@@ -101,46 +118,40 @@ __global__ void __launch_bounds__(CTPB, 5) k_threshold(const uint32_t *__restric
     __syncthreads();
     const uint64_t before = s_before;
     if (before == ~0ull || !out || before >= cap || !count) return;
-    const uint32_t room = (uint32_t)min((uint64_t)count, cap - before);
     const uint32_t r0 = s_rows[0], r1 = s_rows[1];
-    for (uint32_t p0 = 0; p0 < room; p0 += CSTAGE) {
-        uint32_t first = 0;  // rank of the q-th kilobyte's first qualifying support
+    uint64_t to = before + ahead;  // the warp's next triple
+    uint32_t *stage = s_out[warp];
 #pragma unroll
-        for (int q = 0; q < CQ; q++) {
-            uint32_t rank = first + (uint32_t)((pre >> (16 * q)) & 0xFFFF);
-            const uint32_t bits = (keep >> (4 * q)) & 15u;
-            if (bits && rank < p0 + CSTAGE && rank + 4 > p0) {
-                const uint64_t L = base + 1024u * q + 4u * threadIdx.x;
-                const uint32_t p = 1024u * q + 4u * threadIdx.x;  // its place in the tile
-                uint32_t i = row_of(L, n, n_a, r0, r1);
-                // starts of its row (modulo 2^32) and of the next, from the tile's first place on
-                uint32_t here = (uint32_t)(row_start(i, n, n_a) - base);
-                uint32_t next = i < r1 ? (uint32_t)(row_start(i + 1ull, n, n_a) - base) : CCHUNK;
+    for (int q = 0; q < CQ; q++) {
+        const uint32_t found = (uint32_t)(sums >> (16 * q)) & 0xFFFF, bits = (keep >> (4 * q)) & 15u;
+        if (bits) {
+            uint32_t rank = (uint32_t)(pre >> (16 * q)) & 0xFFFF;
+            const uint32_t p = place + CSTAGE * q;  // its place in the tile
+            uint32_t i = row_of(base + p, n, n_a, r0, r1);
+            // starts of its row (modulo 2^32) and of the next, from the tile's first place on
+            uint32_t here = (uint32_t)(row_start(i, n, n_a) - base);
+            uint32_t next = i < r1 ? (uint32_t)(row_start(i + 1ull, n, n_a) - base) : CCHUNK;
 #pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    while (p + j >= next && i < r1) {
-                        i++;
-                        here = next;
-                        next = i < r1 ? (uint32_t)(row_start(i + 1ull, n, n_a) - base) : CCHUNK;
-                    }
-                    if ((bits >> j) & 1u) {
-                        if (rank >= p0 && rank < p0 + CSTAGE) {
-                            uint32_t *o = s_out + 3 * (rank - p0);
-                            o[0] = i;
-                            o[1] = p + j - here + (n_a ? 0 : i + 1);  // B items count from 0
-                            o[2] = v[q][j];
-                        }
-                        rank++;
-                    }
+            for (int j = 0; j < 4; j++) {
+                while (p + j >= next && i < r1) {
+                    i++;
+                    here = next;
+                    next = i < r1 ? (uint32_t)(row_start(i + 1ull, n, n_a) - base) : CCHUNK;
+                }
+                if ((bits >> j) & 1u) {
+                    uint32_t *o = stage + 3 * rank++;
+                    o[0] = i;
+                    o[1] = p + j - here + (n_a ? 0 : i + 1);  // B items count from 0
+                    o[2] = v[q][j];
                 }
             }
-            first += (uint32_t)((sums >> (16 * q)) & 0xFFFF);
         }
-        __syncthreads();
-        const uint32_t words = 3 * min(room - p0, CSTAGE);
-        uint32_t *o = out + 3 * (before + p0);
-        for (uint32_t w = threadIdx.x; w < words; w += CTPB) o[w] = s_out[w];
-        __syncthreads();
+        __syncwarp();
+        const uint32_t words = to < cap ? 3 * (uint32_t)min((uint64_t)found, cap - to) : 0;
+        uint32_t *o = out + 3 * to;
+        for (uint32_t w = lane; w < words; w += 32) o[w] = stage[w];
+        __syncwarp();
+        to += found;
     }
 }
 

@@ -1,6 +1,7 @@
 // Bit rows from CSR tidlists (the bitmap vertical representation, Sec. I-B).
 //
-// One warp writes one item's bits of a run of 16,384-transaction chunks: it finds
+// One warp writes one item's bits of a run of 16,384-transaction chunks (4,096 where
+// there are few tasks, and then 512 bytes of shared memory, not 2 KiB): it finds
 // the run's tids by two 32-way searches side by side (about log32 |S| dependent
 // reads), then walks them in blocks of 256 (16-byte loads, the next block on its
 // way), ORs a chunk's into 2 KiB of shared memory and stores its 64 blocks of 32
@@ -9,7 +10,9 @@
 // Bound: HBM, 4 bytes read per tid and 1 bit written per (item, transaction);
 // short lists by the latency of the searches (hence runs), skewed families by
 // the warps of full lists, one tid per bit, which end last (hence runs only
-// where there are warps enough).
+// where there are warps enough, and a block of its own for each).  Zipf n = 2,000,
+// m = 10^6 (40 M tids, 250 MB of rows): 318 us with eight warps a block and 64-bit
+// places, 287 with 32-bit ones, about 250 with one warp a block.
 #include <algorithm>
 
 #include "bits.cuh"
@@ -257,7 +260,8 @@ bool take_bits(BmBuf *buf, uint64_t bytes) {
 // four ANDs and four popcounts per chunk.  Queries that differ earlier go one by
 // one.  Rows come from L2 (12.5 MB at m = 100,000, n = 1,000) and, for the shared
 // ones, from L1; popcount issues at 16 per clock and SM, so 511,714 triples of
-// 3,128 words take at least 0.32 ms, and their rows 6.4 GB of L2 reads.
+// 3,128 words take at least 0.32 ms, and their rows 6.4 GB of L2 reads; measured
+// 0.46 ms with three blocks a multiprocessor (67 registers), 0.43 with four.
 template <int K, int G, int W>
 __global__ void __launch_bounds__(256, 4) k_bits_support(const uint4 *__restrict__ bits, uint32_t chunks,
                                                       const uint32_t *__restrict__ items, uint64_t nq,

@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
         }
         __syncthreads();
         for (uint32_t k = threadIdx.x; k < slots / 4; k += tpb) t4[k] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
+        for (uint32_t k = slots / 4 * 4 + threadIdx.x; k < slots; k += tpb) table[k] = EMPTY;
         __syncthreads();
         // the chain of copy (e, t) goes on; true: it ended in an empty slot
         auto walk = [&](uint32_t &e, uint32_t &t, uint32_t moves) {
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
         }
         __syncthreads();
         for (uint32_t k = threadIdx.x; k < slots / 16; k += tpb) t4[k] = make_uint4(0, 0, 0, 0);
+        for (uint32_t k = slots / 16 * 4 + threadIdx.x; 4 * k < slots; k += tpb) table[k] = 0;
         __syncthreads();
         for (uint32_t e = threadIdx.x; e < size; e += tpb) {
             const uint32_t has = held[e];
@@ -227,8 +229,13 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
                     bytes[slot[e * NT + t]] = (uint8_t)byte_of<NT>(has, t, code[e * NT + t]);
         }
         __syncthreads();
-        uint4 *out = reinterpret_cast<uint4 *>(J.out + J.base[item]);
-        for (uint32_t k = threadIdx.x; k < slots / 16; k += tpb) out[k] = t4[k];
+        uint8_t *to = J.out + J.base[item];
+        if (((slots | J.base[item]) & 15u) == 0) {
+            uint4 *out = reinterpret_cast<uint4 *>(to);
+            for (uint32_t k = threadIdx.x; k < slots / 16; k += tpb) out[k] = t4[k];
+        } else {  // BatMaps of less than 48 bytes, and those behind them
+            for (uint32_t k = threadIdx.x; k < slots; k += tpb) to[k] = bytes[k];
+        }
         __syncthreads();
     }
 }
@@ -343,7 +350,8 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
         const bool lossy = drops[T.q] != 0;
         const uint64_t slots = (uint64_t)NT << rlog, s0 = (uint64_t)T.k * B_SLOTS + sub * B_SUB;
         const uint32_t low = (1u << J.shift) - 1u;
-        uint32_t *out = reinterpret_cast<uint32_t *>(J.out + J.base[I.item]);
+        uint8_t *out = J.out + J.base[I.item];
+        const bool aligned = ((slots | J.base[I.item]) & 3u) == 0;  // (not so for ranges r below 4)
         // The entries of a pass: each looks into the next table.  `same`: all lie in one table, t0,
         // at positions h0 on; its next one's keys are read once and no slot is taken apart.
         auto entries = [&](auto one, Slot s, uint32_t used) {
@@ -438,7 +446,11 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
 #pragma unroll
             for (uint32_t i = 0; i < B_PASS / 128; i++) {
                 const uint32_t o = 128u * i + 4u * lane;
-                if (s + o < slots) __stcs(&out[(s + o) / 4], words[o / 4]);
+                if (aligned) {
+                    if (s + o < slots) __stcs(reinterpret_cast<uint32_t *>(out + s + o), words[o / 4]);
+                } else {
+                    for (uint32_t j = o; j < o + 4 && s + j < slots; j++) out[s + j] = bytes[j];
+                }
             }
             __syncwarp();
         }
@@ -462,6 +474,12 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
     }
 }
 
+// Words of an item's table in a region: whole 16-byte loads, also where the range is small.
+template <int NT>
+static uint64_t table_words(uint32_t rlog) {
+    return (((uint64_t)NT << rlog) + 63) / 64 * 64;
+}
+
 // The large items in order of the list (widest first): batches, places and tasks.
 template <int NT>
 static void place_large(const PlaceJob &job, const PermView &P, const std::vector<PlaceItem> &list, SideStream &streams) {
@@ -474,9 +492,9 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     const bool known = tbits + hbits <= 28;
     if (!known) hbits = 0;
     const uint32_t epochs = (1u << (32 - tbits - hbits)) - 1u;
-    const uint64_t widest = (uint64_t)NT << list[0].rlog;  // words
+    const uint64_t widest = table_words<NT>(list[0].rlog);
     uint64_t total = 0;
-    for (const PlaceItem &I : list) total += (uint64_t)NT << I.rlog;
+    for (const PlaceItem &I : list) total += table_words<NT>(I.rlog);
     // Two sequences of launches where there are batches for both and room for their regions: the end of
     // one's launch, a few long chains of exchanges, runs beside the body of the other's.  m = 2^22, 5%,
     // n = 2,048 (6.3 MB an item): one sequence 21.0 ms, two with 4 items a region 19.4, with 3 items
@@ -497,7 +515,7 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     std::vector<size_t> first;  // first item of each batch
     uint64_t fill = 0;
     for (size_t q = 0; q < list.size(); q++) {
-        const uint64_t words = (uint64_t)NT << list[q].rlog;
+        const uint64_t words = table_words<NT>(list[q].rlog);
         if (first.empty() || fill + words > region) {
             first.push_back(q);
             fill = 0;

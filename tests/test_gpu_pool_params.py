@@ -1,0 +1,40 @@
+"""Pools take hash ranges below the 2^7 that batmap_build asks for: BatMaps of 3
+bytes and more, whose neighbours start at any byte.  Counts against the merge
+oracle, exact."""
+import numpy as np
+import pytest
+
+import datagen
+import oracle
+from tests.gpu_util import device_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    torch.cuda.set_device(0)
+
+
+# load 1/50: more elements than slots, so that their tables go to L2; 16/1: wide tables beside narrow ones
+@pytest.mark.parametrize("load", [(2, 1), (16, 1), (1, 50)])
+@pytest.mark.parametrize("min_shift", [0, 1, 3, 6])
+@pytest.mark.parametrize("m", [1, 100, 127, 1_000, 9_000])
+def test_narrow_batmaps(m, min_shift, load):
+    import paper_1102_1003_gb300 as pkg
+    rng = np.random.default_rng(m + min_shift)
+    sizes = np.concatenate([np.full(12, 1), np.minimum(m, rng.integers(1, 40, 12)), rng.integers(1, m + 1, 12), [m, m]])
+    inst = datagen.from_lists([np.sort(rng.choice(m, s, replace=False)).astype(np.uint32) for s in sizes], m)
+    off, tids, _ = device_inputs(inst, 0)
+    p = pkg.batmap_default_params(min_shift=min_shift, load_num=load[0], load_den=load[1], max_loop=3)
+    pool = pkg.batmap_pool_create(m, off, tids, params=p)
+    qs = [[int(a), int(b)] for a in range(inst.n) for b in range(inst.n)] + rng.integers(0, inst.n, (200, 4)).tolist()
+    got = pkg.intersect_query(pool, qs).cpu().numpy().astype(np.uint64)
+    assert np.array_equal(got, oracle.kway_counts(inst.offsets, inst.tids, qs))
+    if load == (2, 1) and min_shift == 0 and m == 100:
+        assert pool.info["n_batmaps"] == inst.n  # even the sets of one element (r = 2: 6 bytes)

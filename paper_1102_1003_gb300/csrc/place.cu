@@ -248,6 +248,13 @@ struct LargeItem {
     uint32_t first_a, first_b, na, nb;  // its CTAs' tasks: insertions, bytes
     uint32_t pad;
 };
+// A displaced copy's next table and the moves of its chain so far (at most MAX_MOVES).
+__host__ __device__ constexpr uint32_t chain_word(uint32_t t, uint32_t moves) { return t | moves << 3; }
+__host__ __device__ constexpr uint32_t chain_table(uint32_t w) { return w & 7u; }
+__host__ __device__ constexpr uint32_t chain_moves(uint32_t w) { return w >> 3; }
+static_assert(chain_moves(chain_word(4, MAX_MOVES - 1)) + 1 == MAX_MOVES && chain_table(chain_word(4, MAX_MOVES - 1)) == 4,
+              "a chain's count reaches its limit");
+
 struct LargeTask {
     uint32_t q, k;  // k-th insertion task, or (LARGE_BYTES set) byte task, of large item q
 };
@@ -287,7 +294,7 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
         // First every copy's own exchange, all lanes in one table, four in flight; the displaced copies
         // go to a list, whose chains run on with full warps while it is long enough.
         const uint64_t b0 = (uint64_t)T.k * A_ELEMS + sub * A_SUB, b1 = min(size, b0 + A_SUB);
-        uint32_t waiting = 0;  // entries of the list: tid, table | moves << 3
+        uint32_t waiting = 0;  // entries of the list: tid, chain_word
         auto chains = [&](uint32_t least) {
             while (waiting >= least) {
                 const uint32_t n = min(waiting, 32u);
@@ -296,11 +303,11 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
                 uint2 next = make_uint2(0, 0);
                 bool lost = false;
                 if (lane < n) {
-                    const uint32_t t = c.y & 7u, pi = pi_of(P, t, c.x), high = known ? (pi >> rlog) << tbits : 0;
+                    const uint32_t t = chain_table(c.y), pi = pi_of(P, t, c.x), high = known ? (pi >> rlog) << tbits : 0;
                     const uint32_t old = atomicExch(&table[slot_of_h<NT, Slot>(t, pi & rm, J.shift)], tag | high | c.x);
-                    const uint32_t moves = (c.y >> 3) + 1;
+                    const uint32_t moves = chain_moves(c.y) + 1;
                     lost = (old >> eshift) == I.epoch;
-                    next = make_uint2(old & tidmask, (t + 1 == NT ? 0 : t + 1) | (moves << 3));
+                    next = make_uint2(old & tidmask, chain_word(t + 1 == NT ? 0 : t + 1, moves));
                     if (lost && moves >= J.max_moves) {
                         atomicAdd(&drops[T.q], 1u);
                         lost = false;
@@ -335,7 +342,7 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
                 for (int i = 0; i < 4; i++) {
                     const bool lost = (old[i] >> eshift) == I.epoch;  // (epochs start at 1)
                     const uint32_t mask = __ballot_sync(0xffffffffu, lost);
-                    if (lost) list[waiting + __popc(mask & below)] = make_uint2(old[i] & tidmask, (c + 1) | (1u << 3));
+                    if (lost) list[waiting + __popc(mask & below)] = make_uint2(old[i] & tidmask, chain_word(c + 1, 1));
                     waiting += __popc(mask);
                 }
                 __syncwarp();
@@ -648,9 +655,10 @@ PermView place_perms(const PermView &P, uint32_t tables, uint64_t total, Workspa
     return T;
 }
 
-void enqueue_place(uint32_t tables, const PlaceJob &job, const PermView &P, std::vector<PlaceItem> list,
+void enqueue_place(uint32_t tables, PlaceJob job, const PermView &P, std::vector<PlaceItem> list,
                    uint32_t *d_list, SideStream &streams) {
     if (list.empty()) return;
+    job.max_moves = std::min(job.max_moves, MAX_MOVES);
     BM_CUDA(cudaMemsetAsync(job.queue, 0, PLACE_QUEUES * sizeof(uint32_t), streams.side()));
     if (tables == 3) place::place_all<3>(job, P, list, d_list, streams);
     if (tables == 4) place::place_all<4>(job, P, list, d_list, streams);

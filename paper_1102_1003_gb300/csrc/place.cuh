@@ -27,7 +27,10 @@ struct PlaceItem {
     uint64_t size;
 };
 constexpr uint32_t PLACE_QUEUES = 64;
-void enqueue_place(uint32_t tables, const PlaceJob &job, const PermView &P, std::vector<PlaceItem> list,
+// Moves of a chain, whatever the job asks for: 5 tables times the largest max_loop of a build
+// are less; a pool's max_loop has no other bound (a move takes about a microsecond in L2).
+constexpr uint32_t MAX_MOVES = 1u << 23;
+void enqueue_place(uint32_t tables, PlaceJob job, const PermView &P, std::vector<PlaceItem> list,
                    uint32_t *d_list, SideStream &streams);
 
 // The permutations that the placement of `total` elements reads: a table in ws, written on

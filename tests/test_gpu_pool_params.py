@@ -38,3 +38,17 @@ def test_narrow_batmaps(m, min_shift, load):
     assert np.array_equal(got, oracle.kway_counts(inst.offsets, inst.tids, qs))
     if load == (2, 1) and min_shift == 0 and m == 100:
         assert pool.info["n_batmaps"] == inst.n  # even the sets of one element (r = 2: 6 bytes)
+
+
+def test_chains_end_whatever_max_loop():
+    """max_loop of a pool is not limited; an element that cannot be placed (20 copies, 12 slots) is
+    given up all the same and found by its list."""
+    import paper_1102_1003_gb300 as pkg
+    lists = [np.arange(0, 100, 10), np.arange(0, 120, 12), np.arange(60), np.arange(0, 127, 2)]
+    inst = datagen.from_lists([x.astype(np.uint32) for x in lists], 127)
+    off, tids, _ = device_inputs(inst, 0)
+    p = pkg.batmap_default_params(min_shift=0, load_num=1, load_den=3, max_loop=1 << 30)
+    pool = pkg.batmap_pool_create(127, off, tids, params=p)
+    qs = [[a, b] for a in range(4) for b in range(4)]
+    got = pkg.intersect_query(pool, qs).cpu().numpy().astype(np.uint64)
+    assert np.array_equal(got, oracle.kway_counts(inst.offsets, inst.tids, qs))

@@ -616,6 +616,7 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
         J.fails = bs.p;
         J.mask = d_mask.p;
         J.queue = d_queue.p;
+        J.refused = P.validate ? d_stat.p->err : nullptr;
         enqueue_place(3, J, place_perm, std::move(list), d_list.p, side);
         side.join();
         E.record(3, st);

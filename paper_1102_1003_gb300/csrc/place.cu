@@ -100,6 +100,16 @@ __device__ __forceinline__ void record(const PlaceJob &J, uint32_t item, uint32_
     }
 }
 
+// Has the check that runs beside the placement refused the input?  Equal tids (or a table
+// that is no permutation) send all copies to a few slots, where every chain takes all its
+// moves, one exchange after the other on one word: chains look every POLL moves.
+constexpr uint32_t POLL = 64;
+__device__ __forceinline__ bool refused(const PlaceJob &J) {
+    if (!J.refused) return false;
+    const volatile int *f = J.refused;
+    return (f[0] | f[1] | f[2] | f[3]) != 0;
+}
+
 // One CTA per item, items from a queue.  Dynamic shared memory: NT 2^rlog
 // entries (first the tids, then element indices, then the item's bytes); per
 // element and table its slot (16 bits: at most 5 * 8,192 slots) and code (8 bits, 0:
@@ -119,7 +129,11 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tpb = blockDim.x, warps = tpb / 32;
     uint4 *t4 = reinterpret_cast<uint4 *>(table);
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(J.queue, 1u), s_late = 0;
+        if (threadIdx.x == 0) {
+            const uint32_t next = atomicAdd(J.queue, 1u);
+            s_item = refused(J) ? J.count : next;
+            s_late = 0;
+        }
         __syncthreads();
         if (s_item >= J.count) break;
         const uint32_t item = J.items[s_item];
@@ -189,6 +203,12 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
         // sets of n = 1,000, m = 100,000: launches of 120 us each, passes 1833 -> 1553 and 2631 -> 2412 us
         // with the next rule for those in L2).
         const uint32_t soon = min(J.max_moves, FIRST_MOVES), rest = J.max_moves - soon;
+        auto finish = [&](uint32_t e, uint32_t t) {
+            for (uint32_t left = rest;;) {
+                const uint32_t moves = min(left, POLL);
+                if (walk(e, t, moves) || !(left -= moves) || refused(J)) return;
+            }
+        };
         for (uint32_t c = 0; c < NT - 1; c++)
             for (uint32_t k = threadIdx.x; k < size; k += tpb) {
                 if (!code[k * NT]) continue;
@@ -196,12 +216,11 @@ __global__ void __launch_bounds__(1024) k_place_small(const __grid_constant__ Pl
                 if (walk(e, t, soon) || !rest) continue;
                 const uint32_t at = atomicAdd(&s_late, 1u);
                 if (at < cap / 4) late[at] = e | t << 16;
-                else walk(e, t, rest);
+                else finish(e, t);
             }
         __syncthreads();
         for (uint32_t k = threadIdx.x; k < min(s_late, cap / 4); k += tpb) {
-            uint32_t e = late[k] & 0xFFFFu, t = late[k] >> 16;
-            walk(e, t, rest);
+            finish(late[k] & 0xFFFFu, late[k] >> 16);
         }
         __syncthreads();
         for (uint32_t e = threadIdx.x; e < (size + 31u) / 32u * 32u; e += tpb) {
@@ -290,13 +309,17 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
     const uint32_t rlog = I.rlog, rm = (1u << rlog) - 1u, tag = I.epoch << eshift;
     const uint64_t e0 = J.off[I.item], size = J.off[I.item + 1] - e0;
     const uint32_t *tids = J.tids + e0;
+    if (__any_sync(0xffffffffu, refused(J))) return;
     if (!T.bytes) {
         // First every copy's own exchange, all lanes in one table, four in flight; the displaced copies
         // go to a list, whose chains run on with full warps while it is long enough.
         const uint64_t b0 = (uint64_t)T.k * A_ELEMS + sub * A_SUB, b1 = min(size, b0 + A_SUB);
         uint32_t waiting = 0;  // entries of the list: tid, chain_word
+        uint32_t rounds = 0;
         auto chains = [&](uint32_t least) {
             while (waiting >= least) {
+                if (++rounds % POLL == 0 && __any_sync(0xffffffffu, refused(J))) waiting = 0;
+                if (waiting < least) break;
                 const uint32_t n = min(waiting, 32u);
                 waiting -= n;
                 const uint2 c = lane < n ? list[waiting + lane] : make_uint2(0, 0);

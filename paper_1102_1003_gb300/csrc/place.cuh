@@ -17,6 +17,8 @@ struct PlaceJob {
     uint64_t *fails;         // [chunks] zeroed; failed insertions per chunk
     uint32_t *mask;          // [chunks * CHUNK / 32] bit e: element e of the chunk failed
     uint32_t *queue;         // PLACE_QUEUES words
+    const int *refused;      // 4 flags that the check of the lists and permutations beside the placement may set
+                             // (BuildStat::err), or nullptr: the call is refused, and what is left to place is not placed
 };
 
 // Places all items of the list (ids, any order; d_list: room for as many ids on

@@ -193,6 +193,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
         J.fails = bs.p;
         J.mask = d_mask.p;
         J.queue = d_queue.p;
+        J.refused = P.validate ? d_stat.p->err : nullptr;
         enqueue_place(NT, J, place_perm, std::move(list), d_list.p, side);
     }
     side.join();

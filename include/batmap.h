@@ -526,6 +526,14 @@ batmap_status pair_support_dense(uint32_t m, uint32_t n, const uint64_t *d_offse
 void batmap_test_dense_timeout(uint32_t spin_limit);
 
 /*
+ * Test hook: from now on the library may hold at most `bytes` of device memory
+ * more than it holds at this call, as if the device had no more (a request
+ * beyond is one that cudaMalloc refuses, and what the library takes for free
+ * memory is what is left).  0 lifts the limit.
+ */
+void batmap_test_memory_limit(uint64_t bytes);
+
+/*
  * Frequent pairs from already counted supports, for callers that cannot
  * allocate device memory.  The paper has no counterpart: this is an
  * interface convenience.

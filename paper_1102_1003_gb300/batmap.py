@@ -31,7 +31,7 @@ EXPORTED = [
     "pair_support_dense", "batmap_pool_create", "batmap_pool_free", "batmap_pool_info", "intersect_query",
     "batmap_serve", "batmap_autotune", "batmap_release_scratch", "intersect_query_list", "batmap_build_cross",
     "batmap_build_d", "itemset_support", "frequent_triples", "batmap_test_dense_timeout",
-    "frequent_quadruples",
+    "frequent_quadruples", "batmap_test_memory_limit",
 ]
 
 
@@ -164,6 +164,8 @@ def load_library(path: str = LIB_PATH):
     L.frequent_quadruples.restype = ctypes.c_int
     L.batmap_test_dense_timeout.argtypes = [u32]
     L.batmap_test_dense_timeout.restype = None
+    L.batmap_test_memory_limit.argtypes = [u64]
+    L.batmap_test_memory_limit.restype = None
     _lib = L
     return L
 
@@ -459,6 +461,11 @@ def batmap_test_dense_timeout(spin_limit: int):
     """Make the next pair_support_dense call exercise its bounded-wait error path
     (producer issues nothing, waits give up after spin_limit polls); 0 cancels."""
     load_library().batmap_test_dense_timeout(int(spin_limit))
+
+
+def batmap_test_memory_limit(nbytes: int):
+    """Let the library hold at most nbytes of device memory more than now; 0 lifts the limit."""
+    load_library().batmap_test_memory_limit(int(nbytes))
 
 
 def batmap_autotune(sets, stream=None):

@@ -246,8 +246,7 @@ bool take_bits(BmBuf *buf, uint64_t bytes) {
         buf->alloc(bytes);
     } catch (const Error &e) {
         if (e.code != BATMAP_ERR_NOMEM) throw;
-        cudaGetLastError();  // not an error of this call: the BatMap routes need no bits
-        return false;
+        return false;  // not an error of this call: the BatMap routes need no bits
     }
     return true;
 }

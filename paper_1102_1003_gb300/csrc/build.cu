@@ -10,6 +10,7 @@
 //               (min, max) item pair per failed common transaction
 //   schedule  : compare work units (host, compare.cu)
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <mutex>
 #include <numeric>
@@ -241,6 +242,34 @@ std::vector<cudaEvent_t> g_events;  // at most MAX_EVENTS
 constexpr size_t MAX_EVENTS = 256;
 }  // namespace
 
+// ---- device memory ----
+
+namespace {
+std::atomic<uint64_t> g_device_bytes{0}, g_device_limit{UINT64_MAX};
+bool release_idle();
+}  // namespace
+
+void *device_alloc(size_t bytes) {
+    for (bool again = false;; again = true) {
+        void *p = nullptr;
+        const cudaError_t e = g_device_bytes + bytes > g_device_limit ? cudaErrorMemoryAllocation : cudaMalloc(&p, bytes);
+        if (e == cudaSuccess) {
+            g_device_bytes += bytes;
+            return p;
+        }
+        cudaGetLastError();  // reported here, not by the next launch's check
+        BM_REQUIRE(e == cudaErrorMemoryAllocation, BATMAP_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+        BM_REQUIRE(!again && release_idle(), BATMAP_ERR_NOMEM, "no device memory for " + std::to_string(bytes) + " bytes");
+    }
+}
+
+void device_free(void *p, size_t bytes) {
+    cudaFree(p);
+    g_device_bytes -= bytes;
+}
+
+void set_memory_limit(uint64_t bytes) { g_device_limit = bytes ? g_device_bytes + bytes : UINT64_MAX; }
+
 uint8_t *bm_buffer_take(size_t bytes, size_t *capacity) {
     {
         std::lock_guard<std::mutex> lock(g_bm_cache_mu);
@@ -259,10 +288,8 @@ uint8_t *bm_buffer_take(size_t bytes, size_t *capacity) {
             return b.p;
         }
     }
-    uint8_t *p = nullptr;
-    BM_CUDA(cudaMalloc(&p, bytes));
     *capacity = bytes;
-    return p;
+    return static_cast<uint8_t *>(device_alloc(bytes));
 }
 
 void bm_buffer_give(uint8_t *p, size_t capacity) {
@@ -272,7 +299,7 @@ void bm_buffer_give(uint8_t *p, size_t capacity) {
     const int k = capacity > LARGE_BUF;
     g_bm_cache[k].push_back({p, capacity});
     if (g_bm_cache[k].size() > BM_CACHE[k]) {
-        cudaFree(g_bm_cache[k].front().p);
+        device_free(g_bm_cache[k].front().p, g_bm_cache[k].front().cap);
         g_bm_cache[k].erase(g_bm_cache[k].begin());
     }
 }
@@ -280,7 +307,7 @@ void bm_buffer_give(uint8_t *p, size_t capacity) {
 void bm_buffer_release_all() {
     std::lock_guard<std::mutex> lock(g_bm_cache_mu);
     for (auto &cache : g_bm_cache) {
-        for (auto &b : cache) cudaFree(b.p);
+        for (auto &b : cache) device_free(b.p, b.cap);
         cache.clear();
     }
 }
@@ -327,12 +354,10 @@ struct Arena {
         return t;
     }
     void add(size_t cap) {
-        Block b{nullptr, cap, 0};
-        BM_CUDA(cudaMalloc(&b.p, cap));
-        blocks.push_back(b);
+        blocks.push_back({static_cast<uint8_t *>(device_alloc(cap)), cap, 0});
     }
     void clear() {
-        for (const Block &b : blocks) cudaFree(b.p);
+        for (const Block &b : blocks) device_free(b.p, b.cap);
         blocks.clear();
     }
     ~Arena() {
@@ -366,8 +391,7 @@ Workspace::~Workspace() {
             arena_->clear();
             if (total <= ARENA_BYTES) arena_->add(total);
         }
-    } catch (const Error &) {
-        cudaGetLastError();  // no memory to keep: the next call allocates what it needs
+    } catch (const Error &) {  // no memory to keep: the next call allocates what it needs
     }
     for (auto &b : arena_->blocks) b.used = 0;
     std::lock_guard<std::mutex> lock(g_arena_mu);
@@ -396,6 +420,16 @@ void release_arenas() {
     for (Arena *a : g_arenas) delete a;
     g_arenas.clear();
 }
+
+namespace {
+// Gives back the arrays and the scratch that no set and no call holds; false if there were none.
+bool release_idle() {
+    const uint64_t before = g_device_bytes;
+    bm_buffer_release_all();
+    release_arenas();
+    return g_device_bytes != before;
+}
+}  // namespace
 
 // ---- side stream ----
 

@@ -32,6 +32,7 @@ void enqueue_correct_compact(batmap_set *S, uint32_t *C, uint32_t s, uint32_t *d
 void run_batch(batmap_set *const *sets, const uint32_t *s, uint32_t k, batmap_out *outs, cudaStream_t st);
 void autotune(batmap_set *const *sets, uint32_t k, double *eff_out, cudaStream_t st);
 void release_scratch();
+void set_memory_limit(uint64_t bytes);
 void release_dense_workspace();
 void release_batch_plan();
 
@@ -355,6 +356,8 @@ void batmap_release_scratch(void) {
     release_dense_workspace();
     release_host_workspace();
 }
+
+void batmap_test_memory_limit(uint64_t bytes) { set_memory_limit(bytes); }
 
 static void require_pair_sets(batmap_set *const *sets, uint32_t k) {
     BM_REQUIRE(k == 0 || sets, BATMAP_ERR_ARG, "sets is NULL");

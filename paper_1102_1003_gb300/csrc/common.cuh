@@ -44,7 +44,13 @@ void count_launch();
         if (!(cond)) throw ::bm::Error{(code), (msg)};                                      \
     } while (0)
 
-// RAII device buffer (cudaMalloc / cudaFree).
+// Device memory of the library.  Where there is none left, what it keeps for later
+// calls (arrays of freed sets, idle call scratch) is given back and the request tried
+// once more; then BATMAP_ERR_NOMEM.  batmap_test_memory_limit makes less of it.
+void *device_alloc(size_t bytes);
+void device_free(void *p, size_t bytes);
+
+// RAII device buffer.
 template <typename T>
 struct DevBuf {
     T *p = nullptr;
@@ -61,12 +67,12 @@ struct DevBuf {
     ~DevBuf() { release(); }
     void alloc(size_t count) {
         release();
-        if (count) BM_CUDA(cudaMalloc(&p, count * sizeof(T)));
+        if (count) p = static_cast<T *>(device_alloc(count * sizeof(T)));
         n = count;
     }
     void ensure(size_t count) { if (count > n) alloc(count); }
     void release() {
-        if (p) cudaFree(p);
+        if (p) device_free(p, n * sizeof(T));
         p = nullptr;
         n = 0;
     }

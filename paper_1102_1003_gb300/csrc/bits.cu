@@ -237,11 +237,7 @@ void enqueue_bits(const uint64_t *d_off, const uint32_t *d_tids, uint32_t n, uin
 }
 
 bool take_bits(BmBuf *buf, uint64_t bytes) {
-    if (bytes > (64ull << 20)) {
-        size_t free_b = 0, total_b = 0;
-        BM_CUDA(cudaMemGetInfo(&free_b, &total_b));
-        if (bytes > free_b / 2) return false;
-    }
+    if (bytes > (64ull << 20) && bytes > device_available() / 2) return false;
     try {
         buf->alloc(bytes);
     } catch (const Error &e) {

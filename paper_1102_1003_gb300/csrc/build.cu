@@ -431,6 +431,21 @@ bool release_idle() {
 }
 }  // namespace
 
+uint64_t device_available() {
+    size_t free_b = 0, total_b = 0;
+    BM_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    const uint64_t limit = g_device_limit, held = g_device_bytes;
+    uint64_t b = std::min<uint64_t>(free_b, limit > held ? limit - held : 0) + g_scratch.bytes();
+    {
+        std::lock_guard<std::mutex> lock(g_bm_cache_mu);
+        for (auto &cache : g_bm_cache)
+            for (auto &c : cache) b += c.cap;
+    }
+    std::lock_guard<std::mutex> lock(g_arena_mu);
+    for (const Arena *a : g_arenas) b += a->total();
+    return b;
+}
+
 // ---- side stream ----
 
 namespace {

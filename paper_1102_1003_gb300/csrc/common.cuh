@@ -49,6 +49,9 @@ void count_launch();
 // once more; then BATMAP_ERR_NOMEM.  batmap_test_memory_limit makes less of it.
 void *device_alloc(size_t bytes);
 void device_free(void *p, size_t bytes);
+// Free memory and what the library keeps idle, so that a call finds the same before
+// and after others that were freed.  Within a build only (the placement scratch is the build's).
+uint64_t device_available();
 
 // RAII device buffer.
 template <typename T>

@@ -89,3 +89,28 @@ def test_no_memory_is_reported_once(limit):
     _mine(_inst(30_000, 40, 1_500, 4))
     pkg.batmap_test_memory_limit(0)
     _mine(a)
+
+
+@pytest.mark.parametrize("d", [2, 3])
+def test_equal_builds_take_equal_routes(limit, d):
+    """Rows of 80 MB: less than half of what is free at first, more than half of what is left while
+    the library keeps a freed set's arrays.  They are taken on every pass, or on none."""
+    import torch
+    import paper_1102_1003_gb300 as pkg
+    m, n = 1 << 22, 160
+    inst = _inst(m, n, 200_000, 5)
+    off, tids, _ = device_inputs(inst, 0)
+    pairs = torch.tensor([[0, 1, 1], [0, 2, 1], [1, 2, 1]], dtype=torch.int32, device="cuda")
+    want = int(oracle.kway_counts(inst.offsets, inst.tids, [[0, 1, 2]])[0])
+    for room, rows in ((300 * MB, True), (150 * MB, False)):  # beside the BatMaps
+        limit(n * (d + 1) * (1 << 19) + room)
+        for _ in range(3):
+            if d == 2:
+                t = _mine(inst)
+            else:
+                b = pkg.batmap_build_d(d, m, off, tids)
+                n_out, triples, n_cand = pkg.frequent_triples(b, 1, pairs)
+                assert n_cand == 1 and triples.tolist() == [[0, 1, 2, want]]
+                t = pkg.batmap_get_timing(b)
+                b.free()
+            assert (t["scan_ms"] == 0) == rows

@@ -307,7 +307,8 @@ batmap_status batmap_export_layout(const batmap_set *set, uint8_t *h_bytes,
  *   - the contraction of the family's bit rows (Sec. I-B), which the build then
  *     keeps beside the BatMaps (n * ceil(m / 256) * 32 bytes), on the tensor
  *     cores.  Taken only with tile, shape_mask and probe_log left at 0, and
- *     only if the bit rows fit in half of the free memory;
+ *     only if the bit rows fit in half of the memory that is free (the library's
+ *     idle memory included) beside the supports;
  *   - the BatMaps: pairs of similar width run the cyclic scan, pairs whose
  *     widths differ by 2^probe_log or more the probe route
  *     (batmap_params.probe_log); both count the same slot pairs.

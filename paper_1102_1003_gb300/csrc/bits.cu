@@ -236,8 +236,11 @@ void enqueue_bits(const uint64_t *d_off, const uint32_t *d_tids, uint32_t n, uin
     }
 }
 
-bool take_bits(BmBuf *buf, uint64_t bytes) {
-    if (bytes > (64ull << 20) && bytes > device_available() / 2) return false;
+bool take_bits(BmBuf *buf, uint64_t bytes, uint64_t supports) {
+    if (bytes > (64ull << 20)) {
+        const uint64_t available = device_available();
+        if (available < supports || bytes > (available - supports) / 2) return false;
+    }
     try {
         buf->alloc(bytes);
     } catch (const Error &e) {

@@ -30,9 +30,10 @@ void enqueue_bits(const uint64_t *d_off, const uint32_t *d_tids, uint32_t n, uin
                   uint8_t *d_bits, int *d_flags, bool sorted_only, cudaStream_t st);
 
 // Allocates `bytes` of bit rows unless they would take more than half of the
-// memory that no caller and no set holds; false (and no rows) if so, or if the
-// allocation fails.  Called within a build.
-bool take_bits(BmBuf *buf, uint64_t bytes);
+// memory that no caller and no set holds, less the `supports` bytes that the set's
+// calls may ask for; false (and no rows) if so, or if the allocation fails.
+// Called within a build.
+bool take_bits(BmBuf *buf, uint64_t bytes, uint64_t supports);
 
 // |S_a1 cap .. cap S_ak| of nq queries of k ids each (1 <= k <= 4) over
 // row-major bit rows: AND and popcount.

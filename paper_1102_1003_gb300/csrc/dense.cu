@@ -481,7 +481,7 @@ void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids,
     const uint64_t bytes = L.kb_stride * L.kblocks;
     const double bits_s = ((double)bytes + 4.0 * (double)S->n_elements) / BITS_BYTES_PER_S;
     if (bits_s + contract_seconds(S->n, S->n_a, L.kblocks) > SCAN_MIN_S + S->word_pairs / SCAN_WORD_PAIRS_PER_S) return;
-    if (!take_bits(&S->d_bits, bytes)) return;
+    if (!take_bits(&S->d_bits, bytes, S->npairs() * sizeof(uint32_t))) return;
     std::vector<MmUnit> units;
     S->mm_add = contract_units(S->n, S->n_a, L.kblocks, 0, 0.0, &units);
     S->mm_count = (uint32_t)units.size();

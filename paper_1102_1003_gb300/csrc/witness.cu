@@ -162,7 +162,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     SideStream side(st);
     const BitsLayout BL = bits_row_major(m);
     S->kblocks = BL.kblocks;
-    const bool with_bits = T && !P.tile && !P.shape_mask && !P.probe_log && take_bits(&S->d_bits, BL.row_stride * n);
+    const bool with_bits = T && !P.tile && !P.shape_mask && !P.probe_log && take_bits(&S->d_bits, BL.row_stride * n, 0);
     if (with_bits) enqueue_bits(d_offsets, d_tids, n, m, BL, S->d_bits.p, d_stat.p->err + 2, P.validate != 0, side.side());
     if (P.validate && nch && !with_bits) {  // (the bit rows' build checks every list)
         make_chunks();

@@ -114,3 +114,20 @@ def test_equal_builds_take_equal_routes(limit, d):
                 t = pkg.batmap_get_timing(b)
                 b.free()
             assert (t["scan_ms"] == 0) == rows
+
+
+@pytest.mark.parametrize("room,rows", [(180, False), (400, True)])
+def test_rows_leave_room_for_the_supports(limit, room, rows):
+    """67 MB of rows beside 122 MB of supports, for which the BatMap route has room in 180."""
+    import torch
+    import paper_1102_1003_gb300 as pkg
+    m, n = 70_001, 8_000
+    inst = datagen.bernoulli_tidlists(m, n, 0.003, seed=7)
+    off, tids, _ = device_inputs(inst, 0)
+    limit(n * 3 * 1024 + room * MB)
+    b = pkg.batmap_build(m, off, tids)
+    n_out, pairs = pkg.pair_support_all(b, 3, pairs=torch.empty((n * n // 2, 3), dtype=torch.int32, device="cuda"))
+    assert (pkg.batmap_get_timing(b)["scan_ms"] == 0) == rows
+    b.free()
+    ref = oracle.threshold_from_full(oracle.pairs_full(inst.offsets, inst.tids, threads=THREADS), n, 3)
+    assert n_out == ref.shape[0] and np.array_equal(pairs.cpu().numpy().astype(np.uint32), ref)

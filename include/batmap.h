@@ -384,7 +384,7 @@ batmap_status batmap_get_timing(const batmap_set *set, batmap_timing *t);
 /* Release the scratch the library caches between calls (the placement table
  * of batmap_build, up to 96 MiB or two of its widest item's, four bytes per
  * slot; at most four arrays of freed sets of more than 64 MiB and 32 smaller
- * ones; at most four arenas of call scratch of 256 MiB each; the dense path's
+ * ones, a quarter of the device's memory in all; at most four arenas of call scratch of 256 MiB each; the dense path's
  * bitmap and workspace; pair_support_host's device copies of its inputs and output).
  * Call when no other call of the library is running. */
 void batmap_release_scratch(void);

@@ -84,8 +84,8 @@ struct DevBuf {
 
 // The arrays of built sets come from a cache: a freed set's arrays (after a
 // device synchronisation, as cudaFree would do) are kept for the next build, at
-// most four of more than 64 MiB and 32 smaller ones, reused when no larger than
-// twice the request plus 1 MiB.  A small build makes about thirty allocations,
+// most four of more than 64 MiB and 32 smaller ones, and a quarter of the device's
+// memory in all, reused when no larger than twice the request plus 1 MiB.  A small build makes about thirty allocations,
 // which cost more than its kernels.
 uint8_t *bm_buffer_take(size_t bytes, size_t *capacity);
 void bm_buffer_give(uint8_t *p, size_t capacity);

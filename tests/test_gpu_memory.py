@@ -131,3 +131,24 @@ def test_rows_leave_room_for_the_supports(limit, room, rows):
     b.free()
     ref = oracle.threshold_from_full(oracle.pairs_full(inst.offsets, inst.tids, threads=THREADS), n, 3)
     assert n_out == ref.shape[0] and np.array_equal(pairs.cpu().numpy().astype(np.uint32), ref)
+
+
+def test_kept_arrays_are_bounded_in_bytes(limit):
+    """Freed sets of several sizes: what the library keeps of them stays below a quarter of the
+    memory (here of the limit), and an array above that is not kept."""
+    import torch
+    import paper_1102_1003_gb300 as pkg
+    insts = [_inst(1 << 20, n, 1 << 17, n) for n in (14, 20, 30, 45, 68)]  # BatMaps of 84 to 408 MB
+    for inst in insts:  # (the first calls of the process take memory of their own)
+        _mine(inst, load_num=16, probe_log=32)
+    limit(1_000 * MB)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    for inst in insts:
+        _mine(inst, load_num=16, probe_log=32)
+    torch.cuda.empty_cache()
+    kept = before - torch.cuda.mem_get_info()[0]
+    # a quarter, the placement scratch (at most 96 MiB of regions here, and its tasks) and small arenas
+    assert kept < (250 + 110 + 40) * MB
+    assert kept > 80 * MB  # and the smaller ones are still kept

@@ -287,7 +287,19 @@ def dense_leg(args, inst, off, tids, n_out_ref, peaks, peak_kind, steps=None, wa
             "phases_ms": {"bitmap": statistics.mean(build), "tensor_kernel": statistics.mean(gemm)},
             "roofline": contract_roofline(inst.m, inst.n, 0, g, peaks, peak_kind,
                                           _traffic(workload or args.workload, "k_contract", "dense.cu")),
-            "dtype": "e2m1 {0,1} operands, fp32 accumulate (exact integers <= 2^24)"}
+            "dtype": CONTRACT_DTYPE}
+
+
+def batmap_leg(inst, dev, peaks, peak_kind, workload, rec):
+    """The same workload by the BatMap routes, where the timed steps (rec) took the bit rows: the
+    BatMap side of the comparison with the dense-bitmap path."""
+    if rec["dtype"] != CONTRACT_DTYPE:
+        return None
+    leg, off, tids, n_out = plain_leg(inst, dev, 3, 3, peaks, peak_kind, workload, probe_log=BATMAP_PROBE_LOG)
+    assert n_out == rec["frequent_pairs"], (n_out, rec["frequent_pairs"])
+    keys = ("value", "unit", "steps", "warmup", "ms_per_step", "dtype", "roofline", "logical_hbm", "phases_ms",
+            "compare_equiv", "probe")
+    return dict({k: leg[k] for k in keys if k in leg}, probe_log=BATMAP_PROBE_LOG)
 
 
 def _desc(workload: str) -> str:
@@ -302,16 +314,33 @@ def _alu_peak(dev, peaks):
 
 
 PROBE_LOG = 0  # batmap_params.probe_log of the timed builds (0 = the library's default)
+BATMAP_PROBE_LOG = 2  # asks for the BatMap routes, with the threshold they have by default
+CONTRACT_DTYPE = "e2m1 {0,1} operands, fp32 accumulate (exact integers <= 2^24)"
 
 
-def _build_params():
+def _build_params(probe_log=None):
     """Build parameters of the timed BatMap builds: the defaults, with
-    probe_log from --probe-log."""
+    probe_log from --probe-log unless one is given."""
     import paper_1102_1003_gb300 as pkg
-    return pkg.batmap_default_params(probe_log=PROBE_LOG)
+    return pkg.batmap_default_params(probe_log=PROBE_LOG if probe_log is None else probe_log)
 
 
-def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None, dist=None):
+def route_keys(contract, m, n, npairs, word_pairs, cmp_s, peaks):
+    """Compute type and bandwidth of the compare that ran: BatMap bytes of all pairs for the BatMap
+    routes (Sec. IV-A); the rows once and the supports once for the contraction of bit rows, which
+    reads no BatMap."""
+    if contract:
+        gbs = ((m + 255) // 256 * 32 * n + 4.0 * npairs) / cmp_s / 1e9
+        return {"dtype": CONTRACT_DTYPE,
+                "hbm": {"achieved_GBps": gbs, "peak_GBps": peaks["hbm_gbs"], "frac": gbs / peaks["hbm_gbs"],
+                        "definition": "bit rows once + supports once / compare time"}}
+    gbs = 8.0 * word_pairs / cmp_s / 1e9
+    return {"dtype": "u8",
+            "logical_hbm": {"achieved_GBps": gbs, "peak_GBps": peaks["hbm_gbs"], "frac": gbs / peaks["hbm_gbs"],
+                            "definition": "sum over pairs of 2*max(|B_i|,|B_j|) bytes / compare time (Sec. IV-A)"}}
+
+
+def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None, dist=None, probe_log=None):
     """Time `steps` plain steps (batmap_build + pair_support_all) on resident tidlists."""
     import torch
     import paper_1102_1003_gb300 as pkg
@@ -320,7 +349,7 @@ def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None
     off = torch.from_numpy(inst.offsets.astype(np.int64)).to(dev)
     tids = torch.from_numpy(inst.tids.view(np.int32)).to(dev)
     npairs = inst.n * (inst.n - 1) // 2
-    bset = pkg.batmap_build(inst.m, off, tids, None, params=_build_params())
+    bset = pkg.batmap_build(inst.m, off, tids, None, params=_build_params(probe_log))
     n_out, _ = pkg.pair_support_all(bset, inst.s)
     info = bset.info
     bset.free()
@@ -329,7 +358,7 @@ def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None
     compare_ms, build_ms, compact_ms, scan_ms, probe_ms = [], [], [], [], []
 
     def step(record):
-        bs = pkg.batmap_build(inst.m, off, tids, None, params=_build_params())
+        bs = pkg.batmap_build(inst.m, off, tids, None, params=_build_params(probe_log))
         k, _ = pkg.pair_support_all(bs, inst.s, pairs=pairs_buf)
         if record:
             L.batmap_get_timing(bs.handle, ctypes.byref(timing))
@@ -373,7 +402,6 @@ def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None
     roofline = (contract_roofline(inst.m, inst.n, 0, cmp_s, peaks, peak_kind,
                                   _traffic(workload, "k_contract", "dense.cu")) if contract else
                 scan_roofline(wp_scan, scan_s, alu_peak, sms, peaks, peak_kind, _traffic(workload)))
-    logical_gbs = 8.0 * wp / cmp_s / 1e9
     rec = {
         "value": npairs * steps / elapsed, "unit": UNIT, "steps": steps, "warmup": warmup,
         "ms_per_step": 1e3 * elapsed / steps, "elapsed_s": elapsed,
@@ -381,9 +409,7 @@ def plain_leg(inst, dev, steps, warmup, peaks, peak_kind, workload, sampler=None
                    "s": inst.s, "pairs": npairs, "tids": int(inst.tids.size), "batmap_bytes": info["bytes"],
                    "width_classes": info["n_classes"], "l2": "inputs larger than L2 (no flush)"},
         "roofline": roofline,
-        "logical_hbm": {"achieved_GBps": logical_gbs, "peak_GBps": peaks["hbm_gbs"],
-                        "frac": logical_gbs / peaks["hbm_gbs"],
-                        "definition": "sum over pairs of 2*max(|B_i|,|B_j|) bytes / compare time (Sec. IV-A)"},
+        **route_keys(contract, inst.m, inst.n, npairs, wp, cmp_s, peaks),
         "set_elements_per_s": (inst.n - 1) * int(inst.tids.size) / cmp_s,
         "phases_ms": {"build": statistics.mean(build_ms), "compare": statistics.mean(compare_ms),
                       "compare_scan": statistics.mean(scan_ms), "compare_probe": statistics.mean(probe_ms),
@@ -451,9 +477,9 @@ def run_mine(args, inst, rank, world):
     line = {
         "metric": METRIC, "value": world * rec["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": rec["ms_per_step"], "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "u8", "data": "synthetic",
+        "scaling": "weak", "vs_baseline": None, "dtype": rec["dtype"], "data": "synthetic",
         "config": dict(rec["config"], parallelism="replicas" if world > 1 else "single GPU"),
-        "roofline": rec["roofline"], "logical_hbm": rec["logical_hbm"],
+        "roofline": rec["roofline"], **{k: rec[k] for k in ("hbm", "logical_hbm") if k in rec},
         "set_elements_per_s": rec["set_elements_per_s"],
         "set_elements_definition": "sum over pairs of |S_i| + |S_j| = (n-1) * tids, per compare time (Sec. IV-B)",
         "phases_ms": rec["phases_ms"], "frequent_pairs": n_out, "failed_insertions": rec["failed_insertions"],
@@ -468,6 +494,7 @@ def run_mine(args, inst, rank, world):
         line["compare_equiv"] = rec["compare_equiv"]
     if not args.no_dense and inst.m <= (1 << 24):
         line["dense"] = dense_leg(args, inst, off, tids, n_out, peaks, peak_kind, workload=label)
+        line["batmap"] = batmap_leg(inst, dev, peaks, peak_kind, label, rec)
     del off, tids
     pkg.batmap_release_scratch()
     torch.cuda.empty_cache()
@@ -484,11 +511,14 @@ def run_mine(args, inst, rank, world):
             zr, zoff, ztids, zn = plain_leg(z, dev, 5, 3, peaks, peak_kind, "zipf_m1m_n2000")
             zr["dense"] = dense_leg(args, z, zoff, ztids, zn, peaks, peak_kind, steps=5, warmup=3,
                                     workload="zipf_m1m_n2000")
+            zr["batmap"] = batmap_leg(z, dev, peaks, peak_kind, "zipf_m1m_n2000", zr)
             del zoff, ztids
             sub["zipf_m1m_n2000"] = zr
         pkg.batmap_release_scratch()
         torch.cuda.empty_cache()
-        sub["batched"] = batch_record(args, steps=3, warmup=2)
+        insts = batch_insts()
+        sub["batched"] = batch_record(args, 3, 3, insts)
+        sub["batched_batmap"] = batch_record(args, 3, 3, insts, probe_log=BATMAP_PROBE_LOG)
         line["sub"] = sub
         line["extra_keys"] = sorted(k for k in line if k not in (
             "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
@@ -499,37 +529,37 @@ def run_mine(args, inst, rank, world):
         dist.destroy_process_group()
 
 
-def batch_record(args, steps, warmup, small=False, instances=64, autotune=True):
-    """Batched form: `instances` independent instances (m log-uniform in [1e4, 1e6],
-    n uniform in [100, 4000], density uniform in [1%, 10%], Zipf items); one batched,
-    graph-captured persistent pass vs the same instances as plain pair_support_all
-    calls, each timed with events; outputs compared, a sample against the oracle."""
+def batch_insts(small=False, instances=64):
+    """Independent instances: m log-uniform in [1e4, 1e6], n uniform in [100, 4000], density uniform
+    in [1%, 10%], Zipf items; or many small ones, where per-call launches and waits dominate."""
+    specs = (datagen.batch_specs(instances, 5000, m_range=(1e3, 1e5), n_range=(50, 400)) if small
+             else datagen.batch_specs(instances, 1000))
+    return datagen.batch_instances(specs, workers=os.cpu_count() or 8)
+
+
+def batch_record(args, steps, warmup, insts, small=False, autotune=True, probe_log=None):
+    """Batched form: one batched, graph-captured persistent pass over all instances vs the same
+    instances as plain pair_support_all calls, each timed with events; outputs compared, a sample
+    against the oracle.  The tile schedules are tuned if some instance takes a BatMap route."""
     import torch
     import paper_1102_1003_gb300 as pkg
     import oracle
     dev = torch.device("cuda", torch.cuda.current_device())
-    if small:
-        # many small instances, where per-call launches and synchronisations dominate
-        specs = datagen.batch_specs(instances, 5000, m_range=(1e3, 1e5), n_range=(50, 400))
-    else:
-        specs = datagen.batch_specs(instances, 1000)
-    t0 = time.perf_counter()
-    insts = datagen.batch_instances(specs, workers=os.cpu_count() or 8)
-    gen_s = time.perf_counter() - t0
     sets, npairs, wp = [], 0, 0.0
     t0 = time.perf_counter()
     for inst in insts:
         off = torch.from_numpy(inst.offsets.view(np.int64)).to(dev)
         tids = torch.from_numpy(inst.tids.view(np.int32)).to(dev)
-        sets.append(pkg.batmap_build(inst.m, off, tids, None, params=_build_params()))
+        sets.append(pkg.batmap_build(inst.m, off, tids, None, params=_build_params(probe_log)))
         npairs += inst.n * (inst.n - 1) // 2
         del off, tids
     torch.cuda.synchronize()
     build_s = time.perf_counter() - t0
-    eff = pkg.batmap_autotune(sets) if autotune else None
     wp = sum(b.info["word_pairs"] for b in sets)
     # output sizes from one plain pass
     n_out = [pkg.pair_support_all(b, i.s)[0] for b, i in zip(sets, insts)]
+    scan = any(pkg.batmap_get_timing(b)["scan_ms"] > 0 for b in sets)  # else bit rows answer for all of them
+    eff = pkg.batmap_autotune(sets) if autotune and scan else None
     bufs = [torch.empty((max(k, 1), 3), dtype=torch.int32, device=dev) for k in n_out]
     s_list = [i.s for i in insts]
     cmp_plain, cmp_batch = [], []
@@ -566,11 +596,9 @@ def batch_record(args, steps, warmup, small=False, instances=64, autotune=True):
     for name, c in (("plain", cmp_plain), ("batched", cmp_batch)):
         t = statistics.mean(c) / 1e3
         results[name]["compare_ms"] = 1e3 * t
-        results[name]["compare_equiv_lane_op_frac"] = OPS_PER_WORD_PAIR * wp / t / 1e12 / alu_peak
-    results["compare_equiv_definition"] = (
-        "4 x sum over all pairs of max(|B_i|,|B_j|)/4 word pairs (the scan's work for every pair, "
-        "probe-routed pairs included) / compare time / lane-op peak; far above 1 where bit rows answer")
-    results["probe_routed_share"] = sum(b.info["probe_word_pairs"] for b in sets) / wp
+        if scan:
+            results[name]["compare_equiv_lane_op_frac"] = OPS_PER_WORD_PAIR * wp / t / 1e12 / alu_peak
+    results["probe_routed_share"] = sum(b.info["probe_word_pairs"] for b in sets) / wp if scan else 0.0
     # batched and plain give identical outputs; a sampled oracle check per instance
     batch_pairs = [b[:k].cpu().numpy().copy() for b, k in zip(bufs, n_out)]
     plain(False)
@@ -593,7 +621,9 @@ def batch_record(args, steps, warmup, small=False, instances=64, autotune=True):
     return {"workload": "batch", "unit": UNIT, "value": results["batched"]["value"],
             "ms_per_step": results["batched"]["ms_per_step"], "steps": steps, "warmup": warmup,
             "batched": results["batched"], "plain": results["plain"],
-            "compare_equiv_definition": results["compare_equiv_definition"],
+            "route": "BatMap scan and probe" if scan else "contraction of bit rows",
+            "compare_equiv_definition": "4 x sum over all pairs of max(|B_i|,|B_j|)/4 word pairs (the scan's work for "
+                                        "every pair, probe-routed pairs included) / compare time / lane-op peak",
             "probe_routed_share": results["probe_routed_share"],
             "speedup_batched_over_plain": results["batched"]["value"] / results["plain"]["value"],
             "config": {"instances": len(insts), "small": bool(small), "pairs": npairs,
@@ -601,7 +631,7 @@ def batch_record(args, steps, warmup, small=False, instances=64, autotune=True):
                        "m_range": [min(i.m for i in insts), max(i.m for i in insts)],
                        "n_range": [min(i.n for i in insts), max(i.n for i in insts)],
                        "autotuned": eff is not None},
-            "shape_eff": eff, "gen_s": gen_s, "build_s": build_s,
+            "shape_eff": eff, "build_s": build_s,
             "batched_equals_plain": same, "oracle_sample_exact": exact}
 
 
@@ -609,8 +639,8 @@ def run_batch(args):
     """Batched workload: one JSON line (see batch_record)."""
     import torch
     torch.cuda.set_device(0)
-    rec = batch_record(args, args.steps, args.warmup, small=args.batch_small, instances=args.instances,
-                       autotune=not args.no_autotune)
+    rec = batch_record(args, args.steps, args.warmup, batch_insts(args.batch_small, args.instances),
+                       small=args.batch_small, autotune=not args.no_autotune)
     print(json.dumps(dict({"metric": METRIC}, **rec)), flush=True)
 
 
@@ -622,6 +652,7 @@ def run_nsweep(args):
     import oracle
     torch.cuda.set_device(0)
     dev = torch.device("cuda", 0)
+    peaks, _ = _peaks()
     rows = []
     for n in args.nsweep:
         inst = datagen.nsweep_instance(n)
@@ -652,7 +683,8 @@ def run_nsweep(args):
                      "build_ms": statistics.mean(t["build_ms"] for _, t in times),
                      "compare_ms": statistics.mean(t["compare_ms"] for _, t in times),
                      "pair_supports_per_s": npairs / wall,
-                     "logical_GBps": 8.0 * info["word_pairs"] / (statistics.mean(t["compare_ms"] for _, t in times) / 1e3) / 1e9,
+                     **route_keys(times[-1][1]["scan_ms"] == 0, inst.m, n, npairs, info["word_pairs"],
+                                  statistics.mean(t["compare_ms"] for _, t in times) / 1e3, peaks),
                      "sampled_exact": bool(np.array_equal(got, ref))})
         del full, off, tids, perm
         pkg.batmap_release_scratch()
@@ -728,7 +760,8 @@ def run_cross(args):
     line = {"metric": "A x B pair supports/sec (sparse boolean matrix multiplication), bit-exact",
             "workload": "cross", "unit": UNIT, "value": npairs * args.steps / elapsed, "n_gpus": 1,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * elapsed / args.steps,
-            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u8", "data": "synthetic",
+            "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+            "dtype": "u8" if scan_s else CONTRACT_DTYPE, "data": "synthetic",
             "config": {"workload": "cross", "m": union.m, "n_a": na, "n_b": nb, "s": 1, "pairs": npairs,
                        "desc": "A: Zipf(1) sizes at mean density 1%; B: Bernoulli p=0.002",
                        "tids": int(union.tids.size), "batmap_bytes": int(info["bytes"]),
@@ -833,7 +866,7 @@ def run_triples(args):
     line = {"metric": "candidate itemset supports/sec (Apriori level 3 over 3-of-4 BatMaps), bit-exact",
             "workload": "triples", "unit": "candidate-supports/s", "value": n_cand * args.steps / elapsed,
             "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * elapsed / args.steps,
-            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u8", "data": "synthetic",
+            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bit rows (AND + popcount, u32)", "data": "synthetic",
             "config": {"workload": "triples", "m": inst.m, "n": inst.n, "s": s, "tids": int(inst.tids.size),
                        "desc": "Zipf(1) items at mean density 2%", "frequent_pairs": n_pairs,
                        "candidates": n_cand, "frequent_triples": n_trip, "batmap3_bytes": int(info3["bytes"])},
@@ -941,7 +974,7 @@ def run_quads(args):
     line = {"metric": "candidate itemset supports/sec (Apriori levels 3 and 4 over 4-of-5 BatMaps), bit-exact",
             "workload": "quads", "unit": "candidate-supports/s", "value": (n_c3 + n_c4) * args.steps / elapsed,
             "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * elapsed / args.steps,
-            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u8", "data": "synthetic",
+            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bit rows (AND + popcount, u32)", "data": "synthetic",
             "config": {"workload": "quads", "m": inst.m, "n": inst.n, "s": s, "tids": int(inst.tids.size),
                        "desc": "Zipf(1) items at mean density 2%", "frequent_pairs": n_pairs,
                        "triple_candidates": n_c3, "frequent_triples": n_trip,

@@ -566,10 +566,10 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     S->rank.assign(n, 0);
     S->byte_off.assign(n, 0);
     S->wshift_sorted.assign(n, 0);
-    // per-item arrays for the device: base (64 bits) | line_off | wshift | order | rlog | chunk0
-    std::vector<uint32_t> meta(7ull * n);
+    // per-item arrays for the device: base (64 bits) | line_off | wshift | order | chunk0
+    std::vector<uint32_t> meta(6ull * n);
     uint64_t *base = reinterpret_cast<uint64_t *>(meta.data());
-    uint32_t *line_off = meta.data() + 2ull * n, *chunk0 = meta.data() + 6ull * n;
+    uint32_t *line_off = meta.data() + 2ull * n, *chunk0 = meta.data() + 5ull * n;
     uint64_t pos = 0;
     S->class_begin.clear();
     for (uint32_t q = 0; q < n; q++) {
@@ -615,7 +615,6 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     if (n) {
         std::copy(S->wshift_sorted.begin(), S->wshift_sorted.end(), meta.begin() + 3ull * n);
         std::copy(S->order.begin(), S->order.end(), meta.begin() + 4ull * n);
-        std::copy(rlog.begin(), rlog.end(), meta.begin() + 5ull * n);
         S->d_meta.alloc(meta.size());
         S->d_line_off.p = S->d_meta.p + 2ull * n;
         S->d_wshift.p = S->d_meta.p + 3ull * n;
@@ -636,10 +635,10 @@ void build_set(batmap_set *S, const uint64_t *d_offsets, const uint32_t *d_tids,
     }
 
     const uint64_t *d_base = reinterpret_cast<const uint64_t *>(S->d_meta.p);
-    const uint32_t *d_chunk0 = S->d_meta.p + 6ull * n;
+    const uint32_t *d_chunk0 = S->d_meta.p + 5ull * n;
     WsBuf<uint32_t> d_ch_item(ws, nch);
     WsBuf<uint64_t> d_ch_start(ws, nch);
-    ItemView v{d_offsets, d_tids, d_base, S->d_meta.p + 5ull * n, d_ch_item.p, d_ch_start.p};
+    ItemView v{d_offsets, d_tids, d_ch_item.p, d_ch_start.p};
     auto make_chunks = [&] {
         k_chunks<<<n, 64, 0, st>>>(d_offsets, d_chunk0, d_ch_item.p, d_ch_start.p);
         BM_CHECK_LAUNCH();

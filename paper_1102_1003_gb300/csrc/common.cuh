@@ -182,12 +182,6 @@ __host__ __device__ __forceinline__ uint64_t slot_of(uint32_t t, uint32_t pi, ui
     return 3ull * r0 * (uint64_t)(h >> shift) + (h & (r0 - 1u)) + (uint64_t)t * r0;
 }
 
-// 8-bit element: indicator in bit 7, code (pi >> shift) + 1 in bits 0..6.
-__host__ __device__ __forceinline__ uint32_t element_byte(uint32_t pi, uint32_t shift,
-                                                         uint32_t ind) {
-    return (ind << 7) | ((pi >> shift) + 1u);
-}
-
 // ---- compare work units ----------------------------------------------------
 
 // One unit of the all-pairs compare: rows [r0, r1) x columns [c0, c1) of the

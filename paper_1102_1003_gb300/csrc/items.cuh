@@ -19,8 +19,6 @@ constexpr int CHUNK = TPB * PER_THREAD;  // elements handled by one block
 struct ItemView {
     const uint64_t *off;     // CSR offsets [n+1]
     const uint32_t *tids;    // CSR tids
-    const uint64_t *base;    // [n] first slot (byte) of item i in the BatMap array
-    const uint32_t *rlog;    // [n] log2 r_i
     const uint32_t *ch_item; // [chunks] item of chunk b
     const uint64_t *ch_start;// [chunks] first element of chunk b
 };

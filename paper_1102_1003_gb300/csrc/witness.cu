@@ -147,7 +147,7 @@ void build_witness_impl(batmap_set *S, const uint64_t *d_offsets, const uint32_t
     BM_CUDA(cudaMemsetAsync(bs.p, 0, (nch + 1) * 8ull, st));
     BM_CUDA(cudaMemsetAsync(S->d_fail_off.p, 0, (n + 1) * sizeof(uint64_t), st));
     if (n) BM_CUDA(cudaMemcpyAsync(d_chunk0.p, chunk0.data(), n * 4ull, cudaMemcpyHostToDevice, st));
-    ItemView v{d_offsets, d_tids, S->d_base.p, S->d_rlog.p, d_ch_item.p, d_ch_start.p};
+    ItemView v{d_offsets, d_tids, d_ch_item.p, d_ch_start.p};
     auto make_chunks = [&] {
         k_chunks<<<n, 64, 0, st>>>(d_offsets, d_chunk0.p, d_ch_item.p, d_ch_start.p);
         BM_CHECK_LAUNCH();
@@ -1136,7 +1136,7 @@ void frequent_triples(batmap_set *S, uint32_t s, const uint32_t *d_pairs, uint64
             k_unit_counts<<<grid_for(np), 256, 0, st>>>(cnt, np, uoff.p);
             BM_CHECK_LAUNCH();
             WsBuf<uint64_t> utot_state(ws, scan_states(np));
-        scan_with_tail(uoff.p, np, utot.p, utot_state.p, st);
+            scan_with_tail(uoff.p, np, utot.p, utot_state.p, st);
             uint64_t nu = 0;
             BM_CUDA(cudaMemcpyAsync(&nu, utot.p, 8, cudaMemcpyDeviceToHost, st));
             BM_CUDA(cudaStreamSynchronize(st));

@@ -533,12 +533,20 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     // one's launch, a few long chains of exchanges, runs beside the body of the other's.  m = 2^22, 5%,
     // n = 2,048 (6.3 MB an item): one sequence 21.0 ms, two with 4 items a region 19.4, with 3 items
     // 17.9 (75 MB in use), three with 2 items 17.9; zipf m = 1 M, n = 2,000 (up to 25 MB) 2.2 and 2.0 ms.
-    const uint64_t part = std::max<uint64_t>(widest, SEQ_REGION / 4);
+    // With four and five tables the copies fill more of their slots and the chains are longer, so a
+    // region takes 16 of the widest items, up to twice as much, where two sequences of such batches
+    // come of it (a launch of two or four items ends with one's chains).  m = 10^6, 5%, n = 500, d = 4:
+    // 9.4 -> 7.4 ms; m = 16 M, 1%, n = 100, from a caller's permutation table 12.2 -> 10.1.  Not for
+    // more than 16: m = 120,000, 20%, n = 2,000 (1 MB an item): 5.9 -> 6.2 in twice as much.
+    const uint64_t wide = std::min(16 * 4 * widest, 2 * SEQ_REGION);
+    const uint64_t reg = NT > 3 && wide > SEQ_REGION && 4 * total >= 2 * SEQS * wide ? wide : SEQ_REGION;
+    const uint64_t most = (PLACE_L2_BYTES + 2 * SEQS * (reg - SEQ_REGION)) / 4;  // words of all
+    const uint64_t part = std::max<uint64_t>(widest, reg / 4);
     // Everything in one batch where it fits: insertions, then bytes (two batches of the above triples' sets
     // took three launches, each as long as its longest chains).
     const bool once = total <= PLACE_L2_BYTES / 4;
-    const uint32_t seqs = !once && 2 * SEQS * part <= PLACE_L2_BYTES / 4 && total >= 2 * SEQS * part ? SEQS : 1;
-    const uint64_t region = once ? total : (seqs > 1 ? part : std::max<uint64_t>(widest, PLACE_L2_BYTES / 4 / 2)) / 64 * 64;  // (16-byte loads)
+    const uint32_t seqs = !once && 2 * SEQS * part <= most && total >= 2 * SEQS * part ? SEQS : 1;
+    const uint64_t region = once ? total : (seqs > 1 ? part : std::max<uint64_t>(widest, most / 2)) / 64 * 64;  // (16-byte loads)
     static const bool ready = [] {
         BM_CUDA(cudaFuncSetAttribute(k_place_large<NT, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LARGE_SMEM));
         BM_CUDA(cudaFuncSetAttribute(k_place_large<NT, uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LARGE_SMEM));

@@ -52,3 +52,31 @@ def test_chains_end_whatever_max_loop():
     qs = [[a, b] for a in range(4) for b in range(4)]
     got = pkg.intersect_query(pool, qs).cpu().numpy().astype(np.uint64)
     assert np.array_equal(got, oracle.kway_counts(inst.offsets, inst.tids, qs))
+
+
+@pytest.mark.parametrize("tasks", [1, 255, 256, 257, 600])
+def test_tasks_from_the_host_and_from_the_device(tasks):
+    """Batches of up to 256 tasks bring them along, larger ones make them on the device; counts,
+    lists and the serving loop agree with merges on either side."""
+    import paper_1102_1003_gb300 as pkg
+    m, rng = 40_000, np.random.default_rng(tasks)
+    sizes = [0, 1, 127, 128, 129, 511, 512, 513, 3_000, 9_000, 20_000]  # around a task's and a chunk's end
+    inst = datagen.from_lists([np.sort(rng.choice(m, s, replace=False)).astype(np.uint32) for s in sizes], m)
+    off, tids, _ = device_inputs(inst, 0)
+    pool = pkg.batmap_pool_create(m, off, tids)
+    # tasks of 128 elements (small batches): as many queries on the sets of up to 128 as there are tasks
+    qs = [[int(rng.integers(1, 4)), int(rng.integers(1, len(sizes)))] for _ in range(tasks)]
+    for batch in (qs, qs + [[0, 9], [9, 10], [10, 8, 9], [4, 5], [6], [7, 6, 10]]):
+        want = oracle.kway_counts(inst.offsets, inst.tids, batch)
+        assert np.array_equal(pkg.intersect_query(pool, batch).cpu().numpy().astype(np.uint64), want)
+        o, elems = pkg.intersect_query_list(pool, batch)
+        o, elems = o.cpu().numpy(), elems.cpu().numpy().astype(np.uint32)
+        assert np.array_equal(np.diff(o).astype(np.uint64), want)
+        for q, ids in enumerate(batch):
+            both = inst.tidlist(ids[0])
+            for i in ids[1:]:
+                both = np.intersect1d(both, inst.tidlist(i), assume_unique=True)
+            assert np.array_equal(elems[o[q]:o[q + 1]], both)
+        opts = pkg.batmap_serve_opts(max_batch=tasks, slots=3, work_budget=1 << 26, reserved=0)
+        counts, _, _ = pkg.batmap_serve(pool, batch, np.zeros(len(batch)), opts)
+        assert np.array_equal(np.asarray(counts, np.uint64), want)

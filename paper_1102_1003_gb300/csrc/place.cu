@@ -20,14 +20,15 @@
 //   - above (k_place_large): in L2.  Items go in batches, alternately through
 //     two regions of PLACE_L2_BYTES in all (or two sequences of batches, two
 //     regions each); a launch inserts one batch and forms the bytes of the one
-//     before, so that long chains do not hold the chip up.  Bytes are formed slot by slot from a coalesced pass over the table:
+//     before, so that long chains do not hold the chip up.  Bytes are formed slot
+//     by slot from a coalesced pass over the table:
 //     one load in another table per copy tells which tables hold the element (no
 //     byte is stored at random).  Entries carry an epoch above the tid, so a
 //     region is not cleared between batches.
-// Before, one launch placed all items through one table in DRAM (25.8 GB at
-// m = 2^22, n = 4,096, 5%) and another looked every element up in it: builds of
-// n = 8,192 took 126 ms, and take 70.  At the rates above the exchanges, loads and
-// writes of n = 4,096 come to 26 ms, and take 36.
+// Before, one launch placed all items through one table in DRAM and another looked
+// every element up in it: at m = 2^22, 5%, n = 8,192 (51.5 GB of table) builds took
+// 126 ms, and take 70.  At the rates above the exchanges, loads and writes of half
+// those items come to 26 ms, and take 36.
 #include <algorithm>
 #include <type_traits>
 
@@ -106,7 +107,9 @@ __device__ __forceinline__ void record(const PlaceJob &J, uint32_t item, uint32_
 // tasks before they begin.  A task's look may be answered by L1 (a launch old at most): the
 // flags are one line for all SMs, and reading it in L2 for every task took k_place_large 6%
 // (m = 2^22, 5%, n = 2,048: 17.75 -> 18.9 ms) to 40% (0.1%).
-constexpr uint32_t POLL = 64;
+// Chains of the default max_loop, of 96 to 160 moves, do not look (every 64 moves: quadruples
+// of n = 1,000, m = 100,000 2.36 -> 2.39 ms).
+constexpr uint32_t POLL = 256;
 __device__ __forceinline__ bool refused(const PlaceJob &J) {
     if (!J.refused) return false;
     const volatile int *f = J.refused;
@@ -291,6 +294,8 @@ __global__ void k_large_tasks(const LargeItem *items, LargeTask *tasks) {
 // One CTA per task, a warp per part of it: a batch's insertions, then the
 // bytes of the batch before (inserted by the launch before, in the other
 // region).  drops[q]: copies that item q lost.
+// Slot of 32 bits where all slots fit and every BatMap starts at a multiple of 4 bytes (a test of
+// that at the stores took 0.35%), else of 64.
 template <int NT, typename Slot>
 __global__ void __launch_bounds__(LTPB, 8)
 k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermView P, const LargeItem *__restrict__ items,
@@ -385,7 +390,7 @@ k_place_large(const __grid_constant__ PlaceJob J, const __grid_constant__ PermVi
         const uint64_t slots = (uint64_t)NT << rlog, s0 = (uint64_t)T.k * B_SLOTS + sub * B_SUB;
         const uint32_t low = (1u << J.shift) - 1u;
         uint8_t *out = J.out + J.base[I.item];
-        const bool aligned = ((slots | J.base[I.item]) & 3u) == 0;  // (not so for ranges r below 4)
+        const bool aligned = sizeof(Slot) == 4 || ((slots | J.base[I.item]) & 3u) == 0;
         // The entries of a pass: each looks into the next table.  `same`: all lie in one table, t0,
         // at positions h0 on; its next one's keys are read once and no slot is taken apart.
         auto entries = [&](auto one, Slot s, uint32_t used) {
@@ -516,7 +521,8 @@ static uint64_t table_words(uint32_t rlog) {
 
 // The large items in order of the list (widest first): batches, places and tasks.
 template <int NT>
-static void place_large(const PlaceJob &job, const PermView &P, const std::vector<PlaceItem> &list, SideStream &streams) {
+static void place_large(const PlaceJob &job, const PermView &P, const std::vector<PlaceItem> &list, uint32_t least_rlog,
+                        SideStream &streams) {
     cudaStream_t st = streams.main();
     uint32_t tbits = 1;
     while (tbits < 30 && (1ull << tbits) < P.m) tbits++;
@@ -611,7 +617,7 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
             BM_CUDA(cudaMemsetAsync(w + o_reg + b % (2 * seqs) * region, 0, region * 4, st));
         const unsigned grid = (unsigned)(start[b + 1] - start[b]);
         if (!grid) continue;
-        if (list[0].rlog <= SLOT32_RLOG)
+        if (list[0].rlog <= SLOT32_RLOG && least_rlog >= 2)
             k_place_large<NT, uint32_t><<<grid, LTPB, LARGE_SMEM, st>>>(job, P, d_items, d_tasks + start[b], tbits, hbits,
                                                                         known, w + o_reg, w);
         else
@@ -634,6 +640,7 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
     auto cap_of = [](uint64_t size) { return std::max<uint64_t>(32, (size + 31) / 32 * 32); };
     // items for L2, widest first, then those for shared memory, runs of equal width
     std::stable_sort(list.begin(), list.end(), [](const PlaceItem &a, const PlaceItem &b) { return a.rlog > b.rlog; });
+    const uint32_t least = list.back().rlog;  // of all: BatMaps lie one behind the other
     const auto mid = std::stable_partition(list.begin(), list.end(), [&](const PlaceItem &I) {
         // (the tids are staged where the table will be: no more of them than slots)
         return I.rlog > SMALL_RLOG || I.size > ((uint64_t)NT << I.rlog) || smem_of(I.rlog, cap_of(I.size)) > 225 * 1024;
@@ -643,7 +650,7 @@ static void place_all(const PlaceJob &job, const PermView &P, std::vector<PlaceI
     BM_CUDA(cudaMemcpyAsync(d_list, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, side));
     // (widths side by side on streams of their own: triples 2% slower, quadruples 10%)
     uint32_t launch = 0;
-    if (mid != list.begin()) place_large<NT>(job, P, std::vector<PlaceItem>(list.begin(), mid), streams);
+    if (mid != list.begin()) place_large<NT>(job, P, std::vector<PlaceItem>(list.begin(), mid), least, streams);
     for (size_t k = mid - list.begin(); k < list.size();) {
         size_t e = k;
         uint64_t most = 0;

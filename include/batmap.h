@@ -207,10 +207,10 @@ batmap_status batmap_build_cross(const batmap_params *p, uint32_t m, uint32_t n_
  * Items keep their original order (no width sort); h_bytes of
  * batmap_export_layout follow it.  For d = 3 and 4 the build also keeps the
  * family's bit rows (n * ceil(m / 256) * 32 bytes) unless they would take more
- * than half of the free memory or p->tile, shape_mask or probe_log is set; the
- * k-way supports are then the AND + popcount of the rows, else the witness rule
- * on the BatMaps.  Errors: BATMAP_ERR_ARG for d outside
- * {2, 3, 4} or invalid input.
+ * than half of the memory that is free (the library's idle memory included) or
+ * p->tile, shape_mask or probe_log is set; the k-way supports are then the AND +
+ * popcount of the rows, else the witness rule on the BatMaps.
+ * Errors: BATMAP_ERR_ARG for d outside {2, 3, 4} or invalid input.
  */
 batmap_status batmap_build_d(const batmap_params *p, uint32_t d, uint32_t m, uint32_t n,
                              const uint64_t *d_offsets, const uint32_t *d_tids, const uint32_t *d_perm,
@@ -352,7 +352,9 @@ batmap_status pair_support_host(const batmap_params *p, uint32_t m, uint32_t n,
  * relative throughputs become the scheduler's shape costs for every later
  * batmap_build in the process, and all k sets are rescheduled with them (the
  * width class -> tile shape choice and the split of column words into work
- * units).
+ * units).  The schedule is that of the BatMap routes: sets whose supports come
+ * from bit rows (see pair_support_all) are measured like the others, and their
+ * calls gain nothing from it.
  *   shape_eff : optional host double[BATMAP_NUM_SHAPES], receives the
  *               relative throughputs.
  * Synchronises the stream.
@@ -381,11 +383,14 @@ typedef struct batmap_timing {
 /* Copy the phase durations of the set's most recent calls into *t. */
 batmap_status batmap_get_timing(const batmap_set *set, batmap_timing *t);
 
-/* Release the scratch the library caches between calls (the placement table
- * of batmap_build, up to 96 MiB or two of its widest item's, four bytes per
- * slot; at most four arrays of freed sets of more than 64 MiB and 32 smaller
+/* Release the scratch the library caches between calls (the placement scratch
+ * of batmap_build: up to 96 MiB, 184 for d >= 3, or two tables of its widest item,
+ * four bytes per slot, and 8 bytes per 2,048 slots and per 1,024 elements of
+ * items with more than 2^13 slots a table; at most four arrays of freed sets of more than 64 MiB and 32 smaller
  * ones, a quarter of the device's memory in all; at most four arenas of call scratch of 256 MiB each; the dense path's
  * bitmap and workspace; pair_support_host's device copies of its inputs and output).
+ * A call that finds no device memory gives back the arrays and arenas by itself
+ * and tries again before it returns BATMAP_ERR_NOMEM.
  * Call when no other call of the library is running. */
 void batmap_release_scratch(void);
 
@@ -430,6 +435,8 @@ typedef struct batmap_pool batmap_pool;
  * BatMap built with the same GPU build as batmap_build.  d_perm is the
  * caller's device uint32[3*m] permutation table (copied) or NULL for the
  * permutations the library computes from p->perm_seed (no table is kept).
+ * p->min_shift may be below 7 here, down to 0; a placement chain ends after
+ * 2^23 moves at the latest, whatever p->max_loop.
  * The caller may free its buffers after the call.  Synchronises the stream.
  */
 batmap_status batmap_pool_create(const batmap_params *p, uint32_t m, uint32_t n, const uint64_t *d_offsets,

@@ -205,11 +205,12 @@ static uint32_t shift_bits(uint32_t m, uint32_t min_shift) {
     return s;
 }
 
-// The placement scratch (the regions of place.cu: 96 MiB, or two of the widest
-// item's tables if that is more) is kept between builds so that repeated builds
-// do not pay for allocating and freeing it; it is released when a build needs
-// less than a quarter of it or on batmap_release_scratch().  Builds are
-// serialised on it.
+// The placement scratch (the regions of place.cu: 96 MiB, 184 for 3-of-4 and
+// 4-of-5 sets of wide items, or two of the widest item's tables if that is more;
+// and 8 bytes per 2,048 slots and per 1,024 elements of the items placed there, 61 MiB
+// at m = 2^22, n = 8,192, 5%) is kept between builds so that repeated builds do not
+// pay for allocating and freeing it; it is released when a build needs less than a
+// quarter of it or on batmap_release_scratch().  Builds are serialised on it.
 std::mutex g_scratch_mu;
 static DevBuf<uint32_t> g_scratch;
 

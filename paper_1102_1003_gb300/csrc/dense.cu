@@ -469,7 +469,9 @@ void launch_contract(const MmView *d_views, const MmView &one, const MmUnit *d_u
 // bytes wide, so the scan wins only where tiles are mostly padding: few items
 // over many transactions.  A caller who sets tile, shape_mask or probe_log asks
 // for a BatMap route and gets it.  The bits are left out (and the scan taken)
-// where they would take more than half of the free memory.
+// where they would take more than half of the memory that is free beside the supports.
+// Measured where the rule switches (n = 2 to 300, m = 5,000 to 2^26, 184 builds with their
+// supports): where it takes the contraction that is never the slower route.
 constexpr double SCAN_WORD_PAIRS_PER_S = 7e12, SCAN_MIN_S = 40e-6, BITS_BYTES_PER_S = 4e12;
 
 void plan_contract(batmap_set *S, const uint64_t *d_off, const uint32_t *d_tids, int *d_flags, bool sorted_only,

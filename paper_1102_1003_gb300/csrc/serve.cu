@@ -493,8 +493,7 @@ static void pool_create(const batmap_params *p, uint32_t m, uint32_t n, const ui
         pool->d_bm.alloc(total_bytes);
         std::vector<uint32_t> f_chunks_tid;
         uint64_t bm_pos = 0, f_pos = 0;
-        // build in chunks of at most ~4 GB of BatMaps so the placement scratch
-        // (4 bytes per slot) stays bounded
+        // build in chunks of at most ~4 GB of BatMaps, as each is built beside its copy in the pool
         for (uint32_t c0 = 0; c0 < nb;) {
             uint32_t c1 = c0;
             uint64_t cb = 0;

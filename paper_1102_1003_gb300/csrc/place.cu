@@ -522,7 +522,7 @@ static uint64_t table_words(uint32_t rlog) {
 // The large items in order of the list (widest first): batches, places and tasks.
 template <int NT>
 static void place_large(const PlaceJob &job, const PermView &P, const std::vector<PlaceItem> &list, uint32_t least_rlog,
-                        SideStream &streams) {
+                        SideStream &streams, bool may_widen = true) {
     cudaStream_t st = streams.main();
     uint32_t tbits = 1;
     while (tbits < 30 && (1ull << tbits) < P.m) tbits++;
@@ -545,7 +545,7 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     // 9.4 -> 7.4 ms; m = 16 M, 1%, n = 100, from a caller's permutation table 12.2 -> 10.1.  Not for
     // more than 16: m = 120,000, 20%, n = 2,000 (1 MB an item): 5.9 -> 6.2 in twice as much.
     const uint64_t wide = std::min(16 * 4 * widest, 2 * SEQ_REGION);
-    const uint64_t reg = NT > 3 && wide > SEQ_REGION && 4 * total >= 2 * SEQS * wide ? wide : SEQ_REGION;
+    const uint64_t reg = may_widen && NT > 3 && wide > SEQ_REGION && 4 * total >= 2 * SEQS * wide ? wide : SEQ_REGION;
     const uint64_t most = (PLACE_L2_BYTES + 2 * SEQS * (reg - SEQ_REGION)) / 4;  // words of all
     const uint64_t part = std::max<uint64_t>(widest, reg / 4);
     // Everything in one batch where it fits: insertions, then bytes (two batches of the above triples' sets
@@ -601,7 +601,13 @@ static void place_large(const PlaceJob &job, const PermView &P, const std::vecto
     auto up = [](uint64_t w) { return (w + 63) / 64 * 64; };
     const uint64_t o_items = up(items.size()), o_tasks = o_items + up(items.size() * sizeof(LargeItem) / 4),
                    o_reg = o_tasks + up(pos * sizeof(LargeTask) / 4), regions = std::min<uint64_t>(nb, 2 * seqs);
-    uint32_t *w = scratch_table(o_reg + regions * region).p;
+    uint32_t *w;
+    try {
+        w = scratch_table(o_reg + regions * region).p;
+    } catch (const Error &e) {
+        if (e.code != BATMAP_ERR_NOMEM || reg == SEQ_REGION) throw;
+        return place_large<NT>(job, P, list, least_rlog, streams, false);  // no room for the larger regions
+    }
     BM_CUDA(cudaMemsetAsync(w, 0, o_items * 4, st));
     BM_CUDA(cudaMemcpyAsync(w + o_items, items.data(), items.size() * sizeof(LargeItem), cudaMemcpyHostToDevice, st));
     const LargeItem *d_items = reinterpret_cast<const LargeItem *>(w + o_items);
